@@ -111,6 +111,15 @@ int64_t tree_nodes(const Tree& T) {
   return T.nlevels ? T.offset[T.nlevels - 1] + T.count[T.nlevels - 1] : 0;
 }
 
+// the linear records of `nodes` nodes inside one buffer
+constexpr size_t kLinBytes = 3 * sizeof(float4) + sizeof(float);
+void lin_layout(Tree& T, void* buf, int64_t nodes) {
+  T.ln0 = static_cast<float4*>(buf);
+  T.ln1 = T.ln0 + nodes;
+  T.ln2 = T.ln1 + nodes;
+  T.ln3 = reinterpret_cast<float*>(T.ln2 + nodes);
+}
+
 #define GFS_CK(expr)                         \
   do {                                       \
     cudaError_t e_ = (expr);                 \
@@ -138,7 +147,7 @@ struct gfs_ctx {
   bool built = false;
   DevBuf sph64, keys_in, keys_out, vals_in, vals_out, sph, thr, sid, bound_bits, consts, cnt, cub_temp;
   Tree st{};
-  DevBuf st_lo, st_hi, st_na, st_nb, st_nf;
+  DevBuf st_lo, st_hi, st_na, st_nb, st_nf, st_ln;
   DevBuf st_tight;  // scratch of the internal-ball tightening
   // survivors
   DevBuf surv_raw[2], surv_sorted[2], vt_lo[2], vt_hi[2];
@@ -171,7 +180,7 @@ struct gfs_ctx {
   std::vector<int64_t> b_off, b_qoff, b_soff[2];
   std::vector<Tree> b_st;
   DevBuf b_desc, b_offd, b_qoffd, b_sph64, b_k64in, b_k64out, b_sph, b_thr, b_sid, b_bits, b_bcs;
-  DevBuf b_lo, b_hi, b_na, b_nb, b_nf, b_stdev, b_prefix, b_ctr, b_cnt, b_cviews, b_cw;
+  DevBuf b_lo, b_hi, b_na, b_nb, b_nf, b_ln, b_stdev, b_prefix, b_ctr, b_cnt, b_cviews, b_cw;
   DevBuf b_sraw[2], b_sshape[2], b_ssorted[2], b_vlo[2], b_vhi[2], b_vtdev[2], b_hist;
   DevBuf b_qkin, b_qkout, b_qvin, b_qvout, b_qviews, b_qw, b_qstate;
   std::vector<QueryArgs> b_qv;  // host copies of the per-shape query views
@@ -307,6 +316,8 @@ int build_sphere_hierarchy(gfs_ctx* c, int64_t n, const int* ids = nullptr) {
   c->st.na = c->st_na.as<float4>();
   c->st.nb = c->st_nb.as<float4>();
   c->st.nf = c->st_nf.as<float4>();
+  GFS_TRY(ensure(c->st_ln, size_t(nodes) * kLinBytes));
+  lin_layout(c->st, c->st_ln.p, nodes);
   // the coordinate bound A is needed on the host for the hierarchy's rounding slack
   unsigned int bits[2] = {0, 0};
   GFS_CK(cudaMemcpyAsync(bits, c->bound_bits.p, 8, cudaMemcpyDeviceToHost, st));
@@ -314,7 +325,7 @@ int build_sphere_hierarchy(gfs_ctx* c, int64_t n, const int* ids = nullptr) {
   float Ahost;
   std::memcpy(&Ahost, &bits[0], 4);
   Ahost = std::max(1.0f, Ahost);
-  GFS_TRY(ensure(c->st_tight, size_t(std::max<int64_t>(nodes - c->st.count[0], 1)) * 4 * sizeof(unsigned)));
+  GFS_TRY(ensure(c->st_tight, size_t(std::max<int64_t>(nodes - c->st.count[0], 1)) * 8 * sizeof(unsigned)));
   GFS_CK(launch_build_tree(c->sph.as<float4>(), 1, Ahost, c->st, c->st_tight.as<unsigned>(), st));
   return GFS_OK;
 }
@@ -546,6 +557,8 @@ int gfs_query(gfs_ctx* c, const void* x, int x_is_fp32, int64_t m, float* s_out,
   GFS_CK(cudaMemsetAsync(reinterpret_cast<char*>(c->cnt.p) + offsetof(Counters, q_sphere_ntests), 0,
                          5 * sizeof(unsigned long long), c->stream));
   GFS_CK(cudaMemsetAsync(reinterpret_cast<char*>(c->cnt.p) + offsetof(Counters, ndefer), 0, sizeof(unsigned int),
+                         c->stream));
+  GFS_CK(cudaMemsetAsync(reinterpret_cast<char*>(c->cnt.p) + offsetof(Counters, q_split), 0, 2 * sizeof(unsigned int),
                          c->stream));
   if (c->have_ev) GFS_CK(cudaEventRecord(c->ev[4], c->stream));
   if (c->opt.precision == 0) {
@@ -1403,6 +1416,18 @@ int gfs_batch_build(gfs_ctx* c, const gfs_shape* shapes, int ns) {
   GFS_TRY(ensure(c->b_nf, size_t(nodes) * sizeof(float4)));
   forest_layout(c->b_st, nits, c->b_lo.as<float4>(), c->b_hi.as<float4>(), c->b_na.as<float4>(), c->b_nb.as<float4>(),
                 c->b_nf.as<float4>(), maxL);
+  GFS_TRY(ensure(c->b_ln, size_t(nodes) * kLinBytes));
+  {
+    int64_t base = 0;
+    for (Tree& T : c->b_st) {
+      lin_layout(T, c->b_ln.p, nodes);
+      T.ln0 += base;
+      T.ln1 += base;
+      T.ln2 += base;
+      T.ln3 += base;
+      base += tree_nodes(T);
+    }
+  }
   {
     GFS_TRY(ensure(c->b_stdev, size_t(ns) * sizeof(Tree)));
     GFS_CK(cudaMemcpyAsync(c->b_stdev.p, c->b_st.data(), size_t(ns) * sizeof(Tree), cudaMemcpyHostToDevice, st));
@@ -1860,7 +1885,7 @@ void gfs_destroy(gfs_ctx* c) {
   if (c->side) cudaStreamDestroy(c->side);
   DevBuf* bufs[] = {&c->U32, &c->U64, &c->sph64, &c->keys_in, &c->keys_out, &c->vals_in, &c->vals_out, &c->sph,
                     &c->thr, &c->sid, &c->bound_bits, &c->consts, &c->cnt, &c->cub_temp, &c->st_lo, &c->st_hi,
-                    &c->st_na, &c->st_nb, &c->st_nf, &c->st_tight, &c->qstate, &c->surv_raw[0], &c->surv_raw[1], &c->surv_sorted[0], &c->surv_sorted[1],
+                    &c->st_na, &c->st_nb, &c->st_nf, &c->st_ln, &c->st_tight, &c->qstate, &c->surv_raw[0], &c->surv_raw[1], &c->surv_sorted[0], &c->surv_sorted[1],
                     &c->vt_lo[0], &c->vt_lo[1], &c->vt_hi[0], &c->vt_hi[1], &c->defer, &c->acc, &c->witness64,
                     &c->h_p, &c->h_s, &c->h_x, &c->h_sout, &c->h_arg, &c->h_fl,
                     &c->qk_in, &c->qk_out, &c->qv_in, &c->qv_out, &c->ins_counts,
@@ -1871,7 +1896,7 @@ void gfs_destroy(gfs_ctx* c) {
                     &c->csr_off, &c->scored_status, &c->ud_uncov, &c->ud_cnt, &c->ud_pairs, &c->ud_circ,
                     &c->ud_quad, &c->ud_pts, &c->ud_k0, &c->ud_k1, &c->ud_v0, &c->ud_v1,
                     &c->b_desc, &c->b_offd, &c->b_qoffd, &c->b_sph64, &c->b_k64in, &c->b_k64out, &c->b_sph,
-                    &c->b_thr, &c->b_sid, &c->b_bits, &c->b_bcs, &c->b_lo, &c->b_hi, &c->b_na, &c->b_nb, &c->b_nf,
+                    &c->b_thr, &c->b_sid, &c->b_bits, &c->b_bcs, &c->b_lo, &c->b_hi, &c->b_na, &c->b_nb, &c->b_nf, &c->b_ln,
                     &c->b_stdev, &c->b_prefix, &c->b_ctr, &c->b_cnt, &c->b_cviews, &c->b_cw, &c->b_sraw[0],
                     &c->b_sraw[1], &c->b_sshape[0], &c->b_sshape[1], &c->b_ssorted[0], &c->b_ssorted[1],
                     &c->b_vlo[0], &c->b_vlo[1], &c->b_vhi[0], &c->b_vhi[1], &c->b_vtdev[0], &c->b_vtdev[1],

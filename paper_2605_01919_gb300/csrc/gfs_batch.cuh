@@ -88,12 +88,11 @@ __global__ void k_batch_tree_level(const Tree* __restrict__ trees, const int64_t
   const int64_t j = g - prefix[s];
   if (level == 0) {
     const float4* items = items_base + item_off[s];
-    if (is_sphere) sphere_leaf_node(items, T.nitems, bc[s].A, T.lo, T.hi, T.na, T.nb, T.nf, j);
+    if (is_sphere) sphere_leaf_node(items, bc[s].A, T, j);
     else point_leaf_node(items, T.nitems, T.lo, T.hi, j);
   } else {
     if (is_sphere)
-      sphere_level_node(T.lo, T.hi, T.na, T.nb, T.nf, bc[s].A, T.offset[level - 1], T.count[level - 1],
-                        T.offset[level], j);
+      sphere_level_node(T, bc[s].A, level, j);
     else
       point_level_node(T.lo, T.hi, T.offset[level - 1], T.count[level - 1], T.offset[level], j);
   }
@@ -169,9 +168,9 @@ template <int kPhase>
 __global__ void __launch_bounds__(128) k_batch_query(const QueryArgs* __restrict__ views,
                                                      const int64_t* __restrict__ wprefix, int ns, int64_t limit,
                                                      unsigned long long* __restrict__ ctr) {
-  __shared__ uint32_t s_stack[4][kPStack];
+  using Shared = std::conditional_t<kPhase == 1, SpWarp, uint32_t[kPStack]>;
+  __shared__ Shared s_warp[4];
   const int lane = threadIdx.x & 31;
-  WarpStack W{s_stack[threadIdx.x >> 5], 0};
   for (;;) {
     unsigned long long w = 0;
     if (lane == 0) w = atomicAdd(ctr, 1ull);
@@ -179,7 +178,14 @@ __global__ void __launch_bounds__(128) k_batch_query(const QueryArgs* __restrict
     if (int64_t(w) >= limit) break;
     const int s = find_seg(wprefix, ns, int64_t(w));
     const int64_t wl = int64_t(w) - wprefix[s];
-    query_packet<true, kPhase>(views[s], wl * 32 + lane, W, lane);
+    if constexpr (kPhase == 1) {
+#pragma unroll 1
+      for (int g = 0; g < 32; g += 8)
+        if (wl * 32 + g < views[s].m) sphere_pass_any(views[s], wl * 32 + g, s_warp[threadIdx.x >> 5], lane);
+    } else {
+      WarpStack W{s_warp[threadIdx.x >> 5], 0};
+      query_packet<true>(views[s], wl * 32 + lane, W, lane);
+    }
   }
 }
 
@@ -266,6 +272,8 @@ __global__ void k_batch_surv_layout(const unsigned* __restrict__ counts, int ns,
     T.lo = lo + base;
     T.hi = hi + base;
     T.na = T.nb = T.nf = nullptr;
+    T.ln0 = T.ln1 = T.ln2 = nullptr;
+    T.ln3 = nullptr;
     trees[s] = T;
     for (int l = 0; l < nlev; ++l) {
       int64_t* P = prefix + int64_t(l) * (ns + 1);

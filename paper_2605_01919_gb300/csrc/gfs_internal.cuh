@@ -43,7 +43,39 @@ struct Tree {
   float4* na;                     // sphere trees: (C, max(wp, wn))
   float4* nb;                     // sphere trees: (wp, wn, w0, 0)
   float4* nf;                     // sphere trees: (F, wf)
+  // sphere trees: the linear record of a node (struct Lin), 52 B
+  float4* ln0;                    // (c, h.x)
+  float4* ln1;                    // (h.y, h.z, g.x, g.y)
+  float4* ln2;                    // (g.z, hip, lop, lon)
+  float* ln3;                     // hin
 };
+
+// Linear record of a sphere node: its spheres' centres lie in the box c +- h,
+// and their signed values follow the linear function g . (p - c) within
+//   s <= hip + g . (p - c) over s > 0,   s >= lop + g . (p - c) over s >= 0,
+//   s >= lon + g . (p - c) over s < 0,   s <= hin + g . (p - c) over s <= 0
+// (empty sets: hip, hin = -inf, lop, lon = +inf).  With n = (x - c)/|x - c|,
+// D = |x - c| and the box's support S(v) = sum_i |v_i| h_i, a node bounds
+//   |x - p| - |s| >= D - hip - S(n + g)   over s > 0   (|x - p| >= n . (x - p)),
+//   |x - p| - |s| >= D + lon - S(n - g)   over s < 0,
+//   |x - p| + |s| >= min(D + lop - S(n - g), D - hin - S(n + g)).
+// A ball around the node's balls exceeds their reach by the node's extent a;
+// for samples of a distance field (|g| = 1, n + g small on the facing side)
+// this bound exceeds it by a^2 only, which is what keeps the near ties along
+// a surface normal from opening every node beside it.
+struct Lin {
+  float cx, cy, cz, hx, hy, hz, gx, gy, gz, hip, lop, lon, hin;
+};
+__device__ __forceinline__ void lin_store(const Tree& T, int64_t node, const Lin& r) {
+  T.ln0[node] = make_float4(r.cx, r.cy, r.cz, r.hx);
+  T.ln1[node] = make_float4(r.hy, r.hz, r.gx, r.gy);
+  T.ln2[node] = make_float4(r.gz, r.hip, r.lop, r.lon);
+  T.ln3[node] = r.hin;
+}
+__device__ __forceinline__ Lin lin_load(const Tree& T, int64_t node) {
+  const float4 a = T.ln0[node], b = T.ln1[node], c = T.ln2[node];
+  return Lin{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z, c.w, T.ln3[node]};
+}
 
 __host__ __device__ inline uint32_t pack_node(int level, int64_t idx) {
   return (uint32_t(level) << 27) | uint32_t(idx);
@@ -146,6 +178,7 @@ struct BuildConsts {
   float ed_quad;
   float eprune;   // additive slack for FP32 node pruning
   float pad;
+  float elin;     // margin of the linear node bounds (and of sphere values) against the FP32 error bands
 };
 
 struct Counters {
@@ -161,6 +194,7 @@ struct Counters {
   unsigned long long q_surv_items;     // survivors tested by the survivor pass
   unsigned long long c_ntests;         // child-node coverage tests of the cull (open lanes)
   unsigned long long c_items;          // sphere coverage tests of the cull (open lanes)
+  unsigned int q_split, q_split_next;  // packets the sphere pass left to its point-by-point launch, and that launch's cursor
 };
 
 }  // namespace gfs

@@ -19,6 +19,9 @@
 #include <cub/cub.cuh>
 #include <cooperative_groups.h>
 
+#include <algorithm>
+#include <type_traits>
+
 #include "gfs_internal.cuh"
 #include "gfs_kernels.h"
 
@@ -82,6 +85,11 @@ __device__ BuildConsts make_consts(unsigned int amax_bits, unsigned int rmax_bit
   c.eprune = 4.f * s3 * u * A + 1e-7f;
   // the same for candidate points (their FP32 error is eq)
   c.pad = 4.f * s3 * (c.eq + u * A) + 1e-7f;
+  // linear node bounds against a reference sphere's value at another point of
+  // the packet: about 130 u A + 6 u R of FP32 rounding (the record's box and
+  // residuals, |x - c| and the unit vectors, the sums), plus the widest error
+  // band 2 ea, so that whatever they discard also lies outside that band
+  c.elin = u * (300.f * A + 24.f * R) + 1e-11f;
   return c;
 }
 
@@ -256,9 +264,93 @@ __device__ __forceinline__ void store_sphere_node(float4* __restrict__ na, float
   nf[node] = make_float4(Fc.x, Fc.y, Fc.z, wf);
 }
 
-__device__ void sphere_leaf_node(const float4* __restrict__ items, int64_t nitems, float A, float4* __restrict__ lo,
-                                 float4* __restrict__ hi, float4* __restrict__ na, float4* __restrict__ nb,
-                                 float4* __restrict__ nf, int64_t L) {
+// box part of a linear record from the node's (ulp-widened) box
+__device__ __forceinline__ void lin_box(Lin& r, const float4& lo, const float4& hi, float A) {
+  r.cx = 0.5f * (lo.x + hi.x);
+  r.cy = 0.5f * (lo.y + hi.y);
+  r.cz = 0.5f * (lo.z + hi.z);
+  r.hx = 0.5f * (hi.x - lo.x) * (1.f + 8.f * kU) + 4.f * kU * A;
+  r.hy = 0.5f * (hi.y - lo.y) * (1.f + 8.f * kU) + 4.f * kU * A;
+  r.hz = 0.5f * (hi.z - lo.z) * (1.f + 8.f * kU) + 4.f * kU * A;
+  r.hip = r.hin = -INFINITY;
+  r.lop = r.lon = INFINITY;
+}
+
+// Least-squares gradient of k values (it[i].w at it[i]), slightly
+// regularised (planar or coincident points give 0 across them), at most 1 in
+// norm (signed distances are 1-Lipschitz; noise may exceed it).  Any gradient
+// is valid: the residual bounds are taken against it.
+__device__ void lin_fit(const float4* it, int k, Lin& r) {
+  float mx = 0.f, my = 0.f, mz = 0.f, mw = 0.f;
+  for (int i = 0; i < k; ++i) {
+    mx += it[i].x;
+    my += it[i].y;
+    mz += it[i].z;
+    mw += it[i].w;
+  }
+  const float inv = 1.f / float(k);
+  mx *= inv;
+  my *= inv;
+  mz *= inv;
+  mw *= inv;
+  float xx = 0.f, xy = 0.f, xz = 0.f, yy = 0.f, yz = 0.f, zz = 0.f, bx = 0.f, by = 0.f, bz = 0.f;
+  for (int i = 0; i < k; ++i) {
+    const float dx = it[i].x - mx, dy = it[i].y - my, dz = it[i].z - mz, dw = it[i].w - mw;
+    xx += dx * dx;
+    xy += dx * dy;
+    xz += dx * dz;
+    yy += dy * dy;
+    yz += dy * dz;
+    zz += dz * dz;
+    bx += dx * dw;
+    by += dy * dw;
+    bz += dz * dw;
+  }
+  const float tr = xx + yy + zz;
+  r.gx = r.gy = r.gz = 0.f;
+  if (!(tr > 0.f)) return;
+  const float s = 1.f / tr;
+  xx = xx * s + 1e-4f;
+  yy = yy * s + 1e-4f;
+  zz = zz * s + 1e-4f;
+  xy *= s;
+  xz *= s;
+  yz *= s;
+  bx *= s;
+  by *= s;
+  bz *= s;
+  const float c0 = yy * zz - yz * yz, c1 = xz * yz - xy * zz, c2 = xy * yz - xz * yy;
+  const float det = xx * c0 + xy * c1 + xz * c2;
+  const float id = 1.f / det;
+  float gx = (c0 * bx + c1 * by + c2 * bz) * id;
+  float gy = (c1 * bx + (xx * zz - xz * xz) * by + (xy * xz - xx * yz) * bz) * id;
+  float gz = (c2 * bx + (xy * xz - xx * yz) * by + (xx * yy - xy * xy) * bz) * id;
+  const float n2 = gx * gx + gy * gy + gz * gz;
+  if (!(n2 < 1e30f)) return;  // not finite: no gradient
+  const float f = n2 > 1.f ? rsqrtf(n2) : 1.f;
+  r.gx = gx * f;
+  r.gy = gy * f;
+  r.gz = gz * f;
+}
+
+// residual of one sphere against the record's gradient, and the widening of
+// a residual bound for the rounding of its terms and of the FP32 copies
+__device__ __forceinline__ float lin_res(const Lin& r, const float4& P) {
+  return P.w - (r.gx * (P.x - r.cx) + r.gy * (P.y - r.cy) + r.gz * (P.z - r.cz));
+}
+__device__ __forceinline__ float lin_infl(float s, float A) { return 2e-6f * A + 4e-7f * fabsf(s); }
+
+__device__ __forceinline__ void lin_add(Lin& r, const float4& P, float A) {
+  const float v = lin_res(r, P), e = lin_infl(P.w, A);
+  if (P.w > 0.f) r.hip = fmaxf(r.hip, v + e);
+  if (P.w >= 0.f) r.lop = fminf(r.lop, v - e);
+  if (P.w < 0.f) r.lon = fminf(r.lon, v - e);
+  if (P.w <= 0.f) r.hin = fmaxf(r.hin, v + e);
+}
+
+__device__ void sphere_leaf_node(const float4* __restrict__ items, float A, const Tree& T, int64_t L) {
+  float4 *lo = T.lo, *hi = T.hi, *na = T.na, *nb = T.nb, *nf = T.nf;
+  const int64_t nitems = T.nitems;
   int64_t b = L * kLeaf, e = min(b + kLeaf, nitems);
   float4 Ab[kLeaf], Fb[kLeaf];
   int k = 0;
@@ -289,11 +381,17 @@ __device__ void sphere_leaf_node(const float4* __restrict__ items, int64_t nitem
     wf = fmaxf(wf, radius_up(df, df - r, r, pm));
   }
   store_sphere_node(na, nb, nf, L, C, Fc, wp, wn, w0, wf, A);
+  Lin r;
+  lin_box(r, lo[L], hi[L], A);
+  for (int i = 0; i < k; ++i) Ab[i].w = items[b + i].w;
+  lin_fit(Ab, k, r);
+  for (int i = 0; i < k; ++i) lin_add(r, Ab[i], A);
+  lin_store(T, L, r);
 }
 
-__device__ void sphere_level_node(float4* __restrict__ lo, float4* __restrict__ hi, float4* __restrict__ na,
-                                  float4* __restrict__ nb, float4* __restrict__ nf, float A, int64_t child_off,
-                                  int64_t nchild, int64_t off, int64_t j) {
+__device__ void sphere_level_node(const Tree& T, float A, int level, int64_t j) {
+  float4 *lo = T.lo, *hi = T.hi, *na = T.na, *nb = T.nb, *nf = T.nf;
+  const int64_t child_off = T.offset[level - 1], nchild = T.count[level - 1], off = T.offset[level];
   int64_t b = j * kFan, e = min(b + kFan, nchild);
   float4 L = make_float4(INFINITY, INFINITY, INFINITY, 0.f), H = make_float4(-INFINITY, -INFINITY, -INFINITY, 0.f);
   float4 Ab[kFan], Fb[kFan];
@@ -325,13 +423,34 @@ __device__ void sphere_level_node(float4* __restrict__ lo, float4* __restrict__ 
     wf = fmaxf(wf, radius_up(df, df + cf.w, 0.f, 0.f));
   }
   store_sphere_node(na, nb, nf, off + j, C, Fc, wp, wn, w0, wf, A);
+  // linear record: the gradient from the children's mid values at their box
+  // centres, the residual bounds through the children
+  // (s - g.(p - c) = s - g_k.(p - c_k) - g.(c_k - c) + (g_k - g).(p - c_k))
+  Lin r;
+  lin_box(r, L, H, A);
+  for (int64_t c = b; c < e; ++c) {
+    const Lin q = lin_load(T, child_off + c);
+    const float hi_k = fmaxf(q.hip, q.hin), lo_k = fminf(q.lop, q.lon);
+    const float v = hi_k > -INFINITY ? 0.5f * (hi_k + lo_k) : 0.f;
+    Ab[c - b] = make_float4(q.cx, q.cy, q.cz, v);
+  }
+  lin_fit(Ab, k, r);
+  for (int64_t c = b; c < e; ++c) {
+    const Lin q = lin_load(T, child_off + c);
+    const float sh = r.gx * (q.cx - r.cx) + r.gy * (q.cy - r.cy) + r.gz * (q.cz - r.cz);
+    const float sp = fabsf(q.gx - r.gx) * q.hx + fabsf(q.gy - r.gy) * q.hy + fabsf(q.gz - r.gz) * q.hz;
+    const float e2 = sp * 1.000001f + 2e-6f * A + 4e-7f * fabsf(sh);
+    if (q.hip > -INFINITY) r.hip = fmaxf(r.hip, q.hip - sh + e2 + 4e-7f * fabsf(q.hip));
+    if (q.hin > -INFINITY) r.hin = fmaxf(r.hin, q.hin - sh + e2 + 4e-7f * fabsf(q.hin));
+    if (q.lop < INFINITY) r.lop = fminf(r.lop, q.lop - sh - e2 - 4e-7f * fabsf(q.lop));
+    if (q.lon < INFINITY) r.lon = fminf(r.lon, q.lon - sh - e2 - 4e-7f * fabsf(q.lon));
+  }
+  lin_store(T, off + j, r);
 }
 
-__global__ void k_sphere_leaves(const float4* __restrict__ items, int64_t nitems, float A, float4* __restrict__ lo,
-                                float4* __restrict__ hi, float4* __restrict__ na, float4* __restrict__ nb,
-                                float4* __restrict__ nf, int64_t nleaves) {
+__global__ void k_sphere_leaves(const float4* __restrict__ items, float A, Tree T) {
   int64_t L = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-  if (L < nleaves) sphere_leaf_node(items, nitems, A, lo, hi, na, nb, nf, L);
+  if (L < T.count[0]) sphere_leaf_node(items, A, T, L);
 }
 
 // items of node j at `level`: [j * span, (j + 1) * span), span = kLeaf * kFan^level
@@ -341,11 +460,9 @@ __host__ __device__ inline int64_t level_span(int level) {
   return span;
 }
 
-__global__ void k_sphere_level(float4* __restrict__ lo, float4* __restrict__ hi, float4* __restrict__ na,
-                               float4* __restrict__ nb, float4* __restrict__ nf, float A, int64_t child_off,
-                               int64_t nchild, int64_t off, int64_t nnode) {
+__global__ void k_sphere_level(float A, Tree T, int level) {
   int64_t j = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-  if (j < nnode) sphere_level_node(lo, hi, na, nb, nf, A, child_off, nchild, off, j);
+  if (j < T.count[level]) sphere_level_node(T, A, level, j);
 }
 
 // order-preserving map of floats onto unsigned integers (for atomicMax)
@@ -361,7 +478,8 @@ __device__ __forceinline__ float ord_val(unsigned k) {
 // level >= 1 it evaluates its sphere against the node's centre (a node's
 // spheres are a contiguous range of the Morton order) and raises the node's
 // per-radius maximum (same rounding bounds as the leaves).
-__global__ void k_tighten_items(const float4* __restrict__ items, Tree T, unsigned* __restrict__ keys) {
+constexpr int kTight = 8;  // words per node: the four radii, then hip, -lop, -lon, hin
+__global__ void k_tighten_items(const float4* __restrict__ items, Tree T, float A, unsigned* __restrict__ keys) {
   const int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
   const bool live = i < T.nitems;
   const int lane = threadIdx.x & 31;
@@ -372,7 +490,9 @@ __global__ void k_tighten_items(const float4* __restrict__ items, Tree T, unsign
     // a level-l node spans >= 64 consecutive spheres, so the 32 threads of a
     // warp (32 aligned consecutive spheres) share it
     const int64_t node = T.offset[l] + (live ? i / level_span(l) : 0);
-    float m[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+    float m[kTight];
+#pragma unroll
+    for (int q = 0; q < kTight; ++q) m[q] = -INFINITY;
     if (live) {
       const float4 C = T.na[node], Fc = T.nf[node];
       float dx = v.x - C.x, dy = v.y - C.y, dz = v.z - C.z;
@@ -383,13 +503,20 @@ __global__ void k_tighten_items(const float4* __restrict__ items, Tree T, unsign
       dx = v.x - Fc.x, dy = v.y - Fc.y, dz = v.z - Fc.z;
       const float df = sqrtf(dx * dx + dy * dy + dz * dz);
       m[3] = radius_up(df, df - r, r, pm);
+      Lin L = lin_load(T, node);
+      L.hip = L.hin = -INFINITY;
+      L.lop = L.lon = INFINITY;
+      lin_add(L, v, A);
+      m[4] = L.hip;
+      m[5] = -L.lop;
+      m[6] = -L.lon;
+      m[7] = L.hin;
     }
-    for (int q = 0; q < 4; ++q)
-      for (int o = 16; o > 0; o >>= 1) m[q] = fmaxf(m[q], __shfl_xor_sync(0xffffffffu, m[q], o));
-    if (lane == 0 && live) {
-      const int64_t slot = 4 * (node - T.offset[1]);
-      for (int q = 0; q < 4; ++q)
-        if (m[q] > -INFINITY) atomicMax(keys + slot + q, ord_key(m[q]));
+#pragma unroll
+    for (int q = 0; q < kTight; ++q) {
+      // (fmaxf drops a NaN)
+      const unsigned w = __reduce_max_sync(0xffffffffu, ord_key(fmaxf(m[q], -INFINITY)));
+      if (lane == 0 && live && w > ord_key(-INFINITY)) atomicMax(keys + kTight * (node - T.offset[1]) + q, w);
     }
   }
 }
@@ -404,8 +531,17 @@ __global__ void k_tighten_nodes(Tree T, const unsigned* __restrict__ keys, float
   float4 Fc = T.nf[node];
   float w[4] = {B.x, B.y, B.z, Fc.w};
   for (int q = 0; q < 4; ++q) {
-    const unsigned k = keys[4 * t + q];
+    const unsigned k = keys[kTight * t + q];
     if (k != 0u) w[q] = fminf(w[q], radius_fin(ord_val(k), A));
+  }
+  {
+    Lin r = lin_load(T, node);
+    const unsigned* k = keys + kTight * t + 4;
+    if (k[0] != 0u) r.hip = fminf(r.hip, ord_val(k[0]));
+    if (k[1] != 0u) r.lop = fmaxf(r.lop, -ord_val(k[1]));
+    if (k[2] != 0u) r.lon = fmaxf(r.lon, -ord_val(k[2]));
+    if (k[3] != 0u) r.hin = fminf(r.hin, ord_val(k[3]));
+    lin_store(T, node, r);
   }
   T.nb[node] = make_float4(w[0], w[1], w[2], 0.f);
   Fc.w = w[3];
@@ -700,7 +836,7 @@ __device__ __forceinline__ void top2_init(Top2& t) {
 }
 __device__ __forceinline__ void top2_push(Top2& t, float v, int j) {
   if (v < t.best) {
-    t.sec = t.best;
+    t.sec = fminf(t.sec, t.best);  // sec may hold a seeded threshold before the first push
     t.best = v;
     t.idx = j;
   } else if (v < t.sec) {
@@ -911,10 +1047,13 @@ __device__ __forceinline__ void load_qstate(const uint4* st, int64_t slot, bool&
   c1 = (u2.z & 2u) != 0;
 }
 
-// kPhase 0: the whole query; 1: the sphere pass only, its state stored in
-// a.state; 2: the rest, starting from a.state (phase 1 must have run on the
+}  // namespace gfs
+#include "gfs_sphere_pass.cuh"
+namespace gfs {
+
+// The rest of the query, starting from the sphere pass's state (a.state; the
 // same points in the same order).
-template <bool kInlineExact, int kPhase = 0>
+template <bool kInlineExact>
 __device__ void query_packet(const QueryArgs& a, int64_t slot, WarpStack& W, int lane) {
   const bool active = slot < a.m;
   const int64_t q = active ? int64_t(a.perm ? a.perm[slot] : uint32_t(slot)) : 0;
@@ -922,12 +1061,11 @@ __device__ void query_packet(const QueryArgs& a, int64_t slot, WarpStack& W, int
   double x64 = 0.0, y64 = 0.0, z64 = 0.0;
   if (active) load_query(a, q, x64, y64, z64);
   const float x = float(x64), y = float(y64), z = float(z64);
-  unsigned rechecks = 0, n_nodes = 0, n_items = 0, n_snodes = 0, n_sitems = 0, n_band = 0;
+  unsigned n_snodes = 0, n_sitems = 0, n_band = 0;
   bool defer = active && !(fabs(x64) <= bc.A && fabs(y64) <= bc.A && fabs(z64) <= bc.A);
   bool live = active && !defer;
   const float grow = 1.f + 8.f * kU;
   const float ea2 = 2.f * bc.ea;
-  const float negtol = -a.tol32 + ea2;
   // warp centre, used to order children (nearest first)
   float cx = live ? x : 0.f, cy = live ? y : 0.f, cz = live ? z : 0.f;
   float cnt = live ? 1.f : 0.f;
@@ -942,116 +1080,15 @@ __device__ void query_packet(const QueryArgs& a, int64_t slot, WarpStack& W, int
     cy /= cnt;
     cz /= cnt;
   }
-  // ---- pass over the spheres -------------------------------------------
-  // per-class state as scalars (the class of an item is uniform across the
-  // warp, so branching on it costs nothing; indexing a register array with
-  // it would push the array to local memory)
+  // ---- the sphere pass's results (per-class state as scalars: indexing a
+  // register array would push it to local memory)
   bool cov0 = false, cov1 = false;
   Top2 A0, A1, F;
   top2_init(A0);
   top2_init(A1);
   top2_init(F);
   int sample = INT_MAX;
-  if constexpr (kPhase == 2) {
-    if (active) load_qstate(a.state, slot, cov0, cov1, sample, A0, A1, F);
-  } else if (__any_sync(kFull, live)) {
-    const Tree& T = a.st;
-    auto leaf_items = [&](int64_t idx) {
-        const int64_t b = idx * kLeaf, e = min(b + kLeaf, a.n);
-        n_items += live ? unsigned(e - b) : 0u;
-        for (int64_t j = b; j < e; ++j) {
-          const float4 P = a.sph[j];
-          if (!live) continue;
-          const float dx = x - P.x, dy = y - P.y, dz = z - P.z;
-          const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-          if (d2 == 0.f) {
-            const int o = a.sid[j];
-            const D4 pj = a.sph64[o];
-            if (pj.x == x64 && pj.y == y64 && pj.z == z64 && o < sample) sample = o;
-          }
-          const float r = fabsf(P.w);
-          auto class_item = [&](bool& cv, Top2& Ac) {
-            if (!cv) {
-              const float4 Th = a.thr[j];
-              if (d2 < Th.z) {
-                cv = true;
-              } else if (d2 <= Th.w) {
-                ++rechecks;
-                cv = ex_cov(x64, y64, z64, a.sph64[a.sid[j]], a.tol);
-              }
-            }
-            const float t = r + top2_th(Ac, ea2);
-            if (t > 0.f && d2 < t * t * grow) top2_push(Ac, __fsqrt_rn(d2) - r, int(j));
-          };
-          if (P.w > 0.f) class_item(cov0, A0);
-          else if (P.w < 0.f) class_item(cov1, A1);
-          const float t2 = top2_th(F, ea2) - r;
-          if (t2 > 0.f && d2 < t2 * t2 * grow) top2_push(F, __fsqrt_rn(d2) + r, int(j));
-        }
-    };
-    // seed the thresholds with the leaf nearest the packet centre: a greedy
-    // descent (lanes 0-7 score the 8 children by centre distance) and the
-    // leaf's spheres evaluated by every lane; the walk then skips that leaf
-    const int64_t seeded = warp_descend(T, lane, [&](int64_t node) { return ball_d2(cx, cy, cz, T.na[node]); });
-    leaf_items(seeded);
-    W.push_top(T, lane);
-    while (W.sp > 0) {
-      const uint32_t nd = W.pop();
-      const int lev = node_level(nd);
-      const int64_t idx = node_index(nd);
-      if (lev == 0) {
-        if (idx != seeded) leaf_items(idx);
-      } else {
-        const int64_t cb = idx * kFan, ce = min(cb + kFan, T.count[lev - 1]);
-        const int64_t off = T.offset[lev - 1];
-        float th0 = top2_th(A0, ea2), th1 = top2_th(A1, ea2);
-        if (!cov0) th0 = fmaxf(th0, negtol);
-        if (!cov1) th1 = fmaxf(th1, negtol);
-        const float thf = top2_th(F, ea2);
-        // every child is tested by every lane (unrolled, so the loads of
-        // all children issue together); one warp OR gives the children to
-        // visit and one warp MIN the child nearest the packet centre (its
-        // squared distance with the child number in the low 3 bits)
-        const int nc = int(ce - cb);
-        n_nodes += live ? unsigned(nc) : 0u;
-        unsigned mine = 0, key = 0xffffffffu;
-#pragma unroll
-        for (int c = 0; c < kFan; ++c) {
-          if (c < nc && live) {
-            const float4 B = T.na[off + cb + c];
-            // one distance to the node centre C against the larger of each
-            // class's tangent threshold and the centres ball (a sample equal
-            // to x), then the far bound about its own centre
-            const float4 R = T.nb[off + cb + c];
-            float v = R.z;
-            if (R.x > -INFINITY) v = fmaxf(v, th0 + R.x);
-            if (R.y > -INFINITY) v = fmaxf(v, th1 + R.y);
-            const float t = fmaf(v, grow, bc.eprune);
-            bool nd_c = t > 0.f && ball_d2(x, y, z, B) < t * t;
-            if (!nd_c) {
-              const float4 Fb = T.nf[off + cb + c];
-              const float tf = fmaf(thf + Fb.w, grow, bc.eprune);
-              nd_c = tf > 0.f && ball_d2(x, y, z, Fb) < tf * tf;
-            }
-            if (nd_c) {
-              mine |= 1u << c;
-              key = min(key, (__float_as_uint(ball_d2(cx, cy, cz, B)) & ~7u) | unsigned(c));
-            }
-          }
-        }
-        const unsigned need = __reduce_or_sync(kFull, mine);
-        const int first = need ? int(__reduce_min_sync(kFull, key) & 7u) : -1;
-        W.push(lev - 1, cb, need, first, lane);
-      }
-    }
-  }
-  if constexpr (kPhase == 1) {
-    if (active) store_qstate(a.state, slot, cov0, cov1, sample, A0, A1, F);
-    warp_count(&a.cnt->query_rechecks, rechecks);
-    warp_count(&a.cnt->q_sphere_ntests, n_nodes);
-    warp_count(&a.cnt->q_sphere_items, n_items);
-    return;
-  }
+  if (active) load_qstate(a.state, slot, cov0, cov1, sample, A0, A1, F);
   int code = -1;
   double value = 0.0;
   int64_t arg = -1;
@@ -1252,9 +1289,6 @@ __device__ void query_packet(const QueryArgs& a, int64_t slot, WarpStack& W, int
     if (have_u && ub < __dsub_rn(m, a.tol)) flags |= GFS_FLAG_OPP_VIOL;
     value = cs == 0 ? m : -m;
   }
-  warp_count(&a.cnt->query_rechecks, rechecks);
-  warp_count(&a.cnt->q_sphere_ntests, n_nodes);
-  warp_count(&a.cnt->q_sphere_items, n_items);
   warp_count(&a.cnt->q_surv_ntests, n_snodes);
   warp_count(&a.cnt->q_band_passes, n_band);
   warp_count(&a.cnt->q_surv_items, n_sitems);
@@ -1275,16 +1309,51 @@ __device__ void query_packet(const QueryArgs& a, int64_t slot, WarpStack& W, int
 // survivor pass and the rest.  Each holds less live state than one kernel
 // doing both would, so more warps fit per SM (15% faster on the 64^3 union
 // workload than the fused packet code, which the batched kernel keeps).
-__global__ void __launch_bounds__(128, 8) k_query_spheres(QueryArgs a) {
-  __shared__ uint32_t s_stack[4][kPStack];
-  WarpStack W{s_stack[threadIdx.x >> 5], 0};
-  query_packet<false, 1>(a, blockIdx.x * int64_t(blockDim.x) + threadIdx.x, W, threadIdx.x & 31);
+// One warp per block: packets differ widely in work, and a block of several
+// warps would hold its slots until its slowest one is done.
+// Packets of 16 points from kPacketMin points on, when there are at least as
+// many points as spheres; below, a warp per point (a packet's points then lie
+// many sample spacings apart, and a heavy packet would end long after the
+// rest).  Sphere pass in ms, warp per point / packets of 8 / 16 / 32:
+//   16.2M points on 64^3 samples       101.4 / 38.2 / 30.6 / 36.5
+//   2.1M random points, 96^3 samples    69.8 / 44.0 / 40.3 / 42.9
+//   227k points on 16^3 samples         0.62 / 0.33 / 0.39 / 0.54
+//   100k random points, 32^3 samples    0.42 / 0.46 / 0.63 / 0.95
+//   30k points on 16^3 samples          0.10 / 0.21 / 0.28 / 0.39
+//   32k random points, 64^3 samples     0.52 / 1.01 / 1.28 / 1.81
+// rho_max: a packet of G points of a uniform set of m fills a cube of side
+// 2 cbrt(G / m) of the box; packets half again as wide as that hold a jump of
+// the Morton order and go point by point.
+constexpr int kPacket = 16;
+constexpr int64_t kPacketMin = 131072;
+
+template <int G>
+__global__ void __launch_bounds__(32, 28) k_query_spheres(QueryArgs a, float rho_max) {
+  __shared__ SpWarp S;
+  if (!sphere_pass<G>(a, int64_t(blockIdx.x) * G, S, threadIdx.x, rho_max) && threadIdx.x == 0)
+    a.defer[atomicAdd(&a.cnt->q_split, 1u)] = blockIdx.x;
+}
+
+// The points of the packets that k_query_spheres<G> listed, one at a time.
+template <int G>
+__global__ void __launch_bounds__(32, 28) k_query_spheres_split(QueryArgs a) {
+  __shared__ SpWarp S;
+  const int64_t total = int64_t(a.cnt->q_split) * G;
+  for (;;) {
+    unsigned t = 0;
+    if (threadIdx.x == 0) t = atomicAdd(&a.cnt->q_split_next, 1u);
+    t = __shfl_sync(kFull, t, 0);
+    if (int64_t(t) >= total) return;
+    const int64_t slot = int64_t(a.defer[t / G]) * G + t % G;
+    __syncwarp();
+    if (slot < a.m) sphere_pass<1>(a, slot, S, threadIdx.x, INFINITY);
+  }
 }
 
 __global__ void __launch_bounds__(128, 7) k_query_finish(QueryArgs a) {
   __shared__ uint32_t s_stack[4][kPStack];
   WarpStack W{s_stack[threadIdx.x >> 5], 0};
-  query_packet<false, 2>(a, blockIdx.x * int64_t(blockDim.x) + threadIdx.x, W, threadIdx.x & 31);
+  query_packet<false>(a, blockIdx.x * int64_t(blockDim.x) + threadIdx.x, W, threadIdx.x & 31);
 }
 
 // ---------------------------------------------------------------------------
@@ -1606,19 +1675,17 @@ cudaError_t launch_build_tree(const float4* items, int is_sphere, float A, Tree&
                               cudaStream_t st) {
   if (T.nlevels == 0) return cudaSuccess;
   if (is_sphere) {
-    k_sphere_leaves<<<nblk(T.count[0], 128), 128, 0, st>>>(items, T.nitems, A, T.lo, T.hi, T.na, T.nb, T.nf,
-                                                           T.count[0]);
+    k_sphere_leaves<<<nblk(T.count[0], 128), 128, 0, st>>>(items, A, T);
     ++g_launches;
     for (int l = 1; l < T.nlevels; ++l) {
-      k_sphere_level<<<nblk(T.count[l], 128), 128, 0, st>>>(T.lo, T.hi, T.na, T.nb, T.nf, A, T.offset[l - 1],
-                                                            T.count[l - 1], T.offset[l], T.count[l]);
+      k_sphere_level<<<nblk(T.count[l], 128), 128, 0, st>>>(A, T, l);
       ++g_launches;
     }
     if (scratch && T.nlevels > 1) {
       const int64_t nupper = T.offset[T.nlevels - 1] + T.count[T.nlevels - 1] - T.offset[1];
-      const cudaError_t e = cudaMemsetAsync(scratch, 0, size_t(nupper) * 4 * sizeof(unsigned), st);
+      const cudaError_t e = cudaMemsetAsync(scratch, 0, size_t(nupper) * kTight * sizeof(unsigned), st);
       if (e != cudaSuccess) return e;
-      k_tighten_items<<<nblk(T.nitems, 256), 256, 0, st>>>(items, T, scratch);
+      k_tighten_items<<<nblk(T.nitems, 256), 256, 0, st>>>(items, T, A, scratch);
       k_tighten_nodes<<<nblk(nupper, 128), 128, 0, st>>>(T, scratch, A, nupper);
       g_launches += 2;
     }
@@ -1665,7 +1732,14 @@ cudaError_t launch_cull(const CullArgs& a, cudaStream_t st) {
 
 cudaError_t launch_query_spheres(const QueryArgs& a, cudaStream_t st) {
   if (a.m == 0) return cudaSuccess;
-  k_query_spheres<<<nblk(a.m, 128), 128, 0, st>>>(a);
+  if (a.m < kPacketMin || a.m < a.n) {
+    k_query_spheres<1><<<unsigned(a.m), 32, 0, st>>>(a, INFINITY);
+  } else {
+    const float rho_max = 3.f * cbrtf(float(kPacket) / float(a.m));
+    k_query_spheres<kPacket><<<nblk(a.m, kPacket), 32, 0, st>>>(a, rho_max);
+    k_query_spheres_split<kPacket><<<152 * 28, 32, 0, st>>>(a);
+    ++g_launches;
+  }
   ++g_launches;
   return cudaGetLastError();
 }
