@@ -411,7 +411,7 @@ typedef struct {
 } gfs_shape;
 
 /* P build of many shapes at once: one cull launch covers every shape's
- * candidates, a block per (shape, direction, 128 spheres) item (the library
+ * candidates, in tiles of 32 spheres of one shape (the library
  * keeps the shape table; the caller keeps the buffers alive until the last
  * gfs_batch_query).  Results per shape are those of gfs_build on that shape
  * alone.  Sizes every buffer (the survivor capacity is grown and the cull
@@ -507,7 +507,7 @@ typedef struct {
   int64_t batch_sphere_items;  /* (point, sphere) tests of the last gfs_batch_query */
   int64_t batch_sphere_node_tests; /* its child-node bound tests of the sphere pass */
   int64_t batch_surv_items;    /* its (point, survivor) tests */
-  int64_t batch_cull_tile[3];  /* autotuned cull tile (spheres per block) of the batch's shapes with < 32k,
+  int64_t batch_cull_tile[3];  /* cull tile (spheres per block) of the batch's shapes with < 32k,
                                   < 256k and more samples (0: no such shape) */
   int64_t batch_query_grid;    /* autotuned grid of the persistent batched query (blocks) */
 } gfs_stats_t;

@@ -141,11 +141,13 @@ struct gfs_ctx {
   gfs_options opt{};
   cudaStream_t stream = nullptr;
   int K = 0, KS = 0;
-  DevBuf U32, U64;
+  DevBuf U4, U64, hsrc;
+  int KH = 0;  // directions whose covering balls the cull keeps
+  DevBuf cull_hint, cull_list, cull_count;
   // spheres
   int64_t n = 0;
   bool built = false;
-  DevBuf sph64, keys_in, keys_out, vals_in, vals_out, sph, thr, sid, bound_bits, consts, cnt, cub_temp;
+  DevBuf sph64, keys_in, keys_out, vals_in, vals_out, sph, thr, sid, cvl, bound_bits, consts, cnt, cub_temp;
   Tree st{};
   DevBuf st_lo, st_hi, st_na, st_nb, st_nf, st_ln;
   DevBuf st_tight;  // scratch of the internal-ball tightening
@@ -179,8 +181,8 @@ struct gfs_ctx {
   std::vector<gfs_shape> b_shapes;
   std::vector<int64_t> b_off, b_qoff, b_soff[2];
   std::vector<Tree> b_st;
-  DevBuf b_desc, b_offd, b_qoffd, b_sph64, b_k64in, b_k64out, b_sph, b_thr, b_sid, b_bits, b_bcs;
-  DevBuf b_lo, b_hi, b_na, b_nb, b_nf, b_ln, b_stdev, b_prefix, b_ctr, b_cnt, b_cviews, b_cw;
+  DevBuf b_desc, b_offd, b_qoffd, b_sph64, b_k64in, b_k64out, b_sph, b_thr, b_cvl, b_sid, b_bits, b_bcs;
+  DevBuf b_lo, b_hi, b_na, b_nb, b_nf, b_ln, b_tight, b_stdev, b_prefix, b_ctr, b_cnt, b_cviews;
   DevBuf b_sraw[2], b_sshape[2], b_ssorted[2], b_vlo[2], b_vhi[2], b_vtdev[2], b_hist;
   DevBuf b_qkin, b_qkout, b_qvin, b_qvout, b_qviews, b_qw, b_qstate;
   std::vector<QueryArgs> b_qv;  // host copies of the per-shape query views
@@ -188,14 +190,8 @@ struct gfs_ctx {
   std::vector<int64_t> b_sph_level_total;  // nodes per level of the sample forest, over all shapes
   int b_sph_levels = 0, b_surv_levels = 0, b_end_bit = 32;
   int64_t b_node_cap = 0;
-  // cull tiles per size class (autotuned on the first build): shapes of
-  // class k are views [b_cls_off[k], b_cls_off[k+1]) of b_cviews, with block
-  // prefixes at b_cw + b_cls_off[k] + k
-  int b_tile[3] = {128, 128, 128};
-  bool b_tiles_tuned = false;
-  int b_cls_off[4] = {0, 0, 0, 0};
-  int64_t b_cls_blocks[3] = {0, 0, 0};
-  std::vector<int> b_cls_order;     // shape index of each view, grouped by class
+  int64_t b_nodes = 0;        // nodes of the sample forest
+  int64_t b_cull_tiles = 0;   // 32-sphere tiles of all shapes (prefix behind b_prefix's item offsets)
   unsigned b_cap = 0;
   unsigned b_nsurv[2] = {0, 0};
   int64_t b_M = 0, b_qtotal = 0;
@@ -295,6 +291,7 @@ int build_sphere_hierarchy(gfs_ctx* c, int64_t n, const int* ids = nullptr) {
   GFS_TRY(ensure(c->sph, size_t(n) * sizeof(float4)));
   GFS_TRY(ensure(c->thr, size_t(n) * sizeof(float4)));
   GFS_TRY(ensure(c->sid, size_t(n) * 4));
+  GFS_TRY(ensure(c->cvl, size_t(n) * sizeof(float4)));
   GFS_CK(cudaMemsetAsync(c->bound_bits.p, 0, 16, st));
   GFS_CK(launch_keys_d4(src, n, c->keys_in.as<uint32_t>(), c->vals_in.as<int>(),
                         c->bound_bits.as<unsigned int>(), c->consts.as<BuildConsts>(), st));
@@ -302,7 +299,7 @@ int build_sphere_hierarchy(gfs_ctx* c, int64_t n, const int* ids = nullptr) {
                          c->vals_out.as<int>(), n));
   GFS_CK(launch_gather_spheres(src, c->vals_out.as<int>(), n, c->consts.as<BuildConsts>(),
                                float(c->opt.tol), c->opt.tol, c->sph.as<float4>(), c->thr.as<float4>(),
-                               c->sid.as<int>(), st));
+                               c->cvl.as<float4>(), c->sid.as<int>(), st));
   if (ids) GFS_CK(launch_remap_sid(c->sid.as<int>(), ids, n, st));
   tree_layout(c->st, n);
   const int64_t nodes = tree_nodes(c->st);
@@ -379,14 +376,17 @@ int gfs_create(gfs_ctx** out, const gfs_options* opt, void* cuda_stream) {
   c->K = 10 * (1 << (2 * o.tau)) + 2;
   c->KS = c->K + 1;
   std::vector<double> U(size_t(c->K) * 3);
-  std::vector<float> U32(size_t(c->K) * 3);
-  if (gfs_icosphere(o.tau, U.data(), c->K) != c->K) {
+  std::vector<float> U4(size_t(c->K) * 4);
+  std::vector<int> hsrc(size_t(c->K) * 2);
+  c->KH = o.tau == 0 ? 0 : 10 * (1 << (2 * std::min(o.tau - 1, 3))) + 2;
+  if (gfs_icosphere(o.tau, U.data(), c->K) != c->K || !icosphere_sources(o.tau, c->KH, hsrc.data())) {
     delete c;
     return GFS_ERR_ARG;
   }
-  for (size_t t = 0; t < U.size(); ++t) U32[t] = float(U[t]);
+  for (size_t t = 0; t < U.size(); ++t) U4[t / 3 * 4 + t % 3] = float(U[t]);
   int st = ensure(c->U64, U.size() * 8);
-  if (st == GFS_OK) st = ensure(c->U32, U32.size() * 4);
+  if (st == GFS_OK) st = ensure(c->U4, U4.size() * 4);
+  if (st == GFS_OK) st = ensure(c->hsrc, hsrc.size() * 4);
   if (st == GFS_OK) st = ensure(c->bound_bits, 16);
   if (st == GFS_OK) st = ensure(c->consts, sizeof(BuildConsts));
   if (st == GFS_OK) st = ensure(c->cnt, sizeof(Counters));
@@ -404,7 +404,8 @@ int gfs_create(gfs_ctx** out, const gfs_options* opt, void* cuda_stream) {
     c->have_ev = true;
   }
   if (cudaMemcpy(c->U64.p, U.data(), U.size() * 8, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(c->U32.p, U32.data(), U32.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemcpy(c->U4.p, U4.data(), U4.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemcpy(c->hsrc.p, hsrc.data(), hsrc.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemset(c->cnt.p, 0, sizeof(Counters)) != cudaSuccess) {
     cudaGetLastError();
     gfs_destroy(c);
@@ -428,6 +429,21 @@ int reset_cull_counters(gfs_ctx* c, cudaStream_t st) {
   GFS_CK(cudaMemsetAsync(base + offsetof(Counters, cull_rechecks), 0, sizeof(unsigned long long), st));
   GFS_CK(cudaMemsetAsync(base + offsetof(Counters, nsurv), 0, 2 * sizeof(unsigned int), st));
   GFS_CK(cudaMemsetAsync(base + offsetof(Counters, c_ntests), 0, 2 * sizeof(unsigned long long), st));
+  return GFS_OK;
+}
+
+// The cull's workspace for `tiles` tiles, in chunks of at most 1 GB of
+// covering balls and open-list entries (a chunk's entries number below 2^32).
+int cull_work(gfs_ctx* c, int64_t tiles, CullWork& w) {
+  const int64_t last = c->K - c->KH;  // directions of the last level(s), the largest group
+  const int64_t per = (int64_t(c->KH) + last) * kCullTileSpheres * 4;
+  w.chunk = std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t(1) << 30) / per));
+  GFS_TRY(ensure(c->cull_hint, size_t(w.chunk) * std::max(1, c->KH) * kCullTileSpheres * 4));
+  GFS_TRY(ensure(c->cull_list, size_t(w.chunk) * size_t(last) * kCullTileSpheres * 4));
+  GFS_TRY(ensure(c->cull_count, size_t(cull_launches(c->KH, tiles, w.chunk)) * 8));
+  w.hint = c->cull_hint.as<int>();
+  w.list = c->cull_list.as<uint32_t>();
+  w.count = c->cull_count.as<unsigned>();
   return GFS_OK;
 }
 
@@ -464,7 +480,10 @@ int build_finish(gfs_ctx* c) {
     a.thr = c->thr.as<float4>();
     a.sid = c->sid.as<int>();
     a.sph64 = c->sph64.as<D4>();
-    a.U32 = c->U32.as<float>();
+    a.cvl = c->cvl.as<float4>();
+    a.U4 = c->U4.as<float4>();
+    a.hsrc = c->hsrc.as<int2>();
+    a.KH = c->KH;
     a.U64 = c->U64.as<double>();
     a.K = c->K;
     a.KS = c->KS;
@@ -479,7 +498,10 @@ int build_finish(gfs_ctx* c) {
     a.cap = c->cap;
     a.cnt = c->cnt.as<Counters>();
     if (c->have_ev) GFS_CK(cudaEventRecord(c->ev[1], st));
-    GFS_CK(launch_cull(a, st));
+    CullWork w;
+    const int64_t tiles = (n + kCullTileSpheres - 1) / kCullTileSpheres;
+    GFS_TRY(cull_work(c, tiles, w));
+    GFS_CK(launch_cull(a, nullptr, nullptr, 0, tiles, w, st));
     if (c->have_ev) GFS_CK(cudaEventRecord(c->ev[2], st));
     unsigned int ns[2] = {0, 0};
     GFS_CK(cudaMemcpyAsync(ns, reinterpret_cast<char*>(c->cnt.p) + offsetof(Counters, nsurv), sizeof(ns),
@@ -1278,8 +1300,10 @@ int autotune_grid(gfs_ctx* c, int64_t total) {
 
 namespace {
 
-// Size class of a shape for the cull tile choice: up to 32k, up to 256k, more.
-int batch_size_class(int64_t n) { return n < 32768 ? 0 : (n < 262144 ? 1 : 2); }
+// each shape's first 32-sphere tile (behind the level prefixes and item offsets)
+const int64_t* batch_tiles(const gfs_ctx* c) {
+  return c->b_prefix.as<int64_t>() + size_t(c->b_ns + 1) * std::max(1, c->b_sph_levels) + c->b_ns;
+}
 
 // Levels of the sample forest (static layout uploaded by the first build).
 int batch_sphere_levels(gfs_ctx* c) {
@@ -1289,6 +1313,10 @@ int batch_sphere_levels(gfs_ctx* c) {
     GFS_CK(launch_batch_tree_level(c->b_stdev.as<Tree>(), c->b_prefix.as<int64_t>() + size_t(l) * (ns + 1),
                                    c->b_sph_level_total[size_t(l)], ns, l, c->b_sph.as<float4>(),
                                    c->b_prefix.as<int64_t>() + io, c->b_bcs.as<BuildConsts>(), 1, c->stream));
+  GFS_CK(launch_batch_tighten(c->b_stdev.as<Tree>(), c->b_prefix.as<int64_t>(), c->b_sph_level_total.data(),
+                              c->b_sph_levels, ns, batch_tiles(c), c->b_cull_tiles,
+                              c->b_sph.as<float4>(), c->b_prefix.as<int64_t>() + io, c->b_bcs.as<BuildConsts>(),
+                              c->b_na.as<float4>(), c->b_nodes, c->b_tight.as<unsigned>(), c->stream));
   return GFS_OK;
 }
 
@@ -1306,7 +1334,7 @@ int batch_build_device_samples(gfs_ctx* c) {
                       c->vals_in.as<int>(), c->vals_out.as<int>(), N, c->b_end_bit, st));
   GFS_CK(launch_batch_gather(c->b_sph64.as<D4>(), c->vals_out.as<int>(), c->b_offd.as<int64_t>(), ns, N,
                              c->b_bcs.as<BuildConsts>(), float(c->opt.tol), c->opt.tol, c->b_sph.as<float4>(),
-                             c->b_thr.as<float4>(), c->b_sid.as<int>(), st));
+                             c->b_thr.as<float4>(), c->b_cvl.as<float4>(), c->b_sid.as<int>(), st));
   return batch_sphere_levels(c);
 }
 
@@ -1321,10 +1349,13 @@ int batch_build_device(gfs_ctx* c, bool cull_only) {
   (void)N;
   if (!cull_only) GFS_TRY(batch_build_device_samples(c));
   GFS_CK(cudaMemsetAsync(c->b_cnt.p, 0, sizeof(Counters), st));
-  for (int k = 0; k < 3; ++k)
-    GFS_CK(launch_batch_cull_blocks(c->b_cviews.as<CullArgs>() + c->b_cls_off[k],
-                                    c->b_cw.as<int64_t>() + c->b_cls_off[k] + k, c->b_cls_off[k + 1] - c->b_cls_off[k],
-                                    c->b_cls_blocks[k], c->b_tile[k], st));
+  CullWork w;
+  GFS_TRY(cull_work(c, c->b_cull_tiles, w));  // (sized by the first build)
+  CullArgs one;
+  std::memset(&one, 0, sizeof(one));
+  one.K = c->K;
+  one.KH = c->KH;
+  GFS_CK(launch_cull(one, c->b_cviews.as<CullArgs>(), batch_tiles(c), ns, c->b_cull_tiles, w, st));
   if (cull_only) return GFS_OK;
   for (int k = 0; k < 2; ++k)
     GFS_CK(launch_batch_surv_forest(
@@ -1392,6 +1423,7 @@ int gfs_batch_build(gfs_ctx* c, const gfs_shape* shapes, int ns) {
   GFS_TRY(ensure(c->b_sph, size_t(N) * sizeof(float4)));
   GFS_TRY(ensure(c->b_thr, size_t(N) * sizeof(float4)));
   GFS_TRY(ensure(c->b_sid, size_t(N) * 4));
+  GFS_TRY(ensure(c->b_cvl, size_t(N) * sizeof(float4)));
   GFS_TRY(ensure(c->b_bits, size_t(ns) * 8));
   GFS_TRY(ensure(c->b_bcs, size_t(ns) * sizeof(BuildConsts)));
   GFS_TRY(ensure(c->b_hist, size_t(ns) * 4));
@@ -1431,7 +1463,7 @@ int gfs_batch_build(gfs_ctx* c, const gfs_shape* shapes, int ns) {
   {
     GFS_TRY(ensure(c->b_stdev, size_t(ns) * sizeof(Tree)));
     GFS_CK(cudaMemcpyAsync(c->b_stdev.p, c->b_st.data(), size_t(ns) * sizeof(Tree), cudaMemcpyHostToDevice, st));
-    std::vector<int64_t> pre(size_t(ns + 1) * std::max(1, maxL) + size_t(ns));
+    std::vector<int64_t> pre(size_t(ns + 1) * std::max(1, maxL) + size_t(ns) + size_t(ns + 1));
     c->b_sph_level_total.assign(size_t(std::max(1, maxL)), 0);
     for (int l = 0; l < maxL; ++l) {
       int64_t acc = 0;
@@ -1443,13 +1475,19 @@ int gfs_batch_build(gfs_ctx* c, const gfs_shape* shapes, int ns) {
       c->b_sph_level_total[size_t(l)] = acc;
     }
     const size_t io = size_t(ns + 1) * std::max(1, maxL);
-    for (int s = 0; s < ns; ++s) pre[io + s] = off[s];
+    for (int s = 0; s < ns; ++s) {
+      pre[io + s] = off[s];
+      pre[io + ns + s + 1] = pre[io + ns + s] + (shapes[s].n + kCullTileSpheres - 1) / kCullTileSpheres;
+    }
+    c->b_cull_tiles = pre[io + ns + ns];
+    c->b_nodes = nodes;
+    GFS_TRY(ensure(c->b_tight, size_t(nodes) * 8 * sizeof(unsigned)));
     GFS_TRY(ensure(c->b_prefix, pre.size() * 8));
     GFS_CK(cudaMemcpyAsync(c->b_prefix.p, pre.data(), pre.size() * 8, cudaMemcpyHostToDevice, st));
     GFS_CK(cudaStreamSynchronize(st));  // the pageable host arrays above are copied before they go out of scope
     c->b_sph_levels = maxL;
   }
-  // culling views and work items (shape, direction, 128 spheres)
+  // culling views
   const uint64_t ncand = uint64_t(N) * uint64_t(c->K);
   // survivors are typically < 1% of the candidates; the cull is rerun with
   // room for the counted survivors if this first capacity overflows
@@ -1461,57 +1499,41 @@ int gfs_batch_build(gfs_ctx* c, const gfs_shape* shapes, int ns) {
   // the samples (the cull reads them) -- built once here, then the cull is
   // repeated until its survivor capacity suffices
   GFS_TRY(batch_build_device_samples(c));
-  // size classes of the shapes (the cull tile is chosen per class)
-  c->b_cls_order.clear();
-  for (int k = 0; k < 3; ++k) {
-    c->b_cls_off[k] = int(c->b_cls_order.size());
-    for (int s = 0; s < ns; ++s)
-      if (batch_size_class(shapes[s].n) == k) c->b_cls_order.push_back(s);
-  }
-  c->b_cls_off[3] = ns;
-  // upload the views and the per-class block prefixes for the current tiles
+  // upload the views
   auto upload_cull = [&](unsigned capv) -> int {
     std::vector<CullArgs> cv(ns);
-    std::vector<int64_t> cw(size_t(ns) + 3);
-    for (int k = 0; k < 3; ++k) {
-      int64_t acc = 0;
-      for (int v = c->b_cls_off[k]; v < c->b_cls_off[k + 1]; ++v) {
-        const int s = c->b_cls_order[size_t(v)];
-        CullArgs& a = cv[size_t(v)];
-        std::memset(&a, 0, sizeof(a));
-        a.sph = c->b_sph.as<float4>() + off[s];
-        a.thr = c->b_thr.as<float4>() + off[s];
-        a.sid = c->b_sid.as<int>() + off[s];
-        a.sph64 = c->b_sph64.as<D4>() + off[s];
-        a.U32 = c->U32.as<float>();
-        a.U64 = c->U64.as<double>();
-        a.K = c->K;
-        a.KS = c->KS;
-        a.tree = c->b_st[s];
-        a.tol32 = float(c->opt.tol);
-        a.tol = c->opt.tol;
-        a.box_cull = c->opt.box_cull;
-        a.bc = c->b_bcs.as<BuildConsts>() + s;
-        a.n = shapes[s].n;
-        a.surv[0] = c->b_sraw[0].as<float4>();
-        a.surv[1] = c->b_sraw[1].as<float4>();
-        a.cap = capv;
-        a.cnt = c->b_cnt.as<Counters>();
-        a.surv_shape[0] = c->b_sshape[0].as<uint16_t>();
-        a.surv_shape[1] = c->b_sshape[1].as<uint16_t>();
-        a.shape = s;
-        cw[size_t(v + k)] = acc;
-        acc += (shapes[s].n + c->b_tile[k] - 1) / c->b_tile[k] * c->K;
-      }
-      cw[size_t(c->b_cls_off[k + 1] + k)] = acc;
-      c->b_cls_blocks[k] = acc;
+    for (int s = 0; s < ns; ++s) {
+      CullArgs& a = cv[size_t(s)];
+      std::memset(&a, 0, sizeof(a));
+      a.sph = c->b_sph.as<float4>() + off[s];
+      a.thr = c->b_thr.as<float4>() + off[s];
+      a.sid = c->b_sid.as<int>() + off[s];
+      a.sph64 = c->b_sph64.as<D4>() + off[s];
+      a.cvl = c->b_cvl.as<float4>() + off[s];
+      a.U4 = c->U4.as<float4>();
+      a.hsrc = c->hsrc.as<int2>();
+      a.KH = c->KH;
+      a.U64 = c->U64.as<double>();
+      a.K = c->K;
+      a.KS = c->KS;
+      a.tree = c->b_st[s];
+      a.tol32 = float(c->opt.tol);
+      a.tol = c->opt.tol;
+      a.box_cull = c->opt.box_cull;
+      a.bc = c->b_bcs.as<BuildConsts>() + s;
+      a.n = shapes[s].n;
+      a.surv[0] = c->b_sraw[0].as<float4>();
+      a.surv[1] = c->b_sraw[1].as<float4>();
+      a.cap = capv;
+      a.cnt = c->b_cnt.as<Counters>();
+      a.surv_shape[0] = c->b_sshape[0].as<uint16_t>();
+      a.surv_shape[1] = c->b_sshape[1].as<uint16_t>();
+      a.shape = s;
     }
     GFS_CK(cudaMemcpyAsync(c->b_cviews.p, cv.data(), size_t(ns) * sizeof(CullArgs), cudaMemcpyHostToDevice, st));
-    GFS_CK(cudaMemcpyAsync(c->b_cw.p, cw.data(), cw.size() * 8, cudaMemcpyHostToDevice, st));
     GFS_CK(cudaStreamSynchronize(st));  // pageable sources
     return GFS_OK;
   };
-  GFS_TRY(ensure(c->b_cw, size_t(ns + 3) * 8));
   for (int attempt = 0; attempt < 3; ++attempt) {
     c->b_cap = unsigned(cap);
     for (int k = 0; k < 2; ++k) {
@@ -1529,45 +1551,6 @@ int gfs_batch_build(gfs_ctx* c, const gfs_shape* shapes, int ns) {
     if (need <= c->b_cap) break;
     cap = uint64_t(need) + need / 8 + 1024;
     if (attempt == 2) return GFS_ERR_OOM;
-  }
-  // cull tile per size class: each class's cull timed with tiles of 64, 128
-  // and 256 spheres (the first build only; the fastest is kept), then the
-  // whole cull rerun with the chosen tiles
-  if (!c->b_tiles_tuned) {
-    cudaEvent_t e0, e1;
-    GFS_CK(cudaEventCreate(&e0));
-    GFS_CK(cudaEventCreate(&e1));
-    for (int k = 0; k < 3; ++k) {
-      if (c->b_cls_off[k + 1] == c->b_cls_off[k]) continue;
-      float best = 0.f;
-      int best_tile = 128;
-      for (int tile : {64, 128, 256}) {
-        c->b_tile[k] = tile;
-        if (upload_cull(c->b_cap) != GFS_OK) break;
-        float ms = 0.f;
-        if (cudaMemsetAsync(c->b_cnt.p, 0, sizeof(Counters), st) != cudaSuccess ||
-            cudaEventRecord(e0, st) != cudaSuccess ||
-            launch_batch_cull_blocks(c->b_cviews.as<CullArgs>() + c->b_cls_off[k],
-                                     c->b_cw.as<int64_t>() + c->b_cls_off[k] + k,
-                                     c->b_cls_off[k + 1] - c->b_cls_off[k], c->b_cls_blocks[k], tile, st) !=
-                cudaSuccess ||
-            cudaEventRecord(e1, st) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
-            cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) {
-          cudaGetLastError();
-          break;
-        }
-        if (best == 0.f || ms < best) {
-          best = ms;
-          best_tile = tile;
-        }
-      }
-      c->b_tile[k] = best_tile;
-    }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    c->b_tiles_tuned = true;
-    GFS_TRY(upload_cull(c->b_cap));
-    GFS_TRY(batch_build_device(c, true));
   }
   if (std::max(c->b_nsurv[0], c->b_nsurv[1]) > kMaxSurvivors) return GFS_ERR_TOO_LARGE;
   // survivor forests: sized for the capacity (the layout is computed on the
@@ -1817,7 +1800,8 @@ int gfs_stats(gfs_ctx* c, gfs_stats_t* out) {
     out->batch_sphere_items = int64_t(bc.q_sphere_items);
     out->batch_sphere_node_tests = int64_t(bc.q_sphere_ntests);
     out->batch_surv_items = int64_t(bc.q_surv_items);
-    for (int k = 0; k < 3; ++k) out->batch_cull_tile[k] = c->b_cls_off[k + 1] > c->b_cls_off[k] ? c->b_tile[k] : 0;
+    for (const gfs_shape& sh : c->b_shapes)
+      out->batch_cull_tile[sh.n < 32768 ? 0 : (sh.n < 262144 ? 1 : 2)] = kCullTileSpheres;
     out->batch_query_grid = c->b_grid_query;
   }
   out->insert_sph_exact = int64_t(c->ins_work[0]);
@@ -1883,7 +1867,7 @@ void gfs_destroy(gfs_ctx* c) {
   if (c->sev) cudaEventDestroy(c->sev);
   if (c->sev2) cudaEventDestroy(c->sev2);
   if (c->side) cudaStreamDestroy(c->side);
-  DevBuf* bufs[] = {&c->U32, &c->U64, &c->sph64, &c->keys_in, &c->keys_out, &c->vals_in, &c->vals_out, &c->sph,
+  DevBuf* bufs[] = {&c->U4, &c->hsrc, &c->cvl, &c->b_cvl, &c->cull_hint, &c->cull_list, &c->cull_count, &c->U64, &c->sph64, &c->keys_in, &c->keys_out, &c->vals_in, &c->vals_out, &c->sph,
                     &c->thr, &c->sid, &c->bound_bits, &c->consts, &c->cnt, &c->cub_temp, &c->st_lo, &c->st_hi,
                     &c->st_na, &c->st_nb, &c->st_nf, &c->st_ln, &c->st_tight, &c->qstate, &c->surv_raw[0], &c->surv_raw[1], &c->surv_sorted[0], &c->surv_sorted[1],
                     &c->vt_lo[0], &c->vt_lo[1], &c->vt_hi[0], &c->vt_hi[1], &c->defer, &c->acc, &c->witness64,
@@ -1896,8 +1880,8 @@ void gfs_destroy(gfs_ctx* c) {
                     &c->csr_off, &c->scored_status, &c->ud_uncov, &c->ud_cnt, &c->ud_pairs, &c->ud_circ,
                     &c->ud_quad, &c->ud_pts, &c->ud_k0, &c->ud_k1, &c->ud_v0, &c->ud_v1,
                     &c->b_desc, &c->b_offd, &c->b_qoffd, &c->b_sph64, &c->b_k64in, &c->b_k64out, &c->b_sph,
-                    &c->b_thr, &c->b_sid, &c->b_bits, &c->b_bcs, &c->b_lo, &c->b_hi, &c->b_na, &c->b_nb, &c->b_nf, &c->b_ln,
-                    &c->b_stdev, &c->b_prefix, &c->b_ctr, &c->b_cnt, &c->b_cviews, &c->b_cw, &c->b_sraw[0],
+                    &c->b_thr, &c->b_sid, &c->b_bits, &c->b_bcs, &c->b_lo, &c->b_hi, &c->b_na, &c->b_nb, &c->b_nf, &c->b_ln, &c->b_tight,
+                    &c->b_stdev, &c->b_prefix, &c->b_ctr, &c->b_cnt, &c->b_cviews, &c->b_sraw[0],
                     &c->b_sraw[1], &c->b_sshape[0], &c->b_sshape[1], &c->b_ssorted[0], &c->b_ssorted[1],
                     &c->b_vlo[0], &c->b_vlo[1], &c->b_vhi[0], &c->b_vhi[1], &c->b_vtdev[0], &c->b_vtdev[1],
                     &c->b_hist, &c->b_qkin, &c->b_qkout, &c->b_qvin, &c->b_qvout, &c->b_qviews, &c->b_qw, &c->b_qstate,

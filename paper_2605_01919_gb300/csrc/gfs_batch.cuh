@@ -3,9 +3,9 @@
 // All shapes' samples live in one array, sorted by (shape, Morton code), so
 // each shape owns a contiguous range; every shape gets its own implicit
 // hierarchy inside shared node arrays (a forest).  The hot kernels are
-// persistent: a fixed grid of warps pulls work items -- (shape, 32 spheres,
-// direction k) for the cull, (shape, 32 query points) for the query -- from a
-// global counter, so shapes of very different sizes share the GPU evenly.
+// sized for uneven shapes: the cull's tiles are numbered through all shapes, the
+// query is a fixed grid of warps that pull work items -- (shape, 32
+// query points) -- from a global counter.
 // Each shape is seen through a per-shape argument block ("view") whose
 // pointers are offset to the shape's range and whose indices are local, so
 // the per-warp code is the single-shape packet code.
@@ -17,17 +17,6 @@ namespace gfs {
 namespace {
 
 constexpr unsigned kAllB = 0xffffffffu;
-
-// segment of v in a prefix array (prefix[0] = 0, prefix[ns] = total)
-__device__ __forceinline__ int find_seg(const int64_t* __restrict__ prefix, int ns, int64_t v) {
-  int lo = 0, hi = ns;
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (prefix[mid] <= v) lo = mid;
-    else hi = mid;
-  }
-  return lo;
-}
 
 __device__ __forceinline__ uint32_t morton_of(float x, float y, float z) { return morton3(x, y, z); }
 
@@ -58,7 +47,7 @@ __global__ void k_batch_consts(const unsigned int* __restrict__ bits, int ns, Bu
 __global__ void k_batch_gather(const D4* __restrict__ sph64, const int* __restrict__ order,
                                const int64_t* __restrict__ off, int ns, int64_t N, const BuildConsts* __restrict__ bc,
                                float tol32, double tol, float4* __restrict__ sph, float4* __restrict__ thr,
-                               int* __restrict__ sid) {
+                               float4* __restrict__ cvl, int* __restrict__ sid) {
   const int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
   if (t >= N) return;
   const int o = order[t];
@@ -73,6 +62,7 @@ __global__ void k_batch_gather(const D4* __restrict__ sph64, const int* __restri
   cov_thresholds(d.w, fabsf(w), tol32, tol, bc[s].eq, A, lc, hc);
   cov_thresholds(d.w, fabsf(w), tol32, tol, 5.9604644775390625e-8f * A, A, lq, hq);
   thr[t] = make_float4(lc, hc, lq, hq);
+  cvl[t] = make_float4(float(d.x), float(d.y), float(d.z), lc);
 }
 
 // one level of every shape's hierarchy; prefix[s] = first node of shape s
@@ -96,6 +86,33 @@ __global__ void k_batch_tree_level(const Tree* __restrict__ trees, const int64_t
     else
       point_level_node(T.lo, T.hi, T.offset[level - 1], T.count[level - 1], T.offset[level], j);
   }
+}
+
+// Tightening of every shape's internal bounds (as k_tighten_items /
+// k_tighten_nodes): one warp per 32-sphere tile (tiles: each shape's first
+// tile), then one thread per node of a level; keys: kTight words per node of
+// the forest (zeroed; na0 the forest's first node).
+__global__ void k_batch_tighten_items(const Tree* __restrict__ trees, const int64_t* __restrict__ tiles, int ns,
+                                      const float4* __restrict__ items_base, const int64_t* __restrict__ item_off,
+                                      const BuildConsts* __restrict__ bc, const float4* na0, unsigned* keys) {
+  const int64_t t = (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) >> 5;
+  if (t >= tiles[ns]) return;
+  const int s = find_seg(tiles, ns, t);
+  const Tree& T = trees[s];
+  if (T.nlevels < 2) return;
+  tighten_items(items_base + item_off[s], T, bc[s].A, keys + kTight * (T.na - na0 + T.offset[1]),
+                (t - tiles[s]) * 32 + (threadIdx.x & 31));
+}
+
+__global__ void k_batch_tighten_nodes(const Tree* __restrict__ trees, const int64_t* __restrict__ prefix, int ns,
+                                      int level, const BuildConsts* __restrict__ bc, const float4* na0,
+                                      const unsigned* __restrict__ keys) {
+  const int64_t g = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+  if (g >= prefix[ns]) return;
+  const int s = find_seg(prefix, ns, g);
+  const Tree& T = trees[s];
+  tighten_node(T, keys + kTight * (T.na - na0 + T.offset[1]), bc[s].A,
+               T.offset[level] - T.offset[1] + (g - prefix[s]));
 }
 
 // survivors per (shape, class)
@@ -139,27 +156,6 @@ __global__ void k_batch_qkeys(const ShapeDesc* __restrict__ d, const int64_t* __
   vals[u] = int(i);
 }
 
-// Cull over a group of shapes as one flat launch: block b is item b of
-// (shape, direction k, BS Morton-consecutive spheres) -- BS the group's tile,
-// picked by the autotuner --, so the candidates left open by the neighbour
-// pre-test are packed into full warps as in the single-shape cull, and the
-// hardware schedules the uneven blocks.
-template <int BS>
-__global__ void __launch_bounds__(BS) k_batch_cull_blocks(const CullArgs* __restrict__ views,
-                                                          const int64_t* __restrict__ bprefix, int ns) {
-  __shared__ uint32_t s_stack[BS / 32][kPStack];
-  __shared__ int s_idx[BS], s_wcnt[BS / 32];
-  WarpStack W{s_stack[threadIdx.x >> 5], 0};
-  const int64_t w = blockIdx.x;
-  const int s = find_seg(bprefix, ns, w);
-  const CullArgs& a = views[s];
-  const int64_t local = w - bprefix[s];
-  const int64_t nbs = (a.n + BS - 1) / BS;
-  const int k = int(local / nbs);
-  const int64_t bl = local - int64_t(k) * nbs;
-  cull_packet<true>(a, bl * BS + threadIdx.x, k, W, threadIdx.x & 31, s_idx, s_wcnt);
-}
-
 // Persistent query over all shapes: work item = (shape, 32 consecutive
 // points of the shape's Morton order).
 // kPhase 1: the sphere pass (state per point to the view's state array);
@@ -180,7 +176,7 @@ __global__ void __launch_bounds__(128) k_batch_query(const QueryArgs* __restrict
     const int64_t wl = int64_t(w) - wprefix[s];
     if constexpr (kPhase == 1) {
 #pragma unroll 1
-      for (int g = 0; g < 32; g += 8)
+      for (int g = 0; g < 32; g += kPacket)
         if (wl * 32 + g < views[s].m) sphere_pass_any(views[s], wl * 32 + g, s_warp[threadIdx.x >> 5], lane);
     } else {
       WarpStack W{s_warp[threadIdx.x >> 5], 0};
@@ -337,10 +333,10 @@ cudaError_t sort_pairs64(void* temp, size_t& bytes, const unsigned long long* ki
 }
 
 cudaError_t launch_batch_gather(const D4* sph64, const int* order, const int64_t* off, int ns, int64_t N,
-                                const BuildConsts* bc, float tol32, double tol, float4* sph, float4* thr, int* sid,
-                                cudaStream_t st) {
+                                const BuildConsts* bc, float tol32, double tol, float4* sph, float4* thr, float4* cvl,
+                                int* sid, cudaStream_t st) {
   if (N == 0) return cudaSuccess;
-  k_batch_gather<<<nb(N, 256), 256, 0, st>>>(sph64, order, off, ns, N, bc, tol32, tol, sph, thr, sid);
+  k_batch_gather<<<nb(N, 256), 256, 0, st>>>(sph64, order, off, ns, N, bc, tol32, tol, sph, thr, cvl, sid);
   return cudaGetLastError();
 }
 
@@ -349,6 +345,21 @@ cudaError_t launch_batch_tree_level(const Tree* trees, const int64_t* prefix, in
                                     int is_sphere, cudaStream_t st) {
   if (total == 0) return cudaSuccess;
   k_batch_tree_level<<<nb(total, 128), 128, 0, st>>>(trees, prefix, ns, level, items_base, item_off, bc, is_sphere);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_batch_tighten(const Tree* trees, const int64_t* prefix, const int64_t* level_total, int nlev, int ns,
+                                 const int64_t* tiles, int64_t ntiles, const float4* items_base,
+                                 const int64_t* item_off, const BuildConsts* bc, const float4* na0, int64_t nodes,
+                                 unsigned* keys, cudaStream_t st) {
+  if (nlev < 2) return cudaSuccess;
+  const cudaError_t e = cudaMemsetAsync(keys, 0, size_t(nodes) * kTight * sizeof(unsigned), st);
+  if (e != cudaSuccess) return e;
+  k_batch_tighten_items<<<nb(ntiles, 8), 256, 0, st>>>(trees, tiles, ns, items_base, item_off, bc, na0, keys);
+  for (int l = 1; l < nlev; ++l)
+    if (level_total[l] > 0)
+      k_batch_tighten_nodes<<<nb(level_total[l], 128), 128, 0, st>>>(trees, prefix + int64_t(l) * (ns + 1), ns, l, bc,
+                                                                     na0, keys);
   return cudaGetLastError();
 }
 
@@ -376,17 +387,6 @@ cudaError_t launch_batch_qkeys(const ShapeDesc* d, const int64_t* off, int ns, i
                                int* vals, cudaStream_t st) {
   if (M == 0) return cudaSuccess;
   k_batch_qkeys<<<nb(M, 256), 256, 0, st>>>(d, off, ns, M, keys, vals);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_batch_cull_blocks(const CullArgs* views, const int64_t* bprefix, int ns, int64_t nblocks, int tile,
-                                     cudaStream_t st) {
-  if (nblocks <= 0) return cudaSuccess;
-  if (nblocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-  if (tile == 64) k_batch_cull_blocks<64><<<unsigned(nblocks), 64, 0, st>>>(views, bprefix, ns);
-  else if (tile == 256) k_batch_cull_blocks<256><<<unsigned(nblocks), 256, 0, st>>>(views, bprefix, ns);
-  else if (tile == 128) k_batch_cull_blocks<128><<<unsigned(nblocks), 128, 0, st>>>(views, bprefix, ns);
-  else return cudaErrorInvalidValue;
   return cudaGetLastError();
 }
 

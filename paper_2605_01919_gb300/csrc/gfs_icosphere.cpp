@@ -18,6 +18,7 @@
 #include <cmath>
 #include <cstdint>
 #include <unordered_map>
+#include <utility>
 #include <vector>
 
 #include "gfs.h"
@@ -37,18 +38,16 @@ struct Face {
   int a, b, c;
 };
 
-}  // namespace
-
-extern "C" int gfs_icosphere(int tau, double* out_host, int64_t cap_rows) {
-  if (tau < 0 || tau > 7 || out_host == nullptr) return -1;
+// the table's vertices, and the two vertices each one from 12 on lies between
+bool icosphere_vertices(int tau, std::vector<Vec>& verts, std::vector<std::pair<int, int>>& parents) {
   const int64_t K = 10 * (int64_t(1) << (2 * tau)) + 2;
-  if (cap_rows < K) return -1;
   const double phi = (1.0 + std::sqrt(5.0)) / 2.0;
   const double raw[12][3] = {{-1, phi, 0}, {1, phi, 0}, {-1, -phi, 0}, {1, -phi, 0},
                              {0, -1, phi}, {0, 1, phi}, {0, -1, -phi}, {0, 1, -phi},
                              {phi, 0, -1}, {phi, 0, 1}, {-phi, 0, -1}, {-phi, 0, 1}};
-  std::vector<Vec> verts;
+  verts.clear();
   verts.reserve(size_t(K));
+  parents.assign(12, {-1, -1});
   for (const auto& v : raw) verts.push_back(scaled_unit(v[0], v[1], v[2]));
 
   auto sq = [&](int i, int j) {
@@ -73,7 +72,7 @@ extern "C" int gfs_icosphere(int tau, double* out_host, int64_t cap_rows) {
         faces.push_back(outward ? Face{a, b, c} : Face{a, c, b});
       }
     }
-  if (faces.size() != 20) return -1;
+  if (faces.size() != 20) return false;
 
   for (int level = 0; level < tau; ++level) {
     std::unordered_map<uint64_t, int> mid;
@@ -85,6 +84,7 @@ extern "C" int gfs_icosphere(int tau, double* out_host, int64_t cap_rows) {
       const Vec& va = verts[size_t(a)];
       const Vec& vb = verts[size_t(b)];
       verts.push_back(scaled_unit(va.x + vb.x, va.y + vb.y, va.z + vb.z));
+      parents.emplace_back(a, b);
       int idx = int(verts.size()) - 1;
       mid.emplace(key, idx);
       return idx;
@@ -102,7 +102,36 @@ extern "C" int gfs_icosphere(int tau, double* out_host, int64_t cap_rows) {
     }
     faces.swap(next);
   }
-  if (int64_t(verts.size()) != K) return -1;
+  return int64_t(verts.size()) == K;
+}
+
+}  // namespace
+
+namespace gfs {
+
+bool icosphere_sources(int tau, int Ks, int* src) {
+  std::vector<Vec> verts;
+  std::vector<std::pair<int, int>> parents;
+  if (tau < 0 || tau > 7 || !src || Ks < (tau > 0 ? 12 : 0) || !icosphere_vertices(tau, verts, parents)) return false;
+  for (size_t k = 0; k < verts.size(); ++k) {
+    int e[2] = {parents[k].first, parents[k].second};
+    for (int& v : e)
+      while (v >= Ks) v = parents[size_t(v)].first;
+    src[2 * k] = e[0];
+    src[2 * k + 1] = e[1];
+  }
+  return true;
+}
+
+}  // namespace gfs
+
+extern "C" int gfs_icosphere(int tau, double* out_host, int64_t cap_rows) {
+  if (tau < 0 || tau > 7 || out_host == nullptr) return -1;
+  const int64_t K = 10 * (int64_t(1) << (2 * tau)) + 2;
+  if (cap_rows < K) return -1;
+  std::vector<Vec> verts;
+  std::vector<std::pair<int, int>> parents;
+  if (!icosphere_vertices(tau, verts, parents)) return -1;
   for (int64_t k = 0; k < K; ++k) {
     out_host[3 * k + 0] = verts[size_t(k)].x;
     out_host[3 * k + 1] = verts[size_t(k)].y;

@@ -117,7 +117,8 @@ __device__ __forceinline__ void cov_thresholds(double s64, float r32, float tol3
 
 __global__ void k_gather_spheres(const D4* __restrict__ sph64, const int* __restrict__ order, int64_t n,
                                  const BuildConsts* __restrict__ bc, float tol32, double tol,
-                                 float4* __restrict__ sph, float4* __restrict__ thr, int* __restrict__ sid) {
+                                 float4* __restrict__ sph, float4* __restrict__ thr, float4* __restrict__ cvl,
+                                 int* __restrict__ sid) {
   int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
   if (t >= n) return;
   int o = order[t];
@@ -132,6 +133,7 @@ __global__ void k_gather_spheres(const D4* __restrict__ sph64, const int* __rest
   cov_thresholds(d.w, fabsf(w), tol32, tol, bc->eq, A, lc, hc);
   cov_thresholds(d.w, fabsf(w), tol32, tol, kU * A, A, lq, hq);
   thr[t] = make_float4(lc, hc, lq, hq);
+  cvl[t] = make_float4(S.x, S.y, S.z, lc);
 }
 
 // ---------------------------------------------------------------------------
@@ -479,8 +481,10 @@ __device__ __forceinline__ float ord_val(unsigned k) {
 // spheres are a contiguous range of the Morton order) and raises the node's
 // per-radius maximum (same rounding bounds as the leaves).
 constexpr int kTight = 8;  // words per node: the four radii, then hip, -lop, -lon, hin
-__global__ void k_tighten_items(const float4* __restrict__ items, Tree T, float A, unsigned* __restrict__ keys) {
-  const int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+// (one warp: 32 aligned consecutive spheres of one tree; keys: of the tree's
+// nodes above the leaves)
+__device__ void tighten_items(const float4* __restrict__ items, const Tree& T, float A, unsigned* __restrict__ keys,
+                              int64_t i) {
   const bool live = i < T.nitems;
   const int lane = threadIdx.x & 31;
   const float4 v = live ? items[i] : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -521,11 +525,13 @@ __global__ void k_tighten_items(const float4* __restrict__ items, Tree T, float 
   }
 }
 
+__global__ void k_tighten_items(const float4* __restrict__ items, Tree T, float A, unsigned* __restrict__ keys) {
+  tighten_items(items, T, A, keys, blockIdx.x * int64_t(blockDim.x) + threadIdx.x);
+}
+
 // pass 2: each internal radius becomes the smaller of its bound through the
 // children and the exact maximum over its own spheres (same centre)
-__global__ void k_tighten_nodes(Tree T, const unsigned* __restrict__ keys, float A, int64_t nupper) {
-  const int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-  if (t >= nupper) return;
+__device__ void tighten_node(const Tree& T, const unsigned* __restrict__ keys, float A, int64_t t) {
   const int64_t node = T.offset[1] + t;
   const float4 B = T.nb[node];
   float4 Fc = T.nf[node];
@@ -549,6 +555,11 @@ __global__ void k_tighten_nodes(Tree T, const unsigned* __restrict__ keys, float
   float4 Ca = T.na[node];
   Ca.w = fmaxf(w[0], w[1]);
   T.na[node] = Ca;
+}
+
+__global__ void k_tighten_nodes(Tree T, const unsigned* __restrict__ keys, float A, int64_t nupper) {
+  const int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+  if (t < nupper) tighten_node(T, keys, A, t);
 }
 
 // Morton keys of query points (processing order of the packet kernel)
@@ -601,6 +612,17 @@ __device__ __forceinline__ void warp_count(unsigned long long* dst, unsigned lon
   if ((threadIdx.x & 31) == __ffs(mask) - 1 && v) atomicAdd(dst, v);
 }
 
+// segment of v in a prefix array (prefix[0] = 0, prefix[ns] = total)
+__device__ __forceinline__ int find_seg(const int64_t* __restrict__ prefix, int ns, int64_t v) {
+  int lo = 0, hi = ns;
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (prefix[mid] <= v) lo = mid;
+    else hi = mid;
+  }
+  return lo;
+}
+
 struct WarpStack {
   uint32_t* s;
   int sp;
@@ -629,198 +651,6 @@ struct WarpStack {
     __syncwarp();
   }
 };
-
-// ---------------------------------------------------------------------------
-// P build: coverage culling of the candidates q_ik = p_i + |s_i| u_k
-// ---------------------------------------------------------------------------
-// One lane per candidate; a warp holds 32 Morton-consecutive spheres with the
-// same direction k, so its candidates are spatial neighbours.  The warp walks
-// the sphere hierarchy as a packet (one node at a time, children visited if
-// any lane still needs them); a lane drops out at the first ball that covers
-// its candidate, and the warp stops when every lane is settled.
-// kCompact (single-shape launch, blocks of kCullBlock threads with one
-// direction k): after the neighbour pre-test the candidates still open in
-// the block are packed, in Morton order, into its first warps, so the walks
-// run with full warps (s_idx: one int per thread, s_wcnt: one per warp, in
-// shared memory).  Without it each
-// warp walks for its own lanes (the batched launch, where warps take
-// independent work items).
-template <bool kCompact>
-__device__ void cull_packet(const CullArgs& a, int64_t i, int k, WarpStack& W, int lane, int* s_idx, int* s_wcnt) {
-  bool active = i < a.n;
-  const BuildConsts bc = *a.bc;
-  float4 S = active ? a.sph[i] : make_float4(0.f, 0.f, 0.f, 0.f);
-  float r = fabsf(S.w);
-  const float ux = a.U32[3 * k], uy = a.U32[3 * k + 1], uz = a.U32[3 * k + 2];
-  float qx = fmaf(r, ux, S.x), qy = fmaf(r, uy, S.y), qz = fmaf(r, uz, S.z);
-  bool have64 = false;
-  double qx64 = 0, qy64 = 0, qz64 = 0;
-  unsigned long long rechecks = 0;
-  unsigned n_ntests = 0, n_items = 0;  // tests made for this lane while it is open
-  auto load64 = [&]() {
-    if (!have64) {
-      D4 pi = a.sph64[a.sid[i]];
-      ex_cand(pi, a.U64[3 * k], a.U64[3 * k + 1], a.U64[3 * k + 2], qx64, qy64, qz64);
-      have64 = true;
-    }
-  };
-  bool open = active;  // still looking for a covering ball
-  if (open && a.box_cull) {
-    const float mq = fmaxf(fabsf(qx), fmaxf(fabsf(qy), fabsf(qz)));
-    const float eb = 2.f * bc.eq;
-    if (mq > 1.f + eb) {
-      open = false;
-    } else if (mq >= 1.f - eb) {
-      load64();
-      ++rechecks;
-      if (!ex_inbox(qx64, qy64, qz64)) open = false;
-    }
-  }
-  // the warp's 32 spheres are Morton-consecutive: the spheres of lanes
-  // lane^1, ^2, ^4, ^8, ^16 are near neighbours, the balls most likely to
-  // cover this lane's candidate; a lane they settle skips the walk
-  {
-    const float4 Tho = active ? a.thr[i] : make_float4(-1.f, -1.f, -1.f, -1.f);
-    const int64_t base = i - lane;
-    for (int o = 1; o < 32; o <<= 1) {
-      const int src = lane ^ o;
-      const float4 P = make_float4(__shfl_sync(kFull, S.x, src), __shfl_sync(kFull, S.y, src),
-                                   __shfl_sync(kFull, S.z, src), __shfl_sync(kFull, S.w, src));
-      const float th_lo = __shfl_sync(kFull, Tho.x, src), th_hi = __shfl_sync(kFull, Tho.y, src);
-      const int64_t j = base + src;
-      if (!open || j >= a.n) continue;
-      const float dx = qx - P.x, dy = qy - P.y, dz = qz - P.z;
-      const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-      if (d2 < th_lo) {
-        open = false;
-      } else if (d2 <= th_hi) {
-        load64();
-        ++rechecks;
-        if (ex_cov(qx64, qy64, qz64, a.sph64[a.sid[j]], a.tol)) open = false;
-      }
-    }
-  }
-  // (a candidate that is still open here is in the box)
-  if constexpr (kCompact) {
-    const int wid = threadIdx.x >> 5;
-    const unsigned ballot = __ballot_sync(kFull, open);
-    if (lane == 0) s_wcnt[wid] = __popc(ballot);
-    __syncthreads();
-    int off = 0, total = 0;
-    for (int w = 0; w < int(blockDim.x >> 5); ++w) {
-      const int c = s_wcnt[w];
-      if (w < wid) off += c;
-      total += c;
-    }
-    if (open) s_idx[off + __popc(ballot & ((1u << lane) - 1u))] = int(threadIdx.x);
-    __syncthreads();
-    // this thread now walks for entry threadIdx.x of the packed list
-    if (rechecks) atomicAdd(&a.cnt->cull_rechecks, rechecks);
-    rechecks = 0;
-    if (wid * 32 >= total) return;  // warp-uniform: no entries left for this warp
-    const int64_t blk_base = i - int64_t(threadIdx.x);  // the block's first sphere
-    open = int(threadIdx.x) < total;
-    i = open ? blk_base + s_idx[threadIdx.x] : a.n;
-    active = open;
-    S = open ? a.sph[i] : make_float4(0.f, 0.f, 0.f, 0.f);
-    r = fabsf(S.w);
-    qx = fmaf(r, ux, S.x);
-    qy = fmaf(r, uy, S.y);
-    qz = fmaf(r, uz, S.z);
-    have64 = false;
-  }
-  const bool inbox = open;
-  const Tree& T = a.tree;
-  const float grow = 1.f + 8.f * kU;
-  if (__any_sync(kFull, open)) {
-    W.push_top(T, lane);
-    while (W.sp > 0 && __any_sync(kFull, open)) {
-      const uint32_t nd = W.pop();
-      const int lev = node_level(nd);
-      const int64_t idx = node_index(nd);
-      if (lev == 0) {
-        const int64_t b = idx * kLeaf, e = min(b + kLeaf, a.n);
-        n_items += open ? unsigned(e - b) : 0u;
-#pragma unroll
-        for (int jj = 0; jj < kLeaf; ++jj) {
-          const int64_t j = b + jj;
-          if (j >= e) break;
-          const float4 P = a.sph[j];
-          const float4 Th = a.thr[j];
-          if (!open || j == i) continue;
-          const float dx = qx - P.x, dy = qy - P.y, dz = qz - P.z;
-          const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-          if (d2 < Th.x) {
-            open = false;
-          } else if (d2 <= Th.y) {
-            load64();
-            ++rechecks;
-            if (ex_cov(qx64, qy64, qz64, a.sph64[a.sid[j]], a.tol)) open = false;
-          }
-        }
-      } else {
-        const int64_t cb = idx * kFan, ce = min(cb + kFan, T.count[lev - 1]);
-        const int64_t off = T.offset[lev - 1];
-        unsigned need = 0;
-        int first = -1, firstn = 0;
-        const int nc = int(ce - cb);
-        n_ntests += open ? unsigned(nc) : 0u;
-#pragma unroll
-        for (int c = 0; c < kFan; ++c) {
-          if (c >= nc) break;
-          // the node can hold a covering ball only if q lies in the ball
-          // B(C, max(wp, wn)) shrunk by tol
-          bool nd_c = false;
-          if (open) {
-            const float4 B = T.na[off + cb + c];
-            const float t = fmaf(B.w - a.tol32, grow, bc.pad);
-            nd_c = t > 0.f && ball_d2(qx, qy, qz, B) < t * t;
-          }
-          // visit first the child most lanes need
-          const unsigned votes = __ballot_sync(kFull, nd_c);
-          if (votes) {
-            need |= 1u << unsigned(c);
-            const int nv = __popc(votes);
-            if (nv > firstn) {
-              firstn = nv;
-              first = c;
-            }
-          }
-        }
-        W.push(lev - 1, cb, need, first, lane);
-      }
-    }
-  }
-  if (rechecks) atomicAdd(&a.cnt->cull_rechecks, rechecks);
-  warp_count(&a.cnt->c_ntests, n_ntests);
-  warp_count(&a.cnt->c_items, n_items);
-  if (!(inbox && open)) return;
-  // survivor: append to the list of its sign class (zero spheres: both)
-  const uint32_t g = uint32_t(a.sid[i]) * uint32_t(a.KS) + uint32_t(k);
-  const float4 item = make_float4(qx, qy, qz, __uint_as_float(g));
-  for (int c = 0; c < 2; ++c) {
-    const bool mine = c == 0 ? !(S.w < 0.f) : !(S.w > 0.f);
-    if (!mine) continue;
-    cg::coalesced_group grp = cg::coalesced_threads();
-    unsigned int base = 0;
-    if (grp.thread_rank() == 0) base = atomicAdd(&a.cnt->nsurv[c], grp.size());
-    base = grp.shfl(base, 0) + grp.thread_rank();
-    if (base < a.cap) {
-      a.surv[c][base] = item;
-      if (a.surv_shape[c]) a.surv_shape[c][base] = uint16_t(a.shape);
-    }
-  }
-}
-
-constexpr bool kCullCompact = true;
-constexpr int kCullBlock = 128;
-__global__ void __launch_bounds__(kCullBlock) k_cull(CullArgs a) {
-  __shared__ uint32_t s_stack[kCullBlock / 32][kPStack];
-  __shared__ int s_idx[kCullBlock], s_wcnt[kCullBlock / 32];
-  WarpStack W{s_stack[threadIdx.x >> 5], 0};
-  cull_packet<kCullCompact>(a, blockIdx.x * int64_t(blockDim.x) + threadIdx.x, blockIdx.y, W, threadIdx.x & 31,
-                            s_idx, s_wcnt);
-}
 
 // ---------------------------------------------------------------------------
 // query: FP32 pass with certification
@@ -1049,6 +879,7 @@ __device__ __forceinline__ void load_qstate(const uint4* st, int64_t slot, bool&
 
 }  // namespace gfs
 #include "gfs_sphere_pass.cuh"
+#include "gfs_cull.cuh"
 namespace gfs {
 
 // The rest of the query, starting from the sphere pass's state (a.state; the
@@ -1324,7 +1155,6 @@ __device__ void query_packet(const QueryArgs& a, int64_t slot, WarpStack& W, int
 // rho_max: a packet of G points of a uniform set of m fills a cube of side
 // 2 cbrt(G / m) of the box; packets half again as wide as that hold a jump of
 // the Morton order and go point by point.
-constexpr int kPacket = 16;
 constexpr int64_t kPacketMin = 131072;
 
 template <int G>
@@ -1665,8 +1495,8 @@ cudaError_t sort_keys_u32(void* temp, size_t& temp_bytes, const uint32_t* kin, u
 }
 
 cudaError_t launch_gather_spheres(const D4* sph64, const int* order, int64_t n, const BuildConsts* bc, float tol32,
-                                  double tol, float4* sph, float4* thr, int* sid, cudaStream_t st) {
-  k_gather_spheres<<<nblk(n, 256), 256, 0, st>>>(sph64, order, n, bc, tol32, tol, sph, thr, sid);
+                                  double tol, float4* sph, float4* thr, float4* cvl, int* sid, cudaStream_t st) {
+  k_gather_spheres<<<nblk(n, 256), 256, 0, st>>>(sph64, order, n, bc, tol32, tol, sph, thr, cvl, sid);
   ++g_launches;
   return cudaGetLastError();
 }
@@ -1723,10 +1553,39 @@ cudaError_t launch_gather_points(const float4* src, const int* order, int64_t n,
   return cudaGetLastError();
 }
 
-cudaError_t launch_cull(const CullArgs& a, cudaStream_t st) {
-  dim3 grid(nblk(a.n, kCullBlock), unsigned(a.K));
-  k_cull<<<grid, kCullBlock, 0, st>>>(a);
-  ++g_launches;
+// Level by level over chunks of tiles (the chunk bounds the covering-ball
+// array and the list; a level's list has room for every candidate).
+cudaError_t launch_cull(const CullArgs& one, const CullArgs* views, const int64_t* prefix, int ns, int64_t tiles,
+                        const CullWork& w, cudaStream_t st) {
+  CullSource s;
+  s.views = views;
+  s.prefix = prefix;
+  s.ns = ns;
+  s.hint = w.hint;
+  s.list = w.list;
+  s.KH = one.KH;
+  unsigned* count = w.count;
+  cudaError_t e = cudaMemsetAsync(w.count, 0, size_t(cull_launches(one.KH, tiles, w.chunk)) * 2 * sizeof(unsigned), st);
+  if (e != cudaSuccess) return e;
+  for (s.t0 = 0; s.t0 < tiles; s.t0 += w.chunk) {
+    s.tiles = std::min(w.chunk, tiles - s.t0);
+    s.k0 = 0;
+    for (int k1 = 12;; k1 = 4 * k1 - 6) {  // levels hold 12, 42, 162, ... directions (10 * 4^l + 2)
+      s.k1 = k1 > one.KH ? one.K : k1;     // past the kept levels the directions do not depend on one another
+      s.count = count;
+      count += 2;
+      const int dirs = s.k1 - s.k0;
+      // directions per warp: 16 spread a tile's loads and the list's atomics;
+      // fewer while the launch has less than 16 warps per SM
+      const int D = int(std::max<int64_t>(1, std::min<int64_t>(16, s.tiles * dirs / (152 * 16))));
+      const int chunks = (dirs + D - 1) / D;
+      k_cull_test<<<unsigned((s.tiles * chunks + 3) / 4), 128, 0, st>>>(one, s, D, chunks);
+      k_cull_walk<<<152 * 8, 128, 0, st>>>(one, s);
+      g_launches += 2;
+      if (s.k1 == one.K) break;
+      s.k0 = s.k1;
+    }
+  }
   return cudaGetLastError();
 }
 

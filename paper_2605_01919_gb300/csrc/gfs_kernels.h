@@ -23,12 +23,20 @@ struct ShapeDesc {
   uint16_t* flags_out;
 };
 
+// Two directions below Ks (the directions of the levels kept) for every
+// direction of the icosphere of depth tau from 12 on: its parents, or their
+// first ancestors that are kept.  Host; src: 2 K ints.  false on bad arguments.
+bool icosphere_sources(int tau, int Ks, int* src);
+
 struct CullArgs {
   const float4* sph;     // sorted spheres (x, y, z, s) FP32
   const float4* thr;     // sorted coverage thresholds (lo/hi for candidates, lo/hi for queries)
   const int* sid;        // sorted slot -> input index
   const D4* sph64;       // FP64 spheres in input order
-  const float* U32;      // K x 3 directions, FP32
+  const float4* cvl;     // sorted spheres' centres with the lower candidate threshold (x, y, z, thr.x)
+  const float4* U4;      // K directions, FP32 (x, y, z, -)
+  const int2* hsrc;      // per direction >= 12 two directions below KH near it (its parents, or ancestors of them)
+  int KH;                // directions whose covering balls the cull keeps (levels 0..min(tau - 1, 3))
   const double* U64;     // K x 3 directions, FP64
   int K, KS;             // K directions; KS = K + 1 ids per sphere
   Tree tree;             // sphere hierarchy
@@ -201,7 +209,8 @@ cudaError_t sort_pairs(void* temp, size_t& temp_bytes, const uint32_t* kin, uint
 cudaError_t sort_keys_u32(void* temp, size_t& temp_bytes, const uint32_t* kin, uint32_t* kout, int64_t n,
                           cudaStream_t st);
 cudaError_t launch_gather_spheres(const D4* sph64, const int* order, int64_t n, const BuildConsts* bc, float tol32,
-                                  double tol, float4* sph, float4* thr, int* sid, cudaStream_t st);
+                                  double tol, float4* sph, float4* thr, float4* cvl, int* sid,
+                                  cudaStream_t st);
 // scratch (spheres only, may be null): 8 * (nodes above the leaves) unsigned
 // words for tightening the internal bounds; null skips it
 cudaError_t launch_build_tree(const float4* items, int is_sphere, float A, Tree& T, unsigned* scratch,
@@ -210,7 +219,27 @@ cudaError_t launch_query_keys(const double* x64, const float* x32, int64_t m, ui
                               cudaStream_t st);
 cudaError_t launch_point_keys(const float4* items, int64_t n, uint32_t* keys, int* vals, cudaStream_t st);
 cudaError_t launch_gather_points(const float4* src, const int* order, int64_t n, float4* dst, cudaStream_t st);
-cudaError_t launch_cull(const CullArgs& a, cudaStream_t st);
+// The cull's workspace: covering balls, open list (see gfs_cull.cuh)
+struct CullWork {
+  int* hint;
+  uint32_t* list;
+  unsigned* count;
+  int64_t chunk;  // tiles per chunk
+};
+constexpr int kCullTileSpheres = 32;
+// launches pairs (levels x chunks) and the largest level's directions
+inline int cull_levels(int KH) {
+  int l = 1;
+  for (int k1 = 12; k1 <= KH; k1 = 4 * k1 - 6) ++l;
+  return l;
+}
+inline int64_t cull_launches(int KH, int64_t tiles, int64_t chunk) {
+  return cull_levels(KH) * ((tiles + chunk - 1) / chunk);
+}
+// Cull of one shape (views null: `one` is the shape) or of all shapes of a
+// batch (one: any view, for the options and table sizes)
+cudaError_t launch_cull(const CullArgs& one, const CullArgs* views, const int64_t* prefix, int ns, int64_t tiles,
+                        const CullWork& w, cudaStream_t st);
 // the query in two kernels: phase 1 (sphere pass, state to a.state), phase 2
 // (survivor pass, exact re-evaluation, flags, outputs)
 cudaError_t launch_query_spheres(const QueryArgs& a, cudaStream_t st);
@@ -228,11 +257,17 @@ cudaError_t launch_batch_copy(const ShapeDesc* d, const int64_t* off, int ns, in
 cudaError_t sort_pairs64(void* temp, size_t& bytes, const unsigned long long* kin, unsigned long long* kout,
                          const int* vin, int* vout, int64_t n, int end_bit, cudaStream_t st);
 cudaError_t launch_batch_gather(const D4* sph64, const int* order, const int64_t* off, int ns, int64_t N,
-                                const BuildConsts* bc, float tol32, double tol, float4* sph, float4* thr, int* sid,
-                                cudaStream_t st);
+                                const BuildConsts* bc, float tol32, double tol, float4* sph, float4* thr, float4* cvl,
+                                int* sid, cudaStream_t st);
 cudaError_t launch_batch_tree_level(const Tree* trees, const int64_t* prefix, int64_t total, int ns, int level,
                                     const float4* items_base, const int64_t* item_off, const BuildConsts* bc,
                                     int is_sphere, cudaStream_t st);
+// exact maxima for the internal bounds of all shapes' sample trees (keys: 8
+// words per node of the forest)
+cudaError_t launch_batch_tighten(const Tree* trees, const int64_t* prefix, const int64_t* level_total, int nlev, int ns,
+                                 const int64_t* tiles, int64_t ntiles, const float4* items_base,
+                                 const int64_t* item_off, const BuildConsts* bc, const float4* na0, int64_t nodes,
+                                 unsigned* keys, cudaStream_t st);
 cudaError_t launch_batch_hist(const uint16_t* shape, unsigned n, unsigned* counts, cudaStream_t st);
 cudaError_t launch_batch_surv_keys(const float4* items, const uint16_t* shape, unsigned n, unsigned long long* keys,
                                    int* vals, cudaStream_t st);
@@ -241,11 +276,6 @@ cudaError_t launch_batch_qkeys(const ShapeDesc* d, const int64_t* off, int ns, i
                                int* vals, cudaStream_t st);
 // phase 1: the sphere pass of every (shape, 32 points) item, phase 2: the rest
 // (reset ctr between the two launches)
-// cull over a group of shapes, one block per (shape, k, tile spheres) item
-// (tile 64, 128 or 256): bprefix holds each shape's first item, nblocks the
-// total
-cudaError_t launch_batch_cull_blocks(const CullArgs* views, const int64_t* bprefix, int ns, int64_t nblocks, int tile,
-                                     cudaStream_t st);
 cudaError_t launch_batch_query(const QueryArgs* views, const int64_t* wprefix, int ns, int64_t limit,
                                unsigned long long* ctr, int grid, int phase, cudaStream_t st);
 // the survivor forest of one class laid out and built on the device from the

@@ -345,12 +345,15 @@ __device__ bool sphere_pass(const QueryArgs& a, int64_t first, SpWarp& S, int la
   return true;
 }
 
-// A packet of 8, point by point where it has to be (the batched query; the
+// Points per packet; where packets begin is said at the launch.
+constexpr int kPacket = 16;
+
+// A full packet, point by point where it has to be (the batched query; the
 // single-shape query lists such packets for a second launch instead).
 __device__ void sphere_pass_any(const QueryArgs& a, int64_t first, SpWarp& S, int lane) {
-  if (sphere_pass<8>(a, first, S, lane, INFINITY)) return;
+  if (sphere_pass<kPacket>(a, first, S, lane, INFINITY)) return;
 #pragma unroll 1
-  for (int k = 0; k < 8 && first + k < a.m; ++k) {
+  for (int k = 0; k < kPacket && first + k < a.m; ++k) {
     __syncwarp();
     sphere_pass<1>(a, first + k, S, lane, INFINITY);
   }
