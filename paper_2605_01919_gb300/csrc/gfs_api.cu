@@ -571,7 +571,8 @@ int gfs_query(gfs_ctx* c, const void* x, int x_is_fp32, int64_t m, float* s_out,
     GFS_TRY(sort_u32_pairs(c, c->qk_in.as<uint32_t>(), c->qk_out.as<uint32_t>(), c->qv_in.as<int>(),
                            c->qv_out.as<int>(), m));
     a.perm = reinterpret_cast<const uint32_t*>(c->qv_out.p);
-    GFS_TRY(ensure(c->qstate, size_t(m) * 3 * sizeof(uint4)));
+    a.split = c->qk_in.as<uint32_t>();  // the unsorted keys are done with
+    GFS_TRY(ensure(c->qstate, size_t(m) * 4 * sizeof(uint4)));
     a.state = reinterpret_cast<uint4*>(c->qstate.p);
   }
   GFS_CK(cudaMemsetAsync(reinterpret_cast<char*>(c->cnt.p) + offsetof(Counters, query_rechecks), 0,
@@ -580,7 +581,7 @@ int gfs_query(gfs_ctx* c, const void* x, int x_is_fp32, int64_t m, float* s_out,
                          5 * sizeof(unsigned long long), c->stream));
   GFS_CK(cudaMemsetAsync(reinterpret_cast<char*>(c->cnt.p) + offsetof(Counters, ndefer), 0, sizeof(unsigned int),
                          c->stream));
-  GFS_CK(cudaMemsetAsync(reinterpret_cast<char*>(c->cnt.p) + offsetof(Counters, q_split), 0, 2 * sizeof(unsigned int),
+  GFS_CK(cudaMemsetAsync(reinterpret_cast<char*>(c->cnt.p) + offsetof(Counters, q_split), 0, 6 * sizeof(unsigned int),
                          c->stream));
   if (c->have_ev) GFS_CK(cudaEventRecord(c->ev[4], c->stream));
   if (c->opt.precision == 0) {
@@ -1262,7 +1263,7 @@ float time_grid(gfs_ctx* c, int grid, int64_t limit) {
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
   cudaEventRecord(e0, st);
-  for (int phase = 1; phase <= 2; ++phase) {
+  for (int phase = 1; phase <= 3; ++phase) {
     cudaMemsetAsync(c->b_ctr.p, 0, 8, st);
     launch_batch_query(c->b_qviews.as<QueryArgs>(), c->b_qw.as<int64_t>(), c->b_ns, limit,
                        c->b_ctr.as<unsigned long long>(), grid, phase, st);
@@ -1589,7 +1590,7 @@ int gfs_batch_build(gfs_ctx* c, const gfs_shape* shapes, int ns) {
   GFS_TRY(ensure(c->b_qkout, size_t(std::max<int64_t>(M, 1)) * 8));
   GFS_TRY(ensure(c->b_qvin, size_t(std::max<int64_t>(M, 1)) * 4));
   GFS_TRY(ensure(c->b_qvout, size_t(std::max<int64_t>(M, 1)) * 4));
-  GFS_TRY(ensure(c->b_qstate, size_t(std::max<int64_t>(M, 1)) * 3 * sizeof(uint4)));
+  GFS_TRY(ensure(c->b_qstate, size_t(std::max<int64_t>(M, 1)) * 4 * sizeof(uint4)));
   for (int s = 0; s < ns; ++s) {
     QueryArgs& a = qv[s];
     std::memset(&a, 0, sizeof(a));
@@ -1610,7 +1611,7 @@ int gfs_batch_build(gfs_ctx* c, const gfs_shape* shapes, int ns) {
     else a.x64 = static_cast<const double*>(shapes[s].x);
     a.m = shapes[s].m;
     a.perm = reinterpret_cast<const uint32_t*>(c->b_qvout.as<int>() + qoff[s]);
-    a.state = reinterpret_cast<uint4*>(c->b_qstate.p) + 3 * qoff[s];
+    a.state = reinterpret_cast<uint4*>(c->b_qstate.p) + 4 * qoff[s];
     a.s_out = shapes[s].s_out;
     a.s64_out = shapes[s].s64_out;
     a.arg_out = shapes[s].argmin_out;
@@ -1681,7 +1682,7 @@ int gfs_batch_query(gfs_ctx* c) {
   // the work counters of this query (a memset node under capture)
   GFS_CK(cudaMemsetAsync(reinterpret_cast<char*>(c->b_cnt.p) + offsetof(Counters, q_sphere_ntests), 0,
                          5 * sizeof(unsigned long long), st));
-  for (int phase = 1; phase <= 2; ++phase) {
+  for (int phase = 1; phase <= 3; ++phase) {
     GFS_CK(cudaMemsetAsync(c->b_ctr.p, 0, 8, st));
     GFS_CK(launch_batch_query(c->b_qviews.as<QueryArgs>(), c->b_qw.as<int64_t>(), ns, c->b_qtotal,
                               c->b_ctr.as<unsigned long long>(), grid, phase, st));

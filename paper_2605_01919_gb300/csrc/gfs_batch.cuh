@@ -159,13 +159,13 @@ __global__ void k_batch_qkeys(const ShapeDesc* __restrict__ d, const int64_t* __
 // Persistent query over all shapes: work item = (shape, 32 consecutive
 // points of the shape's Morton order).
 // kPhase 1: the sphere pass (state per point to the view's state array);
-// kPhase 2: the rest of the query (as the single-shape query's two kernels)
+// kPhase 2: the survivor pass; kPhase 3: the decisions (as the single-shape
+// query's kernels)
 template <int kPhase>
 __global__ void __launch_bounds__(128) k_batch_query(const QueryArgs* __restrict__ views,
                                                      const int64_t* __restrict__ wprefix, int ns, int64_t limit,
                                                      unsigned long long* __restrict__ ctr) {
-  using Shared = std::conditional_t<kPhase == 1, SpWarp, uint32_t[kPStack]>;
-  __shared__ Shared s_warp[4];
+  __shared__ SpWarp s_warp[4];
   const int lane = threadIdx.x & 31;
   for (;;) {
     unsigned long long w = 0;
@@ -174,13 +174,13 @@ __global__ void __launch_bounds__(128) k_batch_query(const QueryArgs* __restrict
     if (int64_t(w) >= limit) break;
     const int s = find_seg(wprefix, ns, int64_t(w));
     const int64_t wl = int64_t(w) - wprefix[s];
-    if constexpr (kPhase == 1) {
 #pragma unroll 1
-      for (int g = 0; g < 32; g += kPacket)
-        if (wl * 32 + g < views[s].m) sphere_pass_any(views[s], wl * 32 + g, s_warp[threadIdx.x >> 5], lane);
-    } else {
-      WarpStack W{s_warp[threadIdx.x >> 5], 0};
-      query_packet<true>(views[s], wl * 32 + lane, W, lane);
+    for (int g = 0; g < 32; g += kPacket) {
+      if (wl * 32 + g >= views[s].m) break;
+      if constexpr (kPhase == 1) sphere_pass_any<kPacket>(views[s], wl * 32 + g, s_warp[threadIdx.x >> 5], lane);
+      else if constexpr (kPhase == 2) near_pass_any<kPacket>(views[s], wl * 32 + g, s_warp[threadIdx.x >> 5], lane);
+      else decide_pass_any<kPacket>(views[s], wl * 32 + g, s_warp[threadIdx.x >> 5], lane);
+      __syncwarp();
     }
   }
 }
@@ -393,6 +393,7 @@ cudaError_t launch_batch_qkeys(const ShapeDesc* d, const int64_t* off, int ns, i
 cudaError_t launch_batch_query(const QueryArgs* views, const int64_t* wprefix, int ns, int64_t limit,
                                unsigned long long* ctr, int grid, int phase, cudaStream_t st) {
   if (phase == 1) k_batch_query<1><<<grid, 128, 0, st>>>(views, wprefix, ns, limit, ctr);
+  else if (phase == 3) k_batch_query<3><<<grid, 128, 0, st>>>(views, wprefix, ns, limit, ctr);
   else k_batch_query<2><<<grid, 128, 0, st>>>(views, wprefix, ns, limit, ctr);
   return cudaGetLastError();
 }

@@ -194,7 +194,9 @@ struct Counters {
   unsigned long long q_surv_items;     // survivors tested by the survivor pass
   unsigned long long c_ntests;         // child-node coverage tests of the cull (open lanes)
   unsigned long long c_items;          // sphere coverage tests of the cull (open lanes)
-  unsigned int q_split, q_split_next;  // packets the sphere pass left to its point-by-point launch, and that launch's cursor
+  // packets each of the query's passes (spheres, survivors, decisions) left to its point-by-point launch, and that
+  // launch's cursor
+  unsigned int q_split, q_split_next, f_split, f_split_next, d_split, d_split_next;
 };
 
 }  // namespace gfs

@@ -593,16 +593,6 @@ __global__ void k_gather_points(const float4* __restrict__ src, const int* __res
   dst[i] = src[order[i]];
 }
 
-// ---------------------------------------------------------------------------
-// Warp-cooperative ("packet") traversal.  The 32 lanes of a warp hold 32
-// query points that are neighbours in Morton order; they walk one hierarchy
-// together: the warp pops a node, every lane decides for its own point
-// whether the node can matter, and the node's children (or items) are
-// visited if any lane needs them.  Node and item records are read once per
-// warp (all lanes load the same address), control flow stays uniform, and
-// the stack lives in shared memory.
-// ---------------------------------------------------------------------------
-constexpr int kPStack = 128;  // >= kFan + (kFan-1)*(kMaxLevels-1)
 constexpr unsigned kFull = 0xffffffffu;
 
 // sum of v over the active lanes of the warp, added once to *dst
@@ -622,35 +612,6 @@ __device__ __forceinline__ int find_seg(const int64_t* __restrict__ prefix, int 
   }
   return lo;
 }
-
-struct WarpStack {
-  uint32_t* s;
-  int sp;
-  __device__ void push_top(const Tree& T, int lane) {
-    const int top = T.nlevels - 1;
-    const int cnt = int(T.count[top]);
-    if (lane < cnt) s[lane] = pack_node(top, lane);
-    sp = cnt;
-    __syncwarp();
-  }
-  __device__ uint32_t pop() {
-    const uint32_t nd = s[sp - 1];
-    --sp;
-    __syncwarp();
-    return nd;
-  }
-  // push the children whose bit is set in `need` (lane c writes child c),
-  // `first` last (visited next)
-  __device__ void push(int lev, int64_t cb, unsigned need, int first, int lane) {
-    const unsigned rest = first >= 0 ? need & ~(1u << unsigned(first)) : need;
-    const int nrest = __popc(rest);
-    if (lane < kFan && ((rest >> lane) & 1u))
-      s[sp + __popc(rest & ((1u << lane) - 1u))] = pack_node(lev, cb + lane);
-    if (first >= 0 && lane == 0) s[sp + nrest] = pack_node(lev, cb + first);
-    sp += nrest + (first >= 0 ? 1 : 0);
-    __syncwarp();
-  }
-};
 
 // ---------------------------------------------------------------------------
 // query: FP32 pass with certification
@@ -708,160 +669,21 @@ __device__ __forceinline__ void surv_pos64(const QueryArgs& a, uint32_t g, doubl
   }
 }
 
-// Warp-aggregated counter update (one atomic per warp)
-
-// Packet FP64 band pass over the sphere hierarchy.  A lane with band = true
-// finds, among the spheres whose FP32 value lies at or below its threshold
-// thr, the exact FP64 minimum and its input index (ties to the lowest index).
-// mode 0: |x-p| - r over sign class cls; mode 1: |x-p| + r over all spheres.
-__device__ double packet_band_sphere(const QueryArgs& a, const BuildConsts& bc, WarpStack& W, int lane, bool band,
-                                     double x64, double y64, double z64, float x, float y, float z, int mode,
-                                     int cls, float thr, int& arg) {
-  double best = INFINITY;
-  arg = INT_MAX;
-  if (!__any_sync(kFull, band)) return best;
-  const Tree& T = a.st;
-  const float grow = 1.f + 8.f * kU;
-  W.push_top(T, lane);
-  while (W.sp > 0) {
-    const uint32_t nd = W.pop();
-    const int lev = node_level(nd);
-    const int64_t idx = node_index(nd);
-    if (lev == 0) {
-      const int64_t b = idx * kLeaf, e = min(b + kLeaf, a.n);
-      for (int64_t j = b; j < e; ++j) {
-        const float4 P = a.sph[j];
-        if (!band) continue;
-        if (mode == 0 && (P.w == 0.f || int(P.w < 0.f) != cls)) continue;
-        const float dx = x - P.x, dy = y - P.y, dz = z - P.z;
-        const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-        const float r = fabsf(P.w);
-        const float v = mode == 0 ? __fsqrt_rn(d2) - r : __fsqrt_rn(d2) + r;
-        if (!(v <= thr)) continue;
-        const int o = a.sid[j];
-        const D4 pj = a.sph64[o];
-        const double dl = __dsqrt_rn(ex_d2(x64, y64, z64, pj.x, pj.y, pj.z));
-        const double v64 = mode == 0 ? __dsub_rn(dl, fabs(pj.w)) : __dadd_rn(dl, fabs(pj.w));
-        if (v64 < best || (v64 == best && o < arg)) {
-          best = v64;
-          arg = o;
-        }
-      }
-    } else {
-      const int64_t cb = idx * kFan, ce = min(cb + kFan, T.count[lev - 1]);
-      const int64_t off = T.offset[lev - 1];
-      unsigned need = 0;
-      for (int64_t c = cb; c < ce; ++c) {
-        bool nd_c = false;
-        if (band) {
-          float4 B;
-          float w;
-          if (mode == 1) {
-            B = T.nf[off + c];
-            w = B.w;
-          } else {
-            B = T.na[off + c];
-            const float4 R = T.nb[off + c];
-            w = cls == 0 ? R.x : R.y;
-          }
-          const float t = fmaf(thr + w, grow, bc.eprune);
-          nd_c = t > 0.f && ball_d2(x, y, z, B) < t * t;
-        }
-        if (__any_sync(kFull, nd_c)) need |= 1u << unsigned(c - cb);
-      }
-      W.push(lev - 1, cb, need, -1, lane);
-    }
-  }
-  return best;
-}
-
-// Packet FP64 band pass over the survivor hierarchy of class cls: exact
-// nearest survivor among those whose FP32 distance^2 is at most thr.
-__device__ double packet_band_surv(const QueryArgs& a, const BuildConsts& bc, WarpStack& W, int lane, bool band,
-                                   int cls, double x64, double y64, double z64, float x, float y, float z, float thr,
-                                   uint32_t& gbest) {
-  double best = INFINITY;
-  gbest = 0xffffffffu;
-  if (!__any_sync(kFull, band)) return best;
-  const Tree& T = a.vt[cls];
-  const float4* items = a.surv[cls];
-  const float grow = 1.f + 8.f * kU;
-  const float thn = band ? thr * grow + bc.ed_lin * __fsqrt_rn(thr) + 1e-30f : -1.f;
-  W.push_top(T, lane);
-  while (W.sp > 0) {
-    const uint32_t nd = W.pop();
-    const int lev = node_level(nd);
-    const int64_t idx = node_index(nd);
-    if (lev == 0) {
-      const int64_t b = idx * kLeaf, e = min(b + kLeaf, T.nitems);
-      for (int64_t j = b; j < e; ++j) {
-        const float4 P = items[j];
-        if (!band) continue;
-        const float dx = x - P.x, dy = y - P.y, dz = z - P.z;
-        const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-        if (!(d2 <= thr)) continue;
-        const uint32_t g = __float_as_uint(P.w);
-        double qx, qy, qz;
-        surv_pos64(a, g, qx, qy, qz);
-        const double e2 = ex_d2(x64, y64, z64, qx, qy, qz);
-        if (e2 < best || (e2 == best && g < gbest)) {
-          best = e2;
-          gbest = g;
-        }
-      }
-    } else {
-      const int64_t cb = idx * kFan, ce = min(cb + kFan, T.count[lev - 1]);
-      const int64_t off = T.offset[lev - 1];
-      unsigned need = 0;
-      for (int64_t c = cb; c < ce; ++c) {
-        const bool nd_c = box_d2(x, y, z, T.lo[off + c], T.hi[off + c]) < thn;
-        if (__any_sync(kFull, nd_c)) need |= 1u << unsigned(c - cb);
-      }
-      W.push(lev - 1, cb, need, -1, lane);
-    }
-  }
-  return best;
-}
-
 __device__ void query_exact_one(const QueryArgs& a, int64_t q);
 
-// One lane's query inside a warp-cooperative pass; `slot` indexes the
-// processing order (a.perm), all 32 lanes of the warp must call together.
-// Points outside the coordinate range of the FP32 error model go to the
-// FP64 kernel through a.defer, or (kInlineExact) are evaluated in place.
-// Greedy descent of a whole warp to one leaf: at every level lanes 0-7
-// score the 8 children, the lowest score (lowest child on ties, up to the
-// score's last 3 bits) is followed.  The score must be uniform across the
-// warp.
-template <class Score>
-__device__ int64_t warp_descend(const Tree& T, int lane, Score score) {
-  int lev = T.nlevels - 1;
-  int64_t cb = 0, ce = T.count[lev];
-  for (;;) {
-    const int c = lane & 7;
-    const float v = cb + c < ce ? score(T.offset[lev] + cb + c) : INFINITY;
-    const unsigned key = __reduce_min_sync(kFull, (ord_key(v) & ~7u) | unsigned(c));
-    const int64_t best = cb + (key & 7u);
-    if (lev == 0) return best;
-    cb = best * kFan;
-    ce = min(cb + kFan, T.count[lev - 1]);
-    --lev;
-  }
-}
-
-
-// Per-point state between the two phases of a split query (the sphere pass
-// and the rest), 48 B per processing slot.
+// Per-point state between the query's passes, 64 B per processing slot: the
+// sphere pass's results (48 B), then the nearest survivor (see near_pass).
+constexpr int kStateWords = 4;
 __device__ __forceinline__ void store_qstate(uint4* st, int64_t slot, bool c0, bool c1, int sample, const Top2& A0,
                                              const Top2& A1, const Top2& F) {
-  uint4* p = st + 3 * slot;
+  uint4* p = st + kStateWords * slot;
   p[0] = make_uint4(__float_as_uint(A0.best), __float_as_uint(A0.sec), unsigned(A0.idx), __float_as_uint(A1.best));
   p[1] = make_uint4(__float_as_uint(A1.sec), unsigned(A1.idx), __float_as_uint(F.best), __float_as_uint(F.sec));
   p[2] = make_uint4(unsigned(F.idx), unsigned(sample), (c0 ? 1u : 0u) | (c1 ? 2u : 0u), 0u);
 }
 __device__ __forceinline__ void load_qstate(const uint4* st, int64_t slot, bool& c0, bool& c1, int& sample, Top2& A0,
                                             Top2& A1, Top2& F) {
-  const uint4* p = st + 3 * slot;
+  const uint4* p = st + kStateWords * slot;
   const uint4 u0 = p[0], u1 = p[1], u2 = p[2];
   A0.best = __uint_as_float(u0.x);
   A0.sec = __uint_as_float(u0.y);
@@ -880,266 +702,14 @@ __device__ __forceinline__ void load_qstate(const uint4* st, int64_t slot, bool&
 }  // namespace gfs
 #include "gfs_sphere_pass.cuh"
 #include "gfs_cull.cuh"
+#include "gfs_finish_pass.cuh"
 namespace gfs {
 
-// The rest of the query, starting from the sphere pass's state (a.state; the
-// same points in the same order).
-template <bool kInlineExact>
-__device__ void query_packet(const QueryArgs& a, int64_t slot, WarpStack& W, int lane) {
-  const bool active = slot < a.m;
-  const int64_t q = active ? int64_t(a.perm ? a.perm[slot] : uint32_t(slot)) : 0;
-  const BuildConsts bc = *a.bc;
-  double x64 = 0.0, y64 = 0.0, z64 = 0.0;
-  if (active) load_query(a, q, x64, y64, z64);
-  const float x = float(x64), y = float(y64), z = float(z64);
-  unsigned n_snodes = 0, n_sitems = 0, n_band = 0;
-  bool defer = active && !(fabs(x64) <= bc.A && fabs(y64) <= bc.A && fabs(z64) <= bc.A);
-  bool live = active && !defer;
-  const float grow = 1.f + 8.f * kU;
-  const float ea2 = 2.f * bc.ea;
-  // warp centre, used to order children (nearest first)
-  float cx = live ? x : 0.f, cy = live ? y : 0.f, cz = live ? z : 0.f;
-  float cnt = live ? 1.f : 0.f;
-  for (int o = 16; o > 0; o >>= 1) {
-    cx += __shfl_xor_sync(kFull, cx, o);
-    cy += __shfl_xor_sync(kFull, cy, o);
-    cz += __shfl_xor_sync(kFull, cz, o);
-    cnt += __shfl_xor_sync(kFull, cnt, o);
-  }
-  if (cnt > 0.f) {
-    cx /= cnt;
-    cy /= cnt;
-    cz /= cnt;
-  }
-  // ---- the sphere pass's results (per-class state as scalars: indexing a
-  // register array would push it to local memory)
-  bool cov0 = false, cov1 = false;
-  Top2 A0, A1, F;
-  top2_init(A0);
-  top2_init(A1);
-  top2_init(F);
-  int sample = INT_MAX;
-  if (active) load_qstate(a.state, slot, cov0, cov1, sample, A0, A1, F);
-  int code = -1;
-  double value = 0.0;
-  int64_t arg = -1;
-  int flags = 0;
-  if (live) {
-    if (sample != INT_MAX) {
-      code = GFS_CODE_SAMPLE;
-      value = a.sph64[sample].w;
-      arg = sample;
-    } else if (cov0 && cov1) {
-      code = GFS_CODE_INVALID;
-      value = __longlong_as_double(0x7ff8000000000000LL);
-    } else if (!cov0 && !cov1) {
-      code = GFS_CODE_OUTSIDE;
-    }
-    if (code >= 0) flags = code;
-  }
-  const bool open = live && code < 0;
-  const int cs = cov0 ? 0 : 1, co = 1 - cs;
-  const Top2 As = cs == 0 ? A0 : A1;   // x's own class
-  const Top2 Ao = cs == 0 ? A1 : A0;   // the opposite class
-  // ---- pass over the survivors of each lane's sign ------------------------
-  float bd = INFINITY, sd = INFINITY;
-  uint32_t gbest = 0xffffffffu;
-  auto band = [&](float D) { return bc.ed_lin * __fsqrt_rn(D) + bc.ed_quad * D + 1e-30f; };
-  for (int cl = 0; cl < 2; ++cl) {
-    const bool mine = open && cs == cl;
-    if (!__any_sync(kFull, mine) || a.vt[cl].nlevels == 0) continue;
-    const Tree& T = a.vt[cl];
-    const float4* items = a.surv[cl];
-    float th = mine ? INFINITY : -1.f;   // threshold on d^2
-    float thn = th;                      // widened for node tests
-    auto surv_leaf = [&](int64_t idx) {
-        const int64_t b = idx * kLeaf, e = min(b + kLeaf, T.nitems);
-        n_sitems += mine ? unsigned(e - b) : 0u;
-        for (int64_t j = b; j < e; ++j) {
-          const float4 P = items[j];
-          const float dx = x - P.x, dy = y - P.y, dz = z - P.z;
-          const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-          if (d2 < th) {
-            if (d2 < bd) {
-              sd = bd;
-              bd = d2;
-              gbest = __float_as_uint(P.w);
-            } else {
-              sd = d2;
-            }
-            th = fminf(sd, bd + 2.f * band(bd));
-            thn = th * grow + bc.ed_lin * __fsqrt_rn(th) + 1e-30f;
-          }
-        }
-    };
-    // seed the threshold with the leaf nearest the packet centre (the walk
-    // skips it)
-    const int64_t seeded =
-        warp_descend(T, lane, [&](int64_t node) { return box_d2(cx, cy, cz, T.lo[node], T.hi[node]); });
-    surv_leaf(seeded);
-    W.push_top(T, lane);
-    while (W.sp > 0) {
-      const uint32_t nd = W.pop();
-      const int lev = node_level(nd);
-      const int64_t idx = node_index(nd);
-      if (lev == 0) {
-        if (idx != seeded) surv_leaf(idx);
-      } else {
-        const int64_t cb = idx * kFan, ce = min(cb + kFan, T.count[lev - 1]);
-        const int64_t off = T.offset[lev - 1];
-        const int nc = int(ce - cb);
-        n_snodes += mine ? unsigned(nc) : 0u;
-        unsigned mine_c = 0, key = 0xffffffffu;
-#pragma unroll
-        for (int c = 0; c < kFan; ++c) {
-          if (c < nc && mine) {
-            const float4 L = T.lo[off + cb + c], H = T.hi[off + cb + c];
-            if (box_d2(x, y, z, L, H) < thn) {
-              mine_c |= 1u << c;
-              key = min(key, (__float_as_uint(box_d2(cx, cy, cz, L, H)) & ~7u) | unsigned(c));
-            }
-          }
-        }
-        const unsigned need = __reduce_or_sync(kFull, mine_c);
-        const int first = need ? int(__reduce_min_sync(kFull, key) & 7u) : -1;
-        W.push(lev - 1, cb, need, first, lane);
-      }
-    }
-  }
-  const bool have_s = open && gbest != 0xffffffffu, have_u = open && Ao.idx >= 0;
-  // exact nearest survivor: direct when no other survivor lies in the error
-  // band, else an FP64 pass over the band
-  double ds = INFINITY;
-  bool sband = have_s && !(sd >= bd + 2.f * band(bd));
-  if (have_s && !sband) {
-    double qx, qy, qz;
-    surv_pos64(a, gbest, qx, qy, qz);
-    ds = __dsqrt_rn(ex_d2(x64, y64, z64, qx, qy, qz));
-  }
-  for (int cl = 0; cl < 2; ++cl) {
-    uint32_t g2;
-    const bool mine = sband && cs == cl;
-    const double e2 = packet_band_surv(a, bc, W, lane, mine, cl, x64, y64, z64, x, y, z,
-                                       mine ? bd + 2.f * band(bd) : -1.f, g2);
-    if (mine) {
-      ++n_band;
-      ds = __dsqrt_rn(e2);
-      gbest = g2;
-    }
-  }
-  // exact nearest opposite tangent point
-  double ub = INFINITY;
-  int uj = -1;
-  const bool uband = have_u && !(Ao.sec >= Ao.best + ea2);
-  if (have_u && !uband) {
-    uj = a.sid[Ao.idx];
-    const D4 pj = a.sph64[uj];
-    ub = __dsub_rn(__dsqrt_rn(ex_d2(x64, y64, z64, pj.x, pj.y, pj.z)), fabs(pj.w));
-  }
-  {
-    int j2;
-    const double v = packet_band_sphere(a, bc, W, lane, uband, x64, y64, z64, x, y, z, 0, co,
-                                        uband ? Ao.best + ea2 : -1.f, j2);
-    if (uband) {
-      ++n_band;
-      ub = v;
-      uj = j2;
-    }
-  }
-  // value and the result code
-  double m = 0.0;
-  bool need_lb = false;
-  if (open) {
-    if (have_s && (!a.clamp_opp || ds <= ub)) {
-      code = GFS_CODE_SURVIVOR;
-      m = ds;
-      arg = int64_t(gbest);
-    } else if (a.clamp_opp && have_u) {
-      code = GFS_CODE_OPPOSITE;
-      m = ub;
-      arg = uj;
-    } else {
-      code = GFS_CODE_LOWER;
-      need_lb = true;
-    }
-  }
-  const double E = double(bc.ea) * 1.01 + 1e-15;
-  const double lbt = -double(As.best) - a.tol;
-  const double ft = double(F.best) + a.tol;
-  if (open && code != GFS_CODE_LOWER) {
-    const double mm = m < 0.0 ? 0.0 : m;
-    need_lb = !(mm < lbt - E) && !(mm > lbt + E);
-  }
-  // exact lower bound LB (max over the lane's class of r - |x-p|) if needed
-  double lb = 0.0;
-  int lj = -1;
-  const bool lband = need_lb && !(As.sec >= As.best + ea2);
-  if (need_lb && !lband) {
-    lj = a.sid[As.idx];
-    const D4 pl = a.sph64[lj];
-    lb = __dsub_rn(fabs(pl.w), __dsqrt_rn(ex_d2(x64, y64, z64, pl.x, pl.y, pl.z)));
-  }
-  {
-    int j2;
-    const double v = packet_band_sphere(a, bc, W, lane, lband, x64, y64, z64, x, y, z, 0, cs,
-                                        lband ? As.best + ea2 : -1.f, j2);
-    if (lband) {
-      ++n_band;
-      lb = -v;
-      lj = j2;
-    }
-  }
-  if (open && code == GFS_CODE_LOWER) {
-    m = lb;
-    arg = lj;
-  }
-  if (m < 0.0) m = 0.0;
-  // exact far bound if the FP32 margin does not decide FAR_VIOL
-  const bool need_far = open && !(m > ft + E) && !(m < ft - E);
-  const bool fband = need_far && !(F.sec >= F.best + ea2);
-  double far = INFINITY;
-  if (need_far && !fband) {
-    const D4 pf = a.sph64[a.sid[F.idx]];
-    far = __dadd_rn(__dsqrt_rn(ex_d2(x64, y64, z64, pf.x, pf.y, pf.z)), fabs(pf.w));
-  }
-  {
-    int j2;
-    const double v = packet_band_sphere(a, bc, W, lane, fband, x64, y64, z64, x, y, z, 1, 0,
-                                        fband ? F.best + ea2 : -1.f, j2);
-    if (fband) {
-      ++n_band;
-      far = v;
-    }
-  }
-  if (open) {
-    flags = code;
-    if (m < lbt - E) flags |= GFS_FLAG_LB_VIOL;
-    else if (need_lb && m < __dsub_rn(lb, a.tol)) flags |= GFS_FLAG_LB_VIOL;
-    if (m > ft + E) flags |= GFS_FLAG_FAR_VIOL;
-    else if (need_far && m > __dadd_rn(far, a.tol)) flags |= GFS_FLAG_FAR_VIOL;
-    if (have_u && ub < __dsub_rn(m, a.tol)) flags |= GFS_FLAG_OPP_VIOL;
-    value = cs == 0 ? m : -m;
-  }
-  warp_count(&a.cnt->q_surv_ntests, n_snodes);
-  warp_count(&a.cnt->q_band_passes, n_band);
-  warp_count(&a.cnt->q_surv_items, n_sitems);
-  if (live) {
-    write_result(a, q, value, arg, flags);
-  } else if (defer) {
-    // outside the coordinate range the error bounds assume: FP64 path
-    const unsigned int s2 = atomicAdd(&a.cnt->ndefer, 1u);
-    if constexpr (kInlineExact) {
-      query_exact_one(a, q);
-    } else {
-      if (s2 < a.defer_cap) a.defer[s2] = uint32_t(q);
-    }
-  }
-}
-
-// The query as two kernels: the sphere pass (state to a.state), then the
-// survivor pass and the rest.  Each holds less live state than one kernel
-// doing both would, so more warps fit per SM (15% faster on the 64^3 union
-// workload than the fused packet code, which the batched kernel keeps).
+// The query as three kernels: the sphere pass and the survivor pass (results
+// to a.state), then the decisions.  Each holds less live state and code than
+// one kernel doing all would: with the last two in one, a quarter of the
+// stalls were instruction fetches.
+//
 // One warp per block: packets differ widely in work, and a block of several
 // warps would hold its slots until its slowest one is done.
 // Packets of 16 points from kPacketMin points on, when there are at least as
@@ -1153,15 +723,19 @@ __device__ void query_packet(const QueryArgs& a, int64_t slot, WarpStack& W, int
 //   30k points on 16^3 samples          0.10 / 0.21 / 0.28 / 0.39
 //   32k random points, 64^3 samples     0.52 / 1.01 / 1.28 / 1.81
 // rho_max: a packet of G points of a uniform set of m fills a cube of side
-// 2 cbrt(G / m) of the box; packets half again as wide as that hold a jump of
-// the Morton order and go point by point.
+// 2 cbrt(G / m) of the box; a packet whose radius is three such sides holds a
+// jump of the Morton order and goes point by point (sphere pass of the first
+// two, at 1.5 / 2.5 / 4 sides and without the rule: 30.6 / 21.5 / 20.3 / 22.3 and
+// 40.4 / 38.7 / 39.6 / 40.1 ms; at 1.5 a sixth of the first one's packets,
+// those that straddle the grid's octants, went point by point).
+constexpr float kJump = 6.f;
 constexpr int64_t kPacketMin = 131072;
 
 template <int G>
 __global__ void __launch_bounds__(32, 28) k_query_spheres(QueryArgs a, float rho_max) {
   __shared__ SpWarp S;
   if (!sphere_pass<G>(a, int64_t(blockIdx.x) * G, S, threadIdx.x, rho_max) && threadIdx.x == 0)
-    a.defer[atomicAdd(&a.cnt->q_split, 1u)] = blockIdx.x;
+    a.split[atomicAdd(&a.cnt->q_split, 1u)] = blockIdx.x;
 }
 
 // The points of the packets that k_query_spheres<G> listed, one at a time.
@@ -1174,16 +748,57 @@ __global__ void __launch_bounds__(32, 28) k_query_spheres_split(QueryArgs a) {
     if (threadIdx.x == 0) t = atomicAdd(&a.cnt->q_split_next, 1u);
     t = __shfl_sync(kFull, t, 0);
     if (int64_t(t) >= total) return;
-    const int64_t slot = int64_t(a.defer[t / G]) * G + t % G;
+    const int64_t slot = int64_t(a.split[t / G]) * G + t % G;
     __syncwarp();
     if (slot < a.m) sphere_pass<1>(a, slot, S, threadIdx.x, INFINITY);
   }
 }
 
-__global__ void __launch_bounds__(128, 7) k_query_finish(QueryArgs a) {
-  __shared__ uint32_t s_stack[4][kPStack];
-  WarpStack W{s_stack[threadIdx.x >> 5], 0};
-  query_packet<false>(a, blockIdx.x * int64_t(blockDim.x) + threadIdx.x, W, threadIdx.x & 31);
+// The survivor pass, split the same way.
+template <int G>
+__global__ void __launch_bounds__(32, 28) k_query_near(QueryArgs a, float rho_max) {
+  __shared__ SpWarp S;
+  if (!near_pass<G>(a, int64_t(blockIdx.x) * G, S, threadIdx.x, rho_max) && threadIdx.x == 0)
+    a.split[atomicAdd(&a.cnt->f_split, 1u)] = blockIdx.x;
+}
+
+template <int G>
+__global__ void __launch_bounds__(32, 28) k_query_near_split(QueryArgs a) {
+  __shared__ SpWarp S;
+  const int64_t total = int64_t(a.cnt->f_split) * G;
+  for (;;) {
+    unsigned t = 0;
+    if (threadIdx.x == 0) t = atomicAdd(&a.cnt->f_split_next, 1u);
+    t = __shfl_sync(kFull, t, 0);
+    if (int64_t(t) >= total) return;
+    const int64_t slot = int64_t(a.split[t / G]) * G + t % G;
+    __syncwarp();
+    if (slot < a.m) near_pass<1>(a, slot, S, threadIdx.x, INFINITY);
+  }
+}
+
+// The decisions, split the same way (packets of 8 / 16 / 32 on 16.2M points,
+// 64^3 samples: 18.3 / 14.9 / 15.9 ms; 2.1M random points, 96^3: 8.6 / 9.4 / 12.4).
+template <int G>
+__global__ void __launch_bounds__(32, 24) k_query_decide(QueryArgs a, float rho_max) {
+  __shared__ SpWarp S;
+  if (!decide_pass<G, false>(a, int64_t(blockIdx.x) * G, S, threadIdx.x, rho_max) && threadIdx.x == 0)
+    a.split[atomicAdd(&a.cnt->d_split, 1u)] = blockIdx.x;
+}
+
+template <int G>
+__global__ void __launch_bounds__(32, 24) k_query_decide_split(QueryArgs a) {
+  __shared__ SpWarp S;
+  const int64_t total = int64_t(a.cnt->d_split) * G;
+  for (;;) {
+    unsigned t = 0;
+    if (threadIdx.x == 0) t = atomicAdd(&a.cnt->d_split_next, 1u);
+    t = __shfl_sync(kFull, t, 0);
+    if (int64_t(t) >= total) return;
+    const int64_t slot = int64_t(a.split[t / G]) * G + t % G;
+    __syncwarp();
+    if (slot < a.m) decide_pass<1, false>(a, slot, S, threadIdx.x, INFINITY);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -1594,7 +1209,7 @@ cudaError_t launch_query_spheres(const QueryArgs& a, cudaStream_t st) {
   if (a.m < kPacketMin || a.m < a.n) {
     k_query_spheres<1><<<unsigned(a.m), 32, 0, st>>>(a, INFINITY);
   } else {
-    const float rho_max = 3.f * cbrtf(float(kPacket) / float(a.m));
+    const float rho_max = kJump * cbrtf(float(kPacket) / float(a.m));
     k_query_spheres<kPacket><<<nblk(a.m, kPacket), 32, 0, st>>>(a, rho_max);
     k_query_spheres_split<kPacket><<<152 * 28, 32, 0, st>>>(a);
     ++g_launches;
@@ -1605,7 +1220,17 @@ cudaError_t launch_query_spheres(const QueryArgs& a, cudaStream_t st) {
 
 cudaError_t launch_query_finish(const QueryArgs& a, cudaStream_t st) {
   if (a.m == 0) return cudaSuccess;
-  k_query_finish<<<nblk(a.m, 128), 128, 0, st>>>(a);
+  if (a.m < kPacketMin || a.m < a.n) {
+    k_query_near<1><<<unsigned(a.m), 32, 0, st>>>(a, INFINITY);
+    k_query_decide<1><<<unsigned(a.m), 32, 0, st>>>(a, INFINITY);
+  } else {
+    const float rho_max = kJump * cbrtf(float(kPacket) / float(a.m));
+    k_query_near<kPacket><<<nblk(a.m, kPacket), 32, 0, st>>>(a, rho_max);
+    k_query_near_split<kPacket><<<152 * 28, 32, 0, st>>>(a);
+    k_query_decide<kPacket><<<nblk(a.m, kPacket), 32, 0, st>>>(a, rho_max);
+    k_query_decide_split<kPacket><<<152 * 24, 32, 0, st>>>(a);
+    g_launches += 2;
+  }
   ++g_launches;
   return cudaGetLastError();
 }

@@ -79,7 +79,8 @@ struct QueryArgs {
   uint32_t* defer;
   unsigned int defer_cap;
   Counters* cnt;
-  uint4* state;             // 3 x uint4 per processing slot, between the query's two kernels
+  uint32_t* split;          // packets to take point by point (room for m)
+  uint4* state;             // 4 x uint4 per processing slot, between the query's passes
 };
 
 // One pending step of the insertion window: its value against the state at

@@ -33,12 +33,14 @@ namespace gfs {
 
 constexpr int kSpStack = 448;  // >= kFan + 28 entries per level: 4 popped, at most 32 pushed, deepest level on top
 constexpr int kSpQueue = 64;
+constexpr int kCand = 8;
 
 struct SpWarp {
   uint32_t stk[kSpStack];
   float4 qp[kSpQueue];
   int qi[kSpQueue];
   int2 lv[kMaxLevels];  // (first node, nodes) of each level
+  int cand[kCand * 32]; // per lane: items awaiting their FP64 evaluation (second pass)
 };
 
 __device__ __forceinline__ float sqrt_fast(float v) {
@@ -348,12 +350,13 @@ __device__ bool sphere_pass(const QueryArgs& a, int64_t first, SpWarp& S, int la
 // Points per packet; where packets begin is said at the launch.
 constexpr int kPacket = 16;
 
-// A full packet, point by point where it has to be (the batched query; the
-// single-shape query lists such packets for a second launch instead).
+// A packet of G, point by point where it has to be.
+template <int G>
 __device__ void sphere_pass_any(const QueryArgs& a, int64_t first, SpWarp& S, int lane) {
-  if (sphere_pass<kPacket>(a, first, S, lane, INFINITY)) return;
+  if constexpr (G > 1)
+    if (sphere_pass<G>(a, first, S, lane, INFINITY)) return;
 #pragma unroll 1
-  for (int k = 0; k < kPacket && first + k < a.m; ++k) {
+  for (int k = 0; k < G && first + k < a.m; ++k) {
     __syncwarp();
     sphere_pass<1>(a, first + k, S, lane, INFINITY);
   }
