@@ -482,7 +482,7 @@ int build_finish(gfs_ctx* c) {
     a.sph64 = c->sph64.as<D4>();
     a.cvl = c->cvl.as<float4>();
     a.U4 = c->U4.as<float4>();
-    a.hsrc = c->hsrc.as<int2>();
+    a.hsrc = c->hsrc.as<int>();
     a.KH = c->KH;
     a.U64 = c->U64.as<double>();
     a.K = c->K;
@@ -1512,7 +1512,7 @@ int gfs_batch_build(gfs_ctx* c, const gfs_shape* shapes, int ns) {
       a.sph64 = c->b_sph64.as<D4>() + off[s];
       a.cvl = c->b_cvl.as<float4>() + off[s];
       a.U4 = c->U4.as<float4>();
-      a.hsrc = c->hsrc.as<int2>();
+      a.hsrc = c->hsrc.as<int>();
       a.KH = c->KH;
       a.U64 = c->U64.as<double>();
       a.K = c->K;

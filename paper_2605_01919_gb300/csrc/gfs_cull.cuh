@@ -26,92 +26,6 @@
 namespace gfs {
 
 constexpr int kCullTile = kCullTileSpheres;
-constexpr int kCullStack = 512;
-
-struct CullShared {
-  int2 lv[kMaxLevels];
-};
-
-// A ball other than sphere `own` (sorted slots) that, shrunk by tol, contains
-// the candidate (qx, qy, qz) of direction k, or -1.  The whole warp calls it
-// with the same arguments.  Node test: some sphere of the node satisfies
-// |q - p| - |s| < -tol only if its linear bound stays below -tol and the
-// margins of the bound and of q's FP32 rounding.
-__device__ int cover_walk(const CullArgs& a, const CullShared& C, uint32_t* stk, int lane, float qx, float qy,
-                          float qz, int64_t own, int k, float lim, unsigned& rechecks, unsigned& n_nodes,
-                          unsigned& n_items) {
-  const Tree& T = a.tree;
-  const int top = T.nlevels - 1, grp = lane >> 3, sub = lane & 7;
-  int sp = C.lv[top].y;
-  __syncwarp();
-  if (lane < sp) stk[lane] = pack_node(top, lane);
-  __syncwarp();
-  while (sp > 0) {
-    // past 408 entries one at a time, so that at most 7 per level join them
-    const int take = min(min(sp, 4), max(1, (kCullStack - 96 - sp) / kFan));
-    const uint32_t nd = grp < take ? stk[sp - 1 - grp] : 0xffffffffu;
-    sp -= take;
-    const int lev = node_level(nd);
-    const int c = int(node_index(nd)) * kFan + sub;
-    bool pass = false, cov = false;
-    float v = INFINITY;
-    if (nd != 0xffffffffu) {
-      if (lev == 0) {
-        if (c < a.n) {
-          ++n_items;
-          const float4 P = a.cvl[c];
-          const float hi = a.thr[c].y;
-          const float dx = qx - P.x, dy = qy - P.y, dz = qz - P.z;
-          const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-          if (c != own && d2 <= hi) {
-            cov = d2 < P.w;
-            v = d2 - P.w;
-            if (!cov) {
-              ++rechecks;
-              double x, y, z;
-              ex_cand(a.sph64[a.sid[own]], a.U64[3 * k], a.U64[3 * k + 1], a.U64[3 * k + 2], x, y, z);
-              cov = ex_cov(x, y, z, a.sph64[a.sid[c]], a.tol);
-            }
-          }
-        }
-      } else {
-        const int2 L = C.lv[lev - 1];
-        if (c < L.y) {
-          ++n_nodes;
-          const Lin r = lin_load(T, L.x + c);
-          float nx = qx - r.cx, ny = qy - r.cy, nz = qz - r.cz;
-          const float d = unit3(nx, ny, nz);
-          const float sp_ = fmaf(fabsf(nx + r.gx), r.hx, fmaf(fabsf(ny + r.gy), r.hy, fabsf(nz + r.gz) * r.hz));
-          const float sm_ = fmaf(fabsf(nx - r.gx), r.hx, fmaf(fabsf(ny - r.gy), r.hy, fabsf(nz - r.gz) * r.hz));
-          v = fminf(d - r.hip - sp_, d + r.lon - sm_);
-          pass = v <= lim;
-        }
-      }
-    }
-    // the ball that holds the candidate most deeply is the best hint later
-    if (__any_sync(kFull, cov)) {
-      const unsigned key = cov ? ord_key(v) : 0xffffffffu;
-      return __shfl_sync(kFull, c, __ffs(__ballot_sync(kFull, key == __reduce_min_sync(kFull, key))) - 1);
-    }
-    // the child that reaches deepest around the candidate goes on top, below
-    // it those that reach at least half as deep
-    const unsigned key = pass ? ord_key(v) : 0xffffffffu;
-    const unsigned low = __reduce_min_sync(kFull, key);
-    const unsigned bn = __ballot_sync(kFull, pass);
-    const unsigned bq = __ballot_sync(kFull, pass && v < 0.5f * ord_val(low));
-    if (pass) {
-      const unsigned bb = __ballot_sync(bn, key == low);
-      const unsigned best = bb & (0u - bb), rest = bn & ~bq & ~best, good = bq & ~best, me = 1u << lane;
-      const int at = (me & best) ? __popc(bn) - 1
-                                 : ((me & good) ? __popc(rest) + __popc(good & (me - 1u)) : __popc(rest & (me - 1u)));
-      stk[sp + at] = pack_node(lev - 1, c);
-    }
-    sp += __popc(bn);
-    __syncwarp();
-  }
-  return -1;
-}
-
 // The tile (32 spheres) of one warp: its shape's arguments, first sphere and
 // place in the covering-ball array.
 struct CullTile {
@@ -181,7 +95,7 @@ __global__ void __launch_bounds__(128) k_cull_test(const __grid_constant__ CullA
     }
     if (k >= 12) {
       // d2 < lo: covered for certain (what lies nearer the boundary is left to the walk)
-      const int2 src = a.hsrc[k];
+      const int2 src = reinterpret_cast<const int2*>(a.hsrc)[k];
       const int h0 = tile.hint[src.x * 32 + lane], h1 = tile.hint[src.y * 32 + lane];
       if (open && h0 >= 0) {
         const float4 P = a.cvl[h0];
@@ -236,11 +150,11 @@ __global__ void __launch_bounds__(128) k_cull_test(const __grid_constant__ CullA
 // The listed candidates, a warp each; survivors are gathered 32 at a time
 // (lane l keeps the l-th) for one atomic per class and flush.
 __global__ void __launch_bounds__(128) k_cull_walk(const __grid_constant__ CullArgs one, const CullSource s) {
-  __shared__ uint32_t s_stk[4][kCullStack];
-  __shared__ CullShared s_lv[4];
+  __shared__ uint32_t s_stk[4][kCoverStack];
+  __shared__ LevelTable s_lv[4];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   uint32_t* stk = s_stk[w];
-  CullShared& C = s_lv[w];
+  LevelTable& C = s_lv[w];
   const unsigned n = s.count[0];
   const uint32_t dirs = uint32_t(s.k1 - s.k0);
   unsigned rechecks = 0, n_nodes = 0, n_items = 0;
@@ -301,18 +215,28 @@ __global__ void __launch_bounds__(128) k_cull_walk(const __grid_constant__ CullA
     const CullArgs& a = *tile.a;
     cnt = a.cnt;
     if (loaded != tile.a) {
-      __syncwarp();
-      if (lane < kMaxLevels) C.lv[lane] = make_int2(int(a.tree.offset[lane]), int(a.tree.count[lane]));
+      load_levels(a.tree, C, lane);
       loaded = tile.a;
-      __syncwarp();
     }
     const int64_t i = tile.base + src;
     const float4 S = a.sph[i];
     const float r = fabsf(S.w);
     const float lim = -a.tol32 + a.bc->elin + 4.f * a.bc->eq;
     const float4 u = a.U4[k];
-    const int j = cover_walk(a, C, stk, lane, fmaf(r, u.x, S.x), fmaf(r, u.y, S.y), fmaf(r, u.z, S.z), i, k, lim,
-                             rechecks, n_nodes, n_items);
+    const float qx = fmaf(r, u.x, S.x), qy = fmaf(r, u.y, S.y), qz = fmaf(r, u.z, S.z);
+    const int j = warp_cover_walk(a.tree, C, stk, lane, qx, qy, qz, lim, n_nodes, n_items, [&](int c, float& v) {
+      const float4 P = a.cvl[c];
+      const float hi = a.thr[c].y;
+      const float dx = qx - P.x, dy = qy - P.y, dz = qz - P.z;
+      const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+      if (c == i || !(d2 <= hi)) return false;
+      v = d2 - P.w;
+      if (d2 < P.w) return true;
+      ++rechecks;
+      double x, y, z;
+      ex_cand(a.sph64[a.sid[i]], a.U64[3 * k], a.U64[3 * k + 1], a.U64[3 * k + 2], x, y, z);
+      return ex_cov(x, y, z, a.sph64[a.sid[c]], a.tol);
+    });
     if (j >= 0) {
       if (k < s.KH && lane == 0) tile.hint[k * 32 + src] = j;
     } else {

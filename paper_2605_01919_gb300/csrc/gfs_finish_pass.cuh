@@ -139,12 +139,6 @@ __device__ bool packet_walk(const Tree& T, SpWarp& S, int lane, int budget, Node
   return true;
 }
 
-__device__ __forceinline__ void load_levels(const Tree& T, SpWarp& S, int lane) {
-  __syncwarp();
-  if (lane < kMaxLevels) S.lv[lane] = make_int2(int(T.offset[lane]), int(T.count[lane]));
-  __syncwarp();
-}
-
 // Exact FP64 minimum over the spheres whose FP32 value lies at or below the
 // point's threshold thr, and its input index (ties to the lowest), for the
 // points with band set (idx: the sorted slot of the FP32 minimum).  Returns
@@ -153,7 +147,7 @@ __device__ __forceinline__ void load_levels(const Tree& T, SpWarp& S, int lane) 
 template <int G>
 __device__ bool sphere_band(const QueryArgs& a, const BuildConsts& bc, SpWarp& S, int lane, bool band, int idx,
                             double x64, double y64, double z64, float x, float y, float z, int mode, int cls,
-                            float thr, float rho_max, double& best, int& arg) {
+                            float thr, const PkLimit& lim, double& best, int& arg) {
   constexpr int kParts = 32 / G;
   const int part = lane / G;
   best = INFINITY;
@@ -161,7 +155,7 @@ __device__ bool sphere_band(const QueryArgs& a, const BuildConsts& bc, SpWarp& S
   const unsigned bm = __ballot_sync(kFull, band);
   if (!bm) return true;
   const Pk k = packet_of<G>(band, x, y, z, bc.A);
-  if (G > 1 && k.rho > rho_max * bc.A) return false;
+  if (G > 1 && k.rho > lim.rho * bc.A) return false;
   const Tree& T = a.st;
   // the point's spheres within the band, evaluated in FP64 by all lanes
   // together: done where found they would run one lane at a time on an FP64
@@ -186,7 +180,7 @@ __device__ bool sphere_band(const QueryArgs& a, const BuildConsts& bc, SpWarp& S
   ref_dir(r, k, a.sph[__shfl_sync(kFull, idx, __ffs(bm) - 1)]);
   ref_thr(r, k, band, thr, x, y, z);
   const bool done = packet_walk<G>(
-      T, S, lane, G > 1 ? kSpBudget * G : -1,
+      T, S, lane, G > 1 ? lim.rest * G : -1,
       [&](int64_t nd) {
         const Lin q = lin_load(T, nd);
         float nx = k.cx - q.cx, ny = k.cy - q.cy, nz = k.cz - q.cz;
@@ -353,7 +347,7 @@ __device__ bool near_survivor(const QueryArgs& a, const BuildConsts& bc, SpWarp&
 // is at most thr, for the points with band set (j: the FP32 nearest's slot).
 template <int G>
 __device__ bool surv_band(const QueryArgs& a, const BuildConsts& bc, SpWarp& S, int lane, bool band, int cls, int j,
-                          double x64, double y64, double z64, float x, float y, float z, float thr, float rho_max,
+                          double x64, double y64, double z64, float x, float y, float z, float thr, const PkLimit& lim,
                           double& best, uint32_t& gbest) {
   constexpr int kParts = 32 / G;
   const int part = lane / G;
@@ -362,7 +356,7 @@ __device__ bool surv_band(const QueryArgs& a, const BuildConsts& bc, SpWarp& S, 
   const unsigned bm = __ballot_sync(kFull, band);
   if (!bm) return true;
   const Pk k = packet_of<G>(band, x, y, z, bc.A);
-  if (G > 1 && k.rho > rho_max * bc.A) return false;
+  if (G > 1 && k.rho > lim.rho * bc.A) return false;
   const Tree& T = a.vt[cls];
   const float4* items = a.surv[cls];
   int nc = 0;  // as in sphere_band
@@ -386,7 +380,7 @@ __device__ bool surv_band(const QueryArgs& a, const BuildConsts& bc, SpWarp& S, 
   ref_thr(r, k, band, band ? sqrtf(thr) : 0.f, x, y, z);
   const float margin = bc.elin + 8.f * bc.eq;
   const bool done = packet_walk<G>(
-      T, S, lane, G > 1 ? kSpBudget * G : -1,
+      T, S, lane, G > 1 ? lim.rest * G : -1,
       [&](int64_t nd) {
         float nx, ny, nz;
         const float d = box_dir(k, T.lo[nd], T.hi[nd], nx, ny, nz);
@@ -426,7 +420,7 @@ __device__ bool surv_band(const QueryArgs& a, const BuildConsts& bc, SpWarp& S, 
 // state's fourth word.  false: nothing written, the packet's points go one by
 // one (as in sphere_pass).
 template <int G>
-__device__ bool near_pass(const QueryArgs& a, int64_t first, SpWarp& S, int lane, float rho_max) {
+__device__ bool near_pass(const QueryArgs& a, int64_t first, SpWarp& S, int lane, const PkLimit& lim) {
   const int64_t slot = first + (lane & (G - 1));
   const bool active = slot < a.m;
   const int64_t q = active ? int64_t(a.perm ? a.perm[slot] : uint32_t(slot)) : 0;
@@ -447,7 +441,7 @@ __device__ bool near_pass(const QueryArgs& a, int64_t first, SpWarp& S, int lane
   const bool open = live && sample == INT_MAX && cov0 != cov1;
   const int cs = cov0 ? 0 : 1;
   if constexpr (G > 1) {
-    if (__any_sync(kFull, open) && packet_of<G>(open, x, y, z, bc.A).rho > rho_max * bc.A) return false;
+    if (__any_sync(kFull, open) && packet_of<G>(open, x, y, z, bc.A).rho > lim.rho * bc.A) return false;
   }
   Near N;
   N.bd = N.sd = INFINITY;
@@ -457,7 +451,7 @@ __device__ bool near_pass(const QueryArgs& a, int64_t first, SpWarp& S, int lane
     const bool mine = open && cs == cl;
     if (!__any_sync(kFull, mine) || a.vt[cl].nlevels == 0) continue;
     Near M;
-    if (!near_survivor<G>(a, bc, S, lane, mine, cl, x, y, z, G > 1 ? kSpBudget * G : -1, M, n_nodes, n_items))
+    if (!near_survivor<G>(a, bc, S, lane, mine, cl, x, y, z, G > 1 ? lim.rest * G : -1, M, n_nodes, n_items))
       return false;
     if (mine) N = M;
   }
@@ -474,7 +468,7 @@ __device__ bool near_pass(const QueryArgs& a, int64_t first, SpWarp& S, int lane
 // a.defer, or (kInlineExact) are evaluated in place.  false: nothing written,
 // the packet's points go one by one.
 template <int G, bool kInlineExact>
-__device__ bool decide_pass(const QueryArgs& a, int64_t first, SpWarp& S, int lane, float rho_max) {
+__device__ bool decide_pass(const QueryArgs& a, int64_t first, SpWarp& S, int lane, const PkLimit& lim) {
   const int part = lane / G;
   const int64_t slot = first + (lane & (G - 1));
   const bool active = slot < a.m;
@@ -544,7 +538,7 @@ __device__ bool decide_pass(const QueryArgs& a, int64_t first, SpWarp& S, int la
     uint32_t g2;
     const bool mine = sband && cs == cl;
     double e2;
-    if (!surv_band<G>(a, bc, S, lane, mine, cl, N.j, x64, y64, z64, x, y, z, mine ? sthr : -1.f, rho_max, e2, g2))
+    if (!surv_band<G>(a, bc, S, lane, mine, cl, N.j, x64, y64, z64, x, y, z, mine ? sthr : -1.f, lim, e2, g2))
       return false;
     if (mine) {
       ++n_band;
@@ -567,7 +561,7 @@ __device__ bool decide_pass(const QueryArgs& a, int64_t first, SpWarp& S, int la
     const bool mine = uband && co == cl;
     double v;
     if (!sphere_band<G>(a, bc, S, lane, mine, Ao.idx, x64, y64, z64, x, y, z, 0, cl,
-                        mine ? Ao.best + ea2 : -1.f, rho_max, v, j2))
+                        mine ? Ao.best + ea2 : -1.f, lim, v, j2))
       return false;
     if (mine) {
       ++n_band;
@@ -614,7 +608,7 @@ __device__ bool decide_pass(const QueryArgs& a, int64_t first, SpWarp& S, int la
     const bool mine = lband && cs == cl;
     double v;
     if (!sphere_band<G>(a, bc, S, lane, mine, As.idx, x64, y64, z64, x, y, z, 0, cl,
-                        mine ? As.best + ea2 : -1.f, rho_max, v, j2))
+                        mine ? As.best + ea2 : -1.f, lim, v, j2))
       return false;
     if (mine) {
       ++n_band;
@@ -639,7 +633,7 @@ __device__ bool decide_pass(const QueryArgs& a, int64_t first, SpWarp& S, int la
     int j2;
     double v;
     if (!sphere_band<G>(a, bc, S, lane, fband, F.idx, x64, y64, z64, x, y, z, 1, 0,
-                        fband ? F.best + ea2 : -1.f, rho_max, v, j2))
+                        fband ? F.best + ea2 : -1.f, lim, v, j2))
       return false;
     if (fband) {
       ++n_band;
@@ -675,21 +669,21 @@ __device__ bool decide_pass(const QueryArgs& a, int64_t first, SpWarp& S, int la
 // A packet of G, point by point where it has to be.
 template <int G>
 __device__ void decide_pass_any(const QueryArgs& a, int64_t first, SpWarp& S, int lane) {
-  if (decide_pass<G, true>(a, first, S, lane, INFINITY)) return;
+  if (decide_pass<G, true>(a, first, S, lane, no_jump())) return;
 #pragma unroll 1
   for (int k = 0; k < G && first + k < a.m; ++k) {
     __syncwarp();
-    decide_pass<1, true>(a, first + k, S, lane, INFINITY);
+    decide_pass<1, true>(a, first + k, S, lane, no_jump());
   }
 }
 
 template <int G>
 __device__ void near_pass_any(const QueryArgs& a, int64_t first, SpWarp& S, int lane) {
-  if (near_pass<G>(a, first, S, lane, INFINITY)) return;
+  if (near_pass<G>(a, first, S, lane, no_jump())) return;
 #pragma unroll 1
   for (int k = 0; k < G && first + k < a.m; ++k) {
     __syncwarp();
-    near_pass<1>(a, first + k, S, lane, INFINITY);
+    near_pass<1>(a, first + k, S, lane, no_jump());
   }
 }
 

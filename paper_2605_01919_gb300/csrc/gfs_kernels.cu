@@ -24,6 +24,7 @@
 
 #include "gfs_internal.cuh"
 #include "gfs_kernels.h"
+#include "gfs_warp.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -712,29 +713,43 @@ namespace gfs {
 //
 // One warp per block: packets differ widely in work, and a block of several
 // warps would hold its slots until its slowest one is done.
-// Packets of 16 points from kPacketMin points on, when there are at least as
-// many points as spheres; below, a warp per point (a packet's points then lie
-// many sample spacings apart, and a heavy packet would end long after the
-// rest).  Sphere pass in ms, warp per point / packets of 8 / 16 / 32:
-//   16.2M points on 64^3 samples       101.4 / 38.2 / 30.6 / 36.5
-//   2.1M random points, 96^3 samples    69.8 / 44.0 / 40.3 / 42.9
-//   227k points on 16^3 samples         0.62 / 0.33 / 0.39 / 0.54
-//   100k random points, 32^3 samples    0.42 / 0.46 / 0.63 / 0.95
-//   30k points on 16^3 samples          0.10 / 0.21 / 0.28 / 0.39
-//   32k random points, 64^3 samples     0.52 / 1.01 / 1.28 / 1.81
-// rho_max: a packet of G points of a uniform set of m fills a cube of side
+// Points per packet.  A packet's nodes are tested once for all its points,
+// but the wider it is against the spacing of the spheres the more of them
+// matter to some point, and a heavy packet ends long after the rest, which
+// shows when there are few.  Sphere pass in ms, warp per point / packets of
+// 8 / 16 / 32 (the first without the point-by-point launch: 16 / 38.2 / 32.7):
+//   16.2M points on 64^3 samples       101.4 / 29.3 / 21.6 / 36.5
+//   2.1M random points, 96^3 samples    69.8 / 43.8 / 39.8 / 42.9
+//   118k points on 13^3 samples         0.43 / 0.18 / 0.18
+//   100k random points, 32^3 samples    0.42 / 0.35 / 0.40
+//   30k random points, 32^3 samples     0.16 / 0.47 / 0.75
+//   32k random points, 64^3 samples     0.53 / 1.04 / 1.26
+// lim.rho: a packet of G points of a uniform set of m fills a cube of side
 // 2 cbrt(G / m) of the box; a packet whose radius is three such sides holds a
 // jump of the Morton order and goes point by point (sphere pass of the first
 // two, at 1.5 / 2.5 / 4 sides and without the rule: 30.6 / 21.5 / 20.3 / 22.3 and
 // 40.4 / 38.7 / 39.6 / 40.1 ms; at 1.5 a sixth of the first one's packets,
 // those that straddle the grid's octants, went point by point).
+// lim.spheres, lim.rest: the first two want 600 units a point in the sphere
+// pass (at 300 / 150 the second takes 51 / 74 ms: its packets are heavy
+// throughout) and about 100 in the others (600 / 128 / 64 / 32: 10.9 / 9.0 /
+// 10.0 / 12.6 ms); few points want less, for the sake of the last packets (100k
+// on 32^3, both passes after the spheres: 1.16 / 0.60 / 0.54 / 0.50 ms).
 constexpr float kJump = 6.f;
-constexpr int64_t kPacketMin = 131072;
+static int packet_size(const QueryArgs& a) {
+  if (a.m >= 131072 && a.m >= a.n) return kPacket;
+  if (a.m >= 24576 && a.m >= 3 * a.n) return 8;
+  return 1;
+}
+static PkLimit packet_limit(int G, int64_t m) {
+  const float rho = kJump * cbrtf(float(G) / float(m));
+  return G == 1 ? no_jump() : (G == kPacket ? PkLimit{rho, 600, 100} : PkLimit{rho, 80, 32});
+}
 
 template <int G>
-__global__ void __launch_bounds__(32, 28) k_query_spheres(QueryArgs a, float rho_max) {
+__global__ void __launch_bounds__(32, 28) k_query_spheres(QueryArgs a, PkLimit lim) {
   __shared__ SpWarp S;
-  if (!sphere_pass<G>(a, int64_t(blockIdx.x) * G, S, threadIdx.x, rho_max) && threadIdx.x == 0)
+  if (!sphere_pass<G>(a, int64_t(blockIdx.x) * G, S, threadIdx.x, lim) && threadIdx.x == 0)
     a.split[atomicAdd(&a.cnt->q_split, 1u)] = blockIdx.x;
 }
 
@@ -750,15 +765,15 @@ __global__ void __launch_bounds__(32, 28) k_query_spheres_split(QueryArgs a) {
     if (int64_t(t) >= total) return;
     const int64_t slot = int64_t(a.split[t / G]) * G + t % G;
     __syncwarp();
-    if (slot < a.m) sphere_pass<1>(a, slot, S, threadIdx.x, INFINITY);
+    if (slot < a.m) sphere_pass<1>(a, slot, S, threadIdx.x, no_jump());
   }
 }
 
 // The survivor pass, split the same way.
 template <int G>
-__global__ void __launch_bounds__(32, 28) k_query_near(QueryArgs a, float rho_max) {
+__global__ void __launch_bounds__(32, 28) k_query_near(QueryArgs a, PkLimit lim) {
   __shared__ SpWarp S;
-  if (!near_pass<G>(a, int64_t(blockIdx.x) * G, S, threadIdx.x, rho_max) && threadIdx.x == 0)
+  if (!near_pass<G>(a, int64_t(blockIdx.x) * G, S, threadIdx.x, lim) && threadIdx.x == 0)
     a.split[atomicAdd(&a.cnt->f_split, 1u)] = blockIdx.x;
 }
 
@@ -773,16 +788,16 @@ __global__ void __launch_bounds__(32, 28) k_query_near_split(QueryArgs a) {
     if (int64_t(t) >= total) return;
     const int64_t slot = int64_t(a.split[t / G]) * G + t % G;
     __syncwarp();
-    if (slot < a.m) near_pass<1>(a, slot, S, threadIdx.x, INFINITY);
+    if (slot < a.m) near_pass<1>(a, slot, S, threadIdx.x, no_jump());
   }
 }
 
 // The decisions, split the same way (packets of 8 / 16 / 32 on 16.2M points,
 // 64^3 samples: 18.3 / 14.9 / 15.9 ms; 2.1M random points, 96^3: 8.6 / 9.4 / 12.4).
 template <int G>
-__global__ void __launch_bounds__(32, 24) k_query_decide(QueryArgs a, float rho_max) {
+__global__ void __launch_bounds__(32, 24) k_query_decide(QueryArgs a, PkLimit lim) {
   __shared__ SpWarp S;
-  if (!decide_pass<G, false>(a, int64_t(blockIdx.x) * G, S, threadIdx.x, rho_max) && threadIdx.x == 0)
+  if (!decide_pass<G, false>(a, int64_t(blockIdx.x) * G, S, threadIdx.x, lim) && threadIdx.x == 0)
     a.split[atomicAdd(&a.cnt->d_split, 1u)] = blockIdx.x;
 }
 
@@ -797,7 +812,7 @@ __global__ void __launch_bounds__(32, 24) k_query_decide_split(QueryArgs a) {
     if (int64_t(t) >= total) return;
     const int64_t slot = int64_t(a.split[t / G]) * G + t % G;
     __syncwarp();
-    if (slot < a.m) decide_pass<1, false>(a, slot, S, threadIdx.x, INFINITY);
+    if (slot < a.m) decide_pass<1, false>(a, slot, S, threadIdx.x, no_jump());
   }
 }
 
@@ -1204,34 +1219,43 @@ cudaError_t launch_cull(const CullArgs& one, const CullArgs* views, const int64_
   return cudaGetLastError();
 }
 
-cudaError_t launch_query_spheres(const QueryArgs& a, cudaStream_t st) {
-  if (a.m == 0) return cudaSuccess;
-  if (a.m < kPacketMin || a.m < a.n) {
-    k_query_spheres<1><<<unsigned(a.m), 32, 0, st>>>(a, INFINITY);
-  } else {
-    const float rho_max = kJump * cbrtf(float(kPacket) / float(a.m));
-    k_query_spheres<kPacket><<<nblk(a.m, kPacket), 32, 0, st>>>(a, rho_max);
-    k_query_spheres_split<kPacket><<<152 * 28, 32, 0, st>>>(a);
+template <int G>
+static void query_spheres(const QueryArgs& a, cudaStream_t st) {
+  k_query_spheres<G><<<nblk(a.m, G), 32, 0, st>>>(a, packet_limit(G, a.m));
+  ++g_launches;
+  if constexpr (G > 1) {
+    k_query_spheres_split<G><<<152 * 28, 32, 0, st>>>(a);
     ++g_launches;
   }
-  ++g_launches;
+}
+
+template <int G>
+static void query_rest(const QueryArgs& a, cudaStream_t st) {
+  const PkLimit lim = packet_limit(G, a.m);
+  k_query_near<G><<<nblk(a.m, G), 32, 0, st>>>(a, lim);
+  if constexpr (G > 1) k_query_near_split<G><<<152 * 28, 32, 0, st>>>(a);
+  k_query_decide<G><<<nblk(a.m, G), 32, 0, st>>>(a, lim);
+  if constexpr (G > 1) k_query_decide_split<G><<<152 * 24, 32, 0, st>>>(a);
+  g_launches += G > 1 ? 4 : 2;
+}
+
+cudaError_t launch_query_spheres(const QueryArgs& a, cudaStream_t st) {
+  if (a.m == 0) return cudaSuccess;
+  switch (packet_size(a)) {
+    case 1: query_spheres<1>(a, st); break;
+    case 8: query_spheres<8>(a, st); break;
+    default: query_spheres<kPacket>(a, st);
+  }
   return cudaGetLastError();
 }
 
 cudaError_t launch_query_finish(const QueryArgs& a, cudaStream_t st) {
   if (a.m == 0) return cudaSuccess;
-  if (a.m < kPacketMin || a.m < a.n) {
-    k_query_near<1><<<unsigned(a.m), 32, 0, st>>>(a, INFINITY);
-    k_query_decide<1><<<unsigned(a.m), 32, 0, st>>>(a, INFINITY);
-  } else {
-    const float rho_max = kJump * cbrtf(float(kPacket) / float(a.m));
-    k_query_near<kPacket><<<nblk(a.m, kPacket), 32, 0, st>>>(a, rho_max);
-    k_query_near_split<kPacket><<<152 * 28, 32, 0, st>>>(a);
-    k_query_decide<kPacket><<<nblk(a.m, kPacket), 32, 0, st>>>(a, rho_max);
-    k_query_decide_split<kPacket><<<152 * 24, 32, 0, st>>>(a);
-    g_launches += 2;
+  switch (packet_size(a)) {
+    case 1: query_rest<1>(a, st); break;
+    case 8: query_rest<8>(a, st); break;
+    default: query_rest<kPacket>(a, st);
   }
-  ++g_launches;
   return cudaGetLastError();
 }
 

@@ -35,7 +35,7 @@ struct CullArgs {
   const D4* sph64;       // FP64 spheres in input order
   const float4* cvl;     // sorted spheres' centres with the lower candidate threshold (x, y, z, thr.x)
   const float4* U4;      // K directions, FP32 (x, y, z, -)
-  const int2* hsrc;      // per direction >= 12 two directions below KH near it (its parents, or ancestors of them)
+  const int* hsrc;       // per direction >= 12 two directions below KH near it (its parents, or ancestors of them)
   int KH;                // directions whose covering balls the cull keeps (levels 0..min(tau - 1, 3))
   const double* U64;     // K x 3 directions, FP64
   int K, KS;             // K directions; KS = K + 1 ids per sphere

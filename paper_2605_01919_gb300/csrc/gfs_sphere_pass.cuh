@@ -35,29 +35,12 @@ constexpr int kSpStack = 448;  // >= kFan + 28 entries per level: 4 popped, at m
 constexpr int kSpQueue = 64;
 constexpr int kCand = 8;
 
-struct SpWarp {
+struct SpWarp : LevelTable {
   uint32_t stk[kSpStack];
   float4 qp[kSpQueue];
   int qi[kSpQueue];
-  int2 lv[kMaxLevels];  // (first node, nodes) of each level
   int cand[kCand * 32]; // per lane: items awaiting their FP64 evaluation (second pass)
 };
-
-__device__ __forceinline__ float sqrt_fast(float v) {
-  float r;
-  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
-  return r;
-}
-
-// distance and unit direction of (x, y, z) (direction 0 at distance 0)
-__device__ __forceinline__ float unit3(float& x, float& y, float& z) {
-  const float q = fmaf(x, x, fmaf(y, y, z * z));
-  const float inv = q > 1e-36f ? rsqrtf(q) : 0.f;
-  x *= inv;
-  y *= inv;
-  z *= inv;
-  return q * inv;
-}
 
 // reference sphere of one quantity at the packet centre
 struct SpRef {
@@ -74,13 +57,18 @@ __device__ __forceinline__ void top2_merge(Top2& t, int o) {
   }
 }
 
-// Returns false (nothing stored) when the packet is better served point by
-// point: its points lie far apart (a jump of the Morton order), or the walk
-// has spent kSpBudget units (a round 6, an evaluation 1) per point.
-constexpr int kSpBudget = 600;
+// Limits of a packet beyond which it is better served point by point: the
+// radius (a jump of the Morton order), and the units a walk may spend per
+// point (a round 6, an evaluation 1) in the sphere pass and in the others.
+struct PkLimit {
+  float rho;
+  int spheres, rest;
+};
+__host__ __device__ inline PkLimit no_jump() { return PkLimit{INFINITY, 600, 100}; }
 
+// Returns false (nothing stored) past the limits.
 template <int G>
-__device__ bool sphere_pass(const QueryArgs& a, int64_t first, SpWarp& S, int lane, float rho_max) {
+__device__ bool sphere_pass(const QueryArgs& a, int64_t first, SpWarp& S, int lane, const PkLimit& lim) {
   constexpr int kParts = 32 / G;
   const int part = lane / G;
   const int64_t slot = first + (lane & (G - 1));
@@ -120,7 +108,7 @@ __device__ bool sphere_pass(const QueryArgs& a, int64_t first, SpWarp& S, int la
       rho = sqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
     }
     rho = __uint_as_float(__reduce_max_sync(kFull, __float_as_uint(rho))) * (1.f + 16.f * kU) + 4.f * kU * bc.A;
-    if (G > 1 && rho > rho_max * bc.A) return false;
+    if (G > 1 && rho > lim.rho * bc.A) return false;
     __syncwarp();
     const int top = T.nlevels - 1, grp = lane >> 3, sub = lane & 7;
     // ---- references: a beam of 4 nodes per quantity, down to 4 leaves ------
@@ -277,7 +265,7 @@ __device__ bool sphere_pass(const QueryArgs& a, int64_t first, SpWarp& S, int la
     __syncwarp();
     while (sp > 0) {
       if constexpr (G > 1) {
-        if (spent > kSpBudget * G) return false;
+        if (spent > lim.spheres * G) return false;
         spent += 6;
       }
       const int take = min(min(sp, 4), max(1, (kSpStack - 32 - sp) / kFan));
@@ -354,11 +342,11 @@ constexpr int kPacket = 16;
 template <int G>
 __device__ void sphere_pass_any(const QueryArgs& a, int64_t first, SpWarp& S, int lane) {
   if constexpr (G > 1)
-    if (sphere_pass<G>(a, first, S, lane, INFINITY)) return;
+    if (sphere_pass<G>(a, first, S, lane, no_jump())) return;
 #pragma unroll 1
   for (int k = 0; k < G && first + k < a.m; ++k) {
     __syncwarp();
-    sphere_pass<1>(a, first + k, S, lane, INFINITY);
+    sphere_pass<1>(a, first + k, S, lane, no_jump());
   }
 }
 

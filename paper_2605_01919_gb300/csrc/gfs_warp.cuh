@@ -65,4 +65,106 @@ __device__ void warp_walk_until(const Tree& T, uint32_t* stk, int cap, int lane,
   }
 }
 
+__device__ __forceinline__ float sqrt_fast(float v) {
+  float r;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+  return r;
+}
+
+// distance and unit direction of (x, y, z) (direction 0 at distance 0)
+__device__ __forceinline__ float unit3(float& x, float& y, float& z) {
+  const float q = fmaf(x, x, fmaf(y, y, z * z));
+  const float inv = q > 1e-36f ? rsqrtf(q) : 0.f;
+  x *= inv;
+  y *= inv;
+  z *= inv;
+  return q * inv;
+}
+
+// (first node, nodes) of each level, in shared memory: lanes index it by the
+// level of the entry they hold
+struct LevelTable {
+  int2 lv[kMaxLevels];
+};
+__device__ __forceinline__ void load_levels(const Tree& T, LevelTable& L, int lane) {
+  __syncwarp();
+  if (lane < kMaxLevels) L.lv[lane] = make_int2(int(T.offset[lane]), int(T.count[lane]));
+  __syncwarp();
+}
+
+constexpr int kCoverStack = 512;  // walk stack entries of warp_cover_walk
+
+// A sphere whose shrunk ball contains a point q (FP32 (x, y, z), the same on
+// every lane), as its sorted slot, or -1: the warp walks the sphere hierarchy
+// for the one point, 32 children or spheres a round.  Node test: the linear
+// bound of |q - p| - |s| over the node's spheres stays below lim (-tol and
+// the margins of the bound and of q's rounding); test(slot, v) decides a
+// sphere (v: how deep, the least goes first when several hold the point).  The
+// child that reaches deepest is visited first.  stk: kCoverStack entries.
+template <class Test>
+__device__ int warp_cover_walk(const Tree& T, const LevelTable& C, uint32_t* stk, int lane, float qx, float qy,
+                               float qz, float lim, unsigned& n_nodes, unsigned& n_items, Test test) {
+  const unsigned kAllLanes = 0xffffffffu;
+  const int top = T.nlevels - 1, grp = lane >> 3, sub = lane & 7;
+  auto key_of = [](float v) {  // order-preserving
+    const unsigned b = __float_as_uint(v);
+    return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
+  };
+  int sp = C.lv[top].y;
+  __syncwarp();
+  if (lane < sp) stk[lane] = pack_node(top, lane);
+  __syncwarp();
+  while (sp > 0) {
+    // past 408 entries one at a time, so that at most 7 per level join them
+    const int take = min(min(sp, 4), max(1, (kCoverStack - 96 - sp) / kFan));
+    const uint32_t nd = grp < take ? stk[sp - 1 - grp] : 0xffffffffu;
+    sp -= take;
+    const int lev = node_level(nd);
+    const int c = int(node_index(nd)) * kFan + sub;
+    bool pass = false, cov = false;
+    float v = INFINITY;
+    if (nd != 0xffffffffu) {
+      if (lev == 0) {
+        if (c < T.nitems) {
+          ++n_items;
+          cov = test(c, v);
+        }
+      } else {
+        const int2 L = C.lv[lev - 1];
+        if (c < L.y) {
+          ++n_nodes;
+          const Lin r = lin_load(T, L.x + c);
+          float nx = qx - r.cx, ny = qy - r.cy, nz = qz - r.cz;
+          const float d = unit3(nx, ny, nz);
+          const float sp_ = fmaf(fabsf(nx + r.gx), r.hx, fmaf(fabsf(ny + r.gy), r.hy, fabsf(nz + r.gz) * r.hz));
+          const float sm_ = fmaf(fabsf(nx - r.gx), r.hx, fmaf(fabsf(ny - r.gy), r.hy, fabsf(nz - r.gz) * r.hz));
+          v = fminf(d - r.hip - sp_, d + r.lon - sm_);
+          pass = v <= lim;
+        }
+      }
+    }
+    if (__any_sync(kAllLanes, cov)) {
+      const unsigned key = cov ? key_of(v) : 0xffffffffu;
+      return __shfl_sync(kAllLanes, c, __ffs(__ballot_sync(kAllLanes, key == __reduce_min_sync(kAllLanes, key))) - 1);
+    }
+    // the child that reaches deepest around the point goes on top, below it
+    // those that reach at least half as deep
+    const unsigned key = pass ? key_of(v) : 0xffffffffu;
+    const unsigned low = __reduce_min_sync(kAllLanes, key);
+    const float deep = __uint_as_float((low & 0x80000000u) ? (low & 0x7fffffffu) : ~low);
+    const unsigned bn = __ballot_sync(kAllLanes, pass);
+    const unsigned bq = __ballot_sync(kAllLanes, pass && v < 0.5f * deep);
+    if (pass) {
+      const unsigned bb = __ballot_sync(bn, key == low);
+      const unsigned best = bb & (0u - bb), rest = bn & ~bq & ~best, good = bq & ~best, me = 1u << lane;
+      const int at = (me & best) ? __popc(bn) - 1
+                                 : ((me & good) ? __popc(rest) + __popc(good & (me - 1u)) : __popc(rest & (me - 1u)));
+      stk[sp + at] = pack_node(lev - 1, c);
+    }
+    sp += __popc(bn);
+    __syncwarp();
+  }
+  return -1;
+}
+
 }  // namespace gfs

@@ -38,7 +38,7 @@ def _points(m, p, seed):
     return x[rng.permutation(m)]
 
 
-@pytest.mark.parametrize("m", [1, 31, 33, PACKET_MIN - 1, PACKET_MIN, PACKET_MIN + 5])
+@pytest.mark.parametrize("m", [1, 31, 33, 24575, 24579, PACKET_MIN - 1, PACKET_MIN, PACKET_MIN + 5])
 @pytest.mark.parametrize("case", ["valid", "mixed", "single"])
 @pytest.mark.parametrize("fp32", [False, True])
 def test_packets_match_oracle(G, orc, m, case, fp32):
