@@ -165,7 +165,7 @@ struct gfs_ctx {
   DevBuf ins_present, ins_scan, ins_cmp, ins_dynf4, ins_near, ins_nearcnt;
   // per-sphere survivor lists for the scored value (sorted ids + offsets),
   // valid while csr_state equals state_id (every build or insertion changes it)
-  DevBuf csr_ids, csr_off, scored_status;
+  DevBuf csr_ids, csr_off;
   // uncovered intersection circles and points (raw outputs, sort buffers)
   DevBuf ud_uncov, ud_cnt, ud_pairs, ud_circ, ud_quad, ud_pts, ud_k0, ud_k1, ud_v0, ud_v1;
   int64_t ud_state = -1, ud_nc = 0, ud_np = 0;  // the raw lists hold state ud_state
@@ -873,14 +873,8 @@ int gfs_query_scored(gfs_ctx* c, const void* x, int x_is_fp32, int64_t m, float*
   GFS_TRY(sort_u32_pairs(c, c->qk_in.as<uint32_t>(), c->qk_out.as<uint32_t>(), c->qv_in.as<int>(),
                          c->qv_out.as<int>(), m));
   a.perm = reinterpret_cast<const uint32_t*>(c->qv_out.p);
-  GFS_TRY(ensure(c->scored_status, 16));
-  GFS_CK(cudaMemsetAsync(c->scored_status.p, 0, 4, st));
-  GFS_CK(launch_query_scored(a, c->opt.box_cull, c->csr_ids.as<uint32_t>(), c->csr_off.as<int64_t>(),
-                             c->scored_status.as<unsigned>(), st));
-  unsigned status = 0;
-  GFS_CK(cudaMemcpyAsync(&status, c->scored_status.p, 4, cudaMemcpyDeviceToHost, st));
-  GFS_CK(cudaStreamSynchronize(st));
-  return status ? GFS_ERR_TIMEOUT : GFS_OK;
+  GFS_CK(launch_query_scored(a, c->opt.box_cull, c->csr_ids.as<uint32_t>(), c->csr_off.as<int64_t>(), st));
+  return GFS_OK;
 }
 
 namespace {
@@ -1878,7 +1872,7 @@ void gfs_destroy(gfs_ctx* c) {
                     &c->ins_dtomb[1], &c->ins_misc, &c->ins_maxrem, &c->ins_slot_t, &c->ins_slots, &c->ins_cbuf,
                     &c->ins_new, &c->ins_lost, &c->ins_inserted, &c->ins_codes, &c->ins_dyn, &c->ins_present,
                     &c->ins_scan, &c->ins_cmp, &c->ins_dynf4, &c->ins_near, &c->ins_nearcnt, &c->csr_ids,
-                    &c->csr_off, &c->scored_status, &c->ud_uncov, &c->ud_cnt, &c->ud_pairs, &c->ud_circ,
+                    &c->csr_off, &c->ud_uncov, &c->ud_cnt, &c->ud_pairs, &c->ud_circ,
                     &c->ud_quad, &c->ud_pts, &c->ud_k0, &c->ud_k1, &c->ud_v0, &c->ud_v1,
                     &c->b_desc, &c->b_offd, &c->b_qoffd, &c->b_sph64, &c->b_k64in, &c->b_k64out, &c->b_sph,
                     &c->b_thr, &c->b_sid, &c->b_bits, &c->b_bcs, &c->b_lo, &c->b_hi, &c->b_na, &c->b_nb, &c->b_nf, &c->b_ln, &c->b_tight,

@@ -5,6 +5,7 @@
 #include "gfs.h"
 #include "gfs_scored.cuh"
 #include "gfs_scored.h"
+#include "gfs_scored_warp.cuh"
 
 namespace gfs {
 
@@ -12,11 +13,17 @@ namespace {
 
 unsigned long long g_scored_launches = 0;
 
-__global__ void __launch_bounds__(128) k_query_scored(QueryArgs a, int box_cull, const uint32_t* __restrict__ csr_ids,
-                                                      const int64_t* __restrict__ csr_off, unsigned* status) {
-  const int64_t slot = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-  if (slot >= a.m) return;
-  scored::scored_one(a, box_cull, csr_ids, csr_off, a.perm ? int64_t(a.perm[slot]) : slot, status);
+// one warp per point (gfs_scored_warp.cuh), points in Morton order
+constexpr int kScoreWarps = 4;
+
+__global__ void __launch_bounds__(32 * kScoreWarps) k_query_scored(QueryArgs a, int box_cull,
+                                                                   const uint32_t* __restrict__ csr_ids,
+                                                                   const int64_t* __restrict__ csr_off) {
+  __shared__ uint32_t s_stk[kScoreWarps][tangent::kWarpStack + kFan];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t slot = int64_t(blockIdx.x) * kScoreWarps + w;
+  if (slot >= a.m) return;  // the same for the whole warp
+  scored::warp_scored_one(a, box_cull, csr_ids, csr_off, a.perm ? int64_t(a.perm[slot]) : slot, s_stk[w], lane);
 }
 
 // csr_off[i] = first position of sphere i's ids in the sorted id list
@@ -37,9 +44,10 @@ __global__ void k_csr_offsets(const uint32_t* __restrict__ ids, int64_t nid, int
 }  // namespace
 
 cudaError_t launch_query_scored(const QueryArgs& a, int box_cull, const uint32_t* csr_ids, const int64_t* csr_off,
-                                unsigned* status, cudaStream_t st) {
+                                cudaStream_t st) {
   if (a.m == 0) return cudaSuccess;
-  k_query_scored<<<unsigned((a.m + 127) / 128), 128, 0, st>>>(a, box_cull, csr_ids, csr_off, status);
+  k_query_scored<<<unsigned((a.m + kScoreWarps - 1) / kScoreWarps), 32 * kScoreWarps, 0, st>>>(a, box_cull, csr_ids,
+                                                                                              csr_off);
   ++g_scored_launches;
   return cudaGetLastError();
 }

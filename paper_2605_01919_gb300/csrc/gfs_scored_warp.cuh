@@ -1,0 +1,311 @@
+// Scored value, one warp per point (device code only).
+//
+// The candidates, their order and every FP64 expression are those of
+// scored_one in gfs_scored.cuh (the host build checks that routine against the
+// oracle).  Here the 32 lanes walk the hierarchies for one point together
+// (warp_walk_until): each lane screens and evaluates its own nodes and items
+// and keeps its own best, and between rounds the lanes share the best so far
+// and the balls that covered the latest tangent points.  The chosen candidate
+// is the greatest valid one of a total order, so it does not depend on which
+// lane met it or when: a candidate is only dropped when a better one is known
+// or when it is not valid, and the two least farthest-survivor distances are
+// minima over distinct spheres.
+#pragma once
+
+#include "gfs_scored.cuh"
+#include "gfs_tangent_warp.cuh"
+#include "gfs_warp.cuh"
+
+namespace gfs {
+namespace scored {
+
+constexpr unsigned kLanes = 0xffffffffu;
+
+// the best of the warp's candidates, on every lane
+__device__ __forceinline__ void warp_best(Best& B) {
+  for (int o = 16; o > 0; o >>= 1) {
+    Best c;
+    c.cls = __shfl_xor_sync(kLanes, B.cls, o);
+    c.sr = __shfl_xor_sync(kLanes, B.sr, o);
+    c.key = __shfl_xor_sync(kLanes, (long long)B.key, o);
+    c.sign = __shfl_xor_sync(kLanes, B.sign, o);
+    c.r = __shfl_xor_sync(kLanes, B.r, o);
+    if (c.cls >= 0 && better(c.cls, c.sr, c.key, c.sign, B)) B = c;
+  }
+}
+
+// Walk of one survivor hierarchy: item(g) for every survivor whose FP32 screen
+// allows an exact distance <= R.
+template <class Refresh, class Item>
+__device__ inline void warp_survivors(const QueryArgs& a, const Frame& F, int cls, double R, uint32_t* stk, int lane,
+                                      Refresh refresh, Item item) {
+  const Tree& T = a.vt[cls];
+  const float R32 = f_up(R);
+  const float4* items = a.surv[cls];
+  const float eq4 = 4.f * a.bc->eq;
+  warp_walk_until(
+      T, stk, tangent::kWarpStack, lane, &a.cnt->walk_err, refresh,
+      [&](int64_t node) {
+        const float bd = sqrtf(box_d2(F.x32, F.y32, F.z32, T.lo[node], T.hi[node]));
+        return bd * (1.f - 1e-6f) - eq4 <= R32;
+      },
+      [&](int64_t idx) {
+        const int64_t b = idx * kLeaf, e = imin64(b + kLeaf, T.nitems);
+        for (int64_t j = b; j < e; ++j) {
+          const float4 S = items[j];
+          const float d32 = dist32(F.x32, F.y32, F.z32, S);
+          if (d32 - err32(F.ax, S, d32, 0.f) - eq4 > R32) continue;
+          item(__float_as_uint(S.w));
+        }
+      });
+}
+
+__device__ inline void warp_scored_one(const QueryArgs& a, int box_cull, const uint32_t* __restrict__ csr_ids,
+                                       const int64_t* __restrict__ csr_off, int64_t q, uint32_t* stk, int lane) {
+  const int code = a.fl_out[q] & 15;
+  if (code == GFS_CODE_SAMPLE || code == GFS_CODE_INVALID) return;
+  const double tol = a.tol;
+  Frame F;
+  tangent::load_point(a, q, F.x, F.y, F.z);
+  F.x32 = float(F.x);
+  F.y32 = float(F.y);
+  F.z32 = float(F.z);
+  F.ax = amax3(F.x32, F.y32, F.z32);
+  tangent::SphereBounds SB;
+  tangent::warp_sphere_bounds(a, F.x, F.y, F.z, stk, lane, SB);
+  if (SB.cov[0] && SB.cov[1]) return;  // INVALID (the plain query says so too)
+  F.sig = SB.cov[0] ? 1 : (SB.cov[1] ? -1 : 0);
+  F.ub[0] = SB.bestA[1];
+  F.ub[1] = SB.bestA[0];
+  F.far = SB.bestF;
+  const double R = __dadd_rn(F.far, tol);  // no valid radius exceeds it (V3)
+  // (V2) per lane the two least of its spheres' farthest-survivor distances
+  F.m1 = F.m2 = INFINITY;
+  F.j1 = F.j2 = -1;
+  int64_t seen[4] = {-1, -1, -1, -1};
+  int seen_at = 0;
+  auto v2_sphere = [&](uint32_t g) {
+    const int64_t i = int64_t(g) / a.KS;
+    if (i == F.j1 || i == F.j2 || i == seen[0] || i == seen[1] || i == seen[2] || i == seen[3]) return;
+    seen[seen_at] = i;
+    seen_at = (seen_at + 1) & 3;
+    double md = -1.0;
+    const int64_t u0 = csr_off[i], u1 = imin64(csr_off[i + 1], u0 + a.KS);  // at most KS per sphere
+    for (int64_t u = u0; u < u1; ++u) {
+      double qx, qy, qz;
+      tangent::survivor_pos(a, int64_t(csr_ids[u]), qx, qy, qz);
+      const double d2 = ex_d2(F.x, F.y, F.z, qx, qy, qz);
+      if (d2 > md) md = d2;
+      if (md >= F.m2) return;  // neither of the two least (both only fall)
+    }
+    if (md < 0.0) return;
+    if (md < F.m1) {
+      F.m2 = F.m1;
+      F.j2 = F.j1;
+      F.m1 = md;
+      F.j1 = i;
+    } else if (md < F.m2) {
+      F.m2 = md;
+      F.j2 = i;
+    }
+  };
+  // two least over distinct spheres: a sphere that several lanes measured has
+  // one distance
+  auto v2_merge = [&]() {
+    for (int o = 16; o > 0; o >>= 1) {
+      const double a1 = __shfl_xor_sync(kLanes, F.m1, o), a2 = __shfl_xor_sync(kLanes, F.m2, o);
+      const long long b1 = __shfl_xor_sync(kLanes, (long long)F.j1, o), b2 = __shfl_xor_sync(kLanes, (long long)F.j2, o);
+      auto put = [&](double m, int64_t j) {
+        if (j < 0 || j == F.j1 || j == F.j2) return;
+        if (m < F.m1 || (m == F.m1 && j < F.j1)) {
+          F.m2 = F.m1;
+          F.j2 = F.j1;
+          F.m1 = m;
+          F.j1 = j;
+        } else if (m < F.m2 || (m == F.m2 && j < F.j2)) {
+          F.m2 = m;
+          F.j2 = j;
+        }
+      };
+      put(a1, b1);
+      put(a2, b2);
+    }
+    return true;
+  };
+  warp_survivors(a, F, 0, R, stk, lane, v2_merge, v2_sphere);
+  warp_survivors(a, F, 1, R, stk, lane, v2_merge, v2_sphere);
+  v2_merge();
+  Best B;
+  B.cls = -1;
+  B.sr = B.r = 0.0;
+  B.key = 0;
+  B.sign = 0;
+  auto share = [&]() {
+    warp_best(B);
+    return true;
+  };
+  // survivors (intersection points)
+  auto surv_cand = [&](uint32_t g) {
+    double qx, qy, qz;
+    tangent::survivor_pos(a, int64_t(g), qx, qy, qz);
+    try_candidate(a, F, qx, qy, qz, int64_t(g) / a.KS, false, int64_t(g), B, []() { return true; });
+  };
+  warp_survivors(a, F, 0, R, stk, lane, share, surv_cand);
+  warp_survivors(a, F, 1, R, stk, lane, share, [&](uint32_t g) {
+    // a zero sample's survivors are in both lists: once is enough
+    if (a.sph64[int64_t(g) / a.KS].w == 0.0) return;
+    surv_cand(g);
+  });
+  share();
+  // tangent points: spheres whose near or far tangent point may lie within R
+  {
+    const Tree& T = a.st;
+    const float R32 = f_up(R);
+    // balls that covered the latest tangent points, the same on every lane
+    // (input index; centre in FP32, radius - tol rounded down), and the one
+    // this lane found last
+    constexpr int kHints = 4;
+    int hint[kHints];
+    float4 hintf[kHints];
+    int found = -1, at = 0;
+#pragma unroll
+    for (int u = 0; u < kHints; ++u) hint[u] = -1;
+    auto refresh = [&]() {
+      warp_best(B);
+      // up to two of the balls the lanes found since the last round
+      unsigned m = __ballot_sync(kLanes, found >= 0);
+#pragma unroll
+      for (int n = 0; n < 2; ++n) {
+        if (!m) break;
+        const int o = __shfl_sync(kLanes, found, __ffs(m) - 1);
+        m &= ~__ballot_sync(kLanes, found == o);
+        bool have = false;
+#pragma unroll
+        for (int u = 0; u < kHints; ++u) have = have || hint[u] == o;
+        if (have) continue;
+        const D4 Q = a.sph64[o];
+        const float4 f = make_float4(float(Q.x), float(Q.y), float(Q.z), tangent::f_dn(__dsub_rn(fabs(Q.w), tol)));
+#pragma unroll
+        for (int u = 0; u < kHints; ++u)
+          if (u == at) {
+            hint[u] = o;
+            hintf[u] = f;
+          }
+        at = (at + 1) % kHints;
+      }
+      found = -1;
+      return true;
+    };
+    auto uncovered_tan = [&](double tx, double ty, double tz, int j) -> bool {
+      if (found >= 0 && found != j && ex_cov(tx, ty, tz, a.sph64[found], a.tol)) return false;
+#pragma unroll
+      for (int u = 0; u < kHints; ++u) {
+        const int c = hint[u];
+        if (c >= 0 && c != j && ex_cov(tx, ty, tz, a.sph64[c], a.tol)) return false;
+      }
+      const int o = tangent::covered_except(a, tx, ty, tz, j, -1, -1);
+      if (o < 0) return true;
+      found = o;
+      return false;
+    };
+    // as in scored_one: is the tangent point surely inside one of the balls
+    auto surely_covered = [&](const float4& S, float d32, float sr, int j) -> bool {
+      const float ap = amax3(S.x, S.y, S.z), r = fabsf(sr);
+      if (!(d32 > 1e-3f * (F.ax + ap + r))) return false;
+      const float inv = 1.f / d32;
+      const float tx = S.x + sr * ((F.x32 - S.x) * inv), ty = S.y + sr * ((F.y32 - S.y) * inv),
+                  tz = S.z + sr * ((F.z32 - S.z) * inv);
+      const float mt = 64.f * 5.9604645e-8f * (F.ax + ap + r) * (1.f + r * inv);
+      const float at_ = amax3(tx, ty, tz);
+      bool in = false;
+#pragma unroll
+      for (int u = 0; u < kHints; ++u) {
+        if (hint[u] < 0 || hint[u] == j) continue;
+        const float dd = dist32(tx, ty, tz, hintf[u]);
+        in = in || dd + mt + err32(at_, hintf[u], dd, 0.f) < hintf[u].w;
+      }
+      return in;
+    };
+    warp_walk_until(
+        T, stk, tangent::kWarpStack, lane, &a.cnt->walk_err, refresh,
+        [&](int64_t node) {
+          const float4 Bc = T.na[node], Fb = T.nf[node];
+          const float dC = dist32(F.x32, F.y32, F.z32, Bc), dF = dist32(F.x32, F.y32, F.z32, Fb);
+          return dC - err32(F.ax, Bc, dC, Bc.w) - Bc.w <= R32 || dF - err32(F.ax, Fb, dF, Fb.w) - Fb.w <= R32;
+        },
+        [&](int64_t idx) {
+          const int64_t b = idx * kLeaf, e = imin64(b + kLeaf, a.n);
+          for (int64_t jj = b; jj < e; ++jj) {
+            const float4 S = a.sph[jj];
+            if (S.w == 0.f) continue;
+            const float d32 = dist32(F.x32, F.y32, F.z32, S), r32 = fabsf(S.w);
+            const float er = err32(F.ax, S, d32, r32);
+            bool near_ok = fabsf(d32 - r32) - er <= R32, far_ok = d32 + r32 - er <= R32;
+            if (!near_ok && !far_ok) continue;
+            const int j = a.sid[jj];
+            const int si = S.w > 0.f ? 1 : -1;
+            // FP32 screen against the best so far and V1, as in scored_one
+#pragma unroll
+            for (int side = 0; side < 2; ++side) {
+              bool& ok = side == 0 ? near_ok : far_ok;
+              if (!ok) continue;
+              const float rr = side == 0 ? fabsf(d32 - r32) : d32 + r32;
+              const float r_hi = rr + er, r_lo = rr - er;
+              const int dr = side == 1 ? 0 : (d32 - r32 > er ? 1 : (r32 - d32 > er ? -1 : 2));
+              bool any = false;
+              for (int sgi = 0; sgi < 2 && !any; ++sgi) {
+                const int sign = sgi == 0 ? 1 : -1;
+                if (F.sig != 0 && sign != F.sig) continue;
+                if (double(r_lo) - tol > F.ub[sgi]) continue;  // V1 fails for sure
+                if (B.cls < 0) {
+                  any = true;
+                  break;
+                }
+                int cls;
+                if (side == 1) cls = sign * si > 0 ? 3 : 0;
+                else if (dr == 2) cls = 3;  // undecided: the highest it could be
+                else cls = sign * si * dr < 0 ? 3 : 0;
+                const double sr_hi = double(r_hi) * (sign > 0 ? 1.0 : 2.0);
+                if (cls > B.cls || (cls == B.cls && sr_hi >= B.sr)) any = true;
+              }
+              if (!any || surely_covered(S, d32, side == 0 ? r32 : -r32, j)) ok = false;
+            }
+            if (!near_ok && !far_ok) continue;
+            const D4 P = a.sph64[j];
+            const double r = fabs(P.w);
+            const double vx = __dsub_rn(F.x, P.x), vy = __dsub_rn(F.y, P.y), vz = __dsub_rn(F.z, P.z);
+            const double dv =
+                __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(vx, vx), __dmul_rn(vy, vy)), __dmul_rn(vz, vz)));
+            if (!(dv > 0.0)) continue;
+            for (int side = 0; side < 2; ++side) {
+              if (side == 0 ? !near_ok : !far_ok) continue;
+              const double sr = side == 0 ? r : -r;
+              const double tx = __dadd_rn(P.x, __dmul_rn(sr, __ddiv_rn(vx, dv)));
+              const double ty = __dadd_rn(P.y, __dmul_rn(sr, __ddiv_rn(vy, dv)));
+              const double tz = __dadd_rn(P.z, __dmul_rn(sr, __ddiv_rn(vz, dv)));
+              if (box_cull && !ex_inbox(tx, ty, tz)) continue;
+              try_candidate(a, F, tx, ty, tz, int64_t(j), true, kTanKey + 2 * int64_t(j) + side, B,
+                            [&]() { return uncovered_tan(tx, ty, tz, j); });
+            }
+          }
+        });
+    warp_best(B);
+  }
+  if (lane != 0) return;
+  if (B.cls < 0) {
+    a.fl_out[q] = uint16_t(a.fl_out[q] | GFS_FLAG_SCORE_FALLBACK);
+    return;
+  }
+  const bool tan = B.key >= kTanKey;
+  const double v = B.sign > 0 ? B.r : -B.r;
+  int flags = tan ? GFS_CODE_TANGENT : GFS_CODE_SURVIVOR;
+  const int c = B.sign > 0 ? 0 : 1;
+  if (SB.cov[c] && B.r < __dsub_rn(-SB.bestA[c], tol)) flags |= GFS_FLAG_LB_VIOL;
+  if (a.s_out) a.s_out[q] = float(v);
+  if (a.s64_out) a.s64_out[q] = v;
+  a.arg_out[q] = tan ? B.key - kTanKey : B.key;
+  a.fl_out[q] = uint16_t(flags);
+}
+
+}  // namespace scored
+}  // namespace gfs
