@@ -375,7 +375,7 @@ int gfs_exact_rmin(gfs_ctx* ctx, const double* x, const int8_t* sigma, int64_t m
  * sign, shrunk by tol (the cull's coverage predicate, decided in FP64);
  * counts_out[c] = the number contained (the covered area ratio times sub^3).
  * cells: device, ncells*3 int32.  origin_host: host, 3 FP64.  h > 0.
- * 1 <= sub <= 64.  counts_out: device, ncells uint32.  One warp per cell; no
+ * 1 <= sub <= 64.  counts_out: device, ncells uint32.  One block per cell; no
  * host synchronisation, no allocation.  Errors: GFS_ERR_STATE (no build),
  * GFS_ERR_ARG, GFS_ERR_CUDA. */
 int gfs_cell_coverage(gfs_ctx* ctx, const int32_t* cells, int64_t ncells, const double* origin_host, double h,

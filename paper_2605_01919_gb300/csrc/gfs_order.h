@@ -9,7 +9,7 @@
 namespace gfs {
 
 // counts[c] = covered sub-points of cell c (cells: device, ncells x 3 int32);
-// one warp per cell
+// one block per cell
 cudaError_t launch_cell_coverage(const QueryArgs& a, const int32_t* cells, int64_t ncells, const double* origin,
                                  double h, int sub, uint32_t* counts, cudaStream_t st);
 
