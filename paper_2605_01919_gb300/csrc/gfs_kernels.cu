@@ -180,30 +180,36 @@ __global__ void k_level(float4* __restrict__ lo, float4* __restrict__ hi, int64_
   if (j < nnode) point_level_node(lo, hi, child_off, nchild, off, j);
 }
 
-// Bounding ball of weighted centres (c_i, w_i): a centre c and
-// V >= max_i (|c_i - c| + w_i).  Any centre is valid; subgradient steps from
-// the better of two starts (the item of largest weight, the mean centre) make
-// V small.  V is inflated by 8 ulp of |V| and of the coordinate range, which
-// covers the FP32 evaluation and the rounding of FP64 inputs to FP32.
-__device__ float4 bound_ball(const float4* it, int k, float A) {
-  if (k == 0) return make_float4(0.f, 0.f, 0.f, -INFINITY);
-  auto eval = [&](float cx, float cy, float cz, int& arg) {
+// Centre of a small ball around weighted centres (c_i, w_i): one that makes
+// max_i (|c_i - c| + w_i) small, by subgradient steps from the better of two
+// starts (the item of largest weight, the mean centre).  Any centre is valid
+// (the radii are taken against it afterwards), so the steps use the fast
+// square root and division; a node's steps are a serial chain, and 12 of them
+// leave the walks as they are (24 with IEEE roots and divisions kept the
+// levels of a 16^3 grid's hierarchy waiting 150 us, 12 fast ones on registers under 60 us).
+// it: kFan items, the first k of them given (the rest has w = -inf), so that
+// the loops unroll and the items stay in registers.
+__device__ float4 bound_ball(const float4 (&it)[kFan], int k) {
+  auto eval = [&](float cx, float cy, float cz, float3& far) {
     float best = -INFINITY;
-    arg = 0;
-    for (int i = 0; i < k; ++i) {
+    far = make_float3(cx, cy, cz);
+#pragma unroll
+    for (int i = 0; i < kFan; ++i) {
       const float dx = it[i].x - cx, dy = it[i].y - cy, dz = it[i].z - cz;
-      const float v = sqrtf(dx * dx + dy * dy + dz * dz) + it[i].w;
+      const float v = sqrt_fast(dx * dx + dy * dy + dz * dz) + it[i].w;
       if (v > best) {
         best = v;
-        arg = i;
+        far = make_float3(it[i].x, it[i].y, it[i].z);
       }
     }
     return best;
   };
-  int big = 0;
+  float4 big = it[0];
   float mx = 0.f, my = 0.f, mz = 0.f;
-  for (int i = 0; i < k; ++i) {
-    if (it[i].w > it[big].w) big = i;
+#pragma unroll
+  for (int i = 0; i < kFan; ++i) {
+    if (i >= k) break;
+    if (it[i].w > big.w) big = it[i];
     mx += it[i].x;
     my += it[i].y;
     mz += it[i].z;
@@ -211,36 +217,26 @@ __device__ float4 bound_ball(const float4* it, int k, float A) {
   mx /= float(k);
   my /= float(k);
   mz /= float(k);
-  int j0, j1;
-  const float v0 = eval(it[big].x, it[big].y, it[big].z, j0);
-  const float v1 = eval(mx, my, mz, j1);
-  float cx = v0 <= v1 ? it[big].x : mx, cy = v0 <= v1 ? it[big].y : my, cz = v0 <= v1 ? it[big].z : mz;
+  float3 far;
+  const float v0 = eval(big.x, big.y, big.z, far), v1 = eval(mx, my, mz, far);
+  float cx = v0 <= v1 ? big.x : mx, cy = v0 <= v1 ? big.y : my, cz = v0 <= v1 ? big.z : mz;
   float bx = cx, by = cy, bz = cz, best = fminf(v0, v1);
-  for (int t = 0; t < 24; ++t) {
-    int j;
-    const float v = eval(cx, cy, cz, j);
+  for (int t = 0; t < 12; ++t) {
+    const float v = eval(cx, cy, cz, far);
     if (v < best) {
       best = v;
       bx = cx;
       by = cy;
       bz = cz;
     }
-    const float dx = it[j].x - cx, dy = it[j].y - cy, dz = it[j].z - cz;
-    const float d = sqrtf(dx * dx + dy * dy + dz * dz);
-    if (!(d > 1e-12f)) break;
-    const float step = d / float(t + 2);
-    cx += dx / d * step;
-    cy += dy / d * step;
-    cz += dz / d * step;
+    const float dx = far.x - cx, dy = far.y - cy, dz = far.z - cz;
+    if (!(dx * dx + dy * dy + dz * dz > 1e-24f)) break;
+    const float f = __fdividef(1.f, float(t + 2));  // a step of d / (t + 2) towards the farthest item
+    cx += dx * f;
+    cy += dy * f;
+    cz += dz * f;
   }
-  int j;
-  float v = eval(bx, by, bz, j);
-  // rounding of the evaluation and of the items' FP32 copies (|p| <= A, and
-  // radii up to rmax)
-  float rmax = 0.f;
-  for (int i = 0; i < k; ++i) rmax = fmaxf(rmax, fabsf(it[i].w));
-  v = v + (fabsf(v) + A + rmax) * 4.8e-7f;
-  return make_float4(bx, by, bz, v);
+  return make_float4(bx, by, bz, 0.f);
 }
 
 // Upper bound of a node radius term d = dist (+-) r computed in FP32: the
@@ -283,9 +279,11 @@ __device__ __forceinline__ void lin_box(Lin& r, const float4& lo, const float4& 
 // regularised (planar or coincident points give 0 across them), at most 1 in
 // norm (signed distances are 1-Lipschitz; noise may exceed it).  Any gradient
 // is valid: the residual bounds are taken against it.
-__device__ void lin_fit(const float4* it, int k, Lin& r) {
+__device__ void lin_fit(const float4 (&it)[kFan], int k, Lin& r) {
   float mx = 0.f, my = 0.f, mz = 0.f, mw = 0.f;
-  for (int i = 0; i < k; ++i) {
+#pragma unroll
+  for (int i = 0; i < kFan; ++i) {
+    if (i >= k) break;
     mx += it[i].x;
     my += it[i].y;
     mz += it[i].z;
@@ -297,7 +295,9 @@ __device__ void lin_fit(const float4* it, int k, Lin& r) {
   mz *= inv;
   mw *= inv;
   float xx = 0.f, xy = 0.f, xz = 0.f, yy = 0.f, yz = 0.f, zz = 0.f, bx = 0.f, by = 0.f, bz = 0.f;
-  for (int i = 0; i < k; ++i) {
+#pragma unroll
+  for (int i = 0; i < kFan; ++i) {
+    if (i >= k) break;
     const float dx = it[i].x - mx, dy = it[i].y - my, dz = it[i].z - mz, dw = it[i].w - mw;
     xx += dx * dx;
     xy += dx * dy;
@@ -355,23 +355,26 @@ __device__ void sphere_leaf_node(const float4* __restrict__ items, float A, cons
   float4 *lo = T.lo, *hi = T.hi, *na = T.na, *nb = T.nb, *nf = T.nf;
   const int64_t nitems = T.nitems;
   int64_t b = L * kLeaf, e = min(b + kLeaf, nitems);
-  float4 Ab[kLeaf], Fb[kLeaf];
-  int k = 0;
+  static_assert(kLeaf == kFan, "bound_ball takes kFan items");
+  float4 It[kFan], Ab[kFan], Fb[kFan];
+  const int k = int(e - b);
   float3 mn = make_float3(INFINITY, INFINITY, INFINITY), mx = make_float3(-INFINITY, -INFINITY, -INFINITY);
-  for (int64_t i = b; i < e; ++i) {
-    const float4 v = items[i];
+#pragma unroll
+  for (int c = 0; c < kFan; ++c) {
+    const float4 v = It[c] = items[b + min(c, k - 1)];  // past the end: the last one again, with w = -inf in Ab, Fb
     mn.x = fminf(mn.x, v.x); mn.y = fminf(mn.y, v.y); mn.z = fminf(mn.z, v.z);
     mx.x = fmaxf(mx.x, v.x); mx.y = fmaxf(mx.y, v.y); mx.z = fmaxf(mx.z, v.z);
-    Ab[k] = make_float4(v.x, v.y, v.z, fabsf(v.w));
-    Fb[k++] = make_float4(v.x, v.y, v.z, -fabsf(v.w));
+    Ab[c] = make_float4(v.x, v.y, v.z, c < k ? fabsf(v.w) : -INFINITY);
+    Fb[c] = make_float4(v.x, v.y, v.z, c < k ? -fabsf(v.w) : -INFINITY);
   }
   lo[L] = make_float4(nextafterf(mn.x, -INFINITY), nextafterf(mn.y, -INFINITY), nextafterf(mn.z, -INFINITY), 0.f);
   hi[L] = make_float4(nextafterf(mx.x, INFINITY), nextafterf(mx.y, INFINITY), nextafterf(mx.z, INFINITY), 0.f);
-  const float4 C = bound_ball(Ab, k, A);   // small ball enclosing the balls
-  const float4 Fc = bound_ball(Fb, k, A);  // centre for the far bound
+  const float4 C = bound_ball(Ab, k);   // small ball enclosing the balls
+  const float4 Fc = bound_ball(Fb, k);  // centre for the far bound
   float wp = -INFINITY, wn = -INFINITY, w0 = -INFINITY, wf = -INFINITY;
-  for (int64_t i = b; i < e; ++i) {
-    const float4 v = items[i];
+#pragma unroll
+  for (int c = 0; c < kFan; ++c) {  // (a repeated last item changes no maximum)
+    const float4 v = It[c];
     const float r = fabsf(v.w);
     const float pm = fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fabsf(v.z));
     float dx = v.x - C.x, dy = v.y - C.y, dz = v.z - C.z;
@@ -386,9 +389,9 @@ __device__ void sphere_leaf_node(const float4* __restrict__ items, float A, cons
   store_sphere_node(na, nb, nf, L, C, Fc, wp, wn, w0, wf, A);
   Lin r;
   lin_box(r, lo[L], hi[L], A);
-  for (int i = 0; i < k; ++i) Ab[i].w = items[b + i].w;
-  lin_fit(Ab, k, r);
-  for (int i = 0; i < k; ++i) lin_add(r, Ab[i], A);
+  lin_fit(It, k, r);
+#pragma unroll
+  for (int c = 0; c < kFan; ++c) lin_add(r, It[c], A);
   lin_store(T, L, r);
 }
 
@@ -398,20 +401,23 @@ __device__ void sphere_level_node(const Tree& T, float A, int level, int64_t j) 
   int64_t b = j * kFan, e = min(b + kFan, nchild);
   float4 L = make_float4(INFINITY, INFINITY, INFINITY, 0.f), H = make_float4(-INFINITY, -INFINITY, -INFINITY, 0.f);
   float4 Ab[kFan], Fb[kFan];
-  int k = 0;
-  for (int64_t c = b; c < e; ++c) {
+  const int k = int(e - b);
+#pragma unroll
+  for (int u = 0; u < kFan; ++u) {
+    const int64_t c = b + min(u, k - 1);
     const float4 a = lo[child_off + c], z = hi[child_off + c];
     L.x = fminf(L.x, a.x); L.y = fminf(L.y, a.y); L.z = fminf(L.z, a.z);
     H.x = fmaxf(H.x, z.x); H.y = fmaxf(H.y, z.y); H.z = fmaxf(H.z, z.z);
     const float4 ca = na[child_off + c], cb = nb[child_off + c];
     // a ball around the child that holds all its spheres
-    Ab[k] = make_float4(ca.x, ca.y, ca.z, fmaxf(ca.w, cb.z));
-    Fb[k++] = nf[child_off + c];
+    Ab[u] = make_float4(ca.x, ca.y, ca.z, u < k ? fmaxf(ca.w, cb.z) : -INFINITY);
+    Fb[u] = nf[child_off + c];
+    if (u >= k) Fb[u].w = -INFINITY;
   }
   lo[off + j] = L;
   hi[off + j] = H;
-  const float4 C = bound_ball(Ab, k, A);
-  const float4 Fc = bound_ball(Fb, k, A);
+  const float4 C = bound_ball(Ab, k);
+  const float4 Fc = bound_ball(Fb, k);
   // radii through the children (|p - C| <= |p - C_c| + |C_c - C|)
   float wp = -INFINITY, wn = -INFINITY, w0 = -INFINITY, wf = -INFINITY;
   for (int64_t c = b; c < e; ++c) {
@@ -431,11 +437,13 @@ __device__ void sphere_level_node(const Tree& T, float A, int level, int64_t j) 
   // (s - g.(p - c) = s - g_k.(p - c_k) - g.(c_k - c) + (g_k - g).(p - c_k))
   Lin r;
   lin_box(r, L, H, A);
-  for (int64_t c = b; c < e; ++c) {
-    const Lin q = lin_load(T, child_off + c);
+#pragma unroll
+  for (int u = 0; u < kFan; ++u) {
+    if (u >= k) break;
+    const Lin q = lin_load(T, child_off + b + u);
     const float hi_k = fmaxf(q.hip, q.hin), lo_k = fminf(q.lop, q.lon);
     const float v = hi_k > -INFINITY ? 0.5f * (hi_k + lo_k) : 0.f;
-    Ab[c - b] = make_float4(q.cx, q.cy, q.cz, v);
+    Ab[u] = make_float4(q.cx, q.cy, q.cz, v);
   }
   lin_fit(Ab, k, r);
   for (int64_t c = b; c < e; ++c) {
