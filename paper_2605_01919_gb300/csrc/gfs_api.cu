@@ -688,11 +688,11 @@ int ud_compute(gfs_ctx* c) {
   }
   // raw outputs: a first guess, then exactly the counts (the decisions do not
   // depend on the capacities, so a second run finds the same entries).  The
-  // guess is generous (2 a sphere, at least 2^17: 9 MB), because the second run
-  // repeats the whole search: on a 12^3 union grid, about 8 circles and as
-  // many points a sphere, it doubled the 57 ms.  (Dense small grids have the
-  // most a sphere, 64^3 ones less than one.)
-  int64_t cap_c = std::max<int64_t>(int64_t(1) << 17, 2 * c->n), cap_p = cap_c;
+  // guess is generous (2 a sphere, at least 2^17: 9 MB; up to 2^21, 151 MB, as
+  // many as there are pairs), because the second run repeats the whole search:
+  // it doubled the 57 ms of a 12^3 union grid and the 116 ms of a 14^3 one.
+  // (Dense small grids have the most a sphere, 64^3 ones less than one.)
+  int64_t cap_c = std::max({int64_t(1) << 17, 2 * c->n, std::min(int64_t(hpairs), int64_t(1) << 21)}), cap_p = cap_c;
   unsigned long long hc[2] = {0, 0};
   unsigned hstatus = 0;
   for (int pass = 0; pass < 2; ++pass) {

@@ -166,11 +166,13 @@ __global__ void __launch_bounds__(128) k_ud_pairs(QueryArgs a, const uint8_t* __
 }
 
 // One thread per pair: the circle's certificate and, on an uncovered circle,
-// its uncovered points.
+// its uncovered points.  Bound: the latency of walks whose lanes diverge (1.3
+// active lanes with a pair on every lane), so a warp takes only 32 / spread
+// pairs and the chip is filled with more warps instead; the launch says how far.
 __global__ void __launch_bounds__(128) k_intersections(QueryArgs a, const unsigned long long* __restrict__ pairs,
-                                                       int64_t np, exact::UDOut o) {
-  const int64_t k = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-  if (k >= np) return;
+                                                       int64_t np, exact::UDOut o, int spread) {
+  const int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x, k = t / spread;
+  if (k >= np || t % spread) return;
   const int i = int(pairs[k] >> 32), j = int(pairs[k] & 0xffffffffull);
   int M[exact::kMaxSet];
   uint32_t stacks[2 * kStack];
@@ -212,24 +214,34 @@ __global__ void k_ud_gather(const unsigned long long* __restrict__ ckey, int64_t
   }
 }
 
-// One warp per query point: the lanes split each candidate set (U, D, T in
-// that order) and take the warp's minimum after each, so that later sets are
-// tested against the best point so far.
-__global__ void __launch_bounds__(128) k_exact_rmin(QueryArgs a, int box_cull, exact::UDLists L,
-                                                   const double* __restrict__ x, const int8_t* __restrict__ sigma,
-                                                   int64_t m, double* __restrict__ out) {
-  const int lane = threadIdx.x & 31;
-  const int64_t q = (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) >> 5;
-  if (q >= m) return;  // the same for the whole warp
+// One block per query point: its threads split each candidate set (U, D, T in
+// that order) and take the block's minimum after each, so that later sets are
+// tested against the best point so far.  Bound: FP64 constructions and the
+// latency of the coverage walks; with one warp per point 512 points left most
+// of the chip idle.  Radii of 512 points of a 12^3 union grid, circles included:
+// 85 ms with 1 warp a point, 78 with 4, 72 with 16 (and 50.5 / 48.7 ms with 8 /
+// 16 after the circles were spread over more warps).
+constexpr int kRminWarps = 16;
+__global__ void __launch_bounds__(32 * kRminWarps) k_exact_rmin(QueryArgs a, int box_cull, exact::UDLists L,
+                                                                const double* __restrict__ x,
+                                                                const int8_t* __restrict__ sigma,
+                                                                double* __restrict__ out) {
+  __shared__ double s_best[kRminWarps];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t q = blockIdx.x;
   uint32_t stack[kStack];
   const double xq[3] = {x[3 * q], x[3 * q + 1], x[3 * q + 2]};
   const int sg = sigma[q];
   double best = INFINITY;
   for (int phase = 0; phase < 3; ++phase) {
-    best = exact::rmin_phase(a, box_cull, L, xq, sg, phase, lane, 32, best, stack);
+    best = exact::rmin_phase(a, box_cull, L, xq, sg, phase, threadIdx.x, 32 * kRminWarps, best, stack);
     for (int o = 16; o > 0; o >>= 1) best = fmin(best, __shfl_xor_sync(0xffffffffu, best, o));
+    if (lane == 0) s_best[w] = best;
+    __syncthreads();
+    for (int k = 0; k < kRminWarps; ++k) best = fmin(best, s_best[k]);
+    __syncthreads();
   }
-  if (lane == 0) out[q] = best;
+  if (threadIdx.x == 0) out[q] = best;
 }
 
 unsigned long long g_exact_launches = 0;
@@ -239,7 +251,9 @@ unsigned long long g_exact_launches = 0;
 cudaError_t launch_exact_rmin(const QueryArgs& a, int box_cull, const exact::UDLists& L, const double* x,
                               const int8_t* sigma, int64_t m, double* out, cudaStream_t st) {
   if (m <= 0) return cudaSuccess;
-  k_exact_rmin<<<(unsigned int)((m + 3) / 4), 128, 0, st>>>(a, box_cull, L, x, sigma, m, out);
+  for (int64_t q = 0; q < m; q += 1 << 30)
+    k_exact_rmin<<<unsigned(m - q < (1 << 30) ? m - q : 1 << 30), 32 * kRminWarps, 0, st>>>(a, box_cull, L, x + 3 * q,
+                                                                                        sigma + q, out + q);
   ++g_exact_launches;
   return cudaGetLastError();
 }
@@ -255,7 +269,12 @@ cudaError_t launch_ud_pairs(const QueryArgs& a, const uint8_t* uncov, unsigned l
 cudaError_t launch_intersections(const QueryArgs& a, const unsigned long long* pairs, int64_t np,
                                  const exact::UDOut& o, cudaStream_t st) {
   if (np <= 0) return cudaSuccess;
-  k_intersections<<<(unsigned int)((np + 127) / 128), 128, 0, st>>>(a, pairs, np, o);
+  // One pair a warp while that still leaves few warps a scheduler, 4 a warp
+  // beyond: 171k pairs (12^3 union grid, with the radii of 512 points) 72 ms at
+  // spread 1, 59 at 8, 49 at 32; 16k pairs 7.6, 5.8, 5.1 ms; 419k pairs 284, 232,
+  // 233 ms; 913k pairs 497, 476, 499 ms.
+  const int spread = np <= (int64_t(1) << 18) ? 32 : 8;
+  k_intersections<<<(unsigned int)((np * spread + 127) / 128), 128, 0, st>>>(a, pairs, np, o, spread);
   ++g_exact_launches;
   return cudaGetLastError();
 }
