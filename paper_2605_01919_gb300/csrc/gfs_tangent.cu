@@ -17,11 +17,15 @@ namespace {
 constexpr int kTanWarps = 4;
 
 __global__ void __launch_bounds__(32 * kTanWarps) k_query_tangent(QueryArgs a, int box_cull) {
-  __shared__ uint32_t s_stk[kTanWarps][tangent::kWarpStack + kFan];
+  __shared__ tangent::TanWarp s_w[kTanWarps];
+  __shared__ LevelTable s_lv;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t slot = (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) >> 5;
+  if (threadIdx.x < kMaxLevels)
+    s_lv.lv[threadIdx.x] = make_int2(int(a.st.offset[threadIdx.x]), int(a.st.count[threadIdx.x]));
+  __syncthreads();
   if (slot >= a.m) return;  // the same for the whole warp
-  tangent::warp_tangent_one(a, box_cull, a.perm ? int64_t(a.perm[slot]) : slot, s_stk[w], lane);
+  tangent::warp_tangent_one(a, s_lv, box_cull, a.perm ? int64_t(a.perm[slot]) : slot, s_w[w], lane);
 }
 
 __global__ void __launch_bounds__(128) k_argmin_points(QueryArgs a, const int64_t* __restrict__ argmin,

@@ -20,7 +20,7 @@ namespace gfs {
 namespace tangent {
 
 constexpr unsigned kLanes = 0xffffffffu;
-constexpr int kWarpStack = 512;  // per-warp walk stack entries (plus a reserve of kFan)
+constexpr int kWarpStack = kCoverStack - kFan;  // per-warp walk stack entries (plus a reserve of kFan)
 
 // lexicographic minimum of (v, i) over the warp, on every lane
 __device__ __forceinline__ void warp_min_vi(double& v, int& i) {
@@ -238,14 +238,322 @@ __device__ inline void warp_tangent_search(const QueryArgs& a, int box_cull, dou
   merge();
 }
 
+// ---------------------------------------------------------------------------
+// The same two walks for points in the coordinate range [-A, A]^3 of the FP32
+// bounds: 4 entries a round, each lane tests one child or one sphere, and a
+// node has to pass its linear bounds (struct Lin) instead of the balls around
+// its spheres.  A tangent point that may win is tested against the balls that
+// held the point's latest covered ones, then walked by the whole warp, the
+// nearest first, so an uncovered one ends the search early.  Bound: the latency
+// of those walks (dependent rounds of 4 entries).  31,607 points of a 64^3 union
+// grid take 14 ms, with the lanes walking apart by ball bounds 30 ms, with one
+// point a lane 53 ms.  Points outside the range take the walks above.
+// ---------------------------------------------------------------------------
+
+constexpr int kTanRecent = 8;
+constexpr float kTanU = 5.9604644775390625e-8f;  // 2^-24
+
+struct TanWarp {
+  uint32_t stk[kCoverStack], cstk[kCoverStack];
+  float4 rec[kTanRecent];  // (centre, squared distance below which a point is held for sure)
+  int rec_id[kTanRecent];  // sorted slot
+};
+
+__device__ __forceinline__ unsigned ord_bits(float v) {  // order-preserving
+  const unsigned b = __float_as_uint(v);
+  return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
+}
+__device__ __forceinline__ float ord_value(unsigned k) {
+  return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
+}
+__device__ __forceinline__ float warp_min_f(float v) { return ord_value(__reduce_min_sync(kLanes, ord_bits(v))); }
+
+// node(global node, lin, level) -> visit its children; items(slot or -1) runs
+// on all lanes in rounds that reach leaves.  Stack bound as in warp_cover_walk.
+template <class Node, class Items>
+__device__ __forceinline__ void warp_lin_walk(const Tree& T, const LevelTable& C, uint32_t* stk, int lane, Node node,
+                                              Items items) {
+  const int top = T.nlevels - 1, grp = lane >> 3, sub = lane & 7;
+  int sp = C.lv[top].y;
+  __syncwarp();
+  if (lane < sp) stk[lane] = pack_node(top, lane);
+  __syncwarp();
+  while (sp > 0) {
+    const int take = min(min(sp, 4), max(1, (kCoverStack - 96 - sp) / kFan));
+    const uint32_t nd = grp < take ? stk[sp - 1 - grp] : 0xffffffffu;
+    sp -= take;
+    const int lev = node_level(nd);
+    const int c = int(node_index(nd)) * kFan + sub;
+    const bool leaf = nd != 0xffffffffu && lev == 0;
+    bool pass = false;
+    if (nd != 0xffffffffu && lev > 0) {
+      const int2 L = C.lv[lev - 1];
+      if (c < L.y) pass = node(int64_t(L.x) + c);
+    }
+    const unsigned bn = __ballot_sync(kLanes, pass);
+    // children of the deepest popped entry end up on top
+    if (pass) stk[sp + __popc(bn >> lane >> 1)] = pack_node(lev - 1, c);
+    sp += __popc(bn);
+    if (__any_sync(kLanes, leaf)) items(leaf && c < T.nitems ? c : -1);
+    __syncwarp();
+  }
+}
+
+// warp_sphere_bounds by that walk.
+__device__ inline void warp_sphere_bounds_lin(const QueryArgs& a, const LevelTable& C, double x, double y, double z,
+                                              TanWarp& W, int lane, SphereBounds& R) {
+  const double tol = a.tol;
+  R.cov[0] = R.cov[1] = false;
+  R.bestA[0] = R.bestA[1] = INFINITY;
+  R.idxA[0] = R.idxA[1] = INT_MAX;
+  R.bestF = INFINITY;
+  const Tree& T = a.st;
+  if (T.nlevels == 0) return;
+  const float x32 = float(x), y32 = float(y), z32 = float(z), ax = amax3(x32, y32, z32);
+  const float mg = a.bc->elin + 8.f * kTanU * a.bc->A;
+  float thF = INFINITY, thA[2] = {INFINITY, INFINITY};
+  auto item = [&](int64_t j) -> bool {
+    const float4 S = a.sph[j];
+    const float d32 = dist32(x32, y32, z32, S), r32 = fabsf(S.w);
+    const float er = err32(ax, S, d32, r32);
+    bool need = d32 + r32 - er <= thF;
+    if (S.w != 0.f) need = need || d32 - r32 - er <= (S.w < 0.f ? thA[1] : thA[0]);
+    if (!need) return false;
+    const int o = a.sid[j];
+    const D4 P = a.sph64[o];
+    const double d2 = ex_d2(x, y, z, P.x, P.y, P.z);
+    const double dl = __dsqrt_rn(d2);
+    const double r = fabs(P.w);
+    if (P.w != 0.0) {
+      const bool in = r > tol && d2 < __dmul_rn(__dsub_rn(r, tol), __dsub_rn(r, tol));
+      const double av = __dsub_rn(dl, r);
+#pragma unroll
+      for (int c = 0; c < 2; ++c)
+        if (c == int(P.w < 0.0)) {
+          R.cov[c] = R.cov[c] || in;
+          if (av < R.bestA[c] || (av == R.bestA[c] && o < R.idxA[c])) {
+            R.bestA[c] = av;
+            R.idxA[c] = o;
+          }
+          thA[c] = fminf(thA[c], f_up(R.cov[c] ? R.bestA[c] : fmax(R.bestA[c], -tol)));
+        }
+    }
+    const double f = __dadd_rn(dl, r);
+    if (f < R.bestF) {
+      R.bestF = f;
+      thF = fminf(thF, f_up(f));
+    }
+    return true;
+  };
+  // thresholds of all lanes (a lane's are sound for the warp: its class is
+  // covered if the lane says so, and the least value is at most its own)
+  auto items = [&](int64_t j) {
+    const bool got = j >= 0 && item(j);
+    if (!__any_sync(kLanes, got)) return;
+    thF = warp_min_f(thF);
+    thA[0] = warp_min_f(thA[0]);
+    thA[1] = warp_min_f(thA[1]);
+  };
+  // seed: each group of 8 lanes descends for one quantity (class 0, class 1,
+  // far bound, any ball), the child with the least bound at every level
+  {
+    const int grp = lane >> 3, sub = lane & 7;
+    int lev = T.nlevels - 1;
+    int64_t node = sub;
+    bool valid = sub < C.lv[lev].y;
+    for (;;) {
+      float v = INFINITY;
+      if (valid) {
+        const int64_t nd = C.lv[lev].x + node;
+        const float4 B = grp == 2 ? T.nf[nd] : T.na[nd];
+        float w = B.w;
+        if (grp < 2) w = grp == 0 ? T.nb[nd].x : T.nb[nd].y;
+        v = dist32(x32, y32, z32, B) - w;
+      }
+      unsigned key = v < INFINITY ? (ord_bits(v) & ~7u) | unsigned(sub) : 0xffffffffu;
+      for (int o = 4; o > 0; o >>= 1) key = min(key, __shfl_xor_sync(kLanes, key, o));
+      const int64_t next = __shfl_sync(kLanes, (long long)node, (lane & 24) | int(key & 7u)) * kFan + sub;
+      valid = key != 0xffffffffu;
+      node = next;
+      if (lev == 0) break;
+      --lev;
+      valid = valid && node < C.lv[lev].y;
+    }
+    items(valid && node < T.nitems ? node : -1);
+  }
+  warp_lin_walk(
+      T, C, W.stk, lane,
+      [&](int64_t nd) {
+        const Lin q = lin_load(T, nd);
+        float nx = x32 - q.cx, ny = y32 - q.cy, nz = z32 - q.cz;
+        const float d = unit3(nx, ny, nz);
+        const float sp = fmaf(fabsf(nx + q.gx), q.hx, fmaf(fabsf(ny + q.gy), q.hy, fabsf(nz + q.gz) * q.hz));
+        const float sm = fmaf(fabsf(nx - q.gx), q.hx, fmaf(fabsf(ny - q.gy), q.hy, fabsf(nz - q.gz) * q.hz));
+        // (an absent class: inf - inf compares false)
+        return d - q.hip - sp - thA[0] <= mg || d + q.lon - sm - thA[1] <= mg ||
+               fminf(d + q.lop - sm, d - q.hin - sp) - thF <= mg;
+      },
+      items);
+  R.cov[0] = __any_sync(kLanes, R.cov[0]);
+  R.cov[1] = __any_sync(kLanes, R.cov[1]);
+  warp_min_vi(R.bestA[0], R.idxA[0]);
+  warp_min_vi(R.bestA[1], R.idxA[1]);
+  for (int o = 16; o > 0; o >>= 1) R.bestF = fmin(R.bestF, __shfl_xor_sync(kLanes, R.bestF, o));
+}
+
+// warp_tangent_search by that walk.
+__device__ inline void warp_tangent_search_lin(const QueryArgs& a, const LevelTable& C, int box_cull, double x,
+                                               double y, double z, int cs, int mode, double lim, double lo,
+                                               TanWarp& W, int lane, TanBest& B) {
+  const Tree& T = a.st;
+  if (T.nlevels == 0) return;
+  const float A = a.bc->A;
+  const double lim_d = mode == kBelowSurvivor ? sqrt(lim) : (mode == kWithinOpposite ? lim : INFINITY);
+  const float x32 = float(x), y32 = float(y), z32 = float(z), ax = amax3(x32, y32, z32);
+  const float lo_f = f_dn(lo);
+  const float mg = a.bc->elin + 8.f * kTanU * A;
+  const float cover_lim = -a.tol32 + a.bc->elin;
+  float hi_f = f_up(lim_d * kRel + kAbs);
+  int nrec = 0, at = 0;
+  unsigned n_nodes = 0, n_items = 0;
+  auto tangent_point = [&](int o, int side, double t[3]) -> bool {
+    const D4 P = a.sph64[o];
+    const double r = fabs(P.w);
+    const double vx = __dsub_rn(x, P.x), vy = __dsub_rn(y, P.y), vz = __dsub_rn(z, P.z);
+    const double dv = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(vx, vx), __dmul_rn(vy, vy)), __dmul_rn(vz, vz)));
+    if (!(dv > 0.0)) return false;
+    const double sr = side == 0 ? r : -r;
+    t[0] = __dadd_rn(P.x, __dmul_rn(sr, __ddiv_rn(vx, dv)));
+    t[1] = __dadd_rn(P.y, __dmul_rn(sr, __ddiv_rn(vy, dv)));
+    t[2] = __dadd_rn(P.z, __dmul_rn(sr, __ddiv_rn(vz, dv)));
+    return true;
+  };
+  // one candidate per lane (sphere at sorted slot j, or -1): all are settled
+  auto settle = [&](int j, int o, int side) {
+    bool open = j >= 0;
+    double t[3] = {0.0, 0.0, 0.0}, d2 = INFINITY;
+    if (open) open = tangent_point(o, side, t);
+    if (open && box_cull) open = ex_inbox(t[0], t[1], t[2]);
+    if (open) {
+      d2 = ex_d2(x, y, z, t[0], t[1], t[2]);
+      open = mode == kBelowSurvivor ? d2 < lim : (mode == kWithinOpposite ? __dsqrt_rn(d2) <= lim : true);
+    }
+    const int64_t id = 2 * int64_t(o) + side;
+    const float tx = float(t[0]), ty = float(t[1]), tz = float(t[2]);
+    const bool in_range = fabs(t[0]) <= A && fabs(t[1]) <= A && fabs(t[2]) <= A;
+    auto held = [&](const float4& P) {
+      const float dx = tx - P.x, dy = ty - P.y, dz = tz - P.z;
+      return fmaf(dx, dx, fmaf(dy, dy, dz * dz)) < P.w;
+    };
+    if (open && in_range)
+      for (int u = 0; u < nrec; ++u)
+        if (W.rec_id[u] != j && held(W.rec[u])) open = false;
+    for (;;) {
+      if (open && B.id >= 0 && (d2 > B.d2 || (d2 == B.d2 && id > B.id))) open = false;
+      const unsigned key = open ? __float_as_uint(float(d2)) : 0xffffffffu;
+      const unsigned low = __reduce_min_sync(kLanes, key);
+      const unsigned m = __ballot_sync(kLanes, open && key == low);
+      if (!m) return;
+      const int src = __ffs(m) - 1;
+      const int cj = __shfl_sync(kLanes, j, src);
+      bool covered;
+      if (__shfl_sync(kLanes, int(in_range), src)) {
+        const double qx = __shfl_sync(kLanes, t[0], src), qy = __shfl_sync(kLanes, t[1], src),
+                     qz = __shfl_sync(kLanes, t[2], src);
+        const float qxf = float(qx), qyf = float(qy), qzf = float(qz);
+        const int s = warp_cover_walk(T, C, W.cstk, lane, qxf, qyf, qzf, cover_lim, n_nodes, n_items,
+                                      [&](int c, float& v) {
+                                        if (c == cj) return false;
+                                        const float4 P = a.sph[c], Th = a.thr[c];
+                                        const float dx = qxf - P.x, dy = qyf - P.y, dz = qzf - P.z;
+                                        const float e2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+                                        if (!(e2 <= Th.w)) return false;
+                                        v = e2 - Th.z;
+                                        return e2 < Th.z || ex_cov(qx, qy, qz, a.sph64[a.sid[c]], a.tol);
+                                      });
+        covered = s >= 0;
+        if (covered) {
+          float4 P = a.sph[s];
+          P.w = a.thr[s].z;
+          if (open && in_range && j != s && held(P)) open = false;
+          __syncwarp();
+          if (lane == 0) {
+            W.rec[at] = P;
+            W.rec_id[at] = s;
+          }
+          at = (at + 1) % kTanRecent;
+          nrec = min(nrec + 1, kTanRecent);
+          __syncwarp();
+        }
+      } else {
+        covered = __shfl_sync(kLanes, lane == src ? int(covered_by_other(a, t[0], t[1], t[2], o) >= 0) : 0, src);
+      }
+      if (!covered) {
+        B.d2 = __shfl_sync(kLanes, d2, src);
+        B.id = __shfl_sync(kLanes, (long long)id, src);
+        hi_f = f_up(fmin(lim_d, sqrt(B.d2)) * kRel + kAbs);
+      }
+      if (lane == src) open = false;
+    }
+  };
+  warp_lin_walk(
+      T, C, W.stk, lane,
+      [&](int64_t nd) {
+        // bounds over the node's spheres of the class, d = |x - p| and r = |s|:
+        // linear from below; from above d - r <= D - res + S(n +- g) +
+        // |h|^2 / (2 (D - |h|)) (the chord's excess over its projection on n),
+        // res the least residual of r, or |x - F| + wf
+        const Lin q = lin_load(T, nd);
+        float nx = x32 - q.cx, ny = y32 - q.cy, nz = z32 - q.cz;
+        const float d = unit3(nx, ny, nz);
+        const float sp = fmaf(fabsf(nx + q.gx), q.hx, fmaf(fabsf(ny + q.gy), q.hy, fabsf(nz + q.gz) * q.hz));
+        const float sm = fmaf(fabsf(nx - q.gx), q.hx, fmaf(fabsf(ny - q.gy), q.hy, fabsf(nz - q.gz) * q.hz));
+        const float near_lo = cs == 0 ? d - q.hip - sp : d + q.lon - sm;
+        if (!(near_lo < INFINITY)) return false;  // none of the class
+        const float far_lo = cs == 0 ? d + q.lop - sm : d - q.hin - sp;
+        if (far_lo - hi_f <= mg) return true;
+        if (!(near_lo - hi_f <= mg)) return false;
+        if (-near_lo + mg >= lo_f) return true;
+        const float h2 = fmaf(q.hx, q.hx, fmaf(q.hy, q.hy, q.hz * q.hz)), hn = sqrtf(h2);
+        const float over = d > 2.f * hn ? 0.5f * h2 / (d - hn) * (1.f + 1e-5f) : INFINITY;
+        const float up = (cs == 0 ? d - q.lop + sp : d + q.hin + sm) + over;
+        if (!(up + mg >= lo_f)) return false;
+        const float4 Fb = T.nf[nd];
+        const float df = dist32(x32, y32, z32, Fb);
+        return df + Fb.w + err32(ax, Fb, df, Fb.w) >= lo_f;
+      },
+      [&](int64_t j) {
+        bool near = false, far = false;
+        int o = 0;
+        if (j >= 0) {
+          const float4 S = a.sph[j];
+          if (S.w != 0.f && int(S.w < 0.f) == cs) {
+            // screen: |x - t| is |d - r| (near) or d + r (far)
+            const float d32 = dist32(x32, y32, z32, S), r32 = fabsf(S.w);
+            const float er = err32(ax, S, d32, r32);
+            const float an32 = fabsf(d32 - r32), af32 = d32 + r32;
+            near = an32 + er >= lo_f && an32 - er <= hi_f;
+            far = af32 + er >= lo_f && af32 - er <= hi_f;
+            if (near || far) o = a.sid[j];
+          }
+        }
+        if (__any_sync(kLanes, near)) settle(near ? int(j) : -1, o, 0);
+        if (__any_sync(kLanes, far)) settle(far ? int(j) : -1, o, 1);
+      });
+}
+
 // tangent_one over the warp (lane 0 writes the outputs).
-__device__ inline void warp_tangent_one(const QueryArgs& a, int box_cull, int64_t q, uint32_t* stk, int lane) {
+__device__ inline void warp_tangent_one(const QueryArgs& a, const LevelTable& C, int box_cull, int64_t q, TanWarp& W,
+                                        int lane) {
   const int code = a.fl_out[q] & 15;
   if (code != GFS_CODE_SURVIVOR && code != GFS_CODE_OPPOSITE && code != GFS_CODE_LOWER) return;
   double x, y, z;
   load_point(a, q, x, y, z);
   SphereBounds S;
-  warp_sphere_bounds(a, x, y, z, stk, lane, S);
+  const float A = a.bc->A;
+  const bool lin = fabs(x) <= A && fabs(y) <= A && fabs(z) <= A;
+  if (lin) warp_sphere_bounds_lin(a, C, x, y, z, W, lane, S);
+  else warp_sphere_bounds(a, x, y, z, W.stk, lane, S);
   if (S.cov[0] == S.cov[1]) return;  // OUTSIDE / INVALID: not refined
   const int cs = S.cov[0] ? 0 : 1, co = 1 - cs;
   const bool have_u = S.idxA[co] != INT_MAX;
@@ -267,7 +575,8 @@ __device__ inline void warp_tangent_one(const QueryArgs& a, int box_cull, int64_
   B.d2 = INFINITY;
   B.id = -1;
   __syncwarp();
-  warp_tangent_search(a, box_cull, x, y, z, cs, mode, lim, lo, stk, lane, B);
+  if (lin) warp_tangent_search_lin(a, C, box_cull, x, y, z, cs, mode, lim, lo, W, lane, B);
+  else warp_tangent_search(a, box_cull, x, y, z, cs, mode, lim, lo, W.stk, lane, B);
   if (B.id < 0 || lane != 0) return;
   const double m = __dsqrt_rn(B.d2);
   if (a.clamp_opp && !(m <= ub)) return;  // the opposite tangent point stays the value
