@@ -19,11 +19,15 @@ constexpr int kScoreWarps = 4;
 __global__ void __launch_bounds__(32 * kScoreWarps) k_query_scored(QueryArgs a, int box_cull,
                                                                    const uint32_t* __restrict__ csr_ids,
                                                                    const int64_t* __restrict__ csr_off) {
-  __shared__ uint32_t s_stk[kScoreWarps][tangent::kWarpStack + kFan];
+  __shared__ tangent::TanWarp s_w[kScoreWarps];
+  __shared__ LevelTable s_lv;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t slot = int64_t(blockIdx.x) * kScoreWarps + w;
+  if (threadIdx.x < kMaxLevels)
+    s_lv.lv[threadIdx.x] = make_int2(int(a.st.offset[threadIdx.x]), int(a.st.count[threadIdx.x]));
+  __syncthreads();
   if (slot >= a.m) return;  // the same for the whole warp
-  scored::warp_scored_one(a, box_cull, csr_ids, csr_off, a.perm ? int64_t(a.perm[slot]) : slot, s_stk[w], lane);
+  scored::warp_scored_one(a, box_cull, csr_ids, csr_off, s_lv, a.perm ? int64_t(a.perm[slot]) : slot, s_w[w], lane);
 }
 
 // csr_off[i] = first position of sphere i's ids in the sorted id list

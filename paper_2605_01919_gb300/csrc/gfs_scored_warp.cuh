@@ -2,14 +2,18 @@
 //
 // The candidates, their order and every FP64 expression are those of
 // scored_one in gfs_scored.cuh (the host build checks that routine against the
-// oracle).  Here the 32 lanes walk the hierarchies for one point together
-// (warp_walk_until): each lane screens and evaluates its own nodes and items
-// and keeps its own best, and between rounds the lanes share the best so far
-// and the balls that covered the latest tangent points.  The chosen candidate
+// oracle).  Here the 32 lanes walk the hierarchies for one point together: in
+// the survivor walks (warp_walk_until) each lane screens and evaluates its own
+// nodes and items and keeps its own best, shared between rounds; the tangent
+// points come from the walk by linear bounds (warp_lin_walk), the best open one
+// is settled first, its coverage walked by the whole warp.  The chosen candidate
 // is the greatest valid one of a total order, so it does not depend on which
 // lane met it or when: a candidate is only dropped when a better one is known
 // or when it is not valid, and the two least farthest-survivor distances are
 // minima over distinct spheres.
+// Bound: latency, of the coverage walks and of the FP64 tests.  8,191 points of a
+// 48^3 union grid take 10 ms; 27 ms with ball bounds and a coverage walk per
+// lane, 145 ms with one point a lane.
 #pragma once
 
 #include "gfs_scored.cuh"
@@ -61,7 +65,8 @@ __device__ inline void warp_survivors(const QueryArgs& a, const Frame& F, int cl
 }
 
 __device__ inline void warp_scored_one(const QueryArgs& a, int box_cull, const uint32_t* __restrict__ csr_ids,
-                                       const int64_t* __restrict__ csr_off, int64_t q, uint32_t* stk, int lane) {
+                                       const int64_t* __restrict__ csr_off, const LevelTable& C, int64_t q,
+                                       tangent::TanWarp& W, int lane) {
   const int code = a.fl_out[q] & 15;
   if (code == GFS_CODE_SAMPLE || code == GFS_CODE_INVALID) return;
   const double tol = a.tol;
@@ -72,7 +77,11 @@ __device__ inline void warp_scored_one(const QueryArgs& a, int box_cull, const u
   F.z32 = float(F.z);
   F.ax = amax3(F.x32, F.y32, F.z32);
   tangent::SphereBounds SB;
-  tangent::warp_sphere_bounds(a, F.x, F.y, F.z, stk, lane, SB);
+  uint32_t* const stk = W.stk;
+  const float A = a.bc->A;
+  const bool lin = fabs(F.x) <= A && fabs(F.y) <= A && fabs(F.z) <= A;  // the range of the linear bounds
+  if (lin) tangent::warp_sphere_bounds_lin(a, C, F.x, F.y, F.z, W, lane, SB);
+  else tangent::warp_sphere_bounds(a, F.x, F.y, F.z, stk, lane, SB);
   if (SB.cov[0] && SB.cov[1]) return;  // INVALID (the plain query says so too)
   F.sig = SB.cov[0] ? 1 : (SB.cov[1] ? -1 : 0);
   F.ub[0] = SB.bestA[1];
@@ -161,53 +170,11 @@ __device__ inline void warp_scored_one(const QueryArgs& a, int box_cull, const u
   {
     const Tree& T = a.st;
     const float R32 = f_up(R);
-    // balls that covered the latest tangent points, the same on every lane
-    // (input index; centre in FP32, radius - tol rounded down), and the one
-    // this lane found last
-    constexpr int kHints = 4;
-    int hint[kHints];
-    float4 hintf[kHints];
-    int found = -1, at = 0;
-#pragma unroll
-    for (int u = 0; u < kHints; ++u) hint[u] = -1;
-    auto refresh = [&]() {
-      warp_best(B);
-      // up to two of the balls the lanes found since the last round
-      unsigned m = __ballot_sync(kLanes, found >= 0);
-#pragma unroll
-      for (int n = 0; n < 2; ++n) {
-        if (!m) break;
-        const int o = __shfl_sync(kLanes, found, __ffs(m) - 1);
-        m &= ~__ballot_sync(kLanes, found == o);
-        bool have = false;
-#pragma unroll
-        for (int u = 0; u < kHints; ++u) have = have || hint[u] == o;
-        if (have) continue;
-        const D4 Q = a.sph64[o];
-        const float4 f = make_float4(float(Q.x), float(Q.y), float(Q.z), tangent::f_dn(__dsub_rn(fabs(Q.w), tol)));
-#pragma unroll
-        for (int u = 0; u < kHints; ++u)
-          if (u == at) {
-            hint[u] = o;
-            hintf[u] = f;
-          }
-        at = (at + 1) % kHints;
-      }
-      found = -1;
-      return true;
-    };
-    auto uncovered_tan = [&](double tx, double ty, double tz, int j) -> bool {
-      if (found >= 0 && found != j && ex_cov(tx, ty, tz, a.sph64[found], a.tol)) return false;
-#pragma unroll
-      for (int u = 0; u < kHints; ++u) {
-        const int c = hint[u];
-        if (c >= 0 && c != j && ex_cov(tx, ty, tz, a.sph64[c], a.tol)) return false;
-      }
-      const int o = tangent::covered_except(a, tx, ty, tz, j, -1, -1);
-      if (o < 0) return true;
-      found = o;
-      return false;
-    };
+    // balls that covered the latest tangent points (W.rec: centre in FP32,
+    // radius - tol rounded down; W.rec_id: input index)
+    int nrec = 0, at = 0;
+    unsigned n_nodes = 0, n_items = 0;
+    const float cover_lim = -a.tol32 + a.bc->elin, mg = a.bc->elin + 8.f * tangent::kTanU * A;
     // as in scored_one: is the tangent point surely inside one of the balls
     auto surely_covered = [&](const float4& S, float d32, float sr, int j) -> bool {
       const float ap = amax3(S.x, S.y, S.z), r = fabsf(sr);
@@ -218,78 +185,153 @@ __device__ inline void warp_scored_one(const QueryArgs& a, int box_cull, const u
       const float mt = 64.f * 5.9604645e-8f * (F.ax + ap + r) * (1.f + r * inv);
       const float at_ = amax3(tx, ty, tz);
       bool in = false;
-#pragma unroll
-      for (int u = 0; u < kHints; ++u) {
-        if (hint[u] < 0 || hint[u] == j) continue;
-        const float dd = dist32(tx, ty, tz, hintf[u]);
-        in = in || dd + mt + err32(at_, hintf[u], dd, 0.f) < hintf[u].w;
+      for (int u = 0; u < nrec; ++u) {
+        if (W.rec_id[u] == j) continue;
+        const float4 f = W.rec[u];
+        const float dd = dist32(tx, ty, tz, f);
+        in = in || dd + mt + err32(at_, f, dd, 0.f) < f.w;
       }
       return in;
     };
-    warp_walk_until(
-        T, stk, tangent::kWarpStack, lane, &a.cnt->walk_err, refresh,
+    // one tangent point per lane (sphere at sorted slot jj, input index j; jj < 0
+    // for none): those that would beat the best so far are settled, the best
+    // of them first, its coverage walked by the whole warp
+    auto settle = [&](int jj, int j, int side) {
+      bool open = jj >= 0;
+      double p[3] = {0.0, 0.0, 0.0};
+      Best K = B;
+      auto rate = [&]() {  // the best value of this lane's point that beats B
+        open = false;
+        K = B;
+        try_candidate(a, F, p[0], p[1], p[2], int64_t(j), true, kTanKey + 2 * int64_t(j) + side, K, [&]() {
+          open = true;
+          return true;
+        });
+      };
+      if (open) {
+        const D4 P = a.sph64[j];
+        const double vx = __dsub_rn(F.x, P.x), vy = __dsub_rn(F.y, P.y), vz = __dsub_rn(F.z, P.z);
+        const double dv = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(vx, vx), __dmul_rn(vy, vy)), __dmul_rn(vz, vz)));
+        open = dv > 0.0;
+        if (open) {
+          const double sr = side == 0 ? fabs(P.w) : -fabs(P.w);
+          p[0] = __dadd_rn(P.x, __dmul_rn(sr, __ddiv_rn(vx, dv)));
+          p[1] = __dadd_rn(P.y, __dmul_rn(sr, __ddiv_rn(vy, dv)));
+          p[2] = __dadd_rn(P.z, __dmul_rn(sr, __ddiv_rn(vz, dv)));
+          open = !box_cull || ex_inbox(p[0], p[1], p[2]);
+        }
+        if (open) rate();
+      }
+      const bool in_range = fabs(p[0]) <= A && fabs(p[1]) <= A && fabs(p[2]) <= A;
+      for (;;) {
+        // 2 bits of class, the rest of the ranking value (which is >= 0)
+        const unsigned key = open ? (unsigned(K.cls) << 30) | (__float_as_uint(float(K.sr)) >> 1) : 0u;
+        const unsigned high = __reduce_max_sync(kLanes, key);
+        const unsigned m = __ballot_sync(kLanes, open && key == high);
+        if (!m) return;
+        const int src = __ffs(m) - 1;
+        int ball = -1;  // sorted slot or (out of range) input index of a ball that holds the point
+        const bool ranged = __shfl_sync(kLanes, int(in_range), src) != 0;
+        if (ranged) {
+          const double qx = __shfl_sync(kLanes, p[0], src), qy = __shfl_sync(kLanes, p[1], src),
+                       qz = __shfl_sync(kLanes, p[2], src);
+          const float qxf = float(qx), qyf = float(qy), qzf = float(qz);
+          const int cj = __shfl_sync(kLanes, jj, src);
+          ball = warp_cover_walk(T, C, W.cstk, lane, qxf, qyf, qzf, cover_lim, n_nodes, n_items, [&](int c, float& v) {
+            if (c == cj) return false;
+            const float4 P = a.sph[c], Th = a.thr[c];
+            const float dx = qxf - P.x, dy = qyf - P.y, dz = qzf - P.z;
+            const float e2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+            if (!(e2 <= Th.w)) return false;
+            v = e2 - Th.z;
+            return e2 < Th.z || ex_cov(qx, qy, qz, a.sph64[a.sid[c]], a.tol);
+          });
+          if (ball >= 0) ball = a.sid[ball];
+        } else {
+          if (lane == src) ball = tangent::covered_except(a, p[0], p[1], p[2], j, -1, -1);
+          ball = __shfl_sync(kLanes, ball, src);
+        }
+        if (ball >= 0) {
+          const D4 Q = a.sph64[ball];
+          if (lane == src || (open && ball != j && ex_cov(p[0], p[1], p[2], Q, a.tol))) open = false;
+          __syncwarp();
+          if (lane == 0) {
+            W.rec[at] = make_float4(float(Q.x), float(Q.y), float(Q.z), tangent::f_dn(__dsub_rn(fabs(Q.w), tol)));
+            W.rec_id[at] = ball;
+          }
+          at = (at + 1) % tangent::kTanRecent;
+          nrec = min(nrec + 1, tangent::kTanRecent);
+          __syncwarp();
+        } else {
+          B.cls = __shfl_sync(kLanes, K.cls, src);
+          B.sr = __shfl_sync(kLanes, K.sr, src);
+          B.key = __shfl_sync(kLanes, (long long)K.key, src);
+          B.sign = __shfl_sync(kLanes, K.sign, src);
+          B.r = __shfl_sync(kLanes, K.r, src);
+          if (lane == src) open = false;
+          if (open) rate();
+        }
+      }
+    };
+    tangent::warp_lin_walk(
+        T, C, stk, lane,
         [&](int64_t node) {
-          const float4 Bc = T.na[node], Fb = T.nf[node];
-          const float dC = dist32(F.x32, F.y32, F.z32, Bc), dF = dist32(F.x32, F.y32, F.z32, Fb);
-          return dC - err32(F.ax, Bc, dC, Bc.w) - Bc.w <= R32 || dF - err32(F.ax, Fb, dF, Fb.w) - Fb.w <= R32;
+          if (!lin) {
+            const float4 Bc = T.na[node], Fb = T.nf[node];
+            const float dC = dist32(F.x32, F.y32, F.z32, Bc), dF = dist32(F.x32, F.y32, F.z32, Fb);
+            return dC - err32(F.ax, Bc, dC, Bc.w) - Bc.w <= R32 || dF - err32(F.ax, Fb, dF, Fb.w) - Fb.w <= R32;
+          }
+          // the least d - r and d + r of the node's spheres, d = |x - p|
+          const Lin l = lin_load(T, node);
+          float nx = F.x32 - l.cx, ny = F.y32 - l.cy, nz = F.z32 - l.cz;
+          const float d = unit3(nx, ny, nz);
+          const float sp = fmaf(fabsf(nx + l.gx), l.hx, fmaf(fabsf(ny + l.gy), l.hy, fabsf(nz + l.gz) * l.hz));
+          const float sm = fmaf(fabsf(nx - l.gx), l.hx, fmaf(fabsf(ny - l.gy), l.hy, fabsf(nz - l.gz) * l.hz));
+          return fminf(d - l.hip - sp, d + l.lon - sm) - R32 <= mg || fminf(d + l.lop - sm, d - l.hin - sp) - R32 <= mg;
         },
-        [&](int64_t idx) {
-          const int64_t b = idx * kLeaf, e = imin64(b + kLeaf, a.n);
-          for (int64_t jj = b; jj < e; ++jj) {
+        [&](int64_t jj) {
+          bool near_ok = false, far_ok = false;
+          int j = 0;
+          if (jj >= 0) {
             const float4 S = a.sph[jj];
-            if (S.w == 0.f) continue;
-            const float d32 = dist32(F.x32, F.y32, F.z32, S), r32 = fabsf(S.w);
-            const float er = err32(F.ax, S, d32, r32);
-            bool near_ok = fabsf(d32 - r32) - er <= R32, far_ok = d32 + r32 - er <= R32;
-            if (!near_ok && !far_ok) continue;
-            const int j = a.sid[jj];
-            const int si = S.w > 0.f ? 1 : -1;
-            // FP32 screen against the best so far and V1, as in scored_one
+            if (S.w != 0.f) {
+              const float d32 = dist32(F.x32, F.y32, F.z32, S), r32 = fabsf(S.w);
+              const float er = err32(F.ax, S, d32, r32);
+              near_ok = fabsf(d32 - r32) - er <= R32;
+              far_ok = d32 + r32 - er <= R32;
+              if (near_ok || far_ok) j = a.sid[jj];
+              const int si = S.w > 0.f ? 1 : -1;
+              // FP32 screen against the best so far and V1, as in scored_one
 #pragma unroll
-            for (int side = 0; side < 2; ++side) {
-              bool& ok = side == 0 ? near_ok : far_ok;
-              if (!ok) continue;
-              const float rr = side == 0 ? fabsf(d32 - r32) : d32 + r32;
-              const float r_hi = rr + er, r_lo = rr - er;
-              const int dr = side == 1 ? 0 : (d32 - r32 > er ? 1 : (r32 - d32 > er ? -1 : 2));
-              bool any = false;
-              for (int sgi = 0; sgi < 2 && !any; ++sgi) {
-                const int sign = sgi == 0 ? 1 : -1;
-                if (F.sig != 0 && sign != F.sig) continue;
-                if (double(r_lo) - tol > F.ub[sgi]) continue;  // V1 fails for sure
-                if (B.cls < 0) {
-                  any = true;
-                  break;
+              for (int side = 0; side < 2; ++side) {
+                bool& ok = side == 0 ? near_ok : far_ok;
+                if (!ok) continue;
+                const float rr = side == 0 ? fabsf(d32 - r32) : d32 + r32;
+                const float r_hi = rr + er, r_lo = rr - er;
+                const int dr = side == 1 ? 0 : (d32 - r32 > er ? 1 : (r32 - d32 > er ? -1 : 2));
+                bool any = false;
+                for (int sgi = 0; sgi < 2 && !any; ++sgi) {
+                  const int sign = sgi == 0 ? 1 : -1;
+                  if (F.sig != 0 && sign != F.sig) continue;
+                  if (double(r_lo) - tol > F.ub[sgi]) continue;  // V1 fails for sure
+                  if (B.cls < 0) {
+                    any = true;
+                    break;
+                  }
+                  int cls;
+                  if (side == 1) cls = sign * si > 0 ? 3 : 0;
+                  else if (dr == 2) cls = 3;  // undecided: the highest it could be
+                  else cls = sign * si * dr < 0 ? 3 : 0;
+                  const double sr_hi = double(r_hi) * (sign > 0 ? 1.0 : 2.0);
+                  if (cls > B.cls || (cls == B.cls && sr_hi >= B.sr)) any = true;
                 }
-                int cls;
-                if (side == 1) cls = sign * si > 0 ? 3 : 0;
-                else if (dr == 2) cls = 3;  // undecided: the highest it could be
-                else cls = sign * si * dr < 0 ? 3 : 0;
-                const double sr_hi = double(r_hi) * (sign > 0 ? 1.0 : 2.0);
-                if (cls > B.cls || (cls == B.cls && sr_hi >= B.sr)) any = true;
+                if (!any || surely_covered(S, d32, side == 0 ? r32 : -r32, j)) ok = false;
               }
-              if (!any || surely_covered(S, d32, side == 0 ? r32 : -r32, j)) ok = false;
-            }
-            if (!near_ok && !far_ok) continue;
-            const D4 P = a.sph64[j];
-            const double r = fabs(P.w);
-            const double vx = __dsub_rn(F.x, P.x), vy = __dsub_rn(F.y, P.y), vz = __dsub_rn(F.z, P.z);
-            const double dv =
-                __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(vx, vx), __dmul_rn(vy, vy)), __dmul_rn(vz, vz)));
-            if (!(dv > 0.0)) continue;
-            for (int side = 0; side < 2; ++side) {
-              if (side == 0 ? !near_ok : !far_ok) continue;
-              const double sr = side == 0 ? r : -r;
-              const double tx = __dadd_rn(P.x, __dmul_rn(sr, __ddiv_rn(vx, dv)));
-              const double ty = __dadd_rn(P.y, __dmul_rn(sr, __ddiv_rn(vy, dv)));
-              const double tz = __dadd_rn(P.z, __dmul_rn(sr, __ddiv_rn(vz, dv)));
-              if (box_cull && !ex_inbox(tx, ty, tz)) continue;
-              try_candidate(a, F, tx, ty, tz, int64_t(j), true, kTanKey + 2 * int64_t(j) + side, B,
-                            [&]() { return uncovered_tan(tx, ty, tz, j); });
             }
           }
+          if (__any_sync(kLanes, near_ok)) settle(near_ok ? int(jj) : -1, j, 0);
+          if (__any_sync(kLanes, far_ok)) settle(far_ok ? int(jj) : -1, j, 1);
         });
-    warp_best(B);
   }
   if (lane != 0) return;
   if (B.cls < 0) {
