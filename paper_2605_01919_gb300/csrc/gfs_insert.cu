@@ -58,17 +58,6 @@ __device__ __forceinline__ bool tombed(const uint32_t* bits, int64_t slot) {
   return (bits[slot >> 5] >> (slot & 31)) & 1u;
 }
 
-__device__ __forceinline__ void warp_min_vu(double& v, uint32_t& idx) {
-  for (int o = 16; o > 0; o >>= 1) {
-    const double v2 = __shfl_xor_sync(kAll, v, o);
-    const uint32_t i2 = __shfl_xor_sync(kAll, idx, o);
-    if (v2 < v || (v2 == v && i2 < idx)) {
-      v = v2;
-      idx = i2;
-    }
-  }
-}
-
 // ---------------------------------------------------------------------------
 // Step query: one block of kQT threads.  Every node and item test runs first
 // in FP32 with an error margin that makes it conservative (it never drops a
@@ -82,13 +71,15 @@ constexpr int kQW = kQT / 32;
 constexpr int kQStack = 8192;  // walk stack entries (plus a reserve of kFan)
 constexpr float kRel = 1e-6f;  // ~16 ulp: relative margin of the FP32 filters
 
+constexpr int kDynBatch = 8;   // slots of inserted spheres a thread tests between FP64 passes (at most 8)
 constexpr int kQCap = 288;     // per-warp queue of items awaiting their FP64 evaluation
 static_assert(32 % kLeaf == 0, "a leaf's slots must share one tombstone word");
 
 struct QShared {
   uint32_t stk[kQStack + kFan];
-  double rd[4][kQW];
+  unsigned long long rk[4][kQW];
   uint32_t ri[4][kQW];
+  uint4 th[2][kQW];  // per warp: three FP32 thresholds (ordered bits) and flags, in turn
   int scan[kQW];
   // Survivors that pass a thread's FP32 screen are queued per warp with
   // their FP32 lower bound, while the thread's threshold already tightens to
@@ -103,35 +94,82 @@ struct QShared {
   int qn[kQW];
 };
 
+// order-preserving bits
+__device__ __forceinline__ uint32_t ord32(float v) {
+  const uint32_t b = __float_as_uint(v);
+  return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
+}
+__device__ __forceinline__ float ord32_value(uint32_t k) {
+  return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
+}
+__device__ __forceinline__ unsigned long long ord64(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(__dadd_rn(v, 0.0));  // -0 like +0
+  return (b >> 63) ? ~b : (b | (1ull << 63));
+}
+__device__ __forceinline__ double ord64_value(unsigned long long k) {
+  return __longlong_as_double((long long)((k >> 63) ? (k & ~(1ull << 63)) : ~k));
+}
+
+// lexicographic minimum of (key, index) over the warp
+__device__ __forceinline__ void warp_min_ku(unsigned long long& k, uint32_t& i) {
+  const uint32_t hi = __reduce_min_sync(kAll, uint32_t(k >> 32));
+  const uint32_t l = uint32_t(k >> 32) == hi ? uint32_t(k) : 0xffffffffu;
+  const uint32_t lo = __reduce_min_sync(kAll, l);
+  const bool at = uint32_t(k >> 32) == hi && uint32_t(k) == lo;
+  i = __reduce_min_sync(kAll, at ? i : 0xffffffffu);
+  k = ((unsigned long long)hi << 32) | lo;
+}
+
 // block-wide lexicographic (value, index) minimum of NV pairs; every thread
-// receives the result
+// receives the result.  The values are compared as integers: one FP64 compare
+// holds the SM's FP64 pipe for many cycles a warp, and the exchanges of every
+// walk round kept that pipe 27% busy in a step query of 228 us whose sixteen
+// blocks otherwise wait.  With integers, the round's thresholds in FP32
+// (block_thresholds) and the linear node bounds, the repair of 1,024 samples of
+// a 32^3 grid takes 99 ms instead of 117, 1,536 insertions into a 40^3 grid 17.6
+// instead of 20.5 ms.
 template <int NV>
 __device__ void block_argmin(double (&v)[NV], uint32_t (&idx)[NV], QShared& S) {
+  static_assert(kQW <= 32, "one lane per warp");
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
-  for (int i = 0; i < NV; ++i) warp_min_vu(v[i], idx[i]);
-  if (lane == 0) {
-#pragma unroll
-    for (int i = 0; i < NV; ++i) {
-      S.rd[i][w] = v[i];
+  for (int i = 0; i < NV; ++i) {
+    unsigned long long k = ord64(v[i]);
+    warp_min_ku(k, idx[i]);
+    if (lane == 0) {
+      S.rk[i][w] = k;
       S.ri[i][w] = idx[i];
     }
   }
   __syncthreads();
 #pragma unroll
   for (int i = 0; i < NV; ++i) {
-    v[i] = S.rd[i][0];
-    idx[i] = S.ri[i][0];
-    for (int k = 1; k < kQW; ++k) {
-      const double v2 = S.rd[i][k];
-      const uint32_t i2 = S.ri[i][k];
-      if (v2 < v[i] || (v2 == v[i] && i2 < idx[i])) {
-        v[i] = v2;
-        idx[i] = i2;
-      }
-    }
+    unsigned long long k = lane < kQW ? S.rk[i][lane] : ~0ull;
+    idx[i] = lane < kQW ? S.ri[i][lane] : 0xffffffffu;
+    warp_min_ku(k, idx[i]);
+    v[i] = ord64_value(k);
   }
   __syncthreads();
+}
+
+// block-wide minima of three FP32 thresholds and the or of two flags; turn
+// alternates from call to call, so that one barrier is enough
+__device__ __forceinline__ void block_thresholds(float& a, float& b, float& c, bool& f0, bool& f1, int& turn,
+                                                 QShared& S) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const uint32_t ka = __reduce_min_sync(kAll, ord32(a)), kb = __reduce_min_sync(kAll, ord32(b)),
+                 kc = __reduce_min_sync(kAll, ord32(c));
+  const uint32_t fl = __reduce_or_sync(kAll, (f0 ? 1u : 0u) | (f1 ? 2u : 0u));
+  if (lane == 0) S.th[turn][w] = make_uint4(ka, kb, kc, fl);
+  __syncthreads();
+  const uint4 t = lane < kQW ? S.th[turn][lane] : make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0u);
+  a = ord32_value(__reduce_min_sync(kAll, t.x));
+  b = ord32_value(__reduce_min_sync(kAll, t.y));
+  c = ord32_value(__reduce_min_sync(kAll, t.z));
+  const uint32_t f = __reduce_or_sync(kAll, t.w);
+  f0 = (f & 1u) != 0;
+  f1 = (f & 2u) != 0;
+  turn ^= 1;
 }
 
 // exclusive block prefix sum of cnt; total receives the block sum
@@ -262,14 +300,17 @@ __global__ void __launch_bounds__(kQT) k_ins_query(InsertArgs a) {
   const float xf = float(x), yf = float(y), zf = float(z);
   const float Ax = absmax3(xf, yf, zf);
   const double tol = a.tol;
+  // range and margin of the linear node bounds
+  const float A = a.bc->A, mg = a.bc->elin + 8.f * 5.9604645e-8f * A;
+  const bool in_range = fabs(x) <= A && fabs(y) <= A && fabs(z) <= A;
   // ---- spheres: sample, containment, nearest tangent per class, far bound
   // exact per-thread state (FP64, the oracle's expressions)
   bool cov0 = false, cov1 = false;
   double bA0 = INFINITY, bA1 = INFINITY, bF = INFINITY;
   uint32_t iA0 = 0xffffffffu, iA1 = 0xffffffffu;
   int sample = INT_MAX;
-  // block-wide thresholds of the last refresh
-  double tA0 = INFINITY, tA1 = INFINITY, tF = INFINITY;
+  int turn = 0;  // of the threshold exchange
+  // the block's containment as of the last exchange
   bool cw0 = false, cw1 = false;
   // FP32 upper bounds of min(block threshold, own best), for the filters
   float fA0 = INFINITY, fA1 = INFINITY, fF = INFINITY;
@@ -393,17 +434,11 @@ __global__ void __launch_bounds__(kQT) k_ins_query(InsertArgs a) {
     __syncwarp();
   };
   auto refresh_spheres = [&]() {
-    double v[3] = {bA0, bA1, bF};
-    uint32_t id[3] = {0, 0, 0};
-    block_argmin<3>(v, id, S);
-    tA0 = v[0];
-    tA1 = v[1];
-    tF = v[2];
-    fA0 = fminf(fA0, f_up(tA0));
-    fA1 = fminf(fA1, f_up(tA1));
-    fF = fminf(fF, f_up(tF));
-    cw0 = __syncthreads_or(cov0) != 0;
-    cw1 = __syncthreads_or(cov1) != 0;
+    // (every lane's thresholds are at most the FP32 upper bounds of its minima)
+    bool f0 = cov0, f1 = cov1;
+    block_thresholds(fA0, fA1, fF, f0, f1, turn, S);
+    cw0 = f0;
+    cw1 = f1;
   };
   // seed: warp 0 runs four greedy descents (nearest box, each class's
   // tangent bound, far bound); each group of 8 lanes evaluates the items of
@@ -439,6 +474,19 @@ __global__ void __launch_bounds__(kQT) k_ins_query(InsertArgs a) {
         // lower bounds over the node's spheres of |x-p| - r (per class),
         // |x-p| + r (far) and |x-p| (a sample at x): |x-C| - w, evaluated in
         // FP32 with margin
+        const float th0 = cw0 ? fA0 : fmaxf(fA0, ntol_up);
+        const float th1 = cw1 ? fA1 : fmaxf(fA1, ntol_up);
+        if (in_range) {
+          const Lin q = lin_load(a.st, node);
+          float nx = xf - q.cx, ny = yf - q.cy, nz = zf - q.cz;
+          const bool at = (fabsf(nx) <= q.hx + mg) & (fabsf(ny) <= q.hy + mg) & (fabsf(nz) <= q.hz + mg);
+          const float d = unit3(nx, ny, nz);
+          const float sp = fmaf(fabsf(nx + q.gx), q.hx, fmaf(fabsf(ny + q.gy), q.hy, fabsf(nz + q.gz) * q.hz));
+          const float sm = fmaf(fabsf(nx - q.gx), q.hx, fmaf(fabsf(ny - q.gy), q.hy, fabsf(nz - q.gz) * q.hz));
+          // (an absent class: inf - inf compares false)
+          return bool(at | (d - q.hip - sp - th0 <= mg) | (d + q.lon - sm - th1 <= mg) |
+                      (fminf(d + q.lop - sm, d - q.hin - sp) - fF <= mg));
+        }
         const float4 R = a.st.nb[node], Fb = a.st.nf[node];
         const float dc = sqrtf(ball_d2(xf, yf, zf, a.st.na[node]));
         const float df = sqrtf(ball_d2(xf, yf, zf, Fb));
@@ -447,8 +495,6 @@ __global__ void __launch_bounds__(kQT) k_ins_query(InsertArgs a) {
           const float E = kRel * (d + fabsf(w) + Ax) + 1e-30f;
           return d - w - E <= th;
         };
-        const float th0 = cw0 ? fA0 : fmaxf(fA0, ntol_up);
-        const float th1 = cw1 ? fA1 : fmaxf(fA1, ntol_up);
         return below(dc, R.z, 0.f) || below(dc, R.x, th0) || below(dc, R.y, th1) || below(df, Fb.w, fF);
       },
       [&](int64_t leaf) {
@@ -528,8 +574,8 @@ __global__ void __launch_bounds__(kQT) k_ins_query(InsertArgs a) {
   const double bAs = cs == 0 ? bA0 : bA1, bAo = cs == 0 ? bA1 : bA0;
   const uint32_t iAs = cs == 0 ? iA0 : iA1, iAo = cs == 0 ? iA1 : iA0;
   // ---- nearest live survivor of x's class ----------------------------------
-  double bd = INFINITY, td = INFINITY;  // squared distances: own best, block threshold
-  // FP32 upper bound of sqrt(min(td, bd)); with the opposite clamp a survivor
+  double bd = INFINITY;  // this thread's least squared distance
+  // FP32 upper bound of the distance; with the opposite clamp a survivor
   // farther than UB_opp never sets the value, so the search starts there
   float fd = (a.clamp_opp && iAo != 0xffffffffu) ? fmaxf(f_up(bAo), 0.f) : INFINITY;
   uint32_t gbest = 0xffffffffu;
@@ -576,12 +622,9 @@ __global__ void __launch_bounds__(kQT) k_ins_query(InsertArgs a) {
     __syncwarp();
   };
   auto refresh_surv = [&]() {
-    double v[2] = {bd, double(fd)};
-    uint32_t id[2] = {0, 0};
-    block_argmin<2>(v, id, S);
-    td = v[0];
-    fd = fminf(fd, float(v[1]));  // exact conversion: v[1] is a float
-    if (td < INFINITY) fd = fminf(fd, f_up_sqrt(td));
+    float b = INFINITY, c = INFINITY;
+    bool f0 = false, f1 = false;
+    block_thresholds(fd, b, c, f0, f1, turn, S);
   };
   {
     const Tree& T = a.vt[cs];
@@ -624,12 +667,24 @@ __global__ void __launch_bounds__(kQT) k_ins_query(InsertArgs a) {
       __syncthreads();
       const int tot = min(S.scan[0], kQStack);
       __syncthreads();
-      for (int base = 0; base < tot * a.KS; base += kQT) {
-        const int i = base + tid;
-        if (i < tot * a.KS) {
-          const int64_t slot = int64_t(list[i / a.KS]) * a.KS + i % a.KS;
-          if (!a.dtomb[cs][slot]) surv_filtered(a.dsurv[cs][slot]);
+      // (kDynBatch slots a thread, all loads before the first test: the
+      // iterations are bound by the loads' latency)
+      for (int base = 0; base < tot * a.KS; base += kDynBatch * kQT) {
+        float4 P[kDynBatch];
+        bool live[kDynBatch];
+#pragma unroll
+        for (int k = 0; k < kDynBatch; ++k) {
+          const int i = base + k * kQT + tid;
+          live[k] = false;
+          if (i < tot * a.KS) {
+            const int64_t slot = int64_t(list[i / a.KS]) * a.KS + i % a.KS;
+            live[k] = !a.dtomb[cs][slot];
+            P[k] = a.dsurv[cs][slot];
+          }
         }
+#pragma unroll
+        for (int k = 0; k < kDynBatch; ++k)
+          if (live[k]) surv_filtered(P[k]);
         drain_surv();
       }
       __syncthreads();
