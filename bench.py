@@ -327,7 +327,8 @@ def run_reference(args):
 # ----------------------------------------------------------------------------
 # the CUDA path
 # ----------------------------------------------------------------------------
-KERNEL_TU = ("gfs_kernels.cu", "gfs_internal.cuh", "gfs_kernels.h")
+KERNEL_TU = ("gfs_kernels.cu", "gfs_internal.cuh", "gfs_kernels.h", "gfs_warp.cuh", "gfs_sphere_pass.cuh",
+             "gfs_finish_pass.cuh", "gfs_cull.cuh")
 
 
 def kernel_hash() -> str:
@@ -957,8 +958,8 @@ def run_gfs(args):
                                         if roofline["peak"] else None)
     roofline["frac_of_nominal_peak"] = (roofline["achieved"] / peaks["fp32_tflops_nominal_max_clock"]
                                         if roofline["achieved"] else None)
-    cull_roofline = alu_roofline("k_cull", last["cull_items"], 8,
-                                 "(open candidate, sphere) coverage tests after the neighbour pre-test", cull,
+    cull_roofline = alu_roofline("k_cull_walk", last["cull_items"], 8,
+                                 "(open candidate, sphere) coverage tests of the walks", cull,
                                  peaks, node_tests_per_launch=last["cull_node_tests"])
 
     line = {

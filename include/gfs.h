@@ -122,10 +122,11 @@ int gfs_build(gfs_ctx* ctx, const double* p_xyz, const double* s, int64_t n);
  * s64_out:   device, m FP64 values (nullable).
  * argmin_out:device, m int64 (nullable): candidate id or sphere index, per code.
  * flags_out: device, m uint16 result words (nullable).
- * Runs as two kernels (the pass over the spheres, then the pass over the
- * survivors and the exact re-evaluations) plus, for points outside the FP32
+ * Runs as three kernels (the pass over the spheres, the pass over the
+ * survivors, the decisions with their exact re-evaluations; each with a
+ * second launch for the points it listed) plus, for points outside the FP32
  * error model's coordinate range, the FP64 kernel.  Grows library-owned
- * scratch when m grows (Morton keys and order, 48 B of state per point).
+ * scratch when m grows (Morton keys and order, 64 B of state per point).
  * No host synchronisation.
  * Errors: GFS_ERR_STATE (no build), GFS_ERR_ARG, GFS_ERR_TOO_LARGE
  * (m >= 2^32), GFS_ERR_OOM, GFS_ERR_CUDA. */
@@ -143,7 +144,7 @@ int gfs_query(gfs_ctx* ctx, const void* x, int x_is_fp32, int64_t m, float* s_ou
  * 2j + side) sets the value, clamped by UB_opp as in gfs_query, with the same
  * bound checks; a tangent winner gets code GFS_CODE_TANGENT and argmin
  * 2j + side (side 0 near, 1 far).  Other points are left unchanged.
- * Decisions are taken in FP64 (one thread per point; slower than gfs_query).
+ * Decisions are taken in FP64 (one warp per point; slower than gfs_query).
  * x, m:       the points of the preceding gfs_query on this context.
  * argmin_out, flags_out: that call's outputs (device, required): read, then
  *             rewritten in place where a tangent point wins.

@@ -201,7 +201,7 @@ struct gfs_ctx {
   DevBuf h_p, h_s, h_x, h_sout, h_arg, h_fl;
   cudaStream_t side = nullptr;  // the query points' upload, overlapping the build
   cudaEvent_t sev = nullptr, sev2 = nullptr;  // main -> side, side -> main
-  DevBuf qstate;                // per-slot state between the query's two kernels
+  DevBuf qstate;                // per-slot state between the query's kernels
   // phase events (timing = 1): build start, cull start, cull end, build end,
   // query start, fast end, query end
   cudaEvent_t ev[8] = {};  // + end of the query's sphere pass

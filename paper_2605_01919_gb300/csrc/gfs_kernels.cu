@@ -1,11 +1,13 @@
 // Device kernels of the consistent-SDF hot path.
 //
-//   P build   k_cull          -- candidate generation and coverage culling
+//   P build   k_cull_test     -- candidate generation, coverage by the balls
+//                                that covered their direction's neighbours
+//             k_cull_walk     -- coverage walk of the candidates left open
 //                                (Def. 1 discretised, Prop. 1 (ii))
 //   query     k_query_spheres -- FP32 pass over the spheres (containment,
 //                                tangent and far bounds), state per point
-//             k_query_finish  -- FP32 pass over the survivors, certified
-//                                decisions, value and flags
+//             k_query_near    -- FP32 pass over the survivors
+//             k_query_decide  -- certified decisions, value and flags
 //             k_query_exact   -- FP64 evaluation, used for every decision the
 //                                FP32 path cannot certify (and precision=1)
 //   backward  k_query_grad    -- d s*/d(x, p_i, s_i) through the argmin

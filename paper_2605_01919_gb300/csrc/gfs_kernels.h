@@ -241,8 +241,8 @@ inline int64_t cull_launches(int KH, int64_t tiles, int64_t chunk) {
 // batch (one: any view, for the options and table sizes)
 cudaError_t launch_cull(const CullArgs& one, const CullArgs* views, const int64_t* prefix, int ns, int64_t tiles,
                         const CullWork& w, cudaStream_t st);
-// the query in two kernels: phase 1 (sphere pass, state to a.state), phase 2
-// (survivor pass, exact re-evaluation, flags, outputs)
+// the query: phase 1 (sphere pass, state to a.state), phase 2 (survivor pass,
+// then decisions, flags, outputs)
 cudaError_t launch_query_spheres(const QueryArgs& a, cudaStream_t st);
 cudaError_t launch_query_finish(const QueryArgs& a, cudaStream_t st);
 cudaError_t launch_query_exact(const QueryArgs& a, int all, cudaStream_t st);
