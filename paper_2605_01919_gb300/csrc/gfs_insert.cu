@@ -1095,14 +1095,21 @@ __global__ void __launch_bounds__(256) k_ins_dyn_near(InsertArgs a) {
 }
 
 // The new spheres' candidates and witnesses, culled against every other
-// sphere: one warp per (new sphere, candidate), a warp-parallel walk of the
-// sphere hierarchy that stops at the first covering ball (FP32 decisions
-// where provably away from the boundary, FP64 otherwise), then the spheres
-// inserted since the rebuild.  Survivors join the dynamic lists.
+// sphere: one warp per (new sphere, candidate), first the spheres inserted
+// since the rebuild that reach the new one, then the hierarchy
+// (warp_cover_walk, which stops at the first covering ball; points outside the
+// range of the linear bounds walk by the balls).  FP32 decisions where provably
+// away from the boundary, FP64 otherwise.  Survivors join the dynamic lists.
+// Bound: the latency of the walks' rounds.  INSCULL
 __global__ void __launch_bounds__(128) k_ins_cull_new(InsertArgs a) {
+  static_assert(kUStack + kFan >= kCoverStack, "one stack serves both walks");
   __shared__ uint32_t s_stk[4][kUStack + kFan];
+  __shared__ LevelTable s_lv;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   uint32_t* stk = s_stk[wib];
+  if (threadIdx.x < kMaxLevels)
+    s_lv.lv[threadIdx.x] = make_int2(int(a.st.offset[threadIdx.x]), int(a.st.count[threadIdx.x]));
+  __syncthreads();
   const int KS = a.KS;
   const int per = (KS + 3) / 4;
   const int which = int(blockIdx.x) / per;
@@ -1153,22 +1160,35 @@ __global__ void __launch_bounds__(128) k_ins_cull_new(InsertArgs a) {
     for (int q = lane; q < ndyn && !covered; q += 32)
       if (covered_by(a.dyn_f4[q], a.dyn_ids[q])) covered = true;
   }
-  warp_walk_until(
-      a.st, stk, kUStack, lane, &a.misc->err, [&]() { return !__any_sync(kAll, covered); },
-      [&](int64_t node) {
-        // some sphere of the node has |q-p| - r < -tol only if
-        // |q-C| - max(wp, wn) < -tol
-        const float4 B = a.st.na[node];
-        if (!(B.w > -INFINITY)) return false;
-        const float dc = sqrtf(ball_d2(qxf, qyf, qzf, B));
-        const float E = kRel * (dc + fabsf(B.w) + Aq) + 1e-30f;
-        return dc - B.w - E < ntol_up;
-      },
-      [&](int64_t leaf) {
-        const int64_t b = leaf * kLeaf, e = min(b + kLeaf, a.st.nitems);
-        for (int64_t j = b; j < e && !covered; ++j)
-          if (covered_by(a.sph[j], a.sid[j])) covered = true;
-      });
+  const float A = a.bc->A;
+  if (__any_sync(kAll, covered)) {
+    covered = true;
+  } else if (a.st.nlevels > 0 && fabs(qx) <= A && fabs(qy) <= A && fabs(qz) <= A) {
+    unsigned n_nodes = 0, n_items = 0;
+    covered = warp_cover_walk(a.st, s_lv, stk, lane, qxf, qyf, qzf, ntol_up + a.bc->elin, n_nodes, n_items,
+                              [&](int c, float& v) {
+                                const float4 P = a.sph[c];
+                                v = sqrtf(ball_d2(qxf, qyf, qzf, P)) - fabsf(P.w);
+                                return covered_by(P, a.sid[c]);
+                              }) >= 0;
+  } else {
+    warp_walk_until(
+        a.st, stk, kUStack, lane, &a.misc->err, [&]() { return !__any_sync(kAll, covered); },
+        [&](int64_t node) {
+          // some sphere of the node has |q-p| - r < -tol only if
+          // |q-C| - max(wp, wn) < -tol
+          const float4 B = a.st.na[node];
+          if (!(B.w > -INFINITY)) return false;
+          const float dc = sqrtf(ball_d2(qxf, qyf, qzf, B));
+          const float E = kRel * (dc + fabsf(B.w) + Aq) + 1e-30f;
+          return dc - B.w - E < ntol_up;
+        },
+        [&](int64_t leaf) {
+          const int64_t b = leaf * kLeaf, e = min(b + kLeaf, a.st.nitems);
+          for (int64_t j = b; j < e && !covered; ++j)
+            if (covered_by(a.sph[j], a.sid[j])) covered = true;
+        });
+  }
   covered = __any_sync(kAll, covered);
   if (lane == 0) {
     const uint32_t g = uint32_t(jn) * uint32_t(KS) + uint32_t(k);

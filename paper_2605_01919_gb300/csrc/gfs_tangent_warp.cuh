@@ -20,7 +20,7 @@ namespace gfs {
 namespace tangent {
 
 constexpr unsigned kLanes = 0xffffffffu;
-constexpr int kWarpStack = kCoverStack - kFan;  // per-warp walk stack entries (plus a reserve of kFan)
+constexpr int kWarpStack = 512;  // per-warp walk stack entries (plus a reserve of kFan)
 
 // lexicographic minimum of (v, i) over the warp, on every lane
 __device__ __forceinline__ void warp_min_vi(double& v, int& i) {
@@ -253,8 +253,9 @@ __device__ inline void warp_tangent_search(const QueryArgs& a, int box_cull, dou
 constexpr int kTanRecent = 8;
 constexpr float kTanU = 5.9604644775390625e-8f;  // 2^-24
 
+static_assert(kWarpStack + kFan >= kCoverStack, "warp_lin_walk's stack");
 struct TanWarp {
-  uint32_t stk[kCoverStack], cstk[kCoverStack];
+  uint32_t stk[kWarpStack + kFan], cstk[kCoverStack];  // (the first serves both kinds of walk)
   float4 rec[kTanRecent];  // (centre, squared distance below which a point is held for sure)
   int rec_id[kTanRecent];  // sorted slot
 };
