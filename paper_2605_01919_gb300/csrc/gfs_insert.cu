@@ -1100,7 +1100,9 @@ __global__ void __launch_bounds__(256) k_ins_dyn_near(InsertArgs a) {
 // (warp_cover_walk, which stops at the first covering ball; points outside the
 // range of the linear bounds walk by the balls).  FP32 decisions where provably
 // away from the boundary, FP64 otherwise.  Survivors join the dynamic lists.
-// Bound: the latency of the walks' rounds.  INSCULL
+// Bound: the latency of the walks' rounds.  With the walk by ball bounds, 32
+// nodes a round and their children in turn, 1,536 insertions into a 40^3 grid
+// took 17.7 ms (7.4 of them here), now 14.2.
 __global__ void __launch_bounds__(128) k_ins_cull_new(InsertArgs a) {
   static_assert(kUStack + kFan >= kCoverStack, "one stack serves both walks");
   __shared__ uint32_t s_stk[4][kUStack + kFan];
