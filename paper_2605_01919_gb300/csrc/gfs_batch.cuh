@@ -66,23 +66,23 @@ __global__ void k_batch_gather(const D4* __restrict__ sph64, const int* __restri
 }
 
 // one level of every shape's hierarchy; prefix[s] = first node of shape s
-// at this level in the launch's index space
-__global__ void k_batch_tree_level(const Tree* __restrict__ trees, const int64_t* __restrict__ prefix, int ns,
+// at this level in the launch's index space (spheres: two threads per node)
+__global__ void __launch_bounds__(kNodeBlock) k_batch_tree_level(const Tree* __restrict__ trees, const int64_t* __restrict__ prefix, int ns,
                                    int level, const float4* __restrict__ items_base,
                                    const int64_t* __restrict__ item_off, const BuildConsts* __restrict__ bc,
                                    int is_sphere) {
-  const int64_t g = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+  const int64_t g = is_sphere ? node_of_thread() : blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
   if (g >= prefix[ns]) return;
   const int s = find_seg(prefix, ns, g);
   const Tree& T = trees[s];
   const int64_t j = g - prefix[s];
   if (level == 0) {
     const float4* items = items_base + item_off[s];
-    if (is_sphere) sphere_leaf_node(items, bc[s].A, T, j);
+    if (is_sphere) sphere_leaf_node(items, bc[s].A, T, j, node_part());
     else point_leaf_node(items, T.nitems, T.lo, T.hi, j);
   } else {
     if (is_sphere)
-      sphere_level_node(T, bc[s].A, level, j);
+      sphere_level_node(T, bc[s].A, level, j, node_part());
     else
       point_level_node(T.lo, T.hi, T.offset[level - 1], T.count[level - 1], T.offset[level], j);
   }
@@ -310,8 +310,8 @@ cudaError_t launch_batch_surv_forest(const uint16_t* shape, const float4* raw, c
   // the grid (the kernel reads the exact total from the prefix)
   int64_t bound = int64_t(cap) / kLeaf + ns + 1;
   for (int l = 0; l < nlev; ++l) {
-    k_batch_tree_level<<<nb(bound, 128), 128, 0, st>>>(trees, prefix + int64_t(l) * (ns + 1), ns, l, sorted,
-                                                       soff, nullptr, 0);
+    k_batch_tree_level<<<nb(bound, kNodeBlock), kNodeBlock, 0, st>>>(trees, prefix + int64_t(l) * (ns + 1), ns, l,
+                                                                     sorted, soff, nullptr, 0);
     bound = bound / kFan + ns + 1;
   }
   return cudaGetLastError();
@@ -344,7 +344,7 @@ cudaError_t launch_batch_tree_level(const Tree* trees, const int64_t* prefix, in
                                     const float4* items_base, const int64_t* item_off, const BuildConsts* bc,
                                     int is_sphere, cudaStream_t st) {
   if (total == 0) return cudaSuccess;
-  k_batch_tree_level<<<nb(total, 128), 128, 0, st>>>(trees, prefix, ns, level, items_base, item_off, bc, is_sphere);
+  k_batch_tree_level<<<nb(total, is_sphere ? kNodesPerBlock : kNodeBlock), kNodeBlock, 0, st>>>(trees, prefix, ns, level, items_base, item_off, bc, is_sphere);
   return cudaGetLastError();
 }
 
