@@ -429,7 +429,8 @@ int gfs_batch_build(gfs_ctx* ctx, const gfs_shape* shapes_host, int nshapes);
  * and Morton-sorted, sample forest, cull, survivor forests laid out from the
  * device-side survivor counts, query views -- issues no host
  * synchronisation, no allocation and no host-to-device copy, so it can be
- * captured in a CUDA graph together with gfs_batch_query and replayed.
+ * captured in a CUDA graph together with gfs_batch_query and replayed (until
+ * the next gfs_batch_build; the context's other calls use other buffers).
  * Capacities are the first build's: survivors beyond the survivor capacity
  * are dropped and set a status bit (read with gfs_batch_status; the
  * results of that rebuild are then not valid -- call gfs_batch_build again,

@@ -120,6 +120,11 @@ void lin_layout(Tree& T, void* buf, int64_t nodes) {
   T.ln3 = reinterpret_cast<float*>(T.ln2 + nodes);
 }
 
+// the cull's workspace (see cull_work)
+struct CullBufs {
+  DevBuf hint, list, count;
+};
+
 #define GFS_CK(expr)                         \
   do {                                       \
     cudaError_t e_ = (expr);                 \
@@ -143,7 +148,7 @@ struct gfs_ctx {
   int K = 0, KS = 0;
   DevBuf U4, U64, hsrc;
   int KH = 0;  // directions whose covering balls the cull keeps
-  DevBuf cull_hint, cull_list, cull_count;
+  CullBufs cull;
   // spheres
   int64_t n = 0;
   bool built = false;
@@ -175,7 +180,10 @@ struct gfs_ctx {
   double ins_ms_total = 0.0, ins_ms_rebuild = 0.0, ins_ms_final = 0.0;  // host wall time of its phases
   double ins_ms_query = 0.0, ins_ms_commit = 0.0, ins_ms_update = 0.0;  // device time (timing = 1)
   unsigned long long ins_work[4] = {0, 0, 0, 0};  // step-query work counters (InsMisc::work)
-  // batched shapes
+  // batched shapes.  Everything that gfs_batch_rebuild and gfs_batch_query
+  // touch belongs to the batch (its sort scratch and cull workspace too): a
+  // graph they were captured in keeps these pointers, and the other calls,
+  // which grow (free) the buffers above, must not take them away.
   int b_ns = 0;
   bool b_built = false;
   std::vector<gfs_shape> b_shapes;
@@ -184,7 +192,8 @@ struct gfs_ctx {
   DevBuf b_desc, b_offd, b_qoffd, b_sph64, b_k64in, b_k64out, b_sph, b_thr, b_cvl, b_sid, b_bits, b_bcs;
   DevBuf b_lo, b_hi, b_na, b_nb, b_nf, b_ln, b_tight, b_stdev, b_prefix, b_ctr, b_cnt, b_cviews;
   DevBuf b_sraw[2], b_sshape[2], b_ssorted[2], b_vlo[2], b_vhi[2], b_vtdev[2], b_hist;
-  DevBuf b_qkin, b_qkout, b_qvin, b_qvout, b_qviews, b_qw, b_qstate;
+  DevBuf b_qkin, b_qkout, b_qvin, b_qvout, b_qviews, b_qw, b_qstate, b_vals_in, b_vals_out, b_cub_temp;
+  CullBufs b_cull;
   std::vector<QueryArgs> b_qv;  // host copies of the per-shape query views
   DevBuf b_status, b_vprefix[2], b_sodev[2];
   std::vector<int64_t> b_sph_level_total;  // nodes per level of the sample forest, over all shapes
@@ -434,16 +443,16 @@ int reset_cull_counters(gfs_ctx* c, cudaStream_t st) {
 
 // The cull's workspace for `tiles` tiles, in chunks of at most 1 GB of
 // covering balls and open-list entries (a chunk's entries number below 2^32).
-int cull_work(gfs_ctx* c, int64_t tiles, CullWork& w) {
+int cull_work(gfs_ctx* c, CullBufs& b, int64_t tiles, CullWork& w) {
   const int64_t last = c->K - c->KH;  // directions of the last level(s), the largest group
   const int64_t per = (int64_t(c->KH) + last) * kCullTileSpheres * 4;
   w.chunk = std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t(1) << 30) / per));
-  GFS_TRY(ensure(c->cull_hint, size_t(w.chunk) * std::max(1, c->KH) * kCullTileSpheres * 4));
-  GFS_TRY(ensure(c->cull_list, size_t(w.chunk) * size_t(last) * kCullTileSpheres * 4));
-  GFS_TRY(ensure(c->cull_count, size_t(cull_launches(c->KH, tiles, w.chunk)) * 8));
-  w.hint = c->cull_hint.as<int>();
-  w.list = c->cull_list.as<uint32_t>();
-  w.count = c->cull_count.as<unsigned>();
+  GFS_TRY(ensure(b.hint, size_t(w.chunk) * std::max(1, c->KH) * kCullTileSpheres * 4));
+  GFS_TRY(ensure(b.list, size_t(w.chunk) * size_t(last) * kCullTileSpheres * 4));
+  GFS_TRY(ensure(b.count, size_t(cull_launches(c->KH, tiles, w.chunk)) * 8));
+  w.hint = b.hint.as<int>();
+  w.list = b.list.as<uint32_t>();
+  w.count = b.count.as<unsigned>();
   return GFS_OK;
 }
 
@@ -500,7 +509,7 @@ int build_finish(gfs_ctx* c) {
     if (c->have_ev) GFS_CK(cudaEventRecord(c->ev[1], st));
     CullWork w;
     const int64_t tiles = (n + kCullTileSpheres - 1) / kCullTileSpheres;
-    GFS_TRY(cull_work(c, tiles, w));
+    GFS_TRY(cull_work(c, c->cull, tiles, w));
     GFS_CK(launch_cull(a, nullptr, nullptr, 0, tiles, w, st));
     if (c->have_ev) GFS_CK(cudaEventRecord(c->ev[2], st));
     unsigned int ns[2] = {0, 0};
@@ -1326,12 +1335,12 @@ int batch_build_device_samples(gfs_ctx* c) {
   const int64_t N = c->b_off[size_t(ns)];
   GFS_CK(cudaMemsetAsync(c->b_bits.p, 0, size_t(ns) * 8, st));
   GFS_CK(launch_batch_copy(c->b_desc.as<ShapeDesc>(), c->b_offd.as<int64_t>(), ns, N, c->b_sph64.as<D4>(),
-                           c->b_k64in.as<unsigned long long>(), c->vals_in.as<int>(), c->b_bits.as<unsigned int>(),
+                           c->b_k64in.as<unsigned long long>(), c->b_vals_in.as<int>(), c->b_bits.as<unsigned int>(),
                            c->b_bcs.as<BuildConsts>(), st));
-  size_t bytes = c->cub_temp.bytes;
-  GFS_CK(sort_pairs64(c->cub_temp.p, bytes, c->b_k64in.as<unsigned long long>(), c->b_k64out.as<unsigned long long>(),
-                      c->vals_in.as<int>(), c->vals_out.as<int>(), N, c->b_end_bit, st));
-  GFS_CK(launch_batch_gather(c->b_sph64.as<D4>(), c->vals_out.as<int>(), c->b_offd.as<int64_t>(), ns, N,
+  size_t bytes = c->b_cub_temp.bytes;
+  GFS_CK(sort_pairs64(c->b_cub_temp.p, bytes, c->b_k64in.as<unsigned long long>(), c->b_k64out.as<unsigned long long>(),
+                      c->b_vals_in.as<int>(), c->b_vals_out.as<int>(), N, c->b_end_bit, st));
+  GFS_CK(launch_batch_gather(c->b_sph64.as<D4>(), c->b_vals_out.as<int>(), c->b_offd.as<int64_t>(), ns, N,
                              c->b_bcs.as<BuildConsts>(), float(c->opt.tol), c->opt.tol, c->b_sph.as<float4>(),
                              c->b_thr.as<float4>(), c->b_cvl.as<float4>(), c->b_sid.as<int>(), st));
   return batch_sphere_levels(c);
@@ -1349,7 +1358,7 @@ int batch_build_device(gfs_ctx* c, bool cull_only) {
   if (!cull_only) GFS_TRY(batch_build_device_samples(c));
   GFS_CK(cudaMemsetAsync(c->b_cnt.p, 0, sizeof(Counters), st));
   CullWork w;
-  GFS_TRY(cull_work(c, c->b_cull_tiles, w));  // (sized by the first build)
+  GFS_TRY(cull_work(c, c->b_cull, c->b_cull_tiles, w));  // (sized by the first build)
   CullArgs one;
   std::memset(&one, 0, sizeof(one));
   one.K = c->K;
@@ -1360,7 +1369,7 @@ int batch_build_device(gfs_ctx* c, bool cull_only) {
     GFS_CK(launch_batch_surv_forest(
         c->b_sshape[k].as<uint16_t>(), c->b_sraw[k].as<float4>(), c->b_cnt.as<Counters>(), k, c->b_cap, ns,
         c->b_hist.as<unsigned>(), c->b_k64in.as<unsigned long long>(), c->b_k64out.as<unsigned long long>(),
-        c->vals_in.as<int>(), c->vals_out.as<int>(), c->cub_temp.p, c->cub_temp.bytes, c->b_end_bit,
+        c->b_vals_in.as<int>(), c->b_vals_out.as<int>(), c->b_cub_temp.p, c->b_cub_temp.bytes, c->b_end_bit,
         c->b_ssorted[k].as<float4>(), c->b_node_cap, c->b_vlo[k].as<float4>(), c->b_vhi[k].as<float4>(),
         c->b_vtdev[k].as<Tree>(), c->b_vprefix[k].as<int64_t>(), c->b_surv_levels, c->b_sodev[k].as<int64_t>(),
         c->b_qviews.as<QueryArgs>(), c->b_status.as<unsigned>(), st));
@@ -1417,8 +1426,8 @@ int gfs_batch_build(gfs_ctx* c, const gfs_shape* shapes, int ns) {
   GFS_TRY(ensure(c->b_sph64, size_t(N) * sizeof(D4)));
   GFS_TRY(ensure(c->b_k64in, size_t(std::max(N, M)) * 8));
   GFS_TRY(ensure(c->b_k64out, size_t(std::max(N, M)) * 8));
-  GFS_TRY(ensure(c->vals_in, size_t(N) * 4));
-  GFS_TRY(ensure(c->vals_out, size_t(N) * 4));
+  GFS_TRY(ensure(c->b_vals_in, size_t(N) * 4));
+  GFS_TRY(ensure(c->b_vals_out, size_t(N) * 4));
   GFS_TRY(ensure(c->b_sph, size_t(N) * sizeof(float4)));
   GFS_TRY(ensure(c->b_thr, size_t(N) * sizeof(float4)));
   GFS_TRY(ensure(c->b_sid, size_t(N) * 4));
@@ -1431,8 +1440,8 @@ int gfs_batch_build(gfs_ctx* c, const gfs_shape* shapes, int ns) {
   {
     size_t bytes = 0;
     GFS_CK(sort_pairs64(nullptr, bytes, c->b_k64in.as<unsigned long long>(), c->b_k64out.as<unsigned long long>(),
-                        c->vals_in.as<int>(), c->vals_out.as<int>(), N, c->b_end_bit, st));
-    GFS_TRY(ensure(c->cub_temp, bytes));
+                        c->b_vals_in.as<int>(), c->b_vals_out.as<int>(), N, c->b_end_bit, st));
+    GFS_TRY(ensure(c->b_cub_temp, bytes));
   }
   // sample forest: static layout (depends on the sample counts only)
   c->b_st.assign(ns, Tree{});
@@ -1563,8 +1572,8 @@ int gfs_batch_build(gfs_ctx* c, const gfs_shape* shapes, int ns) {
   }
   GFS_TRY(ensure(c->b_k64in, size_t(std::max<int64_t>(std::max(N, M), capu)) * 8));
   GFS_TRY(ensure(c->b_k64out, size_t(std::max<int64_t>(std::max(N, M), capu)) * 8));
-  GFS_TRY(ensure(c->vals_in, size_t(std::max<int64_t>(N, capu)) * 4));
-  GFS_TRY(ensure(c->vals_out, size_t(std::max<int64_t>(N, capu)) * 4));
+  GFS_TRY(ensure(c->b_vals_in, size_t(std::max<int64_t>(N, capu)) * 4));
+  GFS_TRY(ensure(c->b_vals_out, size_t(std::max<int64_t>(N, capu)) * 4));
   for (int k = 0; k < 2; ++k) {
     GFS_TRY(ensure(c->b_ssorted[k], size_t(capu) * sizeof(float4) + 16));
     GFS_TRY(ensure(c->b_vlo[k], size_t(c->b_node_cap) * sizeof(float4)));
@@ -1576,8 +1585,8 @@ int gfs_batch_build(gfs_ctx* c, const gfs_shape* shapes, int ns) {
   {
     size_t bytes = 0;
     GFS_CK(sort_pairs64(nullptr, bytes, c->b_k64in.as<unsigned long long>(), c->b_k64out.as<unsigned long long>(),
-                        c->vals_in.as<int>(), c->vals_out.as<int>(), int64_t(capu), c->b_end_bit, st));
-    GFS_TRY(ensure(c->cub_temp, bytes));
+                        c->b_vals_in.as<int>(), c->b_vals_out.as<int>(), int64_t(capu), c->b_end_bit, st));
+    GFS_TRY(ensure(c->b_cub_temp, bytes));
   }
   // query views and work items (shape, 32 points); the survivor pointers and
   // trees are filled in by the device-side survivor forests
@@ -1627,14 +1636,14 @@ int gfs_batch_build(gfs_ctx* c, const gfs_shape* shapes, int ns) {
   size_t bytes = 0;
   GFS_CK(sort_pairs64(nullptr, bytes, c->b_qkin.as<unsigned long long>(), c->b_qkout.as<unsigned long long>(),
                       c->b_qvin.as<int>(), c->b_qvout.as<int>(), M, 64, st));
-  GFS_TRY(ensure(c->cub_temp, bytes));
+  GFS_TRY(ensure(c->b_cub_temp, bytes));
   GFS_CK(cudaStreamSynchronize(st));  // qv, qw (pageable) copied before they go out of scope
   // the survivor forests and the views' survivor parts, on the device
   for (int k = 0; k < 2; ++k)
     GFS_CK(launch_batch_surv_forest(
         c->b_sshape[k].as<uint16_t>(), c->b_sraw[k].as<float4>(), c->b_cnt.as<Counters>(), k, c->b_cap, ns,
         c->b_hist.as<unsigned>(), c->b_k64in.as<unsigned long long>(), c->b_k64out.as<unsigned long long>(),
-        c->vals_in.as<int>(), c->vals_out.as<int>(), c->cub_temp.p, c->cub_temp.bytes, c->b_end_bit,
+        c->b_vals_in.as<int>(), c->b_vals_out.as<int>(), c->b_cub_temp.p, c->b_cub_temp.bytes, c->b_end_bit,
         c->b_ssorted[k].as<float4>(), c->b_node_cap, c->b_vlo[k].as<float4>(), c->b_vhi[k].as<float4>(),
         c->b_vtdev[k].as<Tree>(), c->b_vprefix[k].as<int64_t>(), c->b_surv_levels, c->b_sodev[k].as<int64_t>(),
         c->b_qviews.as<QueryArgs>(), c->b_status.as<unsigned>(), st));
@@ -1673,8 +1682,8 @@ int gfs_batch_query(gfs_ctx* c) {
                             c->b_qkin.as<unsigned long long>(), c->b_qvin.as<int>(), st));
   int end_bit = 32;
   while ((int64_t(1) << (end_bit - 32)) < ns) ++end_bit;
-  size_t bytes = c->cub_temp.bytes;
-  GFS_CK(sort_pairs64(c->cub_temp.p, bytes, c->b_qkin.as<unsigned long long>(), c->b_qkout.as<unsigned long long>(),
+  size_t bytes = c->b_cub_temp.bytes;
+  GFS_CK(sort_pairs64(c->b_cub_temp.p, bytes, c->b_qkin.as<unsigned long long>(), c->b_qkout.as<unsigned long long>(),
                       c->b_qvin.as<int>(), c->b_qvout.as<int>(), c->b_M, end_bit, st));
   const int grid = c->b_grid_query ? c->b_grid_query : 152 * 4;
   // the work counters of this query (a memset node under capture)
@@ -1866,7 +1875,8 @@ void gfs_destroy(gfs_ctx* c) {
   if (c->sev) cudaEventDestroy(c->sev);
   if (c->sev2) cudaEventDestroy(c->sev2);
   if (c->side) cudaStreamDestroy(c->side);
-  DevBuf* bufs[] = {&c->U4, &c->hsrc, &c->cvl, &c->b_cvl, &c->cull_hint, &c->cull_list, &c->cull_count, &c->U64, &c->sph64, &c->keys_in, &c->keys_out, &c->vals_in, &c->vals_out, &c->sph,
+  DevBuf* bufs[] = {&c->U4, &c->hsrc, &c->cvl, &c->b_cvl, &c->cull.hint, &c->cull.list, &c->cull.count, &c->b_cull.hint, &c->b_cull.list, &c->b_cull.count,
+                    &c->b_vals_in, &c->b_vals_out, &c->b_cub_temp, &c->U64, &c->sph64, &c->keys_in, &c->keys_out, &c->vals_in, &c->vals_out, &c->sph,
                     &c->thr, &c->sid, &c->bound_bits, &c->consts, &c->cnt, &c->cub_temp, &c->st_lo, &c->st_hi,
                     &c->st_na, &c->st_nb, &c->st_nf, &c->st_ln, &c->st_tight, &c->qstate, &c->surv_raw[0], &c->surv_raw[1], &c->surv_sorted[0], &c->surv_sorted[1],
                     &c->vt_lo[0], &c->vt_lo[1], &c->vt_hi[0], &c->vt_hi[1], &c->defer, &c->acc, &c->witness64,
