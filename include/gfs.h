@@ -182,7 +182,8 @@ int gfs_query_tangent(gfs_ctx* ctx, const void* x, int x_is_fp32, int64_t m, flo
  * and rewritten; s_out, s64_out: its values (device, nullable), rewritten.
  * The first call after a build or an insertion sorts the survivor ids into
  * per-sphere lists (library-owned, synchronises the stream); one warp per
- * point in Morton order, decisions in FP64.
+ * point in Morton order, decisions in FP64.  A walk ends with the hierarchy
+ * (no work limit: every point is completed, none is reported as given up).
  * Errors: GFS_ERR_STATE (no build), GFS_ERR_ARG, GFS_ERR_TOO_LARGE
  * (m >= 2^32), GFS_ERR_OOM, GFS_ERR_CUDA. */
 int gfs_query_scored(gfs_ctx* ctx, const void* x, int x_is_fp32, int64_t m, float* s_out, double* s64_out,

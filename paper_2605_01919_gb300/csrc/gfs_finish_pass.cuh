@@ -102,7 +102,7 @@ __device__ bool packet_walk(const Tree& T, SpWarp& S, int lane, int budget, Node
   while (sp > 0) {
     if (budget >= 0 && spent > budget) return false;
     spent += 6;
-    const int take = min(min(sp, 4), max(1, (kSpStack - 32 - sp) / kFan));
+    const int take = walk_take(sp, kSpStack - kFan, 4);
     const uint32_t nd = grp < take ? S.stk[sp - 1 - grp] : 0xffffffffu;
     sp -= take;
     const int lev = node_level(nd);

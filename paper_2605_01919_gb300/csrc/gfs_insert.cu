@@ -195,14 +195,13 @@ __device__ int block_excl_scan(int cnt, int& total, QShared& S) {
 
 // Block-parallel walk: each round pops up to kQT nodes (one per thread),
 // refreshes the shared thresholds, expands the nodes and pushes the children
-// the caller marks.  A round pops at most (kQStack - sp) / kFan nodes (at
-// least one), so the stack never outgrows kQStack + kFan - 1 entries: a wide
-// frontier turns the walk depth-first instead of overflowing.  Each round
+// the caller marks (walk_take: a wide frontier turns the walk depth-first
+// instead of overflowing the stack).  Each round
 // and the end of the walk call refresh() and then post() (work the previous
 // round queued) on every thread.  Every thread of the block must call it.
 template <class Refresh, class NeedChild, class Leaf, class Post>
-__device__ void block_walk(const Tree& T, QShared& S, unsigned* err, Refresh refresh, NeedChild need_child,
-                           Leaf leaf, Post post) {
+__device__ void block_walk(const Tree& T, QShared& S, Refresh refresh, NeedChild need_child, Leaf leaf,
+                           Post post) {
   if (T.nlevels == 0) return;
   const int tid = threadIdx.x;
   const int top = T.nlevels - 1;
@@ -210,7 +209,7 @@ __device__ void block_walk(const Tree& T, QShared& S, unsigned* err, Refresh ref
   for (int i = tid; i < sp; i += kQT) S.stk[i] = pack_node(top, i);
   __syncthreads();
   while (sp > 0) {
-    const int take = min(min(sp, kQT), max(1, (kQStack - sp) / kFan));
+    const int take = walk_take(sp, kQStack, kQT);
     const uint32_t nd = tid < take ? S.stk[sp - 1 - tid] : 0xffffffffu;
     sp -= take;
     refresh();
@@ -234,10 +233,6 @@ __device__ void block_walk(const Tree& T, QShared& S, unsigned* err, Refresh ref
     const int cnt = __popc(mask);
     int total;
     const int pre = block_excl_scan(cnt, total, S);
-    if (sp + total > kQStack + kFan) {  // cannot happen (see above); kept as a guard
-      if (tid == 0) atomicOr(err, 1u);
-      return;
-    }
     int w = sp + pre;
     for (int c = 0; c < kFan; ++c)
       if ((mask >> c) & 1u) S.stk[w++] = pack_node(lev - 1, cb + c);
@@ -469,7 +464,7 @@ __global__ void __launch_bounds__(kQT) k_ins_query(InsertArgs a) {
     drain_spheres();
   }
   block_walk(
-      a.st, S, &a.misc->err, refresh_spheres,
+      a.st, S, refresh_spheres,
       [&](int64_t node) {
         // lower bounds over the node's spheres of |x-p| - r (per class),
         // |x-p| + r (far) and |x-p| (a sample at x): |x-C| - w, evaluated in
@@ -691,7 +686,7 @@ __global__ void __launch_bounds__(kQT) k_ins_query(InsertArgs a) {
     }
     const float slack = f_up(2.0 * 1.7320508075688772 * double(a.bc->eq) + 1e-12);
     block_walk(
-        T, S, &a.misc->err, refresh_surv,
+        T, S, refresh_surv,
         [&](int64_t node) {
           const float db = sqrtf(box_d2(xf, yf, zf, T.lo[node], T.hi[node]));
           return db - kRel * (db + Ax) - 1e-30f - slack <= fd;
@@ -1020,7 +1015,7 @@ __global__ void __launch_bounds__(64) k_ins_kill_static(InsertArgs a) {
   const float rkill = f_up(rn - a.tol);
   const Tree& T = a.vt[cls];
   warp_walk_until(
-      T, s_stk[cls], kUStack, lane, &a.misc->err, [&]() { return true; },
+      T, s_stk[cls], kUStack, lane, [&]() { return true; },
       [&](int64_t node) {
         const float db = sqrtf(box_d2(nxf, nyf, nzf, T.lo[node], T.hi[node]));
         return db - kRel * (db + An) - 1e-30f < reach;
@@ -1175,7 +1170,7 @@ __global__ void __launch_bounds__(128) k_ins_cull_new(InsertArgs a) {
                               }) >= 0;
   } else {
     warp_walk_until(
-        a.st, stk, kUStack, lane, &a.misc->err, [&]() { return !__any_sync(kAll, covered); },
+        a.st, stk, kUStack, lane, [&]() { return !__any_sync(kAll, covered); },
         [&](int64_t node) {
           // some sphere of the node has |q-p| - r < -tol only if
           // |q-C| - max(wp, wn) < -tol

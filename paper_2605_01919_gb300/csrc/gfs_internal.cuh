@@ -83,6 +83,17 @@ __host__ __device__ inline uint32_t pack_node(int level, int64_t idx) {
 __host__ __device__ inline int node_level(uint32_t v) { return int(v >> 27); }
 __host__ __device__ inline int64_t node_index(uint32_t v) { return int64_t(v & ((1u << 27) - 1)); }
 
+// Entries that a walk with a stack of cap + kFan entries takes off it: up to
+// `width` at once, while every one may leave its kFan children.  At two or more
+// the stack stays below cap - kDepthReserve; past that it goes depth first, one
+// entry at a time, and grows by at most kFan - 1 per level below it.  So it
+// never outgrows cap + kFan entries, and no walk needs a guard or gives up.
+constexpr int kDepthReserve = (kFan - 1) * (kMaxLevels - 1) - kFan;
+__host__ __device__ inline int walk_take(int sp, int cap, int width) {
+  const int room = (cap - kDepthReserve - sp) / kFan, most = sp < width ? sp : width;
+  return room < 1 ? 1 : (room < most ? room : most);
+}
+
 // FP64 sample record in input order: position and signed value.
 struct alignas(32) D4 {
   double x, y, z, w;
@@ -186,7 +197,6 @@ struct Counters {
   unsigned long long query_rechecks;
   unsigned int nsurv[2];
   unsigned int ndefer;
-  unsigned int walk_err;  // bit 0: a warp walk's stack guard tripped (cannot happen)
   unsigned long long q_sphere_ntests;  // child-node bound tests of the query sphere pass
   unsigned long long q_sphere_items;   // spheres tested by the query sphere pass
   unsigned long long q_surv_ntests;    // child-node bound tests of the survivor pass

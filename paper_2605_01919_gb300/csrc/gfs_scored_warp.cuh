@@ -48,7 +48,7 @@ __device__ inline void warp_survivors(const QueryArgs& a, const Frame& F, int cl
   const float4* items = a.surv[cls];
   const float eq4 = 4.f * a.bc->eq;
   warp_walk_until(
-      T, stk, tangent::kWarpStack, lane, &a.cnt->walk_err, refresh,
+      T, stk, tangent::kWarpStack, lane, refresh,
       [&](int64_t node) {
         const float bd = sqrtf(box_d2(F.x32, F.y32, F.z32, T.lo[node], T.hi[node]));
         return bd * (1.f - 1e-6f) - eq4 <= R32;

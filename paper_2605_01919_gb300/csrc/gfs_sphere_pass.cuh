@@ -31,7 +31,7 @@
 
 namespace gfs {
 
-constexpr int kSpStack = 448;  // >= kFan + 28 entries per level: 4 popped, at most 32 pushed, deepest level on top
+constexpr int kSpStack = 448;  // (walk_take keeps within it; 4 popped, at most 32 pushed, deepest level on top, it holds kFan + 28 a level)
 constexpr int kSpQueue = 64;
 constexpr int kCand = 8;
 
@@ -268,7 +268,7 @@ __device__ bool sphere_pass(const QueryArgs& a, int64_t first, SpWarp& S, int la
         if (spent > lim.spheres * G) return false;
         spent += 6;
       }
-      const int take = min(min(sp, 4), max(1, (kSpStack - 32 - sp) / kFan));
+      const int take = walk_take(sp, kSpStack - kFan, 4);
       const uint32_t nd = grp < take ? S.stk[sp - 1 - grp] : 0xffffffffu;
       sp -= take;
       const int lev = node_level(nd);

@@ -20,7 +20,7 @@ namespace gfs {
 namespace tangent {
 
 constexpr unsigned kLanes = 0xffffffffu;
-constexpr int kWarpStack = 512;  // per-warp walk stack entries (plus a reserve of kFan)
+constexpr int kWarpStack = 512 + kDepthReserve;  // per-warp walk stack entries (plus a reserve of kFan)
 
 // lexicographic minimum of (v, i) over the warp, on every lane
 __device__ __forceinline__ void warp_min_vi(double& v, int& i) {
@@ -135,7 +135,7 @@ __device__ inline void warp_sphere_bounds(const QueryArgs& a, double x, double y
     merge();
   }
   warp_walk_until(
-      T, stk, kWarpStack, lane, &a.cnt->walk_err,
+      T, stk, kWarpStack, lane,
       [&]() {
         merge();
         return true;
@@ -176,7 +176,7 @@ __device__ inline void warp_tangent_search(const QueryArgs& a, int box_cull, dou
   };
   merge();
   warp_walk_until(
-      T, stk, kWarpStack, lane, &a.cnt->walk_err,
+      T, stk, kWarpStack, lane,
       [&]() {
         merge();
         return true;
@@ -280,7 +280,7 @@ __device__ __forceinline__ void warp_lin_walk(const Tree& T, const LevelTable& C
   if (lane < sp) stk[lane] = pack_node(top, lane);
   __syncwarp();
   while (sp > 0) {
-    const int take = min(min(sp, 4), max(1, (kCoverStack - 96 - sp) / kFan));
+    const int take = walk_take(sp, kCoverStack - kFan, 4);
     const uint32_t nd = grp < take ? stk[sp - 1 - grp] : 0xffffffffu;
     sp -= take;
     const int lev = node_level(nd);

@@ -8,15 +8,13 @@ namespace gfs {
 
 // A warp's walk over a hierarchy with one stack stk of cap (+ kFan)
 // entries: each round refresh() runs on every lane (false ends the walk),
-// then the lanes take up to 32 nodes off the stack (at most (cap - sp) /
-// kFan, at least one, so the stack stays below cap + kFan); a lane calls
+// then the lanes take up to 32 nodes off the stack (walk_take); a lane calls
 // leaf(index) for a leaf and need_child(node) for each child of an inner
 // node, and the children it needs are pushed in lane order.  The lanes must
-// enter together; *err gets bit 0 if the stack guard ever trips (it cannot,
-// by the bound above).
+// enter together.
 template <class Refresh, class NeedChild, class Leaf>
-__device__ void warp_walk_until(const Tree& T, uint32_t* stk, int cap, int lane, unsigned* err, Refresh refresh,
-                                NeedChild need_child, Leaf leaf) {
+__device__ void warp_walk_until(const Tree& T, uint32_t* stk, int cap, int lane, Refresh refresh, NeedChild need_child,
+                                Leaf leaf) {
   const unsigned kWarpAll = 0xffffffffu;
   if (T.nlevels == 0) return;
   const int top = T.nlevels - 1;
@@ -25,7 +23,7 @@ __device__ void warp_walk_until(const Tree& T, uint32_t* stk, int cap, int lane,
   __syncwarp();
   while (sp > 0) {
     if (!refresh()) return;
-    const int take = min(min(sp, 32), max(1, (cap - sp) / kFan));
+    const int take = walk_take(sp, cap, 32);
     const uint32_t nd = lane < take ? stk[sp - 1 - lane] : 0xffffffffu;
     sp -= take;
     __syncwarp();
@@ -53,10 +51,6 @@ __device__ void warp_walk_until(const Tree& T, uint32_t* stk, int cap, int lane,
     }
     const int total = __shfl_sync(kWarpAll, pre, 31);
     pre -= cnt;
-    if (sp + total > cap + kFan) {  // cannot happen (see above); kept as a guard
-      if (lane == 0) atomicOr(err, 1u);
-      return;
-    }
     int w = sp + pre;
     for (int c = 0; c < kFan; ++c)
       if ((mask >> c) & 1u) stk[w++] = pack_node(lev - 1, cb + c);
@@ -115,8 +109,7 @@ __device__ int warp_cover_walk(const Tree& T, const LevelTable& C, uint32_t* stk
   if (lane < sp) stk[lane] = pack_node(top, lane);
   __syncwarp();
   while (sp > 0) {
-    // past 408 entries one at a time, so that at most 7 per level join them
-    const int take = min(min(sp, 4), max(1, (kCoverStack - 96 - sp) / kFan));
+    const int take = walk_take(sp, kCoverStack - kFan, 4);
     const uint32_t nd = grp < take ? stk[sp - 1 - grp] : 0xffffffffu;
     sp -= take;
     const int lev = node_level(nd);
