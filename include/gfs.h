@@ -111,6 +111,8 @@ int gfs_set_stream(gfs_ctx* ctx, void* cuda_stream);
  * survivor hierarchies.  Inputs are copied; the caller may free them after
  * the call returns.  Synchronises the stream twice (the coordinate bound
  * that sets the hierarchy's rounding slack, and the survivor count).
+ * Library-owned scratch of the cull, kept by the context: n*K*4 bytes, at most
+ * 1 GB and at most an eighth of the free device memory (less if refused).
  * Errors: GFS_ERR_ARG (n < 1, null), GFS_ERR_TOO_LARGE (n*(K+1) >= 2^32, or
  * more than 2^30 survivors of one sign class), GFS_ERR_OOM, GFS_ERR_CUDA. */
 int gfs_build(gfs_ctx* ctx, const double* p_xyz, const double* s, int64_t n);
@@ -416,7 +418,8 @@ typedef struct {
  * candidates, in tiles of 32 spheres of one shape (the library
  * keeps the shape table; the caller keeps the buffers alive until the last
  * gfs_batch_query).  Results per shape are those of gfs_build on that shape
- * alone.  Sizes every buffer (the survivor capacity is grown and the cull
+ * alone.  Sizes every buffer (with a cull scratch of its own, as gfs_build's;
+ * the survivor capacity is grown and the cull
  * rerun until the counts fit) and uploads the shape table, so that
  * gfs_batch_rebuild can later repeat the build without the host.  The first
  * build also picks the persistent query's grid size by timing a few

@@ -13,6 +13,7 @@
 
 #include "gfs.h"
 #include "gfs_kernels.h"
+#include "gfs_chunk.h"
 #include "gfs_exact.h"
 #include "gfs_order.h"
 #include "gfs_scored.h"
@@ -123,7 +124,14 @@ void lin_layout(Tree& T, void* buf, int64_t nodes) {
 // the cull's workspace (see cull_work)
 struct CullBufs {
   DevBuf hint, list, count;
+  int64_t chunk = 0;  // tiles they hold
 };
+void release(CullBufs& b) {
+  release(b.hint);
+  release(b.list);
+  release(b.count);
+  b.chunk = 0;
+}
 
 #define GFS_CK(expr)                         \
   do {                                       \
@@ -441,19 +449,32 @@ int reset_cull_counters(gfs_ctx* c, cudaStream_t st) {
   return GFS_OK;
 }
 
-// The cull's workspace for `tiles` tiles, in chunks of at most 1 GB of
-// covering balls and open-list entries (a chunk's entries number below 2^32).
-int cull_work(gfs_ctx* c, CullBufs& b, int64_t tiles, CullWork& w) {
+// Reserves the cull's workspace for `tiles` tiles (covering balls and open-list
+// entries; a chunk's entries number below 2^32): in chunks as gfs_chunk.h says,
+// smaller ones when the device refuses that much.
+int cull_reserve(gfs_ctx* c, CullBufs& b, int64_t tiles) {
   const int64_t last = c->K - c->KH;  // directions of the last level(s), the largest group
-  const int64_t per = (int64_t(c->KH) + last) * kCullTileSpheres * 4;
-  w.chunk = std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t(1) << 30) / per));
-  GFS_TRY(ensure(b.hint, size_t(w.chunk) * std::max(1, c->KH) * kCullTileSpheres * 4));
-  GFS_TRY(ensure(b.list, size_t(w.chunk) * size_t(last) * kCullTileSpheres * 4));
-  GFS_TRY(ensure(b.count, size_t(cull_launches(c->KH, tiles, w.chunk)) * 8));
-  w.hint = b.hint.as<int>();
-  w.list = b.list.as<uint32_t>();
-  w.count = b.count.as<unsigned>();
-  return GFS_OK;
+  const int64_t per = c->K * int64_t(kCullTileSpheres) * 4;
+  int64_t want = cull_chunk(tiles, per, INT64_MAX);
+  if (b.chunk < want) {
+    size_t free_bytes = 0, total = 0;
+    GFS_CK(cudaMemGetInfo(&free_bytes, &total));
+    want = cull_chunk(tiles, per, int64_t(free_bytes + b.hint.bytes + b.list.bytes));
+    if (b.chunk < want) release(b);
+  }
+  return shrink_until(std::max(want, b.chunk), GFS_ERR_OOM, [&](int64_t chunk) {
+    int r = ensure(b.hint, size_t(chunk) * std::max(1, c->KH) * kCullTileSpheres * 4);
+    if (r == GFS_OK) r = ensure(b.list, size_t(chunk) * size_t(last) * kCullTileSpheres * 4);
+    if (r == GFS_OK) r = ensure(b.count, size_t(cull_launches(c->KH, tiles, chunk)) * 8);
+    if (r == GFS_OK) b.chunk = chunk;
+    else release(b);
+    return r;
+  });
+}
+
+// what cull_reserve left (nothing is allocated here: a batch rebuild may be captured)
+CullWork cull_work(const CullBufs& b) {
+  return CullWork{b.hint.as<int>(), b.list.as<uint32_t>(), b.count.as<unsigned>(), b.chunk};
 }
 
 // a2: inputs copied, counters cleared, sphere hierarchy built
@@ -507,10 +528,9 @@ int build_finish(gfs_ctx* c) {
     a.cap = c->cap;
     a.cnt = c->cnt.as<Counters>();
     if (c->have_ev) GFS_CK(cudaEventRecord(c->ev[1], st));
-    CullWork w;
     const int64_t tiles = (n + kCullTileSpheres - 1) / kCullTileSpheres;
-    GFS_TRY(cull_work(c, c->cull, tiles, w));
-    GFS_CK(launch_cull(a, nullptr, nullptr, 0, tiles, w, st));
+    GFS_TRY(cull_reserve(c, c->cull, tiles));
+    GFS_CK(launch_cull(a, nullptr, nullptr, 0, tiles, cull_work(c->cull), st));
     if (c->have_ev) GFS_CK(cudaEventRecord(c->ev[2], st));
     unsigned int ns[2] = {0, 0};
     GFS_CK(cudaMemcpyAsync(ns, reinterpret_cast<char*>(c->cnt.p) + offsetof(Counters, nsurv), sizeof(ns),
@@ -1357,13 +1377,12 @@ int batch_build_device(gfs_ctx* c, bool cull_only) {
   (void)N;
   if (!cull_only) GFS_TRY(batch_build_device_samples(c));
   GFS_CK(cudaMemsetAsync(c->b_cnt.p, 0, sizeof(Counters), st));
-  CullWork w;
-  GFS_TRY(cull_work(c, c->b_cull, c->b_cull_tiles, w));  // (sized by the first build)
   CullArgs one;
   std::memset(&one, 0, sizeof(one));
   one.K = c->K;
   one.KH = c->KH;
-  GFS_CK(launch_cull(one, c->b_cviews.as<CullArgs>(), batch_tiles(c), ns, c->b_cull_tiles, w, st));
+  GFS_CK(launch_cull(one, c->b_cviews.as<CullArgs>(), batch_tiles(c), ns, c->b_cull_tiles,
+                     cull_work(c->b_cull), st));
   if (cull_only) return GFS_OK;
   for (int k = 0; k < 2; ++k)
     GFS_CK(launch_batch_surv_forest(
@@ -1542,6 +1561,7 @@ int gfs_batch_build(gfs_ctx* c, const gfs_shape* shapes, int ns) {
     GFS_CK(cudaStreamSynchronize(st));  // pageable sources
     return GFS_OK;
   };
+  GFS_TRY(cull_reserve(c, c->b_cull, c->b_cull_tiles));
   for (int attempt = 0; attempt < 3; ++attempt) {
     c->b_cap = unsigned(cap);
     for (int k = 0; k < 2; ++k) {
@@ -1875,8 +1895,9 @@ void gfs_destroy(gfs_ctx* c) {
   if (c->sev) cudaEventDestroy(c->sev);
   if (c->sev2) cudaEventDestroy(c->sev2);
   if (c->side) cudaStreamDestroy(c->side);
-  DevBuf* bufs[] = {&c->U4, &c->hsrc, &c->cvl, &c->b_cvl, &c->cull.hint, &c->cull.list, &c->cull.count, &c->b_cull.hint, &c->b_cull.list, &c->b_cull.count,
-                    &c->b_vals_in, &c->b_vals_out, &c->b_cub_temp, &c->U64, &c->sph64, &c->keys_in, &c->keys_out, &c->vals_in, &c->vals_out, &c->sph,
+  release(c->cull);
+  release(c->b_cull);
+  DevBuf* bufs[] = {&c->U4, &c->hsrc, &c->cvl, &c->b_cvl, &c->b_vals_in, &c->b_vals_out, &c->b_cub_temp, &c->U64, &c->sph64, &c->keys_in, &c->keys_out, &c->vals_in, &c->vals_out, &c->sph,
                     &c->thr, &c->sid, &c->bound_bits, &c->consts, &c->cnt, &c->cub_temp, &c->st_lo, &c->st_hi,
                     &c->st_na, &c->st_nb, &c->st_nf, &c->st_ln, &c->st_tight, &c->qstate, &c->surv_raw[0], &c->surv_raw[1], &c->surv_sorted[0], &c->surv_sorted[1],
                     &c->vt_lo[0], &c->vt_lo[1], &c->vt_hi[0], &c->vt_hi[1], &c->defer, &c->acc, &c->witness64,
