@@ -270,10 +270,13 @@ cudaError_t launch_intersections(const QueryArgs& a, const unsigned long long* p
                                  const exact::UDOut& o, cudaStream_t st) {
   if (np <= 0) return cudaSuccess;
   // One pair a warp while that still leaves few warps a scheduler, 4 a warp
-  // beyond: 171k pairs (12^3 union grid, with the radii of 512 points) 72 ms at
-  // spread 1, 59 at 8, 49 at 32; 16k pairs 7.6, 5.8, 5.1 ms; 419k pairs 284, 232,
-  // 233 ms; 913k pairs 497, 476, 499 ms.
-  const int spread = np <= (int64_t(1) << 18) ? 32 : 8;
+  // beyond, and a pair on every lane once the warps alone fill the chip many
+  // times over (then the lanes' divergence costs less than the empty lanes'
+  // issue).  Circles and points in ms at spread 1 / 8 / 32: 202k pairs (12^3 union
+  // grid) 44.9 / 37.7 / 34.8; 1.1M (16^3) 234 / 204 / 226; 2.9M (24^3 CSG grid)
+  // 887 / 952 / 955; 4.1M (24^3 torus) 2044 / 2201 / 2353; 11M (20^3 union) 2565 /
+  // 2584 / 2819; 36M (64^3 CSG) 9317 / 10122 / 11237.
+  const int spread = np <= (int64_t(1) << 18) ? 32 : (np <= (int64_t(1) << 21) ? 8 : 1);
   k_intersections<<<(unsigned int)((np * spread + 127) / 128), 128, 0, st>>>(a, pairs, np, o, spread);
   ++g_exact_launches;
   return cudaGetLastError();

@@ -25,6 +25,8 @@ def digest(t):
 @pytest.mark.parametrize("grid, N, circles, points, lists, coverage", [
     ("csg", 16, 11085, 18247, ("6bb18785b8cf", "0d514bd0c826", "0c3ac2ed8996"), ("0ec7cdd5434c", "f14c44bc36a3")),
     ("union", 16, 30586, 593729, ("1cfab1321041", "0f79f079b3f6", "c42c540a9d9a"), ("0c7f2cbe5e40", "1387bccb86f4")),
+    # (2.9M pairs: every lane of the circle search has one)
+    ("csg", 24, 49417, 1685021, ("f792cae76e8f", "b2da4f6d11a8", "75ef16f4960b"), ("54650f2dd649", "866c685d9764")),
     ("csg", 32, 48132, 153279, ("218993a25b2e", "03aa1ad48930", "92ba1e3d76d5"), ("7f647172e673", "4a76ac9a6682")),
 ])
 def test_touching_lists_and_witnesses(grid, N, circles, points, lists, coverage):
