@@ -218,10 +218,14 @@ __global__ void k_ud_gather(const unsigned long long* __restrict__ ckey, int64_t
 // that order) and take the block's minimum after each, so that later sets are
 // tested against the best point so far.  Bound: FP64 constructions and the
 // latency of the coverage walks; with one warp per point 512 points left most
-// of the chip idle.  Radii of 512 points of a 12^3 union grid, circles included:
-// 85 ms with 1 warp a point, 78 with 4, 72 with 16 (and 50.5 / 48.7 ms with 8 /
-// 16 after the circles were spread over more warps).
-constexpr int kRminWarps = 16;
+// of the chip idle, and with 16 the threads of many points prune less than one
+// warp's.  Radii in ms with 1 / 4 / 8 / 16 warps a point (the lists prepared):
+// 12^3 union grid, 512 points 11.0 / 4.4 / 4.2 / 4.0, 4,096 points 29.0 / 24.8 /
+// 24.1 / 24.9, 131,072 points 742 / 736 / 737 / 771; 16^3 union grid, 512 points
+// 46.7 / 27.3 / 27.3 / 27.7, 32,768 points 1382 / 1348 / 1345 / 1343.
+// So 16 up to kRminFew points, 8 beyond.
+constexpr int64_t kRminFew = 1024;
+template <int kRminWarps>
 __global__ void __launch_bounds__(32 * kRminWarps) k_exact_rmin(QueryArgs a, int box_cull, exact::UDLists L,
                                                                 const double* __restrict__ x,
                                                                 const int8_t* __restrict__ sigma,
@@ -251,9 +255,11 @@ unsigned long long g_exact_launches = 0;
 cudaError_t launch_exact_rmin(const QueryArgs& a, int box_cull, const exact::UDLists& L, const double* x,
                               const int8_t* sigma, int64_t m, double* out, cudaStream_t st) {
   if (m <= 0) return cudaSuccess;
-  for (int64_t q = 0; q < m; q += 1 << 30)
-    k_exact_rmin<<<unsigned(m - q < (1 << 30) ? m - q : 1 << 30), 32 * kRminWarps, 0, st>>>(a, box_cull, L, x + 3 * q,
-                                                                                        sigma + q, out + q);
+  for (int64_t q = 0; q < m; q += 1 << 30) {
+    const unsigned grid = unsigned(m - q < (1 << 30) ? m - q : 1 << 30);
+    if (m <= kRminFew) k_exact_rmin<16><<<grid, 32 * 16, 0, st>>>(a, box_cull, L, x + 3 * q, sigma + q, out + q);
+    else k_exact_rmin<8><<<grid, 32 * 8, 0, st>>>(a, box_cull, L, x + 3 * q, sigma + q, out + q);
+  }
   ++g_exact_launches;
   return cudaGetLastError();
 }
