@@ -783,84 +783,112 @@ namespace gfs {
 // 10.0 / 12.6 ms); few points want less, for the sake of the last packets (100k
 // on 32^3, both passes after the spheres: 1.16 / 0.60 / 0.54 / 0.50 ms).
 constexpr float kJump = 6.f;
-static int packet_size(const QueryArgs& a) {
-  if (a.m >= 131072 && a.m >= a.n) return kPacket;
-  if (a.m >= 24576 && a.m >= 3 * a.n) return 8;
-  return 1;
-}
-static PkLimit packet_limit(int G, int64_t m) {
-  const float rho = kJump * cbrtf(float(G) / float(m));
-  return G == 1 ? no_jump() : (G == kPacket ? PkLimit{rho, 600, 100} : PkLimit{rho, 80, 32});
+// Fewer points than packet_size's table wants (m < n, m < 3 n) are sparse: a
+// packet of uniform ones spans several spacings of the samples and is better
+// taken point by point, but points in a cluster, on a slice or in one place are
+// as close as dense ones.  So a packet whose radius is below kClose spacings of
+// n uniform samples (2 / cbrt(n) each, in halves) goes as a packet, and the
+// others are marked for launches by points.  ms at kClose 1 / 1.5 / 2, after a
+// warp per point: a cluster of 200k points on 64^3 samples 2.48 | 0.72 / 0.73 /
+// 0.75, of 1M on 128^3 20.4 | 4.1 / 3.9 / 3.9, a slice of 1M on 128^3 32.9 | 27.9 /
+// 21.1 / 21.2, 300k points beside the surface of 128^3 7.26 | 7.34 / 7.35 / 8.44
+// (packets that give up), 1M random points 29.0 | 29.2 / 29.2 / 29.3, 100k on
+// 64^3 1.64 | 1.69 / 1.69 / 1.78.
+constexpr float kClose = 1.5f;
+struct Packets {
+  int G;
+  bool sparse;
+  PkLimit lim;
+};
+static Packets packets_of(const QueryArgs& a) {
+  Packets p{a.m >= 131072 ? kPacket : (a.m >= 24576 ? 8 : 1), false, no_jump()};
+  if (p.G == 1) return p;
+  p.lim = p.G == kPacket ? PkLimit{0.f, 600, 100} : PkLimit{0.f, 80, 32};
+  p.sparse = a.m < (p.G == kPacket ? a.n : 3 * a.n);
+  p.lim.rho = p.sparse ? kClose * cbrtf(1.f / float(a.n)) : kJump * cbrtf(float(p.G) / float(a.m));
+  return p;
 }
 
-template <int G>
+// A packet that pass(slot) does not finish is listed (counter, for the split
+// launch), or marked in a.split (by the packet's number; sparse points), and a
+// packet marked by an earlier pass is left to the launch by points.
+template <bool kSparse, class Pass>
+__device__ __forceinline__ void try_packet(const QueryArgs& a, bool first, unsigned* listed, Pass pass) {
+  if constexpr (kSparse) {
+    if (!first && a.split[blockIdx.x]) return;
+    const bool done = pass();
+    if (threadIdx.x == 0 && (first || !done)) a.split[blockIdx.x] = done ? 0u : 1u;
+  } else {
+    if (!pass() && threadIdx.x == 0) a.split[atomicAdd(listed, 1u)] = blockIdx.x;
+  }
+}
+// the listed packets' points, one at a time
+template <int G, class Pass>
+__device__ __forceinline__ void split_points(const QueryArgs& a, unsigned packets, unsigned* next, Pass pass) {
+  const int64_t total = int64_t(packets) * G;
+  for (;;) {
+    unsigned t = 0;
+    if (threadIdx.x == 0) t = atomicAdd(next, 1u);
+    t = __shfl_sync(kFull, t, 0);
+    if (int64_t(t) >= total) return;
+    const int64_t slot = int64_t(a.split[t / G]) * G + t % G;
+    __syncwarp();
+    if (slot < a.m) pass(slot);
+  }
+}
+
+template <int G, bool kSparse>
 __global__ void __launch_bounds__(32, 28) k_query_spheres(QueryArgs a, PkLimit lim) {
   __shared__ SpWarp S;
-  if (!sphere_pass<G>(a, int64_t(blockIdx.x) * G, S, threadIdx.x, lim) && threadIdx.x == 0)
-    a.split[atomicAdd(&a.cnt->q_split, 1u)] = blockIdx.x;
+  try_packet<kSparse>(a, true, &a.cnt->q_split, [&]() { return sphere_pass<G>(a, int64_t(blockIdx.x) * G, S, threadIdx.x, lim); });
 }
-
-// The points of the packets that k_query_spheres<G> listed, one at a time.
+// The points of the packets that k_query_spheres<G, false> listed, one at a time.
 template <int G>
 __global__ void __launch_bounds__(32, 28) k_query_spheres_split(QueryArgs a) {
   __shared__ SpWarp S;
-  const int64_t total = int64_t(a.cnt->q_split) * G;
-  for (;;) {
-    unsigned t = 0;
-    if (threadIdx.x == 0) t = atomicAdd(&a.cnt->q_split_next, 1u);
-    t = __shfl_sync(kFull, t, 0);
-    if (int64_t(t) >= total) return;
-    const int64_t slot = int64_t(a.split[t / G]) * G + t % G;
-    __syncwarp();
-    if (slot < a.m) sphere_pass<1>(a, slot, S, threadIdx.x, no_jump());
-  }
+  split_points<G>(a, a.cnt->q_split, &a.cnt->q_split_next, [&](int64_t slot) { sphere_pass<1>(a, slot, S, threadIdx.x, no_jump()); });
+}
+// The marked packets' points, a block each (with the cursor of the split launch
+// the survivor pass takes twice as long when nearly all are marked).
+template <int G>
+__global__ void __launch_bounds__(32, 28) k_query_spheres_marked(QueryArgs a) {
+  __shared__ SpWarp S;
+  if (a.split[blockIdx.x / G]) sphere_pass<1>(a, blockIdx.x, S, threadIdx.x, no_jump());
 }
 
 // The survivor pass, split the same way.
-template <int G>
+template <int G, bool kSparse>
 __global__ void __launch_bounds__(32, 28) k_query_near(QueryArgs a, PkLimit lim) {
   __shared__ SpWarp S;
-  if (!near_pass<G>(a, int64_t(blockIdx.x) * G, S, threadIdx.x, lim) && threadIdx.x == 0)
-    a.split[atomicAdd(&a.cnt->f_split, 1u)] = blockIdx.x;
+  try_packet<kSparse>(a, false, &a.cnt->f_split, [&]() { return near_pass<G>(a, int64_t(blockIdx.x) * G, S, threadIdx.x, lim); });
 }
-
 template <int G>
 __global__ void __launch_bounds__(32, 28) k_query_near_split(QueryArgs a) {
   __shared__ SpWarp S;
-  const int64_t total = int64_t(a.cnt->f_split) * G;
-  for (;;) {
-    unsigned t = 0;
-    if (threadIdx.x == 0) t = atomicAdd(&a.cnt->f_split_next, 1u);
-    t = __shfl_sync(kFull, t, 0);
-    if (int64_t(t) >= total) return;
-    const int64_t slot = int64_t(a.split[t / G]) * G + t % G;
-    __syncwarp();
-    if (slot < a.m) near_pass<1>(a, slot, S, threadIdx.x, no_jump());
-  }
+  split_points<G>(a, a.cnt->f_split, &a.cnt->f_split_next, [&](int64_t slot) { near_pass<1>(a, slot, S, threadIdx.x, no_jump()); });
+}
+template <int G>
+__global__ void __launch_bounds__(32, 28) k_query_near_marked(QueryArgs a) {
+  __shared__ SpWarp S;
+  if (a.split[blockIdx.x / G]) near_pass<1>(a, blockIdx.x, S, threadIdx.x, no_jump());
 }
 
 // The decisions, split the same way (packets of 8 / 16 / 32 on 16.2M points,
 // 64^3 samples: 18.3 / 14.9 / 15.9 ms; 2.1M random points, 96^3: 8.6 / 9.4 / 12.4).
-template <int G>
+template <int G, bool kSparse>
 __global__ void __launch_bounds__(32, 24) k_query_decide(QueryArgs a, PkLimit lim) {
   __shared__ SpWarp S;
-  if (!decide_pass<G, false>(a, int64_t(blockIdx.x) * G, S, threadIdx.x, lim) && threadIdx.x == 0)
-    a.split[atomicAdd(&a.cnt->d_split, 1u)] = blockIdx.x;
+  try_packet<kSparse>(a, false, &a.cnt->d_split, [&]() { return decide_pass<G, false>(a, int64_t(blockIdx.x) * G, S, threadIdx.x, lim); });
 }
-
 template <int G>
 __global__ void __launch_bounds__(32, 24) k_query_decide_split(QueryArgs a) {
   __shared__ SpWarp S;
-  const int64_t total = int64_t(a.cnt->d_split) * G;
-  for (;;) {
-    unsigned t = 0;
-    if (threadIdx.x == 0) t = atomicAdd(&a.cnt->d_split_next, 1u);
-    t = __shfl_sync(kFull, t, 0);
-    if (int64_t(t) >= total) return;
-    const int64_t slot = int64_t(a.split[t / G]) * G + t % G;
-    __syncwarp();
-    if (slot < a.m) decide_pass<1, false>(a, slot, S, threadIdx.x, no_jump());
-  }
+  split_points<G>(a, a.cnt->d_split, &a.cnt->d_split_next, [&](int64_t slot) { decide_pass<1, false>(a, slot, S, threadIdx.x, no_jump()); });
+}
+template <int G>
+__global__ void __launch_bounds__(32, 24) k_query_decide_marked(QueryArgs a) {
+  __shared__ SpWarp S;
+  if (a.split[blockIdx.x / G]) decide_pass<1, false>(a, blockIdx.x, S, threadIdx.x, no_jump());
 }
 
 // ---------------------------------------------------------------------------
@@ -1267,41 +1295,51 @@ cudaError_t launch_cull(const CullArgs& one, const CullArgs* views, const int64_
 }
 
 template <int G>
-static void query_spheres(const QueryArgs& a, cudaStream_t st) {
-  k_query_spheres<G><<<nblk(a.m, G), 32, 0, st>>>(a, packet_limit(G, a.m));
-  ++g_launches;
-  if constexpr (G > 1) {
-    k_query_spheres_split<G><<<152 * 28, 32, 0, st>>>(a);
-    ++g_launches;
+static void query_spheres(const QueryArgs& a, const Packets& p, cudaStream_t st) {
+  if (p.sparse) {
+    k_query_spheres<G, true><<<nblk(a.m, G), 32, 0, st>>>(a, p.lim);
+    k_query_spheres_marked<G><<<unsigned(a.m), 32, 0, st>>>(a);
+  } else {
+    k_query_spheres<G, false><<<nblk(a.m, G), 32, 0, st>>>(a, p.lim);
+    if constexpr (G > 1) k_query_spheres_split<G><<<152 * 28, 32, 0, st>>>(a);
   }
+  g_launches += G > 1 ? 2 : 1;
 }
 
 template <int G>
-static void query_rest(const QueryArgs& a, cudaStream_t st) {
-  const PkLimit lim = packet_limit(G, a.m);
-  k_query_near<G><<<nblk(a.m, G), 32, 0, st>>>(a, lim);
-  if constexpr (G > 1) k_query_near_split<G><<<152 * 28, 32, 0, st>>>(a);
-  k_query_decide<G><<<nblk(a.m, G), 32, 0, st>>>(a, lim);
-  if constexpr (G > 1) k_query_decide_split<G><<<152 * 24, 32, 0, st>>>(a);
+static void query_rest(const QueryArgs& a, const Packets& p, cudaStream_t st) {
+  if (p.sparse) {
+    k_query_near<G, true><<<nblk(a.m, G), 32, 0, st>>>(a, p.lim);
+    k_query_near_marked<G><<<unsigned(a.m), 32, 0, st>>>(a);
+    k_query_decide<G, true><<<nblk(a.m, G), 32, 0, st>>>(a, p.lim);
+    k_query_decide_marked<G><<<unsigned(a.m), 32, 0, st>>>(a);
+  } else {
+    k_query_near<G, false><<<nblk(a.m, G), 32, 0, st>>>(a, p.lim);
+    if constexpr (G > 1) k_query_near_split<G><<<152 * 28, 32, 0, st>>>(a);
+    k_query_decide<G, false><<<nblk(a.m, G), 32, 0, st>>>(a, p.lim);
+    if constexpr (G > 1) k_query_decide_split<G><<<152 * 24, 32, 0, st>>>(a);
+  }
   g_launches += G > 1 ? 4 : 2;
 }
 
 cudaError_t launch_query_spheres(const QueryArgs& a, cudaStream_t st) {
   if (a.m == 0) return cudaSuccess;
-  switch (packet_size(a)) {
-    case 1: query_spheres<1>(a, st); break;
-    case 8: query_spheres<8>(a, st); break;
-    default: query_spheres<kPacket>(a, st);
+  const Packets p = packets_of(a);
+  switch (p.G) {
+    case 1: query_spheres<1>(a, p, st); break;
+    case 8: query_spheres<8>(a, p, st); break;
+    default: query_spheres<kPacket>(a, p, st);
   }
   return cudaGetLastError();
 }
 
 cudaError_t launch_query_finish(const QueryArgs& a, cudaStream_t st) {
   if (a.m == 0) return cudaSuccess;
-  switch (packet_size(a)) {
-    case 1: query_rest<1>(a, st); break;
-    case 8: query_rest<8>(a, st); break;
-    default: query_rest<kPacket>(a, st);
+  const Packets p = packets_of(a);
+  switch (p.G) {
+    case 1: query_rest<1>(a, p, st); break;
+    case 8: query_rest<8>(a, p, st); break;
+    default: query_rest<kPacket>(a, p, st);
   }
   return cudaGetLastError();
 }
