@@ -1,6 +1,8 @@
 // Covered area ratio of grid cells for the refinement order (Sec. 4.2).
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "gfs_order.cuh"
 #include "gfs_order.h"
 #include "gfs_warp.cuh"
@@ -9,7 +11,7 @@ namespace gfs {
 
 namespace {
 
-constexpr int kCellWarps = 8, kRecent = 16, kMaxSub = 64;
+constexpr int kRecent = 16, kMaxSub = 64;
 
 // One block per cell.  Each warp takes 32 of its points at a time; the balls
 // that held its latest covered points (kRecent of them, FP32, tested by every
@@ -22,6 +24,7 @@ constexpr int kCellWarps = 8, kRecent = 16, kMaxSub = 64;
 // FP32 decides only what is certain: thr.z is the threshold below which a
 // point rounded to FP32 lies in the ball for sure; points outside the
 // coordinate range of that bound take the FP64 walk of gfs_tangent.cuh.
+template <int kCellWarps>
 __global__ void __launch_bounds__(32 * kCellWarps) k_cell_coverage(QueryArgs a, const int32_t* __restrict__ cells,
                                                                    double ox, double oy, double oz,
                                                                    double h, int sub, uint32_t* __restrict__ counts) {
@@ -112,10 +115,21 @@ unsigned long long g_order_launches = 0;
 cudaError_t launch_cell_coverage(const QueryArgs& a, const int32_t* cells, int64_t ncells, const double* origin,
                                  double h, int sub, uint32_t* counts, cudaStream_t st) {
   if (ncells <= 0) return cudaSuccess;
-  // (grid dimension below 2^31)
-  for (int64_t c0 = 0; c0 < ncells; c0 += 1 << 30)
-    k_cell_coverage<<<unsigned(ncells - c0 < (1 << 30) ? ncells - c0 : 1 << 30), 32 * kCellWarps, 0, st>>>(
-        a, cells + 3 * c0, origin[0], origin[1], origin[2], h, sub, counts + c0);
+  // As many warps as the points fill, at most 8: with 8 throughout the 59,319
+  // cells of a 40^3 union grid took 0.53 / 0.74 / 1.28 / 1.84 / 2.22 ms at 1^3 to 5^3
+  // points, now 0.17 / 0.39 / 0.86 / 1.34 / 1.99, and 237k cells outside the range
+  // (walks per lane) 2.44 / 2.89 / 3.17 / 3.34 / 3.83, now 0.81 / 0.97 / 1.07 / 1.63 /
+  // 2.78.
+  auto run = [&](auto warps) {
+    constexpr int W = decltype(warps)::value;
+    for (int64_t c0 = 0; c0 < ncells; c0 += 1 << 30)  // (grid dimension below 2^31)
+      k_cell_coverage<W><<<unsigned(ncells - c0 < (1 << 30) ? ncells - c0 : 1 << 30), 32 * W, 0, st>>>(
+          a, cells + 3 * c0, origin[0], origin[1], origin[2], h, sub, counts + c0);
+  };
+  if (sub <= 3) run(std::integral_constant<int, 1>());
+  else if (sub == 4) run(std::integral_constant<int, 2>());
+  else if (sub == 5) run(std::integral_constant<int, 4>());
+  else run(std::integral_constant<int, 8>());
   ++g_order_launches;
   return cudaGetLastError();
 }
