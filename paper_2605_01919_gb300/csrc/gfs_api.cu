@@ -123,12 +123,13 @@ void lin_layout(Tree& T, void* buf, int64_t nodes) {
 
 // the cull's workspace (see cull_work)
 struct CullBufs {
-  DevBuf hint, list, count;
+  DevBuf hint, list, groups, count;
   int64_t chunk = 0;  // tiles they hold
 };
 void release(CullBufs& b) {
   release(b.hint);
   release(b.list);
+  release(b.groups);
   release(b.count);
   b.chunk = 0;
 }
@@ -453,19 +454,21 @@ int reset_cull_counters(gfs_ctx* c, cudaStream_t st) {
 // entries; a chunk's entries number below 2^32): in chunks as gfs_chunk.h says,
 // smaller ones when the device refuses that much.
 int cull_reserve(gfs_ctx* c, CullBufs& b, int64_t tiles) {
-  const int64_t last = c->K - c->KH;  // directions of the last level(s), the largest group
-  const int64_t per = c->K * int64_t(kCullTileSpheres) * 4;
+  const int KH = cull_kept(c->KH, tiles);
+  const int64_t last = c->K - KH;  // directions of the last level(s), the largest group
+  const int64_t per = c->K * (int64_t(kCullTileSpheres) * 4 + int64_t(sizeof(uint2)));
   int64_t want = cull_chunk(tiles, per, INT64_MAX);
   if (b.chunk < want) {
     size_t free_bytes = 0, total = 0;
     GFS_CK(cudaMemGetInfo(&free_bytes, &total));
-    want = cull_chunk(tiles, per, int64_t(free_bytes + b.hint.bytes + b.list.bytes));
+    want = cull_chunk(tiles, per, int64_t(free_bytes + b.hint.bytes + b.list.bytes + b.groups.bytes));
     if (b.chunk < want) release(b);
   }
   return shrink_until(std::max(want, b.chunk), GFS_ERR_OOM, [&](int64_t chunk) {
-    int r = ensure(b.hint, size_t(chunk) * std::max(1, c->KH) * kCullTileSpheres * 4);
+    int r = ensure(b.hint, size_t(chunk) * std::max(1, KH) * kCullTileSpheres * 4);
     if (r == GFS_OK) r = ensure(b.list, size_t(chunk) * size_t(last) * kCullTileSpheres * 4);
-    if (r == GFS_OK) r = ensure(b.count, size_t(cull_launches(c->KH, tiles, chunk)) * 8);
+    if (r == GFS_OK) r = ensure(b.groups, size_t(chunk) * size_t(c->K) * sizeof(uint2));
+    if (r == GFS_OK) r = ensure(b.count, size_t(cull_launches(KH, tiles, chunk)) * 2 * sizeof(unsigned));
     if (r == GFS_OK) b.chunk = chunk;
     else release(b);
     return r;
@@ -474,7 +477,7 @@ int cull_reserve(gfs_ctx* c, CullBufs& b, int64_t tiles) {
 
 // what cull_reserve left (nothing is allocated here: a batch rebuild may be captured)
 CullWork cull_work(const CullBufs& b) {
-  return CullWork{b.hint.as<int>(), b.list.as<uint32_t>(), b.count.as<unsigned>(), b.chunk};
+  return CullWork{b.hint.as<int>(), b.list.as<uint32_t>(), b.groups.as<uint2>(), b.count.as<unsigned>(), b.chunk};
 }
 
 // a2: inputs copied, counters cleared, sphere hierarchy built

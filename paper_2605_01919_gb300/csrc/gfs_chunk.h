@@ -11,7 +11,7 @@ namespace gfs {
 // tau 3 with gradients take 67.0 ms at 1 GB (3 chunks), 69.5 at 256 MB, 74.8 at
 // 64 MB; a batch of 16 shapes 62.6, 64.1, 67.2; 64^3 samples and 16.2M points
 // 48.2, 48.4, 49.4.
-constexpr int64_t kCullBytes = int64_t(1) << 30;
+constexpr int64_t kCullBytes = (int64_t(1) << 26) * 17;  // 1.06 GiB
 
 // tiles of a chunk: bytes of workspace per tile, `free_bytes` on the device
 inline int64_t cull_chunk(int64_t tiles, int64_t bytes, int64_t free_bytes) {

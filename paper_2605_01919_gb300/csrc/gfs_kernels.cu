@@ -1259,7 +1259,7 @@ cudaError_t launch_gather_points(const float4* src, const int* order, int64_t n,
 }
 
 // Level by level over chunks of tiles (the chunk bounds the covering-ball
-// array and the list; a level's list has room for every candidate).
+// array and the lists; a level's list has room for every candidate).
 cudaError_t launch_cull(const CullArgs& one, const CullArgs* views, const int64_t* prefix, int ns, int64_t tiles,
                         const CullWork& w, cudaStream_t st) {
   CullSource s;
@@ -1268,15 +1268,20 @@ cudaError_t launch_cull(const CullArgs& one, const CullArgs* views, const int64_
   s.ns = ns;
   s.hint = w.hint;
   s.list = w.list;
-  s.KH = one.KH;
+  s.groups = w.groups;
+  s.K = one.K;
+  s.KH = cull_kept(one.KH, tiles);
+  s.few = tiles <= kCullFewTiles;
   unsigned* count = w.count;
-  cudaError_t e = cudaMemsetAsync(w.count, 0, size_t(cull_launches(one.KH, tiles, w.chunk)) * 2 * sizeof(unsigned), st);
+  cudaError_t e = cudaMemsetAsync(w.count, 0, size_t(cull_launches(s.KH, tiles, w.chunk)) * 2 * sizeof(unsigned), st);
   if (e != cudaSuccess) return e;
   for (s.t0 = 0; s.t0 < tiles; s.t0 += w.chunk) {
     s.tiles = std::min(w.chunk, tiles - s.t0);
     s.k0 = 0;
+    s.gcount = count;
+    count += 2;
     for (int k1 = 12;; k1 = 4 * k1 - 6) {  // levels hold 12, 42, 162, ... directions (10 * 4^l + 2)
-      s.k1 = k1 > one.KH ? one.K : k1;     // past the kept levels the directions do not depend on one another
+      s.k1 = k1 > s.KH ? one.K : k1;       // past the kept levels the directions do not depend on one another
       s.count = count;
       count += 2;
       const int dirs = s.k1 - s.k0;
@@ -1285,10 +1290,17 @@ cudaError_t launch_cull(const CullArgs& one, const CullArgs* views, const int64_
       const int D = int(std::max<int64_t>(1, std::min<int64_t>(16, s.tiles * dirs / (152 * 16))));
       const int chunks = (dirs + D - 1) / D;
       k_cull_test<<<unsigned((s.tiles * chunks + 3) / 4), 128, 0, st>>>(one, s, D, chunks);
-      k_cull_walk<<<152 * 8, 128, 0, st>>>(one, s);
-      g_launches += 2;
+      ++g_launches;
+      if (!s.few) {
+        k_cull_walk<<<152 * 8, 128, 0, st>>>(one, s);
+        ++g_launches;
+      }
       if (s.k1 == one.K) break;
       s.k0 = s.k1;
+    }
+    if (s.few || one.K > 12) {  // (the first level lists no groups)
+      k_cull_groups<<<152 * 8, 128, 0, st>>>(one, s);
+      ++g_launches;
     }
   }
   return cudaGetLastError();

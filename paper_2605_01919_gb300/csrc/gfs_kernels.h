@@ -224,18 +224,22 @@ cudaError_t launch_gather_points(const float4* src, const int* order, int64_t n,
 struct CullWork {
   int* hint;
   uint32_t* list;
+  uint2* groups;
   unsigned* count;
   int64_t chunk;  // tiles per chunk
 };
 constexpr int kCullTileSpheres = 32;
-// launches pairs (levels x chunks) and the largest level's directions
+// Directions whose covering balls the cull keeps (none for few tiles).
+constexpr int64_t kCullFewTiles = 0;
+inline int cull_kept(int KH, int64_t tiles) { return tiles <= kCullFewTiles ? 0 : KH; }
+// pairs of counters: one per level, and one for the groups, of each chunk
 inline int cull_levels(int KH) {
   int l = 1;
   for (int k1 = 12; k1 <= KH; k1 = 4 * k1 - 6) ++l;
   return l;
 }
 inline int64_t cull_launches(int KH, int64_t tiles, int64_t chunk) {
-  return cull_levels(KH) * ((tiles + chunk - 1) / chunk);
+  return (cull_levels(KH) + 1) * ((tiles + chunk - 1) / chunk);
 }
 // Cull of one shape (views null: `one` is the shape) or of all shapes of a
 // batch (one: any view, for the options and table sizes)

@@ -34,8 +34,8 @@ def lib(tmp_path_factory):
 def test_chunk_bounds(lib, tiles, per, free):
     c = lib.chunk_host(tiles, per, free)
     assert 1 <= c <= tiles
-    assert c == 1 or c * per <= min(1 << 30, free // 8)
-    assert c == tiles or (c + 1) * per > min(1 << 30, free // 8)
+    assert c == 1 or c * per <= min(17 << 26, free // 8)
+    assert c == tiles or (c + 1) * per > min(17 << 26, free // 8)
 
 
 @pytest.mark.parametrize("size, fits", [(8192, 8192), (8192, 8191), (8192, 100), (7, 1), (1, 1)])
