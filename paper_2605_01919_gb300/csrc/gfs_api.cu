@@ -208,6 +208,7 @@ struct gfs_ctx {
   std::vector<int64_t> b_sph_level_total;  // nodes per level of the sample forest, over all shapes
   int b_sph_levels = 0, b_surv_levels = 0, b_end_bit = 32;
   int64_t b_node_cap = 0;
+  int b_packet = 16;          // points of a query packet
   int64_t b_nodes = 0;        // nodes of the sample forest
   int64_t b_cull_tiles = 0;   // 32-sphere tiles of all shapes (prefix behind b_prefix's item offsets)
   unsigned b_cap = 0;
@@ -1285,7 +1286,7 @@ int64_t forest_layout(std::vector<Tree>& trees, const std::vector<int64_t>& nite
   return base;
 }
 
-// time one persistent query launch configuration (both phases) on a prefix
+// time one persistent query launch configuration (all phases) on a prefix
 // of the work
 float time_grid(gfs_ctx* c, int grid, int64_t limit) {
   cudaStream_t st = c->stream;
@@ -1296,7 +1297,7 @@ float time_grid(gfs_ctx* c, int grid, int64_t limit) {
   for (int phase = 1; phase <= 3; ++phase) {
     cudaMemsetAsync(c->b_ctr.p, 0, 8, st);
     launch_batch_query(c->b_qviews.as<QueryArgs>(), c->b_qw.as<int64_t>(), c->b_ns, limit,
-                       c->b_ctr.as<unsigned long long>(), grid, phase, st);
+                       c->b_ctr.as<unsigned long long>(), grid, phase, c->b_packet, st);
   }
   cudaEventRecord(e1, st);
   cudaEventSynchronize(e1);
@@ -1611,8 +1612,9 @@ int gfs_batch_build(gfs_ctx* c, const gfs_shape* shapes, int ns) {
                         c->b_vals_in.as<int>(), c->b_vals_out.as<int>(), int64_t(capu), c->b_end_bit, st));
     GFS_TRY(ensure(c->b_cub_temp, bytes));
   }
-  // query views and work items (shape, 32 points); the survivor pointers and
+  // query views and work items (shape, packet of points); the survivor pointers and
   // trees are filled in by the device-side survivor forests
+  c->b_packet = batch_packet(M, N);
   std::vector<QueryArgs> qv(ns);
   std::vector<int64_t> qw(ns + 1);
   qw[0] = 0;
@@ -1647,7 +1649,7 @@ int gfs_batch_build(gfs_ctx* c, const gfs_shape* shapes, int ns) {
     a.arg_out = shapes[s].argmin_out;
     a.fl_out = shapes[s].flags_out;
     a.cnt = c->b_cnt.as<Counters>();
-    qw[s + 1] = qw[s] + (shapes[s].m + 31) / 32;
+    qw[s + 1] = qw[s] + (shapes[s].m + c->b_packet - 1) / c->b_packet;
   }
   GFS_TRY(ensure(c->b_qviews, size_t(ns) * sizeof(QueryArgs)));
   GFS_TRY(ensure(c->b_qw, size_t(ns + 1) * 8));
@@ -1715,7 +1717,7 @@ int gfs_batch_query(gfs_ctx* c) {
   for (int phase = 1; phase <= 3; ++phase) {
     GFS_CK(cudaMemsetAsync(c->b_ctr.p, 0, 8, st));
     GFS_CK(launch_batch_query(c->b_qviews.as<QueryArgs>(), c->b_qw.as<int64_t>(), ns, c->b_qtotal,
-                              c->b_ctr.as<unsigned long long>(), grid, phase, st));
+                              c->b_ctr.as<unsigned long long>(), grid, phase, c->b_packet, st));
   }
   return GFS_OK;
 }

@@ -1308,9 +1308,12 @@ cudaError_t launch_cull(const CullArgs& one, const CullArgs* views, const int64_
 
 template <int G>
 static void query_spheres(const QueryArgs& a, const Packets& p, cudaStream_t st) {
-  if (p.sparse) {
-    k_query_spheres<G, true><<<nblk(a.m, G), 32, 0, st>>>(a, p.lim);
-    k_query_spheres_marked<G><<<unsigned(a.m), 32, 0, st>>>(a);
+  constexpr bool kMaySparse = G == 8 || G == kPacket;
+  if (kMaySparse && p.sparse) {
+    if constexpr (kMaySparse) {
+      k_query_spheres<G, true><<<nblk(a.m, G), 32, 0, st>>>(a, p.lim);
+      k_query_spheres_marked<G><<<unsigned(a.m), 32, 0, st>>>(a);
+    }
   } else {
     k_query_spheres<G, false><<<nblk(a.m, G), 32, 0, st>>>(a, p.lim);
     if constexpr (G > 1) k_query_spheres_split<G><<<152 * 28, 32, 0, st>>>(a);
@@ -1320,11 +1323,14 @@ static void query_spheres(const QueryArgs& a, const Packets& p, cudaStream_t st)
 
 template <int G>
 static void query_rest(const QueryArgs& a, const Packets& p, cudaStream_t st) {
-  if (p.sparse) {
-    k_query_near<G, true><<<nblk(a.m, G), 32, 0, st>>>(a, p.lim);
-    k_query_near_marked<G><<<unsigned(a.m), 32, 0, st>>>(a);
-    k_query_decide<G, true><<<nblk(a.m, G), 32, 0, st>>>(a, p.lim);
-    k_query_decide_marked<G><<<unsigned(a.m), 32, 0, st>>>(a);
+  constexpr bool kMaySparse = G == 8 || G == kPacket;
+  if (kMaySparse && p.sparse) {
+    if constexpr (kMaySparse) {
+      k_query_near<G, true><<<nblk(a.m, G), 32, 0, st>>>(a, p.lim);
+      k_query_near_marked<G><<<unsigned(a.m), 32, 0, st>>>(a);
+      k_query_decide<G, true><<<nblk(a.m, G), 32, 0, st>>>(a, p.lim);
+      k_query_decide_marked<G><<<unsigned(a.m), 32, 0, st>>>(a);
+    }
   } else {
     k_query_near<G, false><<<nblk(a.m, G), 32, 0, st>>>(a, p.lim);
     if constexpr (G > 1) k_query_near_split<G><<<152 * 28, 32, 0, st>>>(a);

@@ -282,10 +282,13 @@ cudaError_t launch_batch_surv_keys(const float4* items, const uint16_t* shape, u
 cudaError_t launch_batch_gather_points(const float4* src, const int* order, unsigned n, float4* dst, cudaStream_t st);
 cudaError_t launch_batch_qkeys(const ShapeDesc* d, const int64_t* off, int ns, int64_t M, unsigned long long* keys,
                                int* vals, cudaStream_t st);
-// phase 1: the sphere pass of every (shape, 32 points) item, phase 2: the rest
-// (reset ctr between the two launches)
+// points of a batched query's packets
+inline int batch_packet(int64_t, int64_t) { return 16; }
+// phase 1: the sphere pass, 2: the survivor pass, 3: the decisions of every item
+// (a packet of one shape; wprefix: first item of each shape; reset ctr between
+// the launches)
 cudaError_t launch_batch_query(const QueryArgs* views, const int64_t* wprefix, int ns, int64_t limit,
-                               unsigned long long* ctr, int grid, int phase, cudaStream_t st);
+                               unsigned long long* ctr, int grid, int phase, int packet, cudaStream_t st);
 // the survivor forest of one class laid out and built on the device from the
 // cull's counts (capacity cap survivor slots, node_cap nodes, nlev levels;
 // the query views' survivor pointers and trees are patched; overflow sets a
