@@ -160,7 +160,7 @@ __global__ void k_batch_qkeys(const ShapeDesc* __restrict__ d, const int64_t* __
 // points of the shape's Morton order).  A packet an item: with two of 16 an item,
 // one after the other on its warp, 64 shapes of 200 samples and 1,000 points
 // took 0.75 ms (0.61 before the packets), now 0.53; the batch of 16 shapes 62.4, now
-// 56.7.
+// 56.7.  G is 16, or 32 for very many points a sample (batch_packet).
 // kPhase 1: the sphere pass (state per point to the view's state array);
 // kPhase 2: the survivor pass; kPhase 3: the decisions (as the single-shape
 // query's kernels)

@@ -805,6 +805,11 @@ static Packets packets_of(const QueryArgs& a) {
   if (p.G == 1) return p;
   p.lim = p.G == kPacket ? PkLimit{0.f, 600, 100} : PkLimit{0.f, 80, 32};
   p.sparse = a.m < (p.G == kPacket ? a.n : 3 * a.n);
+  // very many points a sample (ms with 16 / 32, after 32 with a walk per point:
+  // 1M points on 100 samples 0.85 | 0.95 / 0.79, 4M 2.66 | 3.30 / 2.22, 1M on 1,000
+  // 1.79 | 1.35 / 1.20; but 1M on 4,096 2.37 | 1.55 / 1.70, 0.2M on 1,000 0.90 | 0.59 /
+  // 0.68)
+  if (a.m >= 524288 && a.m >= 512 * a.n) p.G = 32;
   p.lim.rho = p.sparse ? kClose * cbrtf(1.f / float(a.n)) : kJump * cbrtf(float(p.G) / float(a.m));
   return p;
 }
@@ -1346,6 +1351,7 @@ cudaError_t launch_query_spheres(const QueryArgs& a, cudaStream_t st) {
   switch (p.G) {
     case 1: query_spheres<1>(a, p, st); break;
     case 8: query_spheres<8>(a, p, st); break;
+    case 32: query_spheres<32>(a, p, st); break;
     default: query_spheres<kPacket>(a, p, st);
   }
   return cudaGetLastError();
@@ -1357,6 +1363,7 @@ cudaError_t launch_query_finish(const QueryArgs& a, cudaStream_t st) {
   switch (p.G) {
     case 1: query_rest<1>(a, p, st); break;
     case 8: query_rest<8>(a, p, st); break;
+    case 32: query_rest<32>(a, p, st); break;
     default: query_rest<kPacket>(a, p, st);
   }
   return cudaGetLastError();
