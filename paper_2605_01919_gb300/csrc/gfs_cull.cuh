@@ -256,6 +256,7 @@ __global__ void __launch_bounds__(128) k_cull_groups(const __grid_constant__ Cul
   uint32_t* stk = s_stk[w];
   LevelTable& C = s_lv[w];
   const unsigned groups = s.gcount[0];
+  if (!groups) return;
   const uint32_t K = uint32_t(s.K);
   unsigned rechecks = 0, n_nodes = 0, n_items = 0;
   const CullArgs* loaded = nullptr;
