@@ -182,13 +182,8 @@ __device__ bool sphere_band(const QueryArgs& a, const BuildConsts& bc, SpWarp& S
   const bool done = packet_walk<G>(
       T, S, lane, G > 1 ? lim.rest * G : -1,
       [&](int64_t nd) {
-        const Lin q = lin_load(T, nd);
-        float nx = k.cx - q.cx, ny = k.cy - q.cy, nz = k.cz - q.cz;
-        const float d = unit3(nx, ny, nz);
-        const float sp_ = fmaf(fabsf(nx + q.gx), q.hx, fmaf(fabsf(ny + q.gy), q.hy, fabsf(nz + q.gz) * q.hz));
-        const float sm_ = fmaf(fabsf(nx - q.gx), q.hx, fmaf(fabsf(ny - q.gy), q.hy, fabsf(nz - q.gz) * q.hz));
-        const float v = mode == 1 ? fminf(d + q.lop - sm_, d - q.hin - sp_) : (cls == 0 ? d - q.hip - sp_ : d + q.lon - sm_);
-        return pk_reach(r, k.rho, bc.elin, v, nx, ny, nz);
+        const LinAt b = lin_at(lin_load(T, nd), k.cx, k.cy, k.cz);
+        return pk_reach(r, k.rho, bc.elin, mode == 1 ? b.far : (cls == 0 ? b.pos : b.neg), b.nx, b.ny, b.nz);
       },
       [&](int c, float4& P) {
         P = a.sph[c];

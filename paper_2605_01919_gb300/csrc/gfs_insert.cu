@@ -94,14 +94,7 @@ struct QShared {
   int qn[kQW];
 };
 
-// order-preserving bits
-__device__ __forceinline__ uint32_t ord32(float v) {
-  const uint32_t b = __float_as_uint(v);
-  return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-}
-__device__ __forceinline__ float ord32_value(uint32_t k) {
-  return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
-}
+// order-preserving bits of a double, and back
 __device__ __forceinline__ unsigned long long ord64(double v) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(__dadd_rn(v, 0.0));  // -0 like +0
   return (b >> 63) ? ~b : (b | (1ull << 63));
@@ -157,15 +150,15 @@ __device__ void block_argmin(double (&v)[NV], uint32_t (&idx)[NV], QShared& S) {
 __device__ __forceinline__ void block_thresholds(float& a, float& b, float& c, bool& f0, bool& f1, int& turn,
                                                  QShared& S) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const uint32_t ka = __reduce_min_sync(kAll, ord32(a)), kb = __reduce_min_sync(kAll, ord32(b)),
-                 kc = __reduce_min_sync(kAll, ord32(c));
+  const uint32_t ka = __reduce_min_sync(kAll, ord_key(a)), kb = __reduce_min_sync(kAll, ord_key(b)),
+                 kc = __reduce_min_sync(kAll, ord_key(c));
   const uint32_t fl = __reduce_or_sync(kAll, (f0 ? 1u : 0u) | (f1 ? 2u : 0u));
   if (lane == 0) S.th[turn][w] = make_uint4(ka, kb, kc, fl);
   __syncthreads();
   const uint4 t = lane < kQW ? S.th[turn][lane] : make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0u);
-  a = ord32_value(__reduce_min_sync(kAll, t.x));
-  b = ord32_value(__reduce_min_sync(kAll, t.y));
-  c = ord32_value(__reduce_min_sync(kAll, t.z));
+  a = ord_val(__reduce_min_sync(kAll, t.x));
+  b = ord_val(__reduce_min_sync(kAll, t.y));
+  c = ord_val(__reduce_min_sync(kAll, t.z));
   const uint32_t f = __reduce_or_sync(kAll, t.w);
   f0 = (f & 1u) != 0;
   f1 = (f & 2u) != 0;
@@ -296,7 +289,7 @@ __global__ void __launch_bounds__(kQT) k_ins_query(InsertArgs a) {
   const float Ax = absmax3(xf, yf, zf);
   const double tol = a.tol;
   // range and margin of the linear node bounds
-  const float A = a.bc->A, mg = a.bc->elin + 8.f * 5.9604645e-8f * A;
+  const float A = a.bc->A, mg = lin_point_margin(*a.bc);
   const bool in_range = fabs(x) <= A && fabs(y) <= A && fabs(z) <= A;
   // ---- spheres: sample, containment, nearest tangent per class, far bound
   // exact per-thread state (FP64, the oracle's expressions)
@@ -473,14 +466,11 @@ __global__ void __launch_bounds__(kQT) k_ins_query(InsertArgs a) {
         const float th1 = cw1 ? fA1 : fmaxf(fA1, ntol_up);
         if (in_range) {
           const Lin q = lin_load(a.st, node);
-          float nx = xf - q.cx, ny = yf - q.cy, nz = zf - q.cz;
-          const bool at = (fabsf(nx) <= q.hx + mg) & (fabsf(ny) <= q.hy + mg) & (fabsf(nz) <= q.hz + mg);
-          const float d = unit3(nx, ny, nz);
-          const float sp = fmaf(fabsf(nx + q.gx), q.hx, fmaf(fabsf(ny + q.gy), q.hy, fabsf(nz + q.gz) * q.hz));
-          const float sm = fmaf(fabsf(nx - q.gx), q.hx, fmaf(fabsf(ny - q.gy), q.hy, fabsf(nz - q.gz) * q.hz));
+          const bool at = (fabsf(xf - q.cx) <= q.hx + mg) & (fabsf(yf - q.cy) <= q.hy + mg) &
+                          (fabsf(zf - q.cz) <= q.hz + mg);
+          const LinAt b = lin_at(q, xf, yf, zf);
           // (an absent class: inf - inf compares false)
-          return bool(at | (d - q.hip - sp - th0 <= mg) | (d + q.lon - sm - th1 <= mg) |
-                      (fminf(d + q.lop - sm, d - q.hin - sp) - fF <= mg));
+          return bool(at | (b.pos - th0 <= mg) | (b.neg - th1 <= mg) | (b.far - fF <= mg));
         }
         const float4 R = a.st.nb[node], Fb = a.st.nf[node];
         const float dc = sqrtf(ball_d2(xf, yf, zf, a.st.na[node]));

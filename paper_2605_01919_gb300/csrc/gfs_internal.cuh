@@ -158,10 +158,6 @@ __device__ __forceinline__ double ball_d2_64(double x, double y, double z, const
   return dx * dx + dy * dy + dz * dz;
 }
 
-__device__ __forceinline__ bool inside_box(float x, float y, float z, const float4& lo, const float4& hi) {
-  return x >= lo.x && x <= hi.x && y >= lo.y && y <= hi.y && z >= lo.z && z <= hi.z;
-}
-
 // Morton code of a point, 10 bits per axis over [-1, 1] (clamped)
 __device__ __forceinline__ uint32_t spread10(uint32_t v) {
   v &= 1023u;
@@ -187,8 +183,7 @@ struct BuildConsts {
   float ea;       // FP32 error bound on |x-p| -+ r for queries
   float ed_lin;   // survivor distance^2 error: ed_lin * sqrt(D) + ed_quad * D
   float ed_quad;
-  float eprune;   // additive slack for FP32 node pruning
-  float pad;
+  float pad;      // additive slack of the ball bounds of candidate points
   float elin;     // margin of the linear node bounds (and of sphere values) against the FP32 error bands
 };
 

@@ -84,14 +84,14 @@ __device__ BuildConsts make_consts(unsigned int amax_bits, unsigned int rmax_bit
   // survivor distance^2: 2 sqrt3 (eq + uA) sqrt(D) + 5 u D, times 2
   c.ed_lin = 4.f * s3 * (c.eq + u * A);
   c.ed_quad = 10.f * u;
-  // FP32 box-distance slack for a point rounded from FP64
-  c.eprune = 4.f * s3 * u * A + 1e-7f;
-  // the same for candidate points (their FP32 error is eq)
+  // FP32 slack of a ball's distance to a candidate point (its FP32 error is eq)
   c.pad = 4.f * s3 * (c.eq + u * A) + 1e-7f;
   // linear node bounds against a reference sphere's value at another point of
   // the packet: about 130 u A + 6 u R of FP32 rounding (the record's box and
   // residuals, |x - c| and the unit vectors, the sums), plus the widest error
-  // band 2 ea, so that whatever they discard also lies outside that band
+  // band 2 ea, so that whatever they discard also lies outside that band.  A
+  // candidate outside the box lies up to A + R: about 8 u R more, which the R term
+  // holds (and the cull adds 4 eq for the candidate's own rounding)
   c.elin = u * (300.f * A + 24.f * R) + 1e-11f;
   return c;
 }
@@ -513,15 +513,6 @@ __host__ __device__ inline int64_t level_span(int level) {
 __global__ void __launch_bounds__(kNodeBlock) k_sphere_level(float A, Tree T, int level) {
   const int64_t j = node_of_thread();
   if (j < T.count[level]) sphere_level_node(T, A, level, j, node_part());
-}
-
-// order-preserving map of floats onto unsigned integers (for atomicMax)
-__device__ __forceinline__ unsigned ord_key(float v) {
-  const unsigned b = __float_as_uint(v);
-  return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-}
-__device__ __forceinline__ float ord_val(unsigned k) {
-  return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
 }
 
 // Tightening of the internal radii, pass 1: one thread per sphere; at every

@@ -174,7 +174,7 @@ __device__ inline void warp_scored_one(const QueryArgs& a, int box_cull, const u
     // radius - tol rounded down; W.rec_id: input index)
     int nrec = 0, at = 0;
     unsigned n_nodes = 0, n_items = 0;
-    const float cover_lim = -a.tol32 + a.bc->elin, mg = a.bc->elin + 8.f * tangent::kTanU * A;
+    const float cover_lim = -a.tol32 + a.bc->elin, mg = lin_point_margin(*a.bc);
     // as in scored_one: is the tangent point surely inside one of the balls
     auto surely_covered = [&](const float4& S, float d32, float sr, int j) -> bool {
       const float ap = amax3(S.x, S.y, S.z), r = fabsf(sr);
@@ -282,12 +282,8 @@ __device__ inline void warp_scored_one(const QueryArgs& a, int box_cull, const u
             return dC - err32(F.ax, Bc, dC, Bc.w) - Bc.w <= R32 || dF - err32(F.ax, Fb, dF, Fb.w) - Fb.w <= R32;
           }
           // the least d - r and d + r of the node's spheres, d = |x - p|
-          const Lin l = lin_load(T, node);
-          float nx = F.x32 - l.cx, ny = F.y32 - l.cy, nz = F.z32 - l.cz;
-          const float d = unit3(nx, ny, nz);
-          const float sp = fmaf(fabsf(nx + l.gx), l.hx, fmaf(fabsf(ny + l.gy), l.hy, fabsf(nz + l.gz) * l.hz));
-          const float sm = fmaf(fabsf(nx - l.gx), l.hx, fmaf(fabsf(ny - l.gy), l.hy, fabsf(nz - l.gz) * l.hz));
-          return fminf(d - l.hip - sp, d + l.lon - sm) - R32 <= mg || fminf(d + l.lop - sm, d - l.hin - sp) - R32 <= mg;
+          const LinAt b = lin_at(lin_load(T, node), F.x32, F.y32, F.z32);
+          return fminf(b.pos, b.neg) - R32 <= mg || b.far - R32 <= mg;
         },
         [&](int64_t jj) {
           bool near_ok = false, far_ok = false;

@@ -293,14 +293,12 @@ __device__ bool sphere_pass(const QueryArgs& a, int64_t first, SpWarp& S, int la
           if (c < L.y) {
             ++n_nodes;
             const Lin q = lin_load(T, L.x + c);
-            float nx = cx - q.cx, ny = cy - q.cy, nz = cz - q.cz;
             const float lim = rho + margin;
-            const bool at = (fabsf(nx) <= q.hx + lim) & (fabsf(ny) <= q.hy + lim) & (fabsf(nz) <= q.hz + lim);
-            const float d = unit3(nx, ny, nz);
-            const float sp_ = fmaf(fabsf(nx + q.gx), q.hx, fmaf(fabsf(ny + q.gy), q.hy, fabsf(nz + q.gz) * q.hz));
-            const float sm_ = fmaf(fabsf(nx - q.gx), q.hx, fmaf(fabsf(ny - q.gy), q.hy, fabsf(nz - q.gz) * q.hz));
-            pass_n = at | reach(d - q.hip - sp_, nx, ny, nz, R[0]) | reach(d + q.lon - sm_, nx, ny, nz, R[1]) |
-                     reach(fminf(d + q.lop - sm_, d - q.hin - sp_), nx, ny, nz, R[2]);
+            const bool at = (fabsf(cx - q.cx) <= q.hx + lim) & (fabsf(cy - q.cy) <= q.hy + lim) &
+                            (fabsf(cz - q.cz) <= q.hz + lim);
+            const LinAt b = lin_at(q, cx, cy, cz);
+            pass_n = at | reach(b.pos, b.nx, b.ny, b.nz, R[0]) | reach(b.neg, b.nx, b.ny, b.nz, R[1]) |
+                     reach(b.far, b.nx, b.ny, b.nz, R[2]);
           }
         }
       }

@@ -251,7 +251,6 @@ __device__ inline void warp_tangent_search(const QueryArgs& a, int box_cull, dou
 // ---------------------------------------------------------------------------
 
 constexpr int kTanRecent = 8;
-constexpr float kTanU = 5.9604644775390625e-8f;  // 2^-24
 
 static_assert(kWarpStack + kFan >= kCoverStack, "warp_lin_walk's stack");
 struct TanWarp {
@@ -260,14 +259,7 @@ struct TanWarp {
   int rec_id[kTanRecent];  // sorted slot
 };
 
-__device__ __forceinline__ unsigned ord_bits(float v) {  // order-preserving
-  const unsigned b = __float_as_uint(v);
-  return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-}
-__device__ __forceinline__ float ord_value(unsigned k) {
-  return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
-}
-__device__ __forceinline__ float warp_min_f(float v) { return ord_value(__reduce_min_sync(kLanes, ord_bits(v))); }
+__device__ __forceinline__ float warp_min_f(float v) { return ord_val(__reduce_min_sync(kLanes, ord_key(v))); }
 
 // node(global node, lin, level) -> visit its children; items(slot or -1) runs
 // on all lanes in rounds that reach leaves.  Stack bound as in warp_cover_walk.
@@ -311,7 +303,7 @@ __device__ inline void warp_sphere_bounds_lin(const QueryArgs& a, const LevelTab
   const Tree& T = a.st;
   if (T.nlevels == 0) return;
   const float x32 = float(x), y32 = float(y), z32 = float(z), ax = amax3(x32, y32, z32);
-  const float mg = a.bc->elin + 8.f * kTanU * a.bc->A;
+  const float mg = lin_point_margin(*a.bc);
   float thF = INFINITY, thA[2] = {INFINITY, INFINITY};
   auto item = [&](int64_t j) -> bool {
     const float4 S = a.sph[j];
@@ -371,7 +363,7 @@ __device__ inline void warp_sphere_bounds_lin(const QueryArgs& a, const LevelTab
         if (grp < 2) w = grp == 0 ? T.nb[nd].x : T.nb[nd].y;
         v = dist32(x32, y32, z32, B) - w;
       }
-      unsigned key = v < INFINITY ? (ord_bits(v) & ~7u) | unsigned(sub) : 0xffffffffu;
+      unsigned key = v < INFINITY ? (ord_key(v) & ~7u) | unsigned(sub) : 0xffffffffu;
       for (int o = 4; o > 0; o >>= 1) key = min(key, __shfl_xor_sync(kLanes, key, o));
       const int64_t next = __shfl_sync(kLanes, (long long)node, (lane & 24) | int(key & 7u)) * kFan + sub;
       valid = key != 0xffffffffu;
@@ -385,14 +377,9 @@ __device__ inline void warp_sphere_bounds_lin(const QueryArgs& a, const LevelTab
   warp_lin_walk(
       T, C, W.stk, lane,
       [&](int64_t nd) {
-        const Lin q = lin_load(T, nd);
-        float nx = x32 - q.cx, ny = y32 - q.cy, nz = z32 - q.cz;
-        const float d = unit3(nx, ny, nz);
-        const float sp = fmaf(fabsf(nx + q.gx), q.hx, fmaf(fabsf(ny + q.gy), q.hy, fabsf(nz + q.gz) * q.hz));
-        const float sm = fmaf(fabsf(nx - q.gx), q.hx, fmaf(fabsf(ny - q.gy), q.hy, fabsf(nz - q.gz) * q.hz));
+        const LinAt b = lin_at(lin_load(T, nd), x32, y32, z32);
         // (an absent class: inf - inf compares false)
-        return d - q.hip - sp - thA[0] <= mg || d + q.lon - sm - thA[1] <= mg ||
-               fminf(d + q.lop - sm, d - q.hin - sp) - thF <= mg;
+        return b.pos - thA[0] <= mg || b.neg - thA[1] <= mg || b.far - thF <= mg;
       },
       items);
   R.cov[0] = __any_sync(kLanes, R.cov[0]);
@@ -412,7 +399,7 @@ __device__ inline void warp_tangent_search_lin(const QueryArgs& a, const LevelTa
   const double lim_d = mode == kBelowSurvivor ? sqrt(lim) : (mode == kWithinOpposite ? lim : INFINITY);
   const float x32 = float(x), y32 = float(y), z32 = float(z), ax = amax3(x32, y32, z32);
   const float lo_f = f_dn(lo);
-  const float mg = a.bc->elin + 8.f * kTanU * A;
+  const float mg = lin_point_margin(*a.bc);
   const float cover_lim = -a.tol32 + a.bc->elin;
   float hi_f = f_up(lim_d * kRel + kAbs);
   int nrec = 0, at = 0;
@@ -505,19 +492,16 @@ __device__ inline void warp_tangent_search_lin(const QueryArgs& a, const LevelTa
         // |h|^2 / (2 (D - |h|)) (the chord's excess over its projection on n),
         // res the least residual of r, or |x - F| + wf
         const Lin q = lin_load(T, nd);
-        float nx = x32 - q.cx, ny = y32 - q.cy, nz = z32 - q.cz;
-        const float d = unit3(nx, ny, nz);
-        const float sp = fmaf(fabsf(nx + q.gx), q.hx, fmaf(fabsf(ny + q.gy), q.hy, fabsf(nz + q.gz) * q.hz));
-        const float sm = fmaf(fabsf(nx - q.gx), q.hx, fmaf(fabsf(ny - q.gy), q.hy, fabsf(nz - q.gz) * q.hz));
-        const float near_lo = cs == 0 ? d - q.hip - sp : d + q.lon - sm;
+        const LinAt b = lin_at(q, x32, y32, z32);
+        const float near_lo = cs == 0 ? b.pos : b.neg;
         if (!(near_lo < INFINITY)) return false;  // none of the class
-        const float far_lo = cs == 0 ? d + q.lop - sm : d - q.hin - sp;
+        const float far_lo = cs == 0 ? b.d + q.lop - b.sm : b.d - q.hin - b.sp;
         if (far_lo - hi_f <= mg) return true;
         if (!(near_lo - hi_f <= mg)) return false;
         if (-near_lo + mg >= lo_f) return true;
         const float h2 = fmaf(q.hx, q.hx, fmaf(q.hy, q.hy, q.hz * q.hz)), hn = sqrtf(h2);
-        const float over = d > 2.f * hn ? 0.5f * h2 / (d - hn) * (1.f + 1e-5f) : INFINITY;
-        const float up = (cs == 0 ? d - q.lop + sp : d + q.hin + sm) + over;
+        const float over = b.d > 2.f * hn ? 0.5f * h2 / (b.d - hn) * (1.f + 1e-5f) : INFINITY;
+        const float up = (cs == 0 ? b.d - q.lop + b.sp : b.d + q.hin + b.sm) + over;
         if (!(up + mg >= lo_f)) return false;
         const float4 Fb = T.nf[nd];
         const float df = dist32(x32, y32, z32, Fb);

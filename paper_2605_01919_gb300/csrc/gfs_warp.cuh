@@ -75,6 +75,42 @@ __device__ __forceinline__ float unit3(float& x, float& y, float& z) {
   return q * inv;
 }
 
+// order-preserving bits of a float, and back
+__device__ __forceinline__ unsigned ord_key(float v) {
+  const unsigned b = __float_as_uint(v);
+  return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
+}
+__device__ __forceinline__ float ord_val(unsigned k) {
+  return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
+}
+
+// A node's linear bounds (struct Lin) at a point: direction and distance from
+// the centre of its box, the box's support against -g and g (sp, sm), and the
+// least |x - p| - |s| over its positive and negative spheres and |x - p| + |s|
+// over all (an absent class: inf).  They hold within BuildConsts::elin, for
+// points up to A (or A + R, a candidate's range).
+struct LinAt {
+  float nx, ny, nz, d, sp, sm;
+  float pos, neg, far;
+};
+__device__ __forceinline__ LinAt lin_at(const Lin& q, float x, float y, float z) {
+  LinAt r;
+  r.nx = x - q.cx;
+  r.ny = y - q.cy;
+  r.nz = z - q.cz;
+  r.d = unit3(r.nx, r.ny, r.nz);
+  r.sp = fmaf(fabsf(r.nx + q.gx), q.hx, fmaf(fabsf(r.ny + q.gy), q.hy, fabsf(r.nz + q.gz) * q.hz));
+  r.sm = fmaf(fabsf(r.nx - q.gx), q.hx, fmaf(fabsf(r.ny - q.gy), q.hy, fabsf(r.nz - q.gz) * q.hz));
+  r.pos = r.d - q.hip - r.sp;
+  r.neg = r.d + q.lon - r.sm;
+  r.far = fminf(r.d + q.lop - r.sm, r.d - q.hin - r.sp);
+  return r;
+}
+// the bounds' margin for an FP64 point in range rounded to FP32 (8 u A)
+__device__ __forceinline__ float lin_point_margin(const BuildConsts& bc) {
+  return bc.elin + 8.f * 5.9604644775390625e-8f * bc.A;
+}
+
 // (first node, nodes) of each level, in shared memory: lanes index it by the
 // level of the entry they hold
 struct LevelTable {
@@ -100,10 +136,6 @@ __device__ int warp_cover_walk(const Tree& T, const LevelTable& C, uint32_t* stk
                                float qz, float lim, unsigned& n_nodes, unsigned& n_items, Test test) {
   const unsigned kAllLanes = 0xffffffffu;
   const int top = T.nlevels - 1, grp = lane >> 3, sub = lane & 7;
-  auto key_of = [](float v) {  // order-preserving
-    const unsigned b = __float_as_uint(v);
-    return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-  };
   int sp = C.lv[top].y;
   __syncwarp();
   if (lane < sp) stk[lane] = pack_node(top, lane);
@@ -126,25 +158,21 @@ __device__ int warp_cover_walk(const Tree& T, const LevelTable& C, uint32_t* stk
         const int2 L = C.lv[lev - 1];
         if (c < L.y) {
           ++n_nodes;
-          const Lin r = lin_load(T, L.x + c);
-          float nx = qx - r.cx, ny = qy - r.cy, nz = qz - r.cz;
-          const float d = unit3(nx, ny, nz);
-          const float sp_ = fmaf(fabsf(nx + r.gx), r.hx, fmaf(fabsf(ny + r.gy), r.hy, fabsf(nz + r.gz) * r.hz));
-          const float sm_ = fmaf(fabsf(nx - r.gx), r.hx, fmaf(fabsf(ny - r.gy), r.hy, fabsf(nz - r.gz) * r.hz));
-          v = fminf(d - r.hip - sp_, d + r.lon - sm_);
+          const LinAt r = lin_at(lin_load(T, L.x + c), qx, qy, qz);
+          v = fminf(r.pos, r.neg);
           pass = v <= lim;
         }
       }
     }
     if (__any_sync(kAllLanes, cov)) {
-      const unsigned key = cov ? key_of(v) : 0xffffffffu;
+      const unsigned key = cov ? ord_key(v) : 0xffffffffu;
       return __shfl_sync(kAllLanes, c, __ffs(__ballot_sync(kAllLanes, key == __reduce_min_sync(kAllLanes, key))) - 1);
     }
     // the child that reaches deepest around the point goes on top, below it
     // those that reach at least half as deep
-    const unsigned key = pass ? key_of(v) : 0xffffffffu;
+    const unsigned key = pass ? ord_key(v) : 0xffffffffu;
     const unsigned low = __reduce_min_sync(kAllLanes, key);
-    const float deep = __uint_as_float((low & 0x80000000u) ? (low & 0x7fffffffu) : ~low);
+    const float deep = ord_val(low);
     const unsigned bn = __ballot_sync(kAllLanes, pass);
     const unsigned bq = __ballot_sync(kAllLanes, pass && v < 0.5f * deep);
     if (pass) {
