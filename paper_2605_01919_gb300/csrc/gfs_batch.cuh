@@ -71,18 +71,18 @@ __global__ void __launch_bounds__(kNodeBlock) k_batch_tree_level(const Tree* __r
                                    int level, const float4* __restrict__ items_base,
                                    const int64_t* __restrict__ item_off, const BuildConsts* __restrict__ bc,
                                    int is_sphere) {
-  const int64_t g = is_sphere ? node_of_thread() : blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+  const int64_t g = is_sphere ? node_of_thread<false>() : blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
   if (g >= prefix[ns]) return;
   const int s = find_seg(prefix, ns, g);
   const Tree& T = trees[s];
   const int64_t j = g - prefix[s];
   if (level == 0) {
     const float4* items = items_base + item_off[s];
-    if (is_sphere) sphere_leaf_node(items, bc[s].A, T, j, node_part());
+    if (is_sphere) sphere_leaf_node<false>(items, bc[s].A, T, j, node_part());
     else point_leaf_node(items, T.nitems, T.lo, T.hi, j);
   } else {
     if (is_sphere)
-      sphere_level_node(T, bc[s].A, level, j, node_part());
+      sphere_level_node<false>(T, bc[s].A, level, j, node_part());
     else
       point_level_node(T.lo, T.hi, T.offset[level - 1], T.count[level - 1], T.offset[level], j);
   }

@@ -33,6 +33,7 @@ namespace cg = cooperative_groups;
 namespace gfs {
 
 constexpr float kU = 5.9604644775390625e-8f;  // 2^-24, FP32 unit roundoff
+constexpr unsigned kFull = 0xffffffffu;
 
 __device__ __forceinline__ float sqf(float v) { return v * v; }
 
@@ -251,6 +252,74 @@ __device__ float4 bound_ball(const float4 (&it)[kFan], int k) {
   return make_float4(bx, by, bz, 0.f);
 }
 
+// bound_ball by 8 lanes, an item each (the same operations on the same numbers
+// in the same order, so the same centre): a step's roots run side by side.  All
+// 32 lanes call it, for four centres; `mine` has w = -inf past the k-th item.
+__device__ float4 bound_ball8(const float4& mine, int k) {
+  const int lane = threadIdx.x & 31, first = lane & ~(kFan - 1);
+  auto eval = [&](float cx, float cy, float cz, float4& far) {
+    const float dx = mine.x - cx, dy = mine.y - cy, dz = mine.z - cz;
+    const float d = sqrtf(dx * dx + dy * dy + dz * dz);
+    const float v = d + mine.w;
+    float best = fmaxf(v, -INFINITY);
+#pragma unroll
+    for (int o = 1; o < kFan; o <<= 1) best = fmaxf(best, __shfl_xor_sync(kFull, best, o));
+    const unsigned at = (__ballot_sync(kFull, v == best && best > -INFINITY) >> first) & 0xffu;
+    const int src = first + (at ? __ffs(at) - 1 : 0);
+    far = make_float4(__shfl_sync(kFull, mine.x, src), __shfl_sync(kFull, mine.y, src),
+                      __shfl_sync(kFull, mine.z, src), __shfl_sync(kFull, d, src));
+    return best;
+  };
+  int big = first;
+  float bw = __shfl_sync(kFull, mine.w, first), mx = 0.f, my = 0.f, mz = 0.f;
+#pragma unroll
+  for (int i = 0; i < kFan; ++i) {
+    const float x = __shfl_sync(kFull, mine.x, first + i), y = __shfl_sync(kFull, mine.y, first + i),
+                z = __shfl_sync(kFull, mine.z, first + i), w = __shfl_sync(kFull, mine.w, first + i);
+    if (i >= k) continue;
+    if (w > bw) {
+      big = first + i;
+      bw = w;
+    }
+    mx += x;
+    my += y;
+    mz += z;
+  }
+  mx /= float(k);
+  my /= float(k);
+  mz /= float(k);
+  const float gx = __shfl_sync(kFull, mine.x, big), gy = __shfl_sync(kFull, mine.y, big),
+              gz = __shfl_sync(kFull, mine.z, big);
+  float4 far, far1;
+  const float v0 = eval(gx, gy, gz, far), v1 = eval(mx, my, mz, far1);
+  const bool at_big = v0 <= v1;
+  if (!at_big) far = far1;
+  float cx = at_big ? gx : mx, cy = at_big ? gy : my, cz = at_big ? gz : mz;
+  float bx = cx, by = cy, bz = cz, best = fminf(v0, v1);
+  bool moving = true;  // (of this centre; a centre that has stopped keeps its best)
+  for (int t = 0; t < 23; ++t) {
+    moving = moving && far.w > 1e-12f;
+    if (!__any_sync(kFull, moving)) break;
+    const float dx = far.x - cx, dy = far.y - cy, dz = far.z - cz;
+    const float step = far.w / float(t + 2);
+    cx += dx / far.w * step;
+    cy += dy / far.w * step;
+    cz += dz / far.w * step;
+    float4 next;
+    const float v = eval(cx, cy, cz, next);
+    if (moving) {
+      far = next;
+      if (v < best) {
+        best = v;
+        bx = cx;
+        by = cy;
+        bz = cz;
+      }
+    }
+  }
+  return make_float4(bx, by, bz, 0.f);
+}
+
 // Upper bound of a node radius term d = dist (+-) r computed in FP32: the
 // rounding of dist (<= 3.6 ulp relative) and of the sum (1 ulp), and the FP32
 // copy of an FP64 sphere (sqrt3 ulp of |p| = pm, 1 ulp of r), each covered
@@ -267,13 +336,35 @@ __device__ __forceinline__ float radius_fin(float v, float A) {
 // and kFar (centre F and its radius, the linear record), in different warps: a
 // centre's steps are one serial chain, and small hierarchies wait for it
 // (16^3 samples built and queried: 0.67 ms, 0.71 with both chains on one
-// thread; 49^3 samples built: 5.7 ms either way).
+// thread, 0.655 with 8 lanes a centre where nodes are few).
 enum NodePart { kNear, kFar };
-constexpr int kNodeBlock = 128;                  // threads, two per node
+constexpr int kNodeBlock = 128;                  // threads, two per node (wide: two groups of 8)
 constexpr int kNodesPerBlock = kNodeBlock / 2;
+// Up to this many nodes of a level the centres' chains are what takes the time:
+// the levels (leaves) of 16^3 samples 26 (16) us by 8 lanes, 39 (23) by one; of
+// 49^3 55 us with the small levels wide, 77 with none, 78 with all; leaves of 96^3
+// 243 us wide, 77 not.
+constexpr int64_t kWideNodes = 1024;
+__host__ __device__ inline bool wide_nodes(int64_t n) { return n <= kWideNodes; }
+__host__ __device__ inline int nodes_per_block(bool wide) { return wide ? kNodesPerBlock / kFan : kNodesPerBlock; }
 __device__ __forceinline__ NodePart node_part() { return int(threadIdx.x) < kNodesPerBlock ? kNear : kFar; }
+template <bool kWide>
 __device__ __forceinline__ int64_t node_of_thread() {
-  return blockIdx.x * int64_t(kNodesPerBlock) + threadIdx.x % kNodesPerBlock;
+  const int t = threadIdx.x % kNodesPerBlock;
+  return blockIdx.x * int64_t(nodes_per_block(kWide)) + (kWide ? t / kFan : t);
+}
+// centre of a node's items, item(c) = the c-th (w = -inf past the last): kWide,
+// all lanes call it and the first of each group of 8 goes on
+template <bool kWide, class Item>
+__device__ __forceinline__ float4 node_centre(int k, Item item) {
+  if constexpr (kWide) {
+    return bound_ball8(item(int(threadIdx.x) & (kFan - 1)), k);
+  } else {
+    float4 W[kFan];
+#pragma unroll
+    for (int c = 0; c < kFan; ++c) W[c] = item(c);
+    return bound_ball(W, k);
+  }
 }
 
 __device__ __forceinline__ void store_near(const Tree& T, int64_t node, float4 C, float wp, float wn, float w0,
@@ -373,25 +464,32 @@ __device__ __forceinline__ void lin_add(Lin& r, const float4& P, float A) {
   if (P.w <= 0.f) r.hin = fmaxf(r.hin, v + e);
 }
 
-__device__ void sphere_leaf_node(const float4* __restrict__ items, float A, const Tree& T, int64_t L, NodePart part) {
+// (kWide: every lane of the warp calls it; live: the node exists)
+template <bool kWide>
+__device__ void sphere_leaf_node(const float4* __restrict__ items, float A, const Tree& T, int64_t L, NodePart part,
+                                 bool live = true) {
+  if (kWide && !live) L = 0;
   const int64_t b = L * kLeaf, e = min(b + kLeaf, T.nitems);
-  static_assert(kLeaf == kFan, "bound_ball takes kFan items");
-  float4 It[kFan], W[kFan];
+  static_assert(kLeaf == kFan, "a centre takes kFan items");
   const int k = int(e - b);
+  // of a small ball enclosing the balls, or for the far bound
+  const float4 C = node_centre<kWide>(k, [&](int c) {
+    float4 v = items[b + min(c, k - 1)];  // past the end: the last one again, with w = -inf
+    v.w = c < k ? (part == kNear ? fabsf(v.w) : -fabsf(v.w)) : -INFINITY;
+    return v;
+  });
+  if (kWide && (!live || (threadIdx.x & (kFan - 1)))) return;
+  // (a repeated last item changes no maximum below)
+  float4 It[kFan];
   float3 mn = make_float3(INFINITY, INFINITY, INFINITY), mx = make_float3(-INFINITY, -INFINITY, -INFINITY);
 #pragma unroll
   for (int c = 0; c < kFan; ++c) {
-    const float4 v = It[c] = items[b + min(c, k - 1)];  // past the end: the last one again, with w = -inf in W
+    const float4 v = It[c] = items[b + min(c, k - 1)];
     mn.x = fminf(mn.x, v.x); mn.y = fminf(mn.y, v.y); mn.z = fminf(mn.z, v.z);
     mx.x = fmaxf(mx.x, v.x); mx.y = fmaxf(mx.y, v.y); mx.z = fmaxf(mx.z, v.z);
-    const float w = part == kNear ? fabsf(v.w) : -fabsf(v.w);
-    W[c] = make_float4(v.x, v.y, v.z, c < k ? w : -INFINITY);
   }
   const float4 lo = make_float4(nextafterf(mn.x, -INFINITY), nextafterf(mn.y, -INFINITY), nextafterf(mn.z, -INFINITY), 0.f);
   const float4 hi = make_float4(nextafterf(mx.x, INFINITY), nextafterf(mx.y, INFINITY), nextafterf(mx.z, INFINITY), 0.f);
-  // of a small ball enclosing the balls, or for the far bound
-  // (a repeated last item changes no maximum below)
-  const float4 C = bound_ball(W, k);
   if (part == kNear) {
     T.lo[L] = lo;
     T.hi[L] = hi;
@@ -429,24 +527,31 @@ __device__ void sphere_leaf_node(const float4* __restrict__ items, float A, cons
   lin_store(T, L, r);
 }
 
-__device__ void sphere_level_node(const Tree& T, float A, int level, int64_t j, NodePart part) {
+template <bool kWide>
+__device__ void sphere_level_node(const Tree& T, float A, int level, int64_t j, NodePart part, bool live = true) {
+  if (kWide && !live) j = 0;
   const int64_t child_off = T.offset[level - 1], nchild = T.count[level - 1], off = T.offset[level];
   const int64_t b = j * kFan, e = min(b + kFan, nchild);
+  const int k = int(e - b);
+  const float4 C = node_centre<kWide>(k, [&](int u) {
+    // a ball around the child that holds all its spheres, or its far bound
+    const int64_t c = child_off + b + min(u, k - 1);
+    float4 v = part == kNear ? T.na[c] : T.nf[c];
+    if (part == kNear) v.w = fmaxf(v.w, T.nb[c].z);
+    if (u >= k) v.w = -INFINITY;
+    return v;
+  });
+  if (kWide && (!live || (threadIdx.x & (kFan - 1)))) return;
   float4 L = make_float4(INFINITY, INFINITY, INFINITY, 0.f), H = make_float4(-INFINITY, -INFINITY, -INFINITY, 0.f);
   float4 W[kFan];
-  const int k = int(e - b);
 #pragma unroll
   for (int u = 0; u < kFan; ++u) {
     const int64_t c = child_off + b + min(u, k - 1);
     const float4 a = T.lo[c], z = T.hi[c];
     L.x = fminf(L.x, a.x); L.y = fminf(L.y, a.y); L.z = fminf(L.z, a.z);
     H.x = fmaxf(H.x, z.x); H.y = fmaxf(H.y, z.y); H.z = fmaxf(H.z, z.z);
-    // a ball around the child that holds all its spheres, or its far bound
-    W[u] = part == kNear ? T.na[c] : T.nf[c];
-    if (part == kNear) W[u].w = fmaxf(W[u].w, T.nb[c].z);
-    if (u >= k) W[u].w = -INFINITY;
+    W[u] = make_float4(0.f, 0.f, 0.f, 0.f);
   }
-  const float4 C = bound_ball(W, k);
   // radii through the children (|p - C| <= |p - C_c| + |C_c - C|)
   if (part == kNear) {
     T.lo[off + j] = L;
@@ -498,9 +603,10 @@ __device__ void sphere_level_node(const Tree& T, float A, int level, int64_t j, 
   lin_store(T, off + j, r);
 }
 
+template <bool kWide>
 __global__ void __launch_bounds__(kNodeBlock) k_sphere_leaves(const float4* __restrict__ items, float A, Tree T) {
-  const int64_t L = node_of_thread();
-  if (L < T.count[0]) sphere_leaf_node(items, A, T, L, node_part());
+  const int64_t L = node_of_thread<kWide>();
+  if (kWide || L < T.count[0]) sphere_leaf_node<kWide>(items, A, T, L, node_part(), L < T.count[0]);
 }
 
 // items of node j at `level`: [j * span, (j + 1) * span), span = kLeaf * kFan^level
@@ -510,9 +616,10 @@ __host__ __device__ inline int64_t level_span(int level) {
   return span;
 }
 
+template <bool kWide>
 __global__ void __launch_bounds__(kNodeBlock) k_sphere_level(float A, Tree T, int level) {
-  const int64_t j = node_of_thread();
-  if (j < T.count[level]) sphere_level_node(T, A, level, j, node_part());
+  const int64_t j = node_of_thread<kWide>();
+  if (kWide || j < T.count[level]) sphere_level_node<kWide>(T, A, level, j, node_part(), j < T.count[level]);
 }
 
 // Tightening of the internal radii, pass 1: one thread per sphere; at every
@@ -632,7 +739,6 @@ __global__ void k_gather_points(const float4* __restrict__ src, const int* __res
   dst[i] = src[order[i]];
 }
 
-constexpr unsigned kFull = 0xffffffffu;
 
 // sum of v over the active lanes of the warp, added once to *dst
 __device__ __forceinline__ void warp_count(unsigned long long* dst, unsigned long long v) {
@@ -1206,10 +1312,16 @@ cudaError_t launch_build_tree(const float4* items, int is_sphere, float A, Tree&
                               cudaStream_t st) {
   if (T.nlevels == 0) return cudaSuccess;
   if (is_sphere) {
-    k_sphere_leaves<<<nblk(T.count[0], kNodesPerBlock), kNodeBlock, 0, st>>>(items, A, T);
-    ++g_launches;
-    for (int l = 1; l < T.nlevels; ++l) {
-      k_sphere_level<<<nblk(T.count[l], kNodesPerBlock), kNodeBlock, 0, st>>>(A, T, l);
+    for (int l = 0; l < T.nlevels; ++l) {
+      const bool wide = wide_nodes(T.count[l]);
+      const unsigned g = nblk(T.count[l], nodes_per_block(wide));
+      if (l == 0) {
+        if (wide) k_sphere_leaves<true><<<g, kNodeBlock, 0, st>>>(items, A, T);
+        else k_sphere_leaves<false><<<g, kNodeBlock, 0, st>>>(items, A, T);
+      } else {
+        if (wide) k_sphere_level<true><<<g, kNodeBlock, 0, st>>>(A, T, l);
+        else k_sphere_level<false><<<g, kNodeBlock, 0, st>>>(A, T, l);
+      }
       ++g_launches;
     }
     if (scratch && T.nlevels > 1) {
