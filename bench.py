@@ -935,8 +935,8 @@ def run_gfs(args):
                "host_numa_node": numa[0] if numa else None}
 
     # ---- roofline of the dominant kernel --------------------------------------
-    # k_query_spheres, the first of the query's two FP32 kernels (the pass
-    # over the spheres); its duration comes from the library's events around
+    # k_query_spheres, the first of the query's three passes (over the
+    # spheres, with the launch for the packets it gave up); its duration comes from the library's events around
     # it on the stream it is launched on
     last = phases[-1]
     q_sph = float(np.mean([ph_["ms_query_spheres"] for ph_ in phases]))

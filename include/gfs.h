@@ -125,8 +125,8 @@ int gfs_build(gfs_ctx* ctx, const double* p_xyz, const double* s, int64_t n);
  * argmin_out:device, m int64 (nullable): candidate id or sphere index, per code.
  * flags_out: device, m uint16 result words (nullable).
  * Runs as three kernels (the pass over the spheres, the pass over the
- * survivors, the decisions with their exact re-evaluations; each with a
- * second launch for the points it listed) plus, for points outside the FP32
+ * survivors, the decisions with their exact re-evaluations; from 24,576 points
+ * each with a second launch for the points that it left) plus, for points outside the FP32
  * error model's coordinate range, the FP64 kernel.  Grows library-owned
  * scratch when m grows (Morton keys and order, 64 B of state per point).
  * No host synchronisation.
@@ -449,9 +449,9 @@ int gfs_batch_rebuild(gfs_ctx* ctx);
  * Errors: GFS_ERR_ARG (null), GFS_ERR_STATE (no batch build), GFS_ERR_CUDA. */
 int gfs_batch_status(gfs_ctx* ctx, unsigned* status_host);
 
-/* Queries of every shape of the last gfs_batch_build in two persistent
- * launches (the sphere pass of every point, then the rest), into each
- * shape's outputs.  Issues no host synchronisation and no
+/* Queries of every shape of the last gfs_batch_build in three persistent
+ * launches (the sphere pass of every point, the survivor pass, the
+ * decisions), into each shape's outputs.  Issues no host synchronisation and no
  * allocation, so it can be captured in a CUDA graph and replayed (with new
  * point coordinates written into the same buffers).
  * Errors: GFS_ERR_STATE (no batch build), GFS_ERR_CUDA. */
@@ -488,13 +488,13 @@ typedef struct {
   /* phase times of the last build / query in ms (timing = 1 only, else 0) */
   double ms_build_total;       /* whole gfs_build */
   double ms_build_cull;        /* candidate culling kernel */
-  double ms_query_fast;        /* FP32 query kernel */
+  double ms_query_fast;        /* the query's three passes */
   double ms_query_exact;       /* FP64 kernel for queries outside the FP32 error model */
   int64_t kernel_launches;     /* kernels this library has launched in this process (cumulative) */
   int64_t sort_calls;          /* radix-sort calls (each launches a few library-sort kernels) */
   int64_t cull_node_tests;     /* child-node coverage tests of the last build (sum over open candidates) */
   int64_t cull_items;          /* sphere coverage tests of the last build (sum over open candidates) */
-  double ms_query_spheres;     /* first of the query's two FP32 kernels (the pass over the spheres); part of
+  double ms_query_spheres;     /* first of the query's three passes (over the spheres); part of
                                   ms_query_fast (timing = 1 only) */
   int64_t insert_rounds;       /* rounds of the last gfs_insert / gfs_insert_known call */
   int64_t insert_steps;        /* steps it committed (its T) */
@@ -513,7 +513,7 @@ typedef struct {
   int64_t batch_sphere_items;  /* (point, sphere) tests of the last gfs_batch_query */
   int64_t batch_sphere_node_tests; /* its child-node bound tests of the sphere pass */
   int64_t batch_surv_items;    /* its (point, survivor) tests */
-  int64_t batch_cull_tile[3];  /* cull tile (spheres per block) of the batch's shapes with < 32k,
+  int64_t batch_cull_tile[3];  /* cull tile (spheres per warp, always 32) of the batch's shapes with < 32k,
                                   < 256k and more samples (0: no such shape) */
   int64_t batch_query_grid;    /* autotuned grid of the persistent batched query (blocks) */
 } gfs_stats_t;

@@ -457,7 +457,7 @@ int reset_cull_counters(gfs_ctx* c, cudaStream_t st) {
 int cull_reserve(gfs_ctx* c, CullBufs& b, int64_t tiles) {
   const int KH = cull_kept(c->KH, tiles);
   const int64_t last = c->K - KH;  // directions of the last level(s), the largest group
-  const int64_t per = c->K * (int64_t(kCullTileSpheres) * 4 + int64_t(sizeof(uint2)));
+  const int64_t per = c->K * (int64_t(kCullTileSpheres) * 4 + int64_t(sizeof(unsigned long long)));
   int64_t want = cull_chunk(tiles, per, INT64_MAX);
   if (b.chunk < want) {
     size_t free_bytes = 0, total = 0;
@@ -468,7 +468,7 @@ int cull_reserve(gfs_ctx* c, CullBufs& b, int64_t tiles) {
   return shrink_until(std::max(want, b.chunk), GFS_ERR_OOM, [&](int64_t chunk) {
     int r = ensure(b.hint, size_t(chunk) * std::max(1, KH) * kCullTileSpheres * 4);
     if (r == GFS_OK) r = ensure(b.list, size_t(chunk) * size_t(last) * kCullTileSpheres * 4);
-    if (r == GFS_OK) r = ensure(b.groups, size_t(chunk) * size_t(c->K) * sizeof(uint2));
+    if (r == GFS_OK) r = ensure(b.groups, size_t(chunk) * size_t(c->K) * sizeof(unsigned long long));
     if (r == GFS_OK) r = ensure(b.count, size_t(cull_launches(KH, tiles, chunk)) * 2 * sizeof(unsigned));
     if (r == GFS_OK) b.chunk = chunk;
     else release(b);
@@ -478,7 +478,7 @@ int cull_reserve(gfs_ctx* c, CullBufs& b, int64_t tiles) {
 
 // what cull_reserve left (nothing is allocated here: a batch rebuild may be captured)
 CullWork cull_work(const CullBufs& b) {
-  return CullWork{b.hint.as<int>(), b.list.as<uint32_t>(), b.groups.as<uint2>(), b.count.as<unsigned>(), b.chunk};
+  return CullWork{b.hint.as<int>(), b.list.as<uint32_t>(), b.groups.as<unsigned long long>(), b.count.as<unsigned>(), b.chunk};
 }
 
 // a2: inputs copied, counters cleared, sphere hierarchy built

@@ -4,7 +4,7 @@
 // each shape owns a contiguous range; every shape gets its own implicit
 // hierarchy inside shared node arrays (a forest).  The hot kernels are
 // sized for uneven shapes: the cull's tiles are numbered through all shapes, the
-// query is a fixed grid of warps that pull work items -- (shape, 32
+// query is a fixed grid of warps that pull work items -- (shape, packet of
 // query points) -- from a global counter.
 // Each shape is seen through a per-shape argument block ("view") whose
 // pointers are offset to the shape's range and whose indices are local, so

@@ -59,7 +59,7 @@ struct CullSource {
   int* hint;          // tiles x KH x 32 words
   uint32_t* list;     // open candidates: ((tile in the chunk) * (k1 - k0) + k - k0) * 32 + lane
   unsigned* count;    // entries of the list, and the walk's cursor
-  uint2* groups;      // dense groups: (tile in the chunk) * K + k, mask of the lanes
+  unsigned long long* groups;  // dense groups: (tile in the chunk) * K + k, and below the mask of the lanes
   unsigned* gcount;   // their number, and the cursor
   int k0, k1, KH, K;
   bool few;           // few tiles: every open candidate goes to the groups
@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(128) k_cull_test(const __grid_constant__ CullA
       if (lane == 0) at = atomicAdd(s.gcount, unsigned(__popc(dense)));
       at = __shfl_sync(kFull, at, 0) + __popc(dense & ((1u << lane) - 1u));
       if ((dense >> lane) & 1u) {
-        s.groups[at] = make_uint2(uint32_t(t) * uint32_t(a.K) + uint32_t(kb + lane), mine);
+        s.groups[at] = (unsigned long long)(uint32_t(t) * uint32_t(a.K) + uint32_t(kb + lane)) << 32 | mine;
         mine = 0;
       }
     }
@@ -269,10 +269,10 @@ __global__ void __launch_bounds__(128) k_cull_groups(const __grid_constant__ Cul
       if (lane == 0) t = atomicAdd(s.gcount + 1, 1u);
       t = __shfl_sync(kFull, t, 0);
       if (t >= 32u * groups) break;
-      const uint2 g = s.groups[t >> 5];
-      const int src = int(t & 31u), k = int(g.x % K);
-      if (!((g.y >> src) & 1u)) continue;
-      const CullTile tile = cull_tile(one, s, g.x / K);
+      const unsigned long long g = s.groups[t >> 5];
+      const int src = int(t & 31u), k = int(uint32_t(g >> 32) % K);
+      if (!((uint32_t(g) >> src) & 1u)) continue;
+      const CullTile tile = cull_tile(one, s, uint32_t(g >> 32) / K);
       cnt = tile.a->cnt;
       load_levels(tile.a->tree, C, lane);
       const int j = cull_walk_one(*tile.a, tile.base + src, k, C, stk, lane, rechecks, n_nodes, n_items);
@@ -283,10 +283,10 @@ __global__ void __launch_bounds__(128) k_cull_groups(const __grid_constant__ Cul
     if (lane == 0) t = atomicAdd(s.gcount + 1, 1u);
     t = __shfl_sync(kFull, t, 0);
     if (t >= groups) break;
-    const uint2 g = s.groups[t];
-    bool open = (g.y >> lane) & 1u;
-    const int k = int(g.x % K);
-    const CullTile tile = cull_tile(one, s, g.x / K);
+    const unsigned long long g = s.groups[t];
+    bool open = (uint32_t(g) >> lane) & 1u;
+    const int k = int(uint32_t(g >> 32) % K);
+    const CullTile tile = cull_tile(one, s, uint32_t(g >> 32) / K);
     const CullArgs& a = *tile.a;
     cnt = a.cnt;
     if (loaded != tile.a) {

@@ -457,7 +457,7 @@ __device__ bool near_pass(const QueryArgs& a, int64_t first, SpWarp& S, int lane
   return true;
 }
 
-// The decisions of one packet (32 points, or one), from the state of the two
+// The decisions of one packet (or one point), from the state of the two
 // passes before it: FP64 winners, value, flags, outputs.  Points outside the
 // coordinate range of the FP32 error model go to the FP64 kernel through
 // a.defer, or (kInlineExact) are evaluated in place.  false: nothing written,

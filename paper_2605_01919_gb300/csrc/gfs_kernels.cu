@@ -880,7 +880,7 @@ namespace gfs {
 // 10.0 / 12.6 ms); few points want less, for the sake of the last packets (100k
 // on 32^3, both passes after the spheres: 1.16 / 0.60 / 0.54 / 0.50 ms).
 constexpr float kJump = 6.f;
-// Fewer points than packet_size's table wants (m < n, m < 3 n) are sparse: a
+// Fewer points than that table wants (m < n, m < 3 n) are sparse: a
 // packet of uniform ones spans several spacings of the samples and is better
 // taken point by point, but points in a cluster, on a slice or in one place are
 // as close as dense ones.  So a packet whose radius is below kClose spacings of

@@ -224,7 +224,7 @@ cudaError_t launch_gather_points(const float4* src, const int* order, int64_t n,
 struct CullWork {
   int* hint;
   uint32_t* list;
-  uint2* groups;
+  unsigned long long* groups;
   unsigned* count;
   int64_t chunk;  // tiles per chunk
 };

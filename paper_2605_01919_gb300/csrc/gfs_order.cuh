@@ -2,7 +2,9 @@
 // routines.  A cell is sampled at sub^3 regularly spaced points (the centres
 // of a sub x sub x sub split of the cell) and each point is tested for
 // containment in the balls of the current samples, shrunk by tol -- the
-// coverage predicate of the cull, decided in FP64.
+// coverage predicate of the cull, decided in FP64.  (cell_cover_count runs in
+// the host build alone, as the tests' form of the count; the kernel, a block per
+// cell with FP32 screens, is in gfs_order.cu.)
 #pragma once
 
 #include "gfs_tangent.cuh"

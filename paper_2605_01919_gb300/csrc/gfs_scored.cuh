@@ -21,9 +21,13 @@
 // no candidate is valid keep the plain query's result, flagged
 // GFS_FLAG_SCORE_FALLBACK; SAMPLE and INVALID results are kept.
 //
-// One thread per point (Morton order), every decision in FP64 with each
-// operation rounded on its own in the order written; node and item screens in
-// FP32 with a bound on their rounding error only skip what cannot matter.
+// Every decision is in FP64 with each operation rounded on its own in the order
+// written; node and item screens in FP32 with a bound on their rounding error
+// only skip what cannot matter.  The kernel (one warp per point) is
+// warp_scored_one in gfs_scored_warp.cuh, which shares try_candidate, the frame
+// and the ranking with this file; Budget, walk_survivors and scored_one, the
+// same search on one thread, run in the host build alone, where the tests hold
+// the shared routines and the order of the search against the oracle.
 #pragma once
 
 #include <climits>

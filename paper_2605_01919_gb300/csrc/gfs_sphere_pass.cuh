@@ -19,19 +19,21 @@
 // and no containing ball of any point of the packet.  Only the spheres that
 // pass are evaluated per point, from a queue in shared memory.
 //
-// What bounds it: instruction issue (63% of the slots on 253^3 points over a
-// 64^3 union grid, 16 warps resident).  One node test costs the packet one
-// lane instead of 32, and the reference makes the first test already sharp.
+// What bounds it: instruction issue (72% of the slots on 253^3 points over a
+// 64^3 union grid, 36% of the warps resident).  One node test costs the packet
+// one lane instead of 32, and the reference makes the first test already sharp.
 // The walk it replaces tested every node and sphere on every lane, with
 // thresholds found on the way: 81.1 ms on that workload (104k warp
-// instructions per 32 points) against 30.6 ms, 106 against 40 ms for 2.1M
+// instructions per 32 points) against 21.5 ms, 106 against 40 ms for 2.1M
 // random points on a 96^3 torus grid, 2.86 ms against 0.028 ms for 257 random
 // points on a 32^3 grid, where 32 scattered points shared one walk.
 #pragma once
 
 namespace gfs {
 
-constexpr int kSpStack = 448;  // (walk_take keeps within it; 4 popped, at most 32 pushed, deepest level on top, it holds kFan + 28 a level)
+// (walk_take keeps within it; 4 popped and at most 32 pushed a round, the deepest
+// level on top, it holds kFan + 28 entries a level)
+constexpr int kSpStack = 448;
 constexpr int kSpQueue = 64;
 constexpr int kCand = 8;
 
