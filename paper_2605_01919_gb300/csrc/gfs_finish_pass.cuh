@@ -16,7 +16,7 @@
 // gathers before all lanes evaluate theirs together.
 //
 // What bounds it: instruction issue in the walks, the FP64 units in the
-// decisions (41% busy on the union grid).  Both together, against a walk per
+// decisions (70% busy on the union grid).  Both together, against a walk per
 // point with box and ball bounds: 22.3 against 48.6 ms (16.2M points, 64^3
 // union), 10.8 against 55.4 (2.1M random points, 96^3 torus), 0.59 against 8.4
 // (32k random points, 64^3), 0.055 against 1.85 (257 points, 32^3).
