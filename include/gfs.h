@@ -339,7 +339,8 @@ int gfs_sphere_uncovered(gfs_ctx* ctx, uint8_t* out, double* witness);
  * doubles per point.  counts_host (host, 3 int64): the numbers of circles
  * and points, and a status word (bit 0: a circle's certificate outgrew 512
  * members and the circle was taken as uncovered).  Synchronises the
- * context's stream and allocates scratch on the device.
+ * context's stream and allocates scratch on the device (lists for 2 entries a
+ * sphere, up to 151 MB before the counts are known; less if refused).
  * Errors: GFS_ERR_STATE (no build), GFS_ERR_ARG (null pointers, negative
  * capacities, or counts above the capacities: counts_host still set, nothing
  * written), GFS_ERR_TOO_LARGE (2^31 entries or more), GFS_ERR_CUDA. */

@@ -728,10 +728,24 @@ int ud_compute(gfs_ctx* c) {
   int64_t cap_c = std::max({int64_t(1) << 17, 2 * c->n, std::min(int64_t(hpairs), int64_t(1) << 21)}), cap_p = cap_c;
   unsigned long long hc[2] = {0, 0};
   unsigned hstatus = 0;
+  auto reserve = [&](int64_t circles, int64_t points) {
+    int r = ensure(c->ud_circ, size_t(circles) * 16);
+    if (r == GFS_OK) r = ensure(c->ud_quad, size_t(points) * 32);
+    if (r == GFS_OK) r = ensure(c->ud_pts, size_t(points) * 24);
+    if (r != GFS_OK)
+      for (DevBuf* b : {&c->ud_circ, &c->ud_quad, &c->ud_pts}) release(*b);
+    return r;
+  };
   for (int pass = 0; pass < 2; ++pass) {
-    GFS_TRY(ensure(c->ud_circ, size_t(cap_c) * 16));
-    GFS_TRY(ensure(c->ud_quad, size_t(cap_p) * 32));
-    GFS_TRY(ensure(c->ud_pts, size_t(cap_p) * 24));
+    // (a guess that the device refuses is halved)
+    if (pass == 0) {
+      GFS_TRY(shrink_until(cap_c, GFS_ERR_OOM, [&](int64_t cap) {
+        cap_c = cap_p = cap;
+        return reserve(cap, cap);
+      }));
+    } else {
+      GFS_TRY(reserve(cap_c, cap_p));
+    }
     GFS_CK(cudaMemsetAsync(c->ud_cnt.p, 0, 32, st));
     exact::UDOut o{c->ud_cnt.as<unsigned long long>(), cap_c, cap_p, c->ud_circ.as<int64_t>(), c->ud_quad.as<int64_t>(),
                    c->ud_pts.as<double>(), reinterpret_cast<unsigned*>(c->ud_cnt.as<unsigned long long>() + 2)};
